@@ -305,15 +305,11 @@ def _config(w, args):
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none
 #       -k regex:<kernels> -s <2 steps of them> -c <1 step of them> --csv
 #       python bench.py --steps 2 --warmup 3 --no-cpu-baseline --one-form --no-extra
-# (the suffix with regex 'mlp_tc_ws|eloc_assemble|js_hist'; the slot launches,
-# connected set, assembly and partial sum with
-# 'connected_diag|mlp_tc_slots|eloc_assemble|partial_sum'); the adjoint from
+# (the slot launches and the partial sum with 'mlp_tc_slots|partial_sum'); the adjoint from
 # `ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum
 # --clock-control none -c 80 --csv python bench.py --kernel-case`.  A kernel
 # changed since its capture has no entry (traffic null).
-TRAFFIC = {("h2o", "bf16"): {"mlp_tc_suffix_kernel": 1327104, "mlp_tc_parent_kernel": 660480,
-                             "mlp_tc_slot_kernel": 663808, "mlp_tc_grad_kernel": 609792,
-                             "eloc_assemble_kernel": 4674560, "connected_kernel": 64512,
+TRAFFIC = {("h2o", "bf16"): {"mlp_tc_slot_kernel": 663808, "mlp_tc_grad_kernel": 609792,
                              "grad_partial_sum_kernel": 4014336}}
 
 
@@ -715,8 +711,8 @@ def _batch32(args, dev, quick=False):
             extra["autotuner"] = {"times_ms": {nm: round(v, 4) for nm, v in zip(names, t)},
                                   "chosen": {"mode": "static" if mode == _lib.ANQS_BATCH_STATIC else "dynamic",
                                              "chunk": chunk}}
-            # roofline of the persistent amplitude launch: the suffix FLOP (with prefix
-            # reuse) of the sample sets the autotuner timed, over its fastest time
+            # roofline of the persistent amplitude launch: the FLOP of the distinct prefixes
+            # of the sample sets the autotuner timed, over its fastest time
             flop = 0.0
             for sp, pr in zip(specs, probs):
                 nu = int(pr.nu.item())
@@ -727,7 +723,7 @@ def _batch32(args, dev, quick=False):
             extra["roofline"] = {"kernel": "mlp_tc_multi_kernel", "bound": "tensor", "achieved": ach,
                                  "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": ach / peaks["bf16_tflops"],
                                  "traffic": None, "avg_launch_us": best * 1e3, "work_per_launch": flop,
-                                 "note": f"dense bf16 {src} burst peak; suffix FLOP with prefix reuse of the 32 "
+                                 "note": f"dense bf16 {src} burst peak; FLOP of the distinct prefixes of the 32 "
                                          "problems over the autotuner's fastest launch time"}
         bs.capture()
         for _ in range(warm):
@@ -944,62 +940,81 @@ def _compact(sub):
                                                         "vs_baseline", "data")}
 
 
+INDEX_MAX_ORB = 18  # up to here the library evaluates distinct determinants (their distinct prefixes: MLP, NADE)
+
+
+def _distinct_prefixes(A, ham, x):
+    """Distinct prefixes of p = 0..n slots among the samples and their connected determinants."""
+    u = torch.unique(torch.cat([x, A.connected(ham, x)[0].reshape(-1)]))
+    out = [0] * (ham.n + 1)
+    for p in range(ham.n, -1, -1):
+        u = torch.unique(u & ((1 << (2 * p)) - 1))
+        out[p] = u.numel()
+    return np.array(out, dtype=np.float64)
+
+
+def _eloc_bytes(n_x, K):
+    """Local-energy assembly: per connected determinant a rank word, an amplitude and an integral, 8 bytes each."""
+    return 24.0 * n_x * K
+
+
 def _tf_work(A, ham, w, x):
     """Algorithmic FLOP per step of the transformer families for the sample
     set x.  One (sequence, position t) row costs f(t) = L (24 d^2 + 4 (t+1) d)
     + 16 d: the q|k|v, output and FFN projections, the attention scores and
-    weighted sum over the t+1 keys, and the head.  suffix = positions > j(x')
-    of every connected x'; parent = every position of every sample; slot
+    weighted sum over the t+1 keys, and the head.  suffix = every position of
+    every distinct determinant (beyond INDEX_MAX_ORB orbitals: positions > j(x')
+    of every connected x'); parent = every position of every sample; slot
     (sampler) = positions 0..p of every distinct prefix at level p; grad =
     3 x parent (forward plus the two products of the adjoint)."""
     n, d, L = w["n"], w["d_model"], w["n_layers"]
     f = np.array([L * (24 * d * d + 4 * (t + 1) * d) + 16 * d for t in range(n)], dtype=np.float64)
     cf = np.concatenate([[0.0], np.cumsum(f)])
-    xp, hv, js, hd = A.connected(ham, x)
-    j = js.reshape(-1).cpu().numpy().astype(np.int64)
-    suffix = float((cf[n] - cf[j + 1]).sum())
     parent = float(len(x) * cf[n])
     xs = x.cpu().numpy().astype(np.uint64)
     slot = 0.0
     for p in range(n):
         pre = np.unique(xs & np.uint64((1 << (2 * p)) - 1)) if p else np.zeros(1, np.uint64)
         slot += len(pre) * cf[p + 1]
-    eloc_bytes = float((8 + 1 + 8 + 8 + 8 * (n - 1 - j)).sum())
-    return {"tf_tc_suffix_kernel": suffix, "tf_tc_parent_kernel": parent, "tf_tc_slot_kernel": slot,
-            "tf_fp32_kernel": len(j) * cf[n] + parent + slot, "tf_fp32_grad_kernels": 3.0 * parent,
-            "eloc_assemble_kernel": eloc_bytes, "connected_kernel": float(len(j) * (8 + 8 + 1) + len(x) * 8)}
+    out = {"tf_tc_parent_kernel": parent, "tf_tc_slot_kernel": slot, "tf_fp32_grad_kernels": 3.0 * parent}
+    if n <= INDEX_MAX_ORB:
+        full = _distinct_prefixes(A, ham, x)[n] * cf[n]
+        return dict(out, tf_tc_suffix_kernel=full, tf_fp32_kernel=full + slot,
+                    eloc_assemble_kernel=_eloc_bytes(len(x), ham.n_connected))
+    xp, hv, js, hd = A.connected(ham, x)
+    j = js.reshape(-1).cpu().numpy().astype(np.int64)
+    return dict(out, tf_tc_suffix_kernel=float((cf[n] - cf[j + 1]).sum()),
+                tf_fp32_kernel=len(j) * cf[n] + parent + slot,
+                eloc_assemble_kernel=float((8 + 1 + 8 + 8 + 8 * (n - 1 - j)).sum()),
+                connected_kernel=float(len(j) * (8 + 8 + 1) + len(x) * 8))
 
 
 def _tc_work(A, ham, model, w, x):
     """Algorithmic work per step for the sample set x.
 
     FLOP of one slot-p evaluation f(p) = 2 (4p W + (L-1) W^2 + 8 W).
-    suffix = sum over connected x' of f(p) for the slots p > j(x'); parent =
-    every slot of every sample; slot (sampler) = every slot of every distinct
-    prefix of the leaves (the frontier of each level); grad = 3 x parent (the
-    forward recomputed plus the two adjoint products); eloc bytes = per
-    connected x': x' 8 + j 1 + H 8 + parent cache 8 + one 8-byte term per
-    slot p > j."""
+    suffix = f(p) of every distinct prefix of p slots of the connected
+    determinants (16-bit form, up to INDEX_MAX_ORB orbitals); slot (sampler) =
+    every slot of every distinct prefix of the leaves (the frontier of each
+    level); grad = 3 x every slot of every sample (the forward recomputed plus
+    the two adjoint products)."""
     if w["kind"] == "nade":
         return _nade_work(A, ham, w, x)
     if w["kind"] != "mlp":
         return _tf_work(A, ham, w, x)
     n, W, L = w["n"], w["width"], w["n_hidden"]
     f = np.array([2 * (4 * p * W + (L - 1) * W * W + 8 * W) for p in range(n)], dtype=np.float64)
-    cf = np.concatenate([[0.0], np.cumsum(f)])  # cf[p] = sum_{q<p} f[q]
-    xp, hv, js, hd = A.connected(ham, x)
-    j = js.reshape(-1).cpu().numpy().astype(np.int64)
-    suffix = float((cf[n] - cf[j + 1]).sum())
-    parent = float(len(x) * cf[n])
+    parent = float(len(x) * f.sum())
     xs = x.cpu().numpy().astype(np.uint64)
     slot = 0.0
     for p in range(n):
         pre = np.unique(xs & np.uint64((1 << (2 * p)) - 1)) if p else np.zeros(1, np.uint64)
         slot += len(pre) * f[p]
-    eloc_bytes = float((8 + 1 + 8 + 8 + 8 * (n - 1 - j)).sum())
-    return {"mlp_tc_suffix_kernel": suffix, "mlp_tc_parent_kernel": parent, "mlp_tc_slot_kernel": slot,
-            "mlp_fp32_grad_kernel": 3.0 * parent, "mlp_tc_grad_kernel": 3.0 * parent, "eloc_assemble_kernel": eloc_bytes,
-            "connected_kernel": float(len(j) * (8 + 8 + 1) + len(x) * 8)}
+    out = {"mlp_tc_slot_kernel": slot, "mlp_fp32_grad_kernel": 3.0 * parent, "mlp_tc_grad_kernel": 3.0 * parent}
+    if n <= INDEX_MAX_ORB:
+        out["mlp_tc_suffix_kernel"] = float((_distinct_prefixes(A, ham, x)[:n] * f).sum())
+        out["eloc_assemble_kernel"] = _eloc_bytes(len(x), ham.n_connected)
+    return out
 
 
 def _nade_work(A, ham, w, x):
@@ -1008,23 +1023,20 @@ def _nade_work(A, ham, w, x):
     W2 h1 and W3 h2 at 8 FLOP per complex multiply-add, the W1 columns of
     the set bits counted as all i).  parent = the 8 values of every slot of
     every sample, f(2p) + 2 f(2p+1) per slot (qubit 2p+1 for both values of
-    qubit 2p); suffix = the path qubits 2p, 2p+1 of the slots p > j(x') of
-    every connected x'; slot (sampler) = slot p of every distinct prefix at
+    qubit 2p); suffix = the path qubits 2p, 2p+1 of every distinct prefix of
+    p + 1 slots of the connected determinants; slot (sampler) = slot p of every distinct prefix at
     level p; grad = 3 f(i) per (sample, qubit): the forward and the two
     adjoint products."""
     n, W = w["n"], w["width"]
     f = np.array([8 * W * W + 16 * W + 2 * i * W for i in range(2 * n)], dtype=np.float64)
     slot = f[0::2] + 2 * f[1::2]
     path = f[0::2] + f[1::2]
-    cpath = np.concatenate([[0.0], np.cumsum(path)])  # cpath[p] = sum_{q<p} path[q]
-    _, _, js, _ = A.connected(ham, x)
-    j = js.reshape(-1).cpu().numpy().astype(np.int64)
     xs = x.cpu().numpy().astype(np.uint64)
     samp = 0.0
     for p in range(n):
         pre = np.unique(xs & np.uint64((1 << (2 * p)) - 1)) if p else np.zeros(1, np.uint64)
         samp += len(pre) * slot[p]
-    return {"nade_parent_kernel": len(xs) * slot.sum(), "nade_suffix_kernel": float((cpath[n] - cpath[j + 1]).sum()),
+    return {"nade_parent_kernel": len(xs) * slot.sum(), "nade_suffix_kernel": float((_distinct_prefixes(A, ham, x)[1:] * path).sum()),
             "nade_slot_kernel": samp, "nade_grad_kernel": 3.0 * len(xs) * f.sum()}
 
 
@@ -1042,7 +1054,7 @@ def _rooflines(prof, work, steps, peaks, src, traffic):
         if name.startswith(("mlp_tc_", "tf_tc_")):
             bound, unit, peak = "tensor", "TFLOP/s", peaks["bf16_tflops"]
             ach = per_launch / avg_s / 1e12
-            note = f"dense bf16 {src} burst peak; FLOP with prefix reuse"
+            note = f"dense bf16 {src} burst peak; FLOP of the distinct prefixes or rows"
         elif name in ("mlp_fp32_grad_kernel", "tf_fp32_grad_kernels", "tf_fp32_kernel") or name.startswith("nade_"):
             bound, unit, peak = "alu", "TFLOP/s", fp32_peak
             ach = per_launch / avg_s / 1e12

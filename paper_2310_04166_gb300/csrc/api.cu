@@ -118,18 +118,109 @@ int logpsi_dispatch(const anqs_model* M, const anqs_ham* H, const uint64_t* x, C
 }  // namespace anqs
 
 namespace anqs {
-// FP32 form: every connected determinant evaluated over all slots.
-static size_t eloc_plain_ws(const anqs_ham* H, uint64_t n_x, Arena& A, uint64_t** xp, double** hv,
-                            double** hd, float** la_x, float** ph_x, float** la_p, float** ph_p) {
-  uint64_t m = n_x * H->v.K;
-  *xp = A.take<uint64_t>(m);
-  *hv = A.take<double>(m);
-  *hd = A.take<double>(n_x);
-  *la_x = A.take<float>(n_x);
-  *ph_x = A.take<float>(n_x);
-  *la_p = A.take<float>(m);
-  *ph_p = A.take<float>(m);
+// FP32 form (MLP, transformer, table): the distinct connected determinants
+// (the MLP: their distinct prefixes) or, where the sector has no index or the
+// tables of all row variants would grow large, every connected determinant
+// evaluated over all slots.
+struct PlainWs {
+  UniqueWs u;                  // over distinct determinants
+  float2 *terms, *mid, *tab;   // MLP: node terms and path sums; MLP, transformer: per determinant and variant
+  float *la, *ph;              // table: per determinant; else of [n_x][K] connected determinants
+  uint64_t* xp;
+  double* hv;
+  float *la_x, *ph_x;
+  double* part;
+  uint32_t* ticket;
+};
+
+static size_t plan_plain(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique, Arena& A, PlainWs& w) {
+  w = PlainWs{};
+  const uint64_t m = n_x * H->v.K;
+  if (unique) {
+    const bool mlp = M->d.kind == ANQS_MODEL_MLP;
+    plan_unique(H, n_x, mlp, A, w.u);
+    if (mlp) {
+      const uint64_t V = mlp_fp32_variants();
+      w.terms = A.take<float2>((w.u.max_nodes - w.u.max_leaves) * V * 4);
+      w.mid = A.take<float2>(path_sums_mid(H, n_x) * V);
+      w.tab = A.take<float2>(w.u.max_leaves * V);
+    } else if (M->d.kind == ANQS_MODEL_TF) {
+      w.tab = A.take<float2>(w.u.max_leaves * tf_fp32_variants(M->tf));
+    } else {
+      w.la = A.take<float>(w.u.max_leaves);
+      w.ph = A.take<float>(w.u.max_leaves);
+    }
+    return A.off;
+  }
+  w.xp = A.take<uint64_t>(m);
+  w.hv = A.take<double>(m);
+  w.la_x = A.take<float>(n_x);
+  w.ph_x = A.take<float>(n_x);
+  w.la = A.take<float>(m);
+  w.ph = A.take<float>(m);
+  w.part = A.take<double>(eloc_partials(H, n_x));
+  w.ticket = A.take<uint32_t>(1);
   return A.off;
+}
+
+static size_t plain_ws_bytes(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique) {
+  Arena A(nullptr, 0);
+  PlainWs w;
+  return plan_plain(M, H, n_x, unique, A, w);
+}
+
+// The variants' tables take up to 1 KB per prefix (MLP): they may use twice
+// the memory of the form without them, or 1 GiB.
+static bool plain_prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  return unique_applies(H, n_x) && plain_ws_bytes(M, H, n_x, true) <=
+                                       std::max<size_t>(size_t(1) << 30, 2 * plain_ws_bytes(M, H, n_x, false));
+}
+
+int run_eloc_array(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, uint64_t* xp, double* hv,
+                   float* la_x, float* ph_x, float* la, float* ph, double* part, uint32_t* ticket, double* ere,
+                   double* eim, const uint64_t* counts, double* stats, cudaStream_t s) {
+  ANQS_CUDA(cudaMemsetAsync(ticket, 0, sizeof(uint32_t), s));
+  ANQS_TRY(launch_connected(H->v, x, n_x, xp, hv, nullptr, nullptr, s));
+  ANQS_TRY(logpsi_dispatch(M, H, x, n_x, la_x, ph_x, s));
+  ANQS_TRY(logpsi_dispatch(M, H, xp, scaled(n_x, H->v.K), la, ph, s));
+  AmpSrc amp{};
+  amp.mode = AMP_ARRAY;
+  amp.la = la;
+  amp.ph = ph;
+  amp.la_x = la_x;
+  amp.ph_x = ph_x;
+  return launch_eloc_direct(H, x, n_x, NodeView{}, amp, ere, eim, part, StatsOut{counts, stats, ticket}, s);
+}
+
+static int run_eloc_plain(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere,
+                          double* eim, const uint64_t* counts, double* stats, void* ws, size_t ws_bytes,
+                          cudaStream_t s) {
+  const bool unique = use_unique(H, plain_prefers_unique(M, H, n_x.n), plain_ws_bytes(M, H, n_x.n, false),
+                                 H->has_index ? plain_ws_bytes(M, H, n_x.n, true) : 0, ws_bytes);
+  Arena A(ws, ws_bytes);
+  PlainWs w;
+  plan_plain(M, H, n_x.n, unique, A, w);
+  if (!A.fits() || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+  if (!unique)
+    return run_eloc_array(M, H, x, n_x, w.xp, w.hv, w.la_x, w.ph_x, w.la, w.ph, w.part, w.ticket, ere, eim, counts,
+                          stats, s);
+  ANQS_TRY(launch_unique(H, x, n_x, w.u, s));
+  AmpSrc amp{};
+  amp.mode = AMP_SUM;
+  amp.tab = w.tab;
+  if (M->d.kind == ANQS_MODEL_MLP) {
+    amp.variants = mlp_fp32_variants();
+    ANQS_TRY(launch_mlp_fp32_nodes(M->mlp, H->v, w.u.nodes, w.u.max_nodes - w.u.max_leaves, w.terms, s));
+    ANQS_TRY(launch_path_sums(H, w.u, w.terms, w.mid, w.tab, s, amp.variants));
+  } else if (M->d.kind == ANQS_MODEL_TF) {
+    amp.variants = tf_fp32_variants(M->tf);
+    ANQS_TRY(launch_tf_fp32_variants(M->tf, H->v, unique_leaf_x(H, w.u), unique_leaves(w.u), w.tab, s));
+  } else {
+    amp.la = w.la;
+    amp.ph = w.ph;
+    ANQS_TRY(logpsi_dispatch(M, H, unique_leaf_x(H, w.u), unique_leaves(w.u), w.la, w.ph, s));
+  }
+  return launch_eloc_direct(H, x, n_x, w.u.nodes, amp, ere, eim, w.u.part, StatsOut{counts, stats, w.u.ticket}, s);
 }
 }  // namespace anqs
 
@@ -292,6 +383,74 @@ static int build_prefix_table(anqs_ham* H) {
   return ANQS_OK;
 }
 
+// Ranks of the sector's prefixes (SectorView) for up to IDX_MAX_ORB orbitals
+// and 2^30 determinants, and the list of all prefixes when levels 0..n-1 hold
+// at most kPrefixTable of them and level n at most four times that.
+static int build_index(anqs_ham* H) {
+  const int n = H->v.n;
+  if (n > IDX_MAX_ORB) return ANQS_OK;
+  SectorView& sv = H->sv;
+  sv.n = n;
+  std::vector<uint32_t> tab[2], str[2];  // rank tables, strings
+  for (int s = 0; s < 2; ++s) {
+    const int ne = s ? H->v.nb : H->v.na;
+    tab[s].assign(size_t(2) << n, 0u);
+    for (int p = 0; p <= n; ++p) {
+      (s ? sv.sob : sv.soa)[p] = uint32_t(str[s].size());
+      uint32_t r = 0;
+      for (uint32_t v = 0; v < (1u << p); ++v) {
+        const int e = __builtin_popcount(v);
+        if (e > ne || e + (n - p) < ne) continue;
+        tab[s][(size_t(1) << p) + v] = r++;
+        str[s].push_back(v);
+      }
+      (s ? sv.nb_p : sv.na_p)[p] = r;
+    }
+  }
+  uint64_t words = 0, below = 0;
+  for (int p = 0; p <= n; ++p) {
+    sv.woff[p] = uint32_t(words);
+    const uint64_t c = uint64_t(sv.na_p[p]) * sv.nb_p[p];
+    if (c > (1ull << 30)) return ANQS_OK;
+    words += (c + 31) / 32;
+    if (p < n) below += c;
+  }
+  sv.woff[n + 1] = uint32_t(words);
+  const uint64_t leaves = uint64_t(sv.na_p[n]) * sv.nb_p[n];
+  std::vector<uint32_t> all;
+  for (int s = 0; s < 2; ++s) all.insert(all.end(), tab[s].begin(), tab[s].end());
+  const size_t st0 = all.size();
+  for (int s = 0; s < 2; ++s) all.insert(all.end(), str[s].begin(), str[s].end());
+  ANQS_CUDA(cudaMalloc(&H->d_idx, all.size() * sizeof(uint32_t)));
+  ANQS_CUDA(cudaMemcpy(H->d_idx, all.data(), all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+  sv.rka = H->d_idx;
+  sv.rkb = H->d_idx + tab[0].size();
+  sv.sta = H->d_idx + st0;
+  sv.stb = sv.sta + str[0].size();
+  H->has_index = true;
+  if (below > kPrefixTable || leaves > 4 * kPrefixTable) return ANQS_OK;
+  auto spread = [](uint32_t v) {
+    uint64_t x = 0;
+    for (int i = 0; i < 32; ++i) x |= uint64_t((v >> i) & 1u) << (2 * i);
+    return x;
+  };
+  std::vector<uint64_t> xs;
+  for (int p = 0; p <= n; ++p) {
+    H->full_off.push_back(uint32_t(xs.size()));
+    for (uint32_t a = 0; a < sv.na_p[p]; ++a)
+      for (uint32_t b = 0; b < sv.nb_p[p]; ++b)
+        xs.push_back(spread(str[0][sv.soa[p] + a]) | spread(str[1][sv.sob[p] + b]) << 1);
+  }
+  H->full_off.push_back(uint32_t(xs.size()));
+  ANQS_CUDA(cudaMalloc(&H->d_full_x, xs.size() * sizeof(uint64_t)));
+  ANQS_CUDA(cudaMemcpy(H->d_full_x, xs.data(), xs.size() * sizeof(uint64_t), cudaMemcpyHostToDevice));
+  ANQS_CUDA(cudaMalloc(&H->d_full_off, H->full_off.size() * sizeof(uint32_t)));
+  ANQS_CUDA(cudaMemcpy(H->d_full_off, H->full_off.data(), H->full_off.size() * sizeof(uint32_t),
+                       cudaMemcpyHostToDevice));
+  H->has_full = true;
+  return ANQS_OK;
+}
+
 extern "C" {
 
 const char* anqs_version(void) { return "anqs 0.1 (sm_103a)"; }
@@ -358,7 +517,7 @@ int anqs_hamiltonian_create(anqs_ham** out, int n, int na, int nb, const double*
   v.g = H->d_g;
   v.mask = H->d_mask;
   v.mu_lv = n;
-  if (build_prefix_table(H) != ANQS_OK) {
+  if (build_prefix_table(H) != ANQS_OK || build_index(H) != ANQS_OK) {
     anqs_hamiltonian_destroy(H);
     return ANQS_ERR_CUDA;
   }
@@ -414,6 +573,9 @@ int anqs_hamiltonian_destroy(anqs_ham* H) {
   cudaFree(H->d_pt_x);
   cudaFree(H->d_pt_child);
   cudaFree(H->d_status);
+  cudaFree(H->d_idx);
+  cudaFree(H->d_full_x);
+  cudaFree(H->d_full_off);
   delete H;
   return ANQS_OK;
 }
@@ -719,24 +881,30 @@ int anqs_stats_combine(const double* stats_in, int world, double* stats_out, voi
 // prefix-reuse local energy: the BF16 forms and the NADE
 static bool uses_tc_eloc(const anqs_model* M) { return M->d.form == ANQS_FORM_BF16 || M->d.kind == ANQS_MODEL_NADE; }
 
-static size_t tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
-  if (M->d.kind == ANQS_MODEL_NADE) return nade_eloc_workspace(H, n_x);
-  return M->d.kind == ANQS_MODEL_TF ? tf_tc_eloc_workspace(M, H, n_x) : eloc_tc_workspace(M, H, n_x);
+static size_t eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique) {
+  if (!uses_tc_eloc(M)) return plain_ws_bytes(M, H, n_x, unique);
+  if (M->d.kind == ANQS_MODEL_NADE) return nade_eloc_workspace(H, n_x, unique);
+  return M->d.kind == ANQS_MODEL_TF ? tf_tc_eloc_workspace(M, H, n_x, unique) : eloc_tc_workspace(H, n_x, unique);
+}
+
+static bool prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  return uses_tc_eloc(M) ? unique_applies(H, n_x) : plain_prefers_unique(M, H, n_x);
 }
 
 int anqs_local_energy_workspace_size(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
   ANQS_TRY(check_pair(M, H));
   if (!bytes) return set_error(ANQS_ERR_ARG, "null output");
-  if (uses_tc_eloc(M)) {
-    *bytes = tc_eloc_workspace(M, H, n_x);
-    return ANQS_OK;
-  }
-  Arena A(nullptr, 0);
-  uint64_t* a;
-  double *b, *c;
-  float *d, *e, *f, *g;
-  *bytes = eloc_plain_ws(H, n_x, A, &a, &b, &c, &d, &e, &f, &g);
+  *bytes = eloc_workspace(M, H, n_x, prefers_unique(M, H, n_x));
   return ANQS_OK;
+}
+
+// a workspace large enough for one of the call's forms
+static int check_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, const void* ws, size_t ws_bytes) {
+  const bool pref = prefers_unique(M, H, n_x);
+  const size_t need = eloc_workspace(M, H, n_x, pref);
+  if (ws && ws_bytes >= need) return ANQS_OK;
+  if (ws && H->has_index && ws_bytes >= eloc_workspace(M, H, n_x, !pref)) return ANQS_OK;
+  return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
 }
 
 int anqs_local_energy(const anqs_model* M, const anqs_ham* H, const uint64_t* x, const uint64_t* counts,
@@ -748,29 +916,12 @@ int anqs_local_energy(const anqs_model* M, const anqs_ham* H, const uint64_t* x,
   if (counts && !stats) return set_error(ANQS_ERR_ARG, "counts given without stats output");
   cudaStream_t s = (cudaStream_t)stream;
   const Count nc{n_x, n_x_dev, 1};
-  if (uses_tc_eloc(M)) {
-    size_t need = tc_eloc_workspace(M, H, n_x);
-    if (ws_bytes < need || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
-    // the assembly kernel also writes the statistics (counts set)
-    if (M->d.kind == ANQS_MODEL_NADE) ANQS_TRY(run_eloc_nade(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s));
-    else if (M->d.kind == ANQS_MODEL_TF)
-      ANQS_TRY(run_eloc_tf_tc(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s));
-    else ANQS_TRY(run_eloc_tc(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s));
-    return ANQS_OK;
-  } else {
-    Arena A(ws, ws_bytes);
-    uint64_t* xp;
-    double *hv, *hd;
-    float *la_x, *ph_x, *la_p, *ph_p;
-    size_t need = eloc_plain_ws(H, n_x, A, &xp, &hv, &hd, &la_x, &ph_x, &la_p, &ph_p);
-    if (ws_bytes < need || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
-    ANQS_TRY(launch_connected(H->v, x, nc, xp, hv, nullptr, hd, s));
-    ANQS_TRY(logpsi_dispatch(M, H, x, nc, la_x, ph_x, s));
-    ANQS_TRY(logpsi_dispatch(M, H, xp, scaled(nc, H->v.K), la_p, ph_p, s));
-    ANQS_TRY(launch_eloc_sum(H->v, nc, hv, hd, la_x, ph_x, la_p, ph_p, ere, eim, s));
-  }
-  if (counts) ANQS_TRY(launch_stats(ere, eim, counts, nc, stats, s));
-  return ANQS_OK;
+  ANQS_TRY(check_eloc_workspace(M, H, n_x, ws, ws_bytes));
+  // the last kernel of each form also writes the statistics (counts set)
+  if (!uses_tc_eloc(M)) return run_eloc_plain(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s);
+  if (M->d.kind == ANQS_MODEL_NADE) return run_eloc_nade(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s);
+  if (M->d.kind == ANQS_MODEL_TF) return run_eloc_tf_tc(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s);
+  return run_eloc_tc(M, H, x, nc, ere, eim, counts, stats, ws, ws_bytes, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -832,9 +983,7 @@ static int check_problem(const anqs_eloc_problem& q, int device) {
   if (q.n_x == 0) return set_error(ANQS_ERR_ARG, "n_x must be >= 1");
   if (!q.x_dev || !q.eloc_re_dev || !q.eloc_im_dev) return set_error(ANQS_ERR_ARG, "null array argument");
   if (q.counts_dev && !q.stats_dev) return set_error(ANQS_ERR_ARG, "counts given without stats output");
-  size_t need = 0;
-  ANQS_TRY(anqs_local_energy_workspace_size(q.model, q.ham, q.n_x, &need));
-  if (q.workspace_bytes < need || !q.workspace_dev) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
+  ANQS_TRY(check_eloc_workspace(q.model, q.ham, q.n_x, q.workspace_dev, q.workspace_bytes));
   if (uses_tc_eloc(q.model) && q.n_x * uint64_t(q.ham->v.K) > 0xffffffffull)
     return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
   return ANQS_OK;
@@ -953,7 +1102,7 @@ int anqs_batched_local_energy(anqs_batch* b, const anqs_eloc_problem* q, int n, 
           break;
         }
         const Count nc{q[k].n_x, q[k].n_x_dev, 1};
-        r = eloc_tc_post(q[k].ham, nc, q[k].eloc_re_dev, q[k].eloc_im_dev, q[k].counts_dev, q[k].stats_dev,
+        r = eloc_tc_post(q[k].ham, q[k].x_dev, nc, q[k].eloc_re_dev, q[k].eloc_im_dev, q[k].counts_dev, q[k].stats_dev,
                          q[k].workspace_dev, q[k].workspace_bytes, sk);
         if (cudaEventRecord(b->done[k], sk) == cudaSuccess) join[k] = 2;
         else fail("event record");

@@ -254,6 +254,66 @@ __device__ __forceinline__ unsigned norm_mask(const HamView& hv, int p, unsigned
 }
 #endif
 
+// Ranks of the sector's prefixes.  A prefix of p slots is a pair of spin
+// strings (alpha, beta bits of its slots); with na_p[p] alpha and nb_p[p] beta
+// strings that can still reach the sector, prefix (a, b) of level p has the
+// index rank(a) * nb_p[p] + rank(b).  Level n holds the determinants.
+// Tables: rank of the p-bit string s at rk[(1 << p) + s], string of rank r of
+// level p at st[so[p] + r].  Z2 symmetries do not enter (they leave part of
+// the indices unused).
+constexpr int IDX_MAX_ORB = 18;
+struct SectorView {
+  int n;
+  uint32_t na_p[IDX_MAX_ORB + 1], nb_p[IDX_MAX_ORB + 1];
+  uint32_t soa[IDX_MAX_ORB + 1], sob[IDX_MAX_ORB + 1];
+  uint32_t woff[IDX_MAX_ORB + 2];  // first 32-bit word of each level in a bitmap over all levels
+  const uint32_t *rka, *rkb, *sta, *stb;
+};
+
+// Distinct prefixes ("nodes") of a call's determinants, level by level in
+// index order: node ids [off[p], off[p + 1]) are level p's.  With packed set,
+// the id of index i of level p is packed[w].y + popc of the lower bits of
+// packed[w].x, w = woff[p] + i / 32 (the node is there only if its bit is
+// set); without it every prefix of the sector is a node and the id is
+// off[p] + i.
+struct NodeView {
+  const uint64_t* x;    // [nodes] prefix bits
+  const uint32_t* off;  // [n + 2], device
+  const uint2* packed;
+};
+#ifdef __CUDACC__
+// even bits of x, packed
+__device__ __forceinline__ uint32_t even_bits(uint64_t x) {
+  x &= 0x5555555555555555ull;
+  x = (x | (x >> 1)) & 0x3333333333333333ull;
+  x = (x | (x >> 2)) & 0x0F0F0F0F0F0F0F0Full;
+  x = (x | (x >> 4)) & 0x00FF00FF00FF00FFull;
+  x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
+  x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
+  return uint32_t(x);
+}
+__device__ __forceinline__ uint64_t spread_bits(uint32_t v) {
+  uint64_t x = v;
+  x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
+  x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
+  x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
+  x = (x | (x << 2)) & 0x3333333333333333ull;
+  x = (x | (x << 1)) & 0x5555555555555555ull;
+  return x;
+}
+// index of the level-p prefix of the strings (a, b)
+__device__ __forceinline__ uint32_t prefix_index(const SectorView& sv, int p, uint32_t a, uint32_t b) {
+  const uint32_t m = (1u << p) - 1u;
+  return __ldg(sv.rka + (m + 1u) + (a & m)) * sv.nb_p[p] + __ldg(sv.rkb + (m + 1u) + (b & m));
+}
+__device__ __forceinline__ uint32_t node_id(const SectorView& sv, const NodeView& nv, int p, uint32_t idx) {
+  // through L2: both may have been written by the kernel just before
+  if (!nv.packed) return __ldcg(nv.off + p) + idx;
+  const uint2 w = __ldcg(nv.packed + sv.woff[p] + (idx >> 5));
+  return w.y + uint32_t(__popc(w.x & ((1u << (idx & 31u)) - 1u)));
+}
+#endif
+
 // Cotangents of an adjoint: the given arrays cl, cp (log|psi|, arg psi per
 // row), or, when stats is set, those of the VMC gradient computed per row:
 // 2 (n_l / S) Re(E_loc,l - E) and 2 (n_l / S) Im(E_loc,l - E).
@@ -328,6 +388,14 @@ struct anqs_ham {
   std::vector<int32_t> pt_child;
   uint64_t* d_pt_x;
   int32_t* d_pt_child;
+  // Prefix ranks (null tables: too many orbitals or determinants) and, for
+  // small sectors, the list of all prefixes with its level offsets
+  bool has_index = false, has_full = false;
+  SectorView sv{};
+  uint32_t* d_idx = nullptr;        // rank and string tables
+  uint64_t* d_full_x = nullptr;     // all prefixes of levels 0..n
+  uint32_t* d_full_off = nullptr;   // [n + 2]
+  std::vector<uint32_t> full_off;
   unsigned* d_status;  // HamView::status
   double* d_h;
   double* d_g;
@@ -385,6 +453,12 @@ int launch_connected(const HamView& hv, const uint64_t* x, Count n_x, uint64_t* 
 // mlp_fp32.cu
 int launch_mlp_fp32_logpsi(const MlpView& m, const HamView& hv, const uint64_t* x, Count n_x,
                            float* la, float* ph, cudaStream_t s);
+// terms [node][mlp_fp32_variants()][4] of every node below level n: the masked
+// half-log-probability and the phase of each outcome, as the rows
+// 0..variants-1 of a tile would have them
+uint32_t mlp_fp32_variants();
+int launch_mlp_fp32_nodes(const MlpView& m, const HamView& hv, const NodeView& nodes, uint64_t max_nodes,
+                          float2* terms, cudaStream_t s);
 int launch_mlp_fp32_slot_logits(const MlpView& m, int p, const uint64_t* prefixes,
                                 const uint64_t* n_rows_dev, uint64_t max_rows, float* out8,
                                 cudaStream_t s);
@@ -402,6 +476,11 @@ size_t mlp_fp32_grad_partial_floats(const MlpView& m, uint64_t n_x);
 // table.cu
 int launch_tf_fp32_logpsi(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float* la, float* ph,
                           cudaStream_t s);
+// out [determinant][tf_fp32_variants(m)]: (log|psi|, phase) as each sequence
+// of a tile would have it
+uint32_t tf_fp32_variants(const TfView& m);
+int launch_tf_fp32_variants(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float2* out,
+                            cudaStream_t s);
 int launch_tf_fp32_slot_logits(const TfView& m, int p, const uint64_t* pre, const uint64_t* nr, uint64_t max_rows,
                                float* out, cudaStream_t s);
 size_t tf_grad_workspace(const TfView& m, uint64_t n_x, bool recompute);  // recompute: block inputs only
@@ -413,13 +492,67 @@ int launch_table_slot_logits(const anqs_model* md, int p, const uint64_t* prefix
                              const uint64_t* n_rows_dev, uint64_t max_rows, float* out8,
                              cudaStream_t s);
 
+// eloc_unique.cu: local energies over the distinct connected determinants
+// Scratch of one call.  `full`: every prefix of the sector is a node.
+struct UniqueWs {
+  bool full, levels;
+  NodeView nodes;
+  uint64_t max_nodes, max_leaves;  // bounds: all levels, level n
+  uint32_t* ticket;
+  uint32_t* bits;      // bitmap over all levels (not full)
+  size_t bits_bytes;   // with the ticket and n_leaves before it
+  uint2* packed;
+  uint32_t* bsum;      // per-block node counts
+  uint64_t* n_leaves;  // device count (not full)
+  uint64_t *node_x, *leaf_x;
+  uint32_t* off;
+  double* part;        // partial sums when a sample is split over CTAs
+};
+bool unique_applies(const anqs_ham* H, uint64_t n_x);
+// Which form a call takes: the preferred one if its scratch fits into the
+// workspace, else the other if that fits (a workspace may have been sized for
+// more samples, in the other form).
+bool use_unique(const anqs_ham* H, bool preferred, size_t plain, size_t unique, size_t ws_bytes);
+// levels: the prefixes of the determinants are nodes too
+void plan_unique(const anqs_ham* H, uint64_t n_x, bool levels, Arena& A, UniqueWs& w);
+// the distinct determinants of the samples' connected sets into w.nodes; zeroes the ticket
+int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueWs& w, cudaStream_t s);
+Count unique_leaves(const UniqueWs& w);
+const uint64_t* unique_leaf_x(const anqs_ham* H, const UniqueWs& w);  // full, or planned without levels
+int launch_path_terms(const anqs_ham* H, const UniqueWs& w, const float2* per, float2* out, cudaStream_t s);
+int launch_byj(const HamView& hv, const uint64_t* x, Count rows, const float* raw, float2* tab, cudaStream_t s);
+int launch_chunk_counts(const uint64_t* total, uint64_t chunk, int n, uint64_t* out, cudaStream_t s);
+// per determinant, the sum of the node terms of its path (float2 [node][4]:
+// log|psi| and phase of each outcome) in slot order
+// (`variants` of each: terms [node][variants][4], sums [determinant][variants])
+int launch_path_sums(const anqs_ham* H, const UniqueWs& w, const float2* terms, float2* mid, float2* sums,
+                     cudaStream_t s, uint32_t variants = 1);
+uint64_t path_sums_mid(const anqs_ham* H, uint64_t n_x);  // float2 entries of `mid`, per variant
+// Amplitudes of the assembly.  SUM: one (log|psi|, phase) per distinct
+// determinant.  BYJ: [n + 1] per distinct determinant, entry j for a
+// connected determinant with first differing slot j, entry n for a sample.
+// TERMS: the parents' cache, plus the path terms [n] of each distinct
+// determinant.  ARRAY: one per sample and connected determinant.
+enum AmpMode { AMP_SUM = 0, AMP_BYJ = 1, AMP_TERMS = 2, AMP_ARRAY = 3 };
+struct AmpSrc {
+  AmpMode mode;
+  const float2* tab;           // SUM, BYJ, TERMS
+  const float *la, *ph;        // SUM without tab: per determinant; ARRAY: [n_x][K]
+  const float *la_x, *ph_x;    // TERMS, ARRAY: per sample
+  const float* cache;          // TERMS
+  // SUM: entries per determinant.  The FP32 MLP and transformer start the dot
+  // products of their head at an input that depends on the row of the tile, so
+  // the last bits of an amplitude depend on the row: entry r serves the rows
+  // r mod variants of the [n_x][K] connected determinants (and of the samples).
+  uint32_t variants = 1;
+};
+uint64_t eloc_partials(const anqs_ham* H, uint64_t n_x);  // doubles
+// E_loc and (counts set) the statistics; the ticket must be zero
+int launch_eloc_direct(const anqs_ham* H, const uint64_t* x, Count n_x, const NodeView& nodes, const AmpSrc& amp,
+                       double* ere, double* eim, double* part, const StatsOut& so, cudaStream_t s);
+
 // eloc.cu
-int launch_eloc_sum(const HamView& hv, Count n_x, const double* hval, const double* hdiag,
-                    const float* la_x, const float* ph_x, const float* la_p, const float* ph_p,
-                    double* ere, double* eim, cudaStream_t s);
 int launch_stats_combine(const double* in, int world, double* out, cudaStream_t s);
-int launch_stats(const double* ere, const double* eim, const uint64_t* counts, Count n_x,
-                 double* stats, cudaStream_t s);
 int launch_grad_cotangents(const double* ere, const double* eim, const uint64_t* counts,
                            const double* stats, Count n_x, float* cot_la, float* cot_ph,
                            cudaStream_t s);
@@ -427,7 +560,7 @@ int launch_grad_cotangents(const double* ere, const double* eim, const uint64_t*
 // mlp_tc.cu (BF16 tensor-core form)
 int mlp_tc_pack_alloc(anqs_model* m);
 int mlp_tc_pack(anqs_model* m, cudaStream_t s);
-size_t eloc_tc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x);
+size_t eloc_tc_workspace(const anqs_ham* H, uint64_t n_x, bool unique);
 // 16-bit MLP local energy in stages (pre: connected set, parents, sort; post:
 // assembly) and the suffix stage of many problems in one persistent launch
 struct MultiEloc {
@@ -441,7 +574,7 @@ struct MultiEloc {
 // beside the connected set and the sort (joined back into s before returning)
 int eloc_tc_pre(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, void* ws, size_t ws_bytes,
                 cudaStream_t s, bool fork = false);
-int eloc_tc_post(const anqs_ham* H, Count n_x, double* ere, double* eim, const uint64_t* counts, double* stats,
+int eloc_tc_post(const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim, const uint64_t* counts, double* stats,
                  void* ws, size_t ws_bytes, cudaStream_t s);
 int mlp_tc_multi_max();
 size_t mlp_tc_multi_groups_bytes();
@@ -449,6 +582,9 @@ int launch_mlp_tc_multi(const MultiEloc* q, int n, int chunk, int dynamic, void*
                         cudaStream_t s);
 int run_eloc_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere,
                 double* eim, const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s);
+// terms [node][4] of every node below level n: the masked half-log-probability
+// and the phase of each outcome of its slot
+int launch_mlp_tc_nodes(const anqs_model* M, const HamView& hv, const NodeView& nodes, float2* terms, cudaStream_t s);
 int launch_mlp_tc_logpsi(const anqs_model* M, const HamView& hv, const uint64_t* x, uint64_t n_x, float* la,
                          float* ph, cudaStream_t s);
 int launch_mlp_tc_slot_logits(const anqs_model* M, const HamView& hv, int p, const uint64_t* pre,
@@ -478,7 +614,7 @@ int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const
 int tf_tc_pack_alloc(anqs_model* m);
 int tf_tc_pack(anqs_model* m, cudaStream_t s);
 int tf_tc_status(const anqs_model* M, int* status);
-size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x);
+size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique);
 int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                    const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s);
 int launch_tf_tc_logpsi(const anqs_model* M, const HamView& hv, const uint64_t* x, uint64_t n_x, float* la,
@@ -495,13 +631,19 @@ int launch_nade_slot_logits(const NadeView& m, const HamView& hv, int p, const u
 int launch_nade_grad(const NadeView& m, const HamView& hv, const uint64_t* x, Count n_x, const CotSrc& cot,
                      float* grad, uint64_t n_params, float* part, cudaStream_t s);
 size_t nade_grad_partial_floats(const NadeView& m, uint64_t n_params, uint64_t n_x);
-size_t nade_eloc_workspace(const anqs_ham* H, uint64_t n_x);
+size_t nade_eloc_workspace(const anqs_ham* H, uint64_t n_x, bool unique);
 int run_eloc_nade(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                   const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s);
 
 // api.cu
 int logpsi_dispatch(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, float* la,
                     float* ph, cudaStream_t s);
+
+// the local energy from the amplitude of every connected determinant; part:
+// 2 n_x K / 512 doubles at most (eloc_partials), may alias hv
+int run_eloc_array(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, uint64_t* xp, double* hv,
+                   float* la_x, float* ph_x, float* la, float* ph, double* part, uint32_t* ticket, double* ere,
+                   double* eim, const uint64_t* counts, double* stats, cudaStream_t s);
 
 // sampler.cu
 size_t sampler_workspace(const anqs_ham* ham, uint64_t n_samples);

@@ -235,6 +235,85 @@ __global__ void __launch_bounds__(NT) logpsi_kernel(MlpView m, HamView hv, const
   }
 }
 
+// Slot terms of the distinct prefixes of a call's determinants (eloc_unique.cu):
+// 32 nodes of one level per tile.  slot_forward starts row r's head sums at
+// input r, so a prefix's outputs differ in the last bits from row to row; here
+// all 32 starting points are evaluated for every node (lane = starting point:
+// the activations and the head's weights are read at consecutive addresses),
+// which costs as much as one hidden layer.
+template <int W>
+__global__ void __launch_bounds__(NT) nodes_kernel(MlpView m, HamView hv, const uint64_t* __restrict__ xs,
+                                                   const uint32_t* __restrict__ off_, float2* __restrict__ terms) {
+  ANQS_PDL_ENTRY();
+  extern __shared__ float smem[];
+  float* act = smem;
+  float* ws = act + 2 * R * W;
+  float* out8 = ws + Smem<W>::ws_floats;
+  __shared__ uint64_t xt[R];
+  __shared__ float hw[8 * W];
+  __shared__ uint32_t off[ANQS_MAX_ORB + 1];
+  const int n = m.n, lane = threadIdx.x & 31, wg = threadIdx.x >> 5;
+  if (threadIdx.x <= n) off[threadIdx.x] = __ldcg(off_ + threadIdx.x);
+  __syncthreads();
+  uint32_t first = 0;  // first tile of level p
+  int p = 0;
+  for (uint32_t tile = blockIdx.x;; tile += gridDim.x) {
+    uint32_t nt;
+    while (p < n && tile >= first + (nt = (off[p + 1] - off[p] + R - 1) / R)) {
+      first += nt;
+      ++p;
+    }
+    if (p >= n) break;
+    const uint32_t row0 = off[p] + (tile - first) * R;
+    const int nrows = int(min(uint32_t(R), off[p + 1] - row0));
+    const MlpPtr P = slot_ptrs(m, p);
+    if (threadIdx.x < R)
+      xt[threadIdx.x] = threadIdx.x < nrows
+                            ? __ldcg(reinterpret_cast<const unsigned long long*>(xs) + row0 + threadIdx.x) : 0ull;
+    for (int i = threadIdx.x; i < 8 * W; i += NT) hw[i] = __ldg(P.Wh + i);
+    __syncthreads();
+    const int cur = slot_forward<W>(m, p, xt, nrows, act, 2, ws, out8);
+    const float* h = act + size_t(cur) * R * W + size_t(wg) * (R / 8) * W;
+    float acc[R / 8][8];
+#pragma unroll
+    for (int i = 0; i < R / 8; ++i)
+#pragma unroll
+      for (int o = 0; o < 8; ++o) acc[i][o] = __ldg(P.bh + o);
+    for (int k = 0; k < W; ++k) {
+      const int kk = (k + lane) & (W - 1);
+      float a[R / 8];
+#pragma unroll
+      for (int i = 0; i < R / 8; ++i) a[i] = h[i * W + kk];
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        const float w = hw[o * W + kk];
+#pragma unroll
+        for (int i = 0; i < R / 8; ++i) acc[i][o] = fmaf(a[i], w, acc[i][o]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R / 8; ++i) {
+      const int r = wg * (R / 8) + i;
+      if (r >= nrows) break;
+      const uint64_t x = xt[r];
+      const unsigned pm = slot_mask(hv, p, __popcll(x & 0x5555555555555555ull), __popcll(x & 0xAAAAAAAAAAAAAAAAull), x);
+      const unsigned nm = norm_mask(hv, p, pm);
+      float t[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        float la = 0.f, ph = 0.f;
+        bool dead = false;
+        slot_term(acc[i], nm, pm, v, la, ph, dead);
+        t[v] = dead ? -INFINITY : la;
+      }
+      float4* d = reinterpret_cast<float4*>(terms + (size_t(row0 + r) * R + lane) * 4);
+      d[0] = make_float4(t[0], acc[i][4], t[1], acc[i][5]);
+      d[1] = make_float4(t[2], acc[i][6], t[3], acc[i][7]);
+    }
+    __syncthreads();
+  }
+}
+
 template <int W>
 __global__ void __launch_bounds__(NT) slot_logits_kernel(MlpView m, int p, const uint64_t* __restrict__ prefixes,
                                                          const uint64_t* __restrict__ n_rows_dev,
@@ -520,6 +599,16 @@ int logpsi_w(const MlpView& m, const HamView& hv, const uint64_t* x, Count n_x, 
 }
 
 template <int W>
+int nodes_w(const MlpView& m, const HamView& hv, const NodeView& nodes, uint64_t max_nodes, float2* terms,
+            cudaStream_t s) {
+  const size_t sm = Smem<W>::bytes(2);
+  ANQS_TRY(set_smem(nodes_kernel<W>, sm));
+  ProfScope ps(PROF_MLP_FP32_LOGPSI, s);
+  ANQS_CUDA_LAUNCH("mlp nodes_kernel", launch_k(nodes_kernel<W>, dim3(grid_for(max_nodes / R + m.n, 152 * 8)), dim3(NT), sm, s, m, hv, nodes.x, nodes.off, terms));
+  return ANQS_OK;
+}
+
+template <int W>
 int logits_w(const MlpView& m, int p, const uint64_t* pre, const uint64_t* nr, uint64_t max_rows, float* out,
              cudaStream_t s) {
   size_t sm = Smem<W>::bytes(2);
@@ -586,6 +675,18 @@ int launch_mlp_fp32_logpsi(const MlpView& m, const HamView& hv, const uint64_t* 
     case 256: return logpsi_w<256>(m, hv, x, n_x, la, ph, s);
   }
   return set_error(ANQS_ERR_UNSUPPORTED, "width %d", m.width);
+}
+
+uint32_t mlp_fp32_variants() { return R; }
+
+int launch_mlp_fp32_nodes(const MlpView& m, const HamView& hv, const NodeView& nodes, uint64_t max_nodes,
+                          float2* terms, cudaStream_t s) {
+  switch (m.width) {
+    case 64: return nodes_w<64>(m, hv, nodes, max_nodes, terms, s);
+    case 128: return nodes_w<128>(m, hv, nodes, max_nodes, terms, s);
+    case 256: return nodes_w<256>(m, hv, nodes, max_nodes, terms, s);
+  }
+  return set_error(ANQS_ERR_UNSUPPORTED, "MLP width %d", m.width);
 }
 
 int launch_mlp_fp32_slot_logits(const MlpView& m, int p, const uint64_t* pre, const uint64_t* nr,

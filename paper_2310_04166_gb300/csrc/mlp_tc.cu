@@ -590,6 +590,117 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_ws_kernel(TcView tv, HamView hv,
   teardown<W>(tv, s_tmem, s_abort);
 }
 
+// One 128-row tile of the nodes of level p (rows [r0, r1) of the node list):
+// the masked terms of slot p's four outcomes of each prefix, in the same
+// expressions as the suffix rows and finalize_kernel.
+template <int W>
+__device__ __forceinline__ bool node_tile(const Ctx& c, uint32_t& ph_m, int p, uint32_t row, bool valid, uint64_t x,
+                                          const HamView& hv, const SlotLayout& Sl, uint32_t img_addr,
+                                          const unsigned char* img, float2* terms) {
+  unsigned pmk = 0, mk = 0;
+  if (valid) {
+    pmk = slot_mask(hv, p, __popcll(x & 0x5555555555555555ull), __popcll(x & 0xAAAAAAAAAAAAAAAAull), x);
+    mk = norm_mask(hv, p, pmk);
+  }
+  float out[8];
+  const bool ok = tile_slot<W>(c, ph_m, p, x, Sl, img_addr, img, out);
+  if (ok && valid) {
+    float mx = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if ((mk >> u) & 1u) mx = fmaxf(mx, out[u]);
+    float sum = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if ((mk >> u) & 1u) sum += __expf(out[u] - mx);
+    const float lse = mx + __logf(sum);
+    float t[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) t[u] = ((pmk >> u) & 1u) ? 0.5f * (out[u] - lse) : -INFINITY;
+    float4* d = reinterpret_cast<float4*>(terms + uint64_t(row) * 4);
+    d[0] = make_float4(t[0], out[4], t[1], out[5]);
+    d[1] = make_float4(t[2], out[6], t[3], out[7]);
+  }
+  return ok;
+}
+
+// NODES (weight-stationary): every distinct prefix of a call's determinants
+// once.  Work split as in mlp_tc_ws_kernel.
+template <int W>
+__global__ void __launch_bounds__(NT, 1) mlp_tc_nodes_kernel(TcView tv, HamView hv, const uint64_t* __restrict__ xs,
+                                                             const uint32_t* __restrict__ off,
+                                                             float2* __restrict__ terms) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bars[2 + NWG];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_abort;
+  const int wg = threadIdx.x / MT, t = threadIdx.x % MT;
+  const int n = tv.n;
+  setup<W>(bars, &s_tmem, &s_abort);
+  ANQS_PDL_WAIT();
+  ANQS_PDL_TRIGGER();
+  const uint32_t img_stride = round_up(tv.max_img, 1024u);
+  Ctx c;
+  c.tv = &tv;
+  c.s_a = smem + img_stride + wg * (MT * tv.kmax * 2u);
+  c.a_addr = tc::smem_u32(c.s_a);
+  c.tmem = s_tmem + uint32_t(wg) * W;
+  c.lane_base = uint32_t(t & ~31) << 16;
+  c.bar_m = tc::smem_u32(&bars[2 + wg]);
+  c.wg = wg;
+  c.t = t;
+  __shared__ uint32_t s_off[ANQS_MAX_ORB + 1];
+  if (threadIdx.x <= n) s_off[threadIdx.x] = __ldcg(off + threadIdx.x);
+  __syncthreads();
+  auto tiles = [&](int p) { return (s_off[p + 1] - s_off[p] + MT - 1) / MT; };
+  uint64_t total = 0;
+  int S = 0;
+  for (int p = 0; p < n; ++p) {
+    total += tiles(p);
+    S += tiles(p) ? 1 : 0;
+  }
+  int my_p = -1;
+  uint32_t li = 0, gp = 0;
+  if (total) {
+    const uint64_t G = gridDim.x, spare = G > uint64_t(S) ? G - S : 0;
+    uint64_t start = 0;
+    for (int p = 0; p < n; ++p) {
+      if (!tiles(p)) continue;
+      const uint64_t g = 1 + spare * tiles(p) / total;
+      if (blockIdx.x >= start && blockIdx.x < start + g) {
+        my_p = p;
+        li = uint32_t(blockIdx.x - start);
+        gp = uint32_t(g);
+      }
+      start += g;
+    }
+  }
+  if (my_p >= 0 && li < tiles(my_p)) {
+    const int p = my_p;
+    const uint32_t r0 = s_off[p], r1 = s_off[p + 1], nt = tiles(p);
+    const SlotLayout Sl = slot_layout(p, W, tv.L, tv.lo);
+    const uint32_t img_addr = tc::smem_u32(smem);
+    if (threadIdx.x == 0) load_slot(tv, p, img_addr, tc::smem_u32(&bars[0]), W, tv.L);
+    // the next tile's rows are loaded while this tile runs (the first while the weights come in)
+    uint32_t tile = li + gp * wg;
+    auto row_x = [&](uint32_t k) -> uint64_t {
+      const uint32_t r = r0 + k * MT + t;
+      return k < nt && r < r1 ? __ldcg(reinterpret_cast<const unsigned long long*>(xs) + r) : 0ull;
+    };
+    uint64_t nx = row_x(tile);
+    bool ok = __syncthreads_and(wait_bar(tc::smem_u32(&bars[0]), 0));
+    uint32_t ph_m = 0;
+    for (; ok && tile < nt; tile += gp * NWG) {
+      const uint64_t x = nx;
+      const uint32_t r = r0 + tile * MT + t;
+      nx = row_x(tile + gp * NWG);
+      ok = node_tile<W>(c, ph_m, p, r, r < r1, x, hv, Sl, img_addr, smem, terms);
+    }
+    if (!ok) s_abort = 1;
+  }
+  teardown<W>(tv, s_tmem, s_abort);
+}
+
 // ---- many problems in one persistent launch ---------------------------------
 //
 // The suffix work of up to kMaxBatch independent problems (each its own
@@ -612,7 +723,8 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_ws_kernel(TcView tv, HamView hv,
 struct MultiProblem {
   TcView tv;
   HamView hv;
-  const uint64_t* xp;
+  int nodes;                // rows of slot p: the nodes [offsets[p], offsets[p + 1]), terms to T[node][4];
+  const uint64_t* xp;       // else the first offsets[p] entries of perm, terms to T[row][n]
   const uint32_t* perm;
   const uint32_t* offsets;
   float2* T;
@@ -640,7 +752,10 @@ __global__ void multi_plan_kernel(const __grid_constant__ MultiArgs a) {
   for (int i = threadIdx.x; i < kMaxBatch * ANQS_MAX_ORB; i += blockDim.x) {
     const int b = i / ANQS_MAX_ORB, p = i % ANQS_MAX_ORB;
     uint32_t t = 0;
-    if (b < a.n_prob && p < a.prob[b].tv.n) t = (__ldcg(a.prob[b].offsets + p) + MT - 1) / MT;
+    if (b < a.n_prob && p < a.prob[b].tv.n) {
+      const uint32_t* o = a.prob[b].offsets + p;
+      t = ((a.prob[b].nodes ? __ldcg(o + 1) - __ldcg(o) : __ldcg(o)) + MT - 1) / MT;
+    }
     tiles[b][p] = t;
   }
   __syncthreads();
@@ -717,8 +832,25 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_multi_kernel(const __grid_consta
       loaded = bp;
       if (!ok) return false;
     }
-    const uint64_t rows = __ldcg(P.offsets + p);
     bool ok = true;
+    if (P.nodes) {
+      const uint32_t r0 = __ldcg(P.offsets + p), r1 = __ldcg(P.offsets + p + 1);
+      auto row_x = [&](uint32_t k) -> uint64_t {
+        const uint32_t r = r0 + k * MT + c.t;
+        return k < t_hi && r < r1 ? __ldcg(reinterpret_cast<const unsigned long long*>(P.xp) + r) : 0ull;
+      };
+      uint64_t nx = row_x(t_lo + wg);
+      for (uint32_t tile = t_lo + wg; ok && tile < t_hi; tile += NWG) {
+        const uint64_t x = nx;
+        const uint32_t r = r0 + tile * MT + c.t;
+        nx = row_x(tile + NWG);
+        ok = node_tile<W>(c, ph_m, p, r, r < r1, x, P.hv, Sl, img_addr, smem, P.T);
+      }
+      tc::fence_async_smem();
+      tc::fence_before_sync();
+      return __syncthreads_and(ok);
+    }
+    const uint64_t rows = __ldcg(P.offsets + p);
     for (uint32_t tile = t_lo + wg; ok && tile < t_hi; tile += NWG)
       ok = suffix_tile<W>(c, ph_m, p, P.tv.n, tile, rows, suffix_row(tile, rows, c.t, P.perm, P.xp), P.hv, Sl, img_addr,
                           smem, P.T);
@@ -1548,6 +1680,25 @@ size_t plan_eloc(const anqs_ham* H, uint64_t n_x, Arena& A, ElocWs& w) {
   return A.off;
 }
 
+// Scratch of the form over distinct prefixes (eloc_unique.cu)
+struct NodeWs {
+  UniqueWs u;
+  float2 *terms, *mid, *sums;
+};
+
+size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NodeWs& w) {
+  plan_unique(H, n_x, true, A, w.u);
+  w.terms = A.take<float2>((w.u.max_nodes - w.u.max_leaves) * 4);
+  w.mid = A.take<float2>(path_sums_mid(H, n_x));
+  w.sums = A.take<float2>(w.u.max_leaves);
+  return A.off;
+}
+
+bool nodes_form(const anqs_ham* H, uint64_t n_x, size_t ws_bytes) {
+  return use_unique(H, unique_applies(H, n_x), eloc_tc_workspace(H, n_x, false), H->has_index ? eloc_tc_workspace(H, n_x, true) : 0,
+                    ws_bytes);
+}
+
 template <int W>
 int launch_ws_w(const TcView& tv, const HamView& hv, const ElocWs& w, cudaStream_t s) {
   const size_t sm = smem_bytes(tv, 1);
@@ -1679,9 +1830,12 @@ int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const
   return ANQS_OK;
 }
 
-size_t eloc_tc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
-  (void)M;
+size_t eloc_tc_workspace(const anqs_ham* H, uint64_t n_x, bool unique) {
   Arena A(nullptr, 0);
+  if (unique) {
+    NodeWs v;
+    return plan_nodes(H, n_x, A, v);
+  }
   ElocWs w;
   return plan_eloc(H, n_x, A, w);
 }
@@ -1691,6 +1845,28 @@ size_t eloc_tc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
 //   pre:    connected set, parents' slots and caches, sort by first slot
 //   suffix: the connected determinants' slots p > j (mlp_tc_ws_kernel)
 //   post:   E_loc assembly
+static int plan_nodes_ws(const anqs_ham* H, Count n_x, void* ws, size_t ws_bytes, NodeWs& w) {
+  Arena A(ws, ws_bytes);
+  plan_nodes(H, n_x.n, A, w);
+  if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+  if (n_x.n * H->v.K > 0xffffffffull)
+    return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
+  return ANQS_OK;
+}
+
+int launch_mlp_tc_nodes(const anqs_model* M, const HamView& hv, const NodeView& nodes, float2* terms, cudaStream_t s) {
+  const TcView tv = make_view(M);
+  const size_t sm = smem_bytes(tv, 1);
+  const unsigned grid = unsigned(std::max(num_sms(), tv.n));
+  ProfScope ps(PROF_TC_SUFFIX, s);
+  auto go = [&](auto kern) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+    return e != cudaSuccess ? e : launch_k(kern, dim3(grid), dim3(NT), sm, s, tv, hv, nodes.x, nodes.off, terms);
+  };
+  ANQS_CUDA_LAUNCH("mlp_tc_nodes_kernel", tv.W == 128 ? go(mlp_tc_nodes_kernel<128>) : go(mlp_tc_nodes_kernel<64>));
+  return ANQS_OK;
+}
+
 static int plan_ws(const anqs_ham* H, Count n_x, void* ws, size_t ws_bytes, ElocWs& w) {
   Arena A(ws, ws_bytes);
   plan_eloc(H, n_x.n, A, w);
@@ -1706,6 +1882,11 @@ static int plan_ws(const anqs_ham* H, Count n_x, void* ws, size_t ws_bytes, Eloc
 // kernel, on the stream of the histogram and the assembly that use them.
 int eloc_tc_pre(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, void* ws, size_t ws_bytes,
                 cudaStream_t s, bool fork) {
+  if (nodes_form(H, n_x.n, ws_bytes)) {
+    NodeWs v;
+    ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
+    return launch_unique(H, x, n_x, v.u, s);
+  }
   ElocWs w;
   ANQS_TRY(plan_ws(H, n_x, ws, ws_bytes, w));
   const Count mc = scaled(n_x, H->v.K);
@@ -1742,8 +1923,17 @@ int eloc_tc_pre(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count
   return r;
 }
 
-int eloc_tc_post(const anqs_ham* H, Count n_x, double* ere, double* eim, const uint64_t* counts, double* stats,
-                 void* ws, size_t ws_bytes, cudaStream_t s) {
+int eloc_tc_post(const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim, const uint64_t* counts,
+                 double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
+  if (nodes_form(H, n_x.n, ws_bytes)) {
+    NodeWs v;
+    ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
+    ANQS_TRY(launch_path_sums(H, v.u, v.terms, v.mid, v.sums, s));
+    AmpSrc amp{};
+    amp.mode = AMP_SUM;
+    amp.tab = v.sums;
+    return launch_eloc_direct(H, x, n_x, v.u.nodes, amp, ere, eim, v.u.part, StatsOut{counts, stats, v.u.ticket}, s);
+  }
   ElocWs w;
   ANQS_TRY(plan_ws(H, n_x, ws, ws_bytes, w));
   ProfScope ps(PROF_TC_ELOC, s);
@@ -1753,15 +1943,19 @@ int eloc_tc_post(const anqs_ham* H, Count n_x, double* ere, double* eim, const u
 
 int run_eloc_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                 const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
-  ElocWs w;
-  ANQS_TRY(plan_ws(H, n_x, ws, ws_bytes, w));
   ANQS_TRY(eloc_tc_pre(M, H, x, n_x, ws, ws_bytes, s, true));
-  {
+  if (nodes_form(H, n_x.n, ws_bytes)) {
+    NodeWs v;
+    ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
+    ANQS_TRY(launch_mlp_tc_nodes(M, H->v, v.u.nodes, v.terms, s));
+  } else {
+    ElocWs w;
+    ANQS_TRY(plan_ws(H, n_x, ws, ws_bytes, w));
     TcView tv = make_view(M);
     ProfScope ps(PROF_TC_SUFFIX, s);
     ANQS_TRY(tv.W == 128 ? launch_ws_w<128>(tv, H->v, w, s) : launch_ws_w<64>(tv, H->v, w, s));
   }
-  return eloc_tc_post(H, n_x, ere, eim, counts, stats, ws, ws_bytes, s);
+  return eloc_tc_post(H, x, n_x, ere, eim, counts, stats, ws, ws_bytes, s);
 }
 
 // Shared memory of the tensor-core adjoint of model M (0 when it does not
@@ -1834,14 +2028,23 @@ int launch_mlp_tc_multi(const MultiEloc* q, int n, int chunk, int dynamic, void*
     const TcView tv = make_view(q[k].model);
     if (k == 0) W = tv.W;
     if (tv.W != W) return set_error(ANQS_ERR_ARG, "multi-problem launch needs one network width");
-    ElocWs w;
-    ANQS_TRY(plan_ws(q[k].ham, host_count(q[k].n_x), q[k].ws, q[k].ws_bytes, w));
     a.prob[k].tv = tv;
     a.prob[k].hv = q[k].ham->v;
-    a.prob[k].xp = w.xp;
-    a.prob[k].perm = w.perm;
-    a.prob[k].offsets = w.offsets;
-    a.prob[k].T = w.T;
+    a.prob[k].nodes = nodes_form(q[k].ham, q[k].n_x, q[k].ws_bytes) ? 1 : 0;
+    if (a.prob[k].nodes) {
+      NodeWs v;
+      ANQS_TRY(plan_nodes_ws(q[k].ham, host_count(q[k].n_x), q[k].ws, q[k].ws_bytes, v));
+      a.prob[k].xp = v.u.nodes.x;
+      a.prob[k].offsets = v.u.nodes.off;
+      a.prob[k].T = v.terms;
+    } else {
+      ElocWs w;
+      ANQS_TRY(plan_ws(q[k].ham, host_count(q[k].n_x), q[k].ws, q[k].ws_bytes, w));
+      a.prob[k].xp = w.xp;
+      a.prob[k].perm = w.perm;
+      a.prob[k].offsets = w.offsets;
+      a.prob[k].T = w.T;
+    }
     a.max_img = std::max(a.max_img, tv.max_img);
     a.kmax = std::max(a.kmax, tv.kmax);
   }

@@ -30,7 +30,8 @@
 // of every slot of every row: the parent pass of the local energy), SUFFIX
 // (for each connected x', sorted by its first differing slot j, the path terms
 // of the slots p > j: prefix reuse, the slots <= j come from the parent), and
-// LOGITS (slot p's 8 values for the sampler's prefixes).
+// LOGITS (slot p's 8 values for the sampler's prefixes), NODES (each distinct
+// prefix of p + 1 slots: the path term of its slot p).
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -332,7 +333,7 @@ __device__ void slot_values(const HamView& hv, int p, uint64_t x, const float2* 
   }
 }
 
-enum { MODE_LOGPSI = 0, MODE_RAW = 1, MODE_SUFFIX = 2, MODE_LOGITS = 3 };
+enum { MODE_LOGPSI = 0, MODE_RAW = 1, MODE_SUFFIX = 2, MODE_LOGITS = 3, MODE_NODES = 4 };
 
 struct FwdArgs {
   const uint64_t* x;        // rows (LOGPSI, RAW, LOGITS) or connected determinants (SUFFIX)
@@ -343,7 +344,7 @@ struct FwdArgs {
   const uint8_t* js;        // SUFFIX: first differing slot of each connected row
   const uint32_t* perm;     // SUFFIX: connected rows in ascending js
   const uint32_t* offsets;  // SUFFIX: offsets[p] = rows with js < p
-  float2* T;                // SUFFIX: [row][n] path terms of the slots > js
+  float2* T;                // SUFFIX: [row][n] path terms of the slots > js; NODES: [node]
 };
 
 template <int W, int RJ, int MODE>
@@ -357,9 +358,40 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
   __shared__ int dead[TR], jr[TR];
   __shared__ uint32_t rid[TR];
   const int n = m.n, tid = threadIdx.x;
-  const uint64_t rows = MODE == MODE_SUFFIX ? uint64_t(A.offsets[n - 1]) : A.rows.get();
   int staged = -1;
   bool pending = false;
+  if constexpr (MODE == MODE_NODES) {
+    // tiles of the levels 1..n in order; offsets[q] = first node of level q
+    __shared__ uint32_t off[2 * ANQS_MAX_ORB];
+    if (tid <= n + 1) off[tid] = __ldcg(A.offsets + tid);
+    __syncthreads();
+    uint32_t first = 0;  // first tile of slot p's level
+    int p = 0;
+    for (uint32_t tile = blockIdx.x;; tile += gridDim.x) {
+      uint32_t nt;
+      while (p < n && tile >= first + (nt = (off[p + 2] - off[p + 1] + TR - 1) / TR)) {
+        first += nt;
+        ++p;
+      }
+      if (p >= n) break;
+      const uint32_t row = off[p + 1] + (tile - first) * TR + tid;
+      const bool valid = tid < TR && row < off[p + 2];
+      if (tid < TR) xt[tid] = valid ? __ldcg(reinterpret_cast<const unsigned long long*>(A.x) + row) : 0ull;
+      __syncthreads();
+      float tr[2] = {0.f, 0.f}, ti[2];
+      bool ok[2];
+      for (int e = 0; e < 2; ++e) {
+        const int i = 2 * p + e;
+        eval_qubit<W, RJ>(m, i, i, 0, xt, S, S.Z3, staged, pending, e == 0 ? i + 1 : -1);
+        if (valid) ok[e] = path_term(hv, i, xt[tid], S.Z3[tid * 2], S.Z3[tid * 2 + 1], tr[e], ti[e]);
+      }
+      if (valid) A.T[row] = make_float2(ok[1] ? (ok[0] ? tr[0] : -INFINITY) + tr[1] : -INFINITY, ti[0] + ti[1]);
+      __syncthreads();
+    }
+    if (pending) cp_async_wait_all();
+    return;
+  }
+  const uint64_t rows = MODE == MODE_SUFFIX ? uint64_t(A.offsets[n - 1]) : A.rows.get();
   for (uint64_t base = uint64_t(blockIdx.x) * TR; base < rows; base += uint64_t(gridDim.x) * TR) {
     if (tid < TR) {
       const uint64_t l = base + tid;
@@ -478,6 +510,26 @@ int fwd_launch(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t 
   return ANQS_OK;
 }
 
+// NODES: the register tile that the suffix launch over all `rows` connected
+// determinants would take (the head's partial sums, hence the terms' last
+// bits, depend on it)
+template <int W>
+int nodes_w(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t rows, uint64_t max_nodes, cudaStream_t s) {
+  const uint64_t big_tiles = (rows + Tile<W, 4>::TR - 1) / Tile<W, 4>::TR;
+  max_nodes += uint64_t(m.n) * Tile<W, 4>::TR;  // a level's last tile may be partial
+  if (big_tiles >= 152) return fwd_launch<W, 4, MODE_NODES>(m, hv, a, max_nodes, PROF_NADE_SUFFIX, s);
+  return fwd_launch<W, 1, MODE_NODES>(m, hv, a, max_nodes, PROF_NADE_SUFFIX, s);
+}
+
+int nodes(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t rows, uint64_t max_nodes, cudaStream_t s) {
+  switch (m.w) {
+    case 32: return nodes_w<32>(m, hv, a, rows, max_nodes, s);
+    case 64: return nodes_w<64>(m, hv, a, rows, max_nodes, s);
+    case 128: return nodes_w<128>(m, hv, a, rows, max_nodes, s);
+  }
+  return set_error(ANQS_ERR_UNSUPPORTED, "NADE width %d", m.w);
+}
+
 template <int W, int MODE>
 int fwd_w(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t max_rows, int prof, cudaStream_t s) {
   const uint64_t ny = MODE == MODE_RAW ? 3ull * uint64_t(m.n) : (clustered<MODE>() ? 3ull : 1ull);
@@ -525,6 +577,25 @@ size_t plan_eloc(const anqs_ham* H, uint64_t n_x, Arena& A, NadeElocWs& w) {
   return A.off;
 }
 
+// Scratch of the form over distinct prefixes (eloc_unique.cu)
+struct NadeNodeWs {
+  UniqueWs u;
+  float *la_x, *ph_x, *raw, *cache;
+  float2 *per, *T;  // per node, per determinant and slot
+};
+
+size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NadeNodeWs& w) {
+  const uint64_t n = uint64_t(H->v.n);
+  plan_unique(H, n_x, true, A, w.u);
+  w.la_x = A.take<float>(n_x);
+  w.ph_x = A.take<float>(n_x);
+  w.raw = A.take<float>(n_x * n * 8);
+  w.cache = A.take<float>(n_x * n * TC_CACHE_F);
+  w.per = A.take<float2>(w.u.max_nodes);
+  w.T = A.take<float2>(w.u.max_leaves * n);
+  return A.off;
+}
+
 }  // namespace
 
 int launch_nade_logpsi(const NadeView& m, const HamView& hv, const uint64_t* x, Count n_x, float* la, float* ph,
@@ -548,8 +619,12 @@ int launch_nade_slot_logits(const NadeView& m, const HamView& hv, int p, const u
   return fwd<MODE_LOGITS>(m, hv, a, max_rows, PROF_NADE_SLOT, s);
 }
 
-size_t nade_eloc_workspace(const anqs_ham* H, uint64_t n_x) {
+size_t nade_eloc_workspace(const anqs_ham* H, uint64_t n_x, bool unique) {
   Arena A(nullptr, 0);
+  if (unique) {
+    NadeNodeWs v;
+    return plan_nodes(H, n_x, A, v);
+  }
   NadeElocWs w;
   return plan_eloc(H, n_x, A, w);
 }
@@ -557,11 +632,43 @@ size_t nade_eloc_workspace(const anqs_ham* H, uint64_t n_x) {
 // Local energy with prefix reuse: the parents' slot values (RAW) give log psi(x)
 // and, per slot, the prefix sums and the slot's masked terms; each connected
 // x' then needs only the path terms of the slots above its first differing
-// slot j (SUFFIX, rows sorted by j); the assembly adds them up and sums
+// slot j: of every distinct prefix (NODES), or row by row where the sector has
+// no index (SUFFIX, rows sorted by j).  The assembly adds them up and sums
 // H_xx' psi(x')/psi(x) in FP64.
 int run_eloc_nade(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                   const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
   Arena A(ws, ws_bytes);
+  if (use_unique(H, unique_applies(H, n_x.n), nade_eloc_workspace(H, n_x.n, false),
+                 H->has_index ? nade_eloc_workspace(H, n_x.n, true) : 0, ws_bytes)) {
+    NadeNodeWs v;
+    plan_nodes(H, n_x.n, A, v);
+    if (!A.fits() || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+    if (n_x.n * H->v.K > 0xffffffffull)
+      return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
+    ANQS_TRY(launch_unique(H, x, n_x, v.u, s));
+    FwdArgs a{};
+    a.x = x;
+    a.rows = n_x;
+    a.out8 = v.raw;
+    ANQS_TRY(fwd<MODE_RAW>(M->nade, H->v, a, n_x.n, PROF_NADE_PARENT, s));
+    {
+      ProfScope ps(PROF_TC_FINALIZE, s);
+      ANQS_TRY(launch_tc_finalize(H->v, x, n_x, v.raw, v.la_x, v.ph_x, v.cache, s));
+    }
+    FwdArgs b{};
+    b.x = v.u.nodes.x;
+    b.offsets = v.u.nodes.off;
+    b.T = v.per;
+    ANQS_TRY(nodes(M->nade, H->v, b, n_x.n * H->v.K, v.u.max_nodes, s));
+    ANQS_TRY(launch_path_terms(H, v.u, v.per, v.T, s));
+    AmpSrc amp{};
+    amp.mode = AMP_TERMS;
+    amp.tab = v.T;
+    amp.la_x = v.la_x;
+    amp.ph_x = v.ph_x;
+    amp.cache = v.cache;
+    return launch_eloc_direct(H, x, n_x, v.u.nodes, amp, ere, eim, v.u.part, StatsOut{counts, stats, v.u.ticket}, s);
+  }
   NadeElocWs w;
   plan_eloc(H, n_x.n, A, w);
   if (!A.fits() || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);

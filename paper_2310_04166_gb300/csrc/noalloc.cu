@@ -131,11 +131,8 @@ extern "C" int anqs_local_energy_static(const anqs_model* M, const anqs_ham* H, 
   float* la_p = S.take<float>(m);
   float* ph_p = S.take<float>(m);
   cudaStream_t s = (cudaStream_t)stream;
-  const Count nc = host_count(n_x);
-  ANQS_TRY(launch_connected(H->v, x, nc, xp, hv, nullptr, hd, s));
-  ANQS_TRY(logpsi_dispatch(M, H, x, nc, la_x, ph_x, s));
-  ANQS_TRY(logpsi_dispatch(M, H, xp, host_count(m), la_p, ph_p, s));
-  ANQS_TRY(launch_eloc_sum(H->v, nc, hv, hd, la_x, ph_x, la_p, ph_p, ere, eim, s));
-  if (counts) ANQS_TRY(launch_stats(ere, eim, counts, nc, stats, s));
-  return ANQS_OK;
+  // the parts of samples split over CTAs go where the matrix elements were (at
+  // most one part per 512 excitations), the ticket where the diagonal would be
+  return run_eloc_array(M, H, x, host_count(n_x), xp, hv, la_x, ph_x, la_p, ph_p, hv, reinterpret_cast<uint32_t*>(hd),
+                        ere, eim, counts, stats, s);
 }

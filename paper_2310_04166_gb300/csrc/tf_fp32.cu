@@ -146,6 +146,27 @@ __device__ __forceinline__ void layer_norm(const float* x, float* y, const float
   __syncthreads();
 }
 
+// The 8 outputs of every row from the final LayerNorm's output a.  Row r's sums
+// start at input rot + r (the rows' different starts spread the shared-memory
+// banks).
+template <int D>
+__device__ __forceinline__ void head(const TfView& m, const float* a, float* out8, int rot) {
+  constexpr int MT = Cfg<D>::MT;
+  const float* hw = tf_tail(m) + 2 * D;
+  const float* hb = hw + 8 * D;
+  for (int task = threadIdx.x; task < MT * 8; task += NT) {
+    const int r = task >> 3, o = task & 7;
+    float acc = __ldg(hb + o);
+    const float* wr = hw + o * D;
+    for (int k = 0; k < D; ++k) {
+      const int kk = (k + rot + r) & (D - 1);
+      acc = fmaf(a[r * D + kk], __ldg(wr + kk), acc);
+    }
+    out8[task] = acc;
+  }
+  __syncthreads();
+}
+
 // Forward of a tile: rows r = s T + t for s < S sequences (determinant or
 // prefix xs[s]) and t < T positions.  Leaves the 8 outputs of every row in
 // out8[MT][8].
@@ -222,19 +243,7 @@ __device__ void tile_forward(const TfView& m, const uint64_t* xs, int S, int T, 
   }
   const float* tail = tf_tail(m);
   layer_norm<D>(h, a, tail, tail + D);
-  const float* hw = tail + 2 * D;
-  const float* hb = hw + 8 * D;
-  for (int task = threadIdx.x; task < MT * 8; task += NT) {
-    const int r = task >> 3, o = task & 7;
-    float acc = __ldg(hb + o);
-    const float* wr = hw + o * D;
-    for (int k = 0; k < D; ++k) {
-      const int kk = (k + r) & (D - 1);  // rotate the start to spread shared-memory banks
-      acc = fmaf(a[r * D + kk], __ldg(wr + kk), acc);
-    }
-    out8[task] = acc;
-  }
-  __syncthreads();
+  head<D>(m, a, out8, 0);
 }
 
 // log-softmax term of the chosen outcome (FP32), as for the MLP: normalised
@@ -295,6 +304,52 @@ __global__ void __launch_bounds__(NT, 1) tf_logpsi_kernel(TfView m, HamView hv, 
   }
 }
 
+// log psi of the distinct determinants of a call (eloc_unique.cu), as each of
+// the S sequences of a tile would have it: sequence s's row of position t is
+// s T + t, so for variant q the sums of sequence s start (q - s) T further on
+// (D a power of two: the start counts modulo D).
+template <int D>
+__global__ void __launch_bounds__(NT, 1) tf_variants_kernel(TfView m, HamView hv, const uint64_t* __restrict__ xs,
+                                                            Count n_x_, float2* __restrict__ out) {
+  ANQS_PDL_ENTRY();
+  extern __shared__ float smem[];
+  constexpr int MT = Cfg<D>::MT;
+  __shared__ uint64_t xt[MT];
+  float* out8 = smem + Cfg<D>::floats - MT * 8;
+  const uint64_t n_x = n_x_.get();
+  const int T = m.n, S = MT / T;
+  const uint64_t n_tiles = (n_x + S - 1) / S;
+  for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const uint64_t base = tile * S;
+    const int ns = int(n_x - base < uint64_t(S) ? n_x - base : uint64_t(S));
+    if (threadIdx.x < S)
+      xt[threadIdx.x] = threadIdx.x < ns ? __ldcg(reinterpret_cast<const unsigned long long*>(xs) + base + threadIdx.x) : 0ull;
+    __syncthreads();
+    tile_forward<D>(m, xt, ns, T, smem);
+    // shift d = q - s mod S' over all (sequence, variant) pairs: with the sums
+    // shifted by d rows, sequence s holds variant s + d (for d < 0 too)
+    for (int d = 1 - S; d < S; ++d) {
+      head<D>(m, smem + MT * D, out8, ((d * T) % D + D) & (D - 1));
+      const int s = threadIdx.x, q = s + d;
+      if (s < ns && q >= 0 && q < S) {
+        const uint64_t x = xt[s];
+        float la = 0.f, ph = 0.f;
+        bool dead = false;
+        int ca = 0, cb = 0;
+        for (int p = 0; p < T; ++p) {
+          const int v = int((x >> (2 * p)) & 3ull);
+          const unsigned pm = slot_mask(hv, p, ca, cb, x);
+          slot_term(out8 + (s * T + p) * 8, norm_mask(hv, p, pm), pm, v, la, ph, dead);
+          ca += v & 1;
+          cb += v >> 1;
+        }
+        out[(base + s) * S + q] = make_float2(dead ? -INFINITY : la, ph);
+      }
+      __syncthreads();
+    }
+  }
+}
+
 template <int D>
 __global__ void __launch_bounds__(NT, 1) tf_slot_logits_kernel(TfView m, int p, const uint64_t* __restrict__ pre,
                                                                const uint64_t* __restrict__ n_rows_dev,
@@ -334,6 +389,19 @@ int logpsi_d(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, f
 }
 
 template <int D>
+int variants_d(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float2* out, cudaStream_t s) {
+  const int S = Cfg<D>::MT / m.n;
+  const uint64_t tiles = (n_x.n + S - 1) / S;
+  const unsigned grid = unsigned(tiles < 152 ? (tiles ? tiles : 1) : 152);
+  ANQS_CUDA(cudaFuncSetAttribute(tf_variants_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(Cfg<D>::bytes)));
+  ProfScope ps(PROF_TF, s);
+  ANQS_CUDA_LAUNCH("tf_variants_kernel",
+                   launch_k(tf_variants_kernel<D>, dim3(grid), dim3(NT), Cfg<D>::bytes, s, m, hv, x, n_x, out));
+  return ANQS_OK;
+}
+
+template <int D>
 int logits_d(const TfView& m, int p, const uint64_t* pre, const uint64_t* nr, uint64_t max_rows, float* out,
              cudaStream_t s) {
   const int S = Cfg<D>::MT / (p + 1);
@@ -357,6 +425,23 @@ int launch_tf_fp32_logpsi(const TfView& m, const HamView& hv, const uint64_t* x,
     case 64: return logpsi_d<64>(m, hv, x, n_x, la, ph, s);
     case 128: return logpsi_d<128>(m, hv, x, n_x, la, ph, s);
     case 256: return logpsi_d<256>(m, hv, x, n_x, la, ph, s);
+  }
+  return set_error(ANQS_ERR_UNSUPPORTED, "d_model %d", m.d);
+}
+
+uint32_t tf_fp32_variants(const TfView& m) {
+  const int mt = m.d <= 64 ? Cfg<64>::MT : m.d == 128 ? Cfg<128>::MT : Cfg<256>::MT;
+  return uint32_t(mt / m.n);
+}
+
+int launch_tf_fp32_variants(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float2* out,
+                            cudaStream_t s) {
+  if (n_x.n == 0) return ANQS_OK;
+  switch (m.d) {
+    case 32: return variants_d<32>(m, hv, x, n_x, out, s);
+    case 64: return variants_d<64>(m, hv, x, n_x, out, s);
+    case 128: return variants_d<128>(m, hv, x, n_x, out, s);
+    case 256: return variants_d<256>(m, hv, x, n_x, out, s);
   }
   return set_error(ANQS_ERR_UNSUPPORTED, "d_model %d", m.d);
 }

@@ -774,6 +774,25 @@ size_t plan(const anqs_model* M, const anqs_ham* H, uint64_t n_x, Arena& A, TfEl
   return A.off;
 }
 
+// Scratch of the form over distinct determinants (eloc_unique.cu): every
+// position of each is evaluated, in chunks of at most kChunk determinants
+constexpr uint64_t kChunk = 1 << 20;
+struct TfLeafWs {
+  UniqueWs u;
+  float* raw;        // [chunk][n][8]
+  float2* tab;       // [determinants][n + 1]
+  uint64_t* counts;  // determinants of each chunk
+};
+
+size_t plan_leaves(const anqs_ham* H, uint64_t n_x, Arena& A, TfLeafWs& w) {
+  const uint64_t n = H->v.n;
+  plan_unique(H, n_x, false, A, w.u);
+  w.raw = A.take<float>(std::min(w.u.max_leaves, kChunk) * n * 8);
+  w.tab = A.take<float2>(w.u.max_leaves * (n + 1));
+  w.counts = A.take<uint64_t>((w.u.max_leaves + kChunk - 1) / kChunk);
+  return A.off;
+}
+
 }  // namespace
 
 int tf_tc_pack_alloc(anqs_model* M) {
@@ -833,8 +852,12 @@ int launch_tf_tc_slot_logits(const anqs_model* M, int p, const uint64_t* pre, co
   return launch(M, a, (max_rows + S - 1) / S, PROF_TF_TC_SLOT, s);
 }
 
-size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique) {
   Arena A(nullptr, 0);
+  if (unique) {
+    TfLeafWs v;
+    return plan_leaves(H, n_x, A, v);
+  }
   TfElocWs w;
   return plan(M, H, n_x, A, w);
 }
@@ -842,6 +865,35 @@ size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x
 int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                    const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
   Arena A(ws, ws_bytes);
+  if (use_unique(H, unique_applies(H, n_x.n), tf_tc_eloc_workspace(M, H, n_x.n, false),
+                 H->has_index ? tf_tc_eloc_workspace(M, H, n_x.n, true) : 0, ws_bytes)) {
+    TfLeafWs v;
+    plan_leaves(H, n_x.n, A, v);
+    if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+    if (n_x.n * H->v.K > 0xffffffffull)
+      return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
+    const int n = H->v.n;
+    ANQS_TRY(launch_unique(H, x, n_x, v.u, s));
+    const uint64_t* lx = unique_leaf_x(H, v.u);
+    const Count leaves = unique_leaves(v.u);
+    const int chunks = int((leaves.n + kChunk - 1) / kChunk);
+    if (chunks > 1 && leaves.dev) ANQS_TRY(launch_chunk_counts(leaves.dev, kChunk, chunks, v.counts, s));
+    for (int c = 0; c < chunks; ++c) {
+      const uint64_t lo = uint64_t(c) * kChunk, most = std::min<uint64_t>(kChunk, leaves.n - lo);
+      const Count rows{most, leaves.dev ? (chunks > 1 ? v.counts + c : leaves.dev) : nullptr, 1};
+      if (M->d.d_model == 128) {
+        ANQS_TRY(launch_tf128_full(M, H->v, lx + lo, rows, n, 0, v.raw, nullptr, PROF_TF_TC_SUFFIX, s));
+      } else {
+        const Args a = full_args(lx + lo, rows, n, 0, v.raw, nullptr, H->v);
+        ANQS_TRY(launch(M, a, (most + MT / n - 1) / (MT / n), PROF_TF_TC_SUFFIX, s));
+      }
+      ANQS_TRY(launch_byj(H->v, lx + lo, rows, v.raw, v.tab + lo * (n + 1), s));
+    }
+    AmpSrc amp{};
+    amp.mode = AMP_BYJ;
+    amp.tab = v.tab;
+    return launch_eloc_direct(H, x, n_x, v.u.nodes, amp, ere, eim, v.u.part, StatsOut{counts, stats, v.u.ticket}, s);
+  }
   TfElocWs w;
   plan(M, H, n_x.n, A, w);
   if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);

@@ -1,0 +1,143 @@
+"""Local energies over distinct connected determinants (csrc/eloc_unique.cu).
+
+The FP32 forms are compared with the static-scratch entry point, which
+evaluates every connected determinant by itself through the same assembly:
+the results are equal bit for bit.  The 16-bit and NADE forms are compared
+with the sum over anqs_connected's list and anqs_logpsi's amplitudes: the same
+terms added in another order, so each log-amplitude differs by float32
+rounding (n sums of values below about 20: 2e-5), and E_loc by that times the
+sum of |H psi'/psi|.
+"""
+import ctypes as C
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def A():
+    import paper_2310_04166_gb300 as A
+    return A
+
+
+def _problem(A, kind, form, n, na, nb, seed, z2=False, du=0):
+    from synthetic import (flatten_mlp, flatten_nade, flatten_tf, integrals, integrals_z2, mlp_params, nade_params,
+                           tf_params, z2_qubit_masks)
+    labels = [p % 2 for p in range(n)]
+    h, g, e = integrals_z2(seed, n, 2 * n, labels) if z2 else integrals(seed, n, 2 * n)
+    ham = A.Hamiltonian(h, g, e, na, nb)
+    if z2:
+        ham.set_z2(z2_qubit_masks(labels))
+    if du:
+        ham.set_pruning(du)
+    t = lambda a: torch.tensor(a, device="cuda")
+    if kind == "mlp":
+        return A.Model.mlp(n, 64, 2, t(flatten_mlp(mlp_params(seed, n, 64, 2, 0.2))), form), ham
+    if kind == "nade":
+        return A.Model.nade(n, 32, t(flatten_nade(nade_params(seed, n, 32, 0.1)))), ham
+    return A.Model.transformer(n, 64, 4, 1, t(flatten_tf(tf_params(seed, n, 64, 1, 0.1))), form), ham
+
+
+def _dets(n, na, nb, m, seed, parity=None):
+    rng = np.random.default_rng(seed)
+    out = set()
+    for _ in range(50 * m):
+        x = sum(1 << (2 * int(p)) for p in rng.choice(n, na, replace=False))
+        x += sum(1 << (2 * int(p) + 1) for p in rng.choice(n, nb, replace=False))
+        if parity is None or bin(x & parity[0]).count("1") % 2 == parity[1]:
+            out.add(x)
+        if len(out) == m:
+            break
+    return torch.tensor(sorted(out), dtype=torch.int64, device="cuda")
+
+
+def _static(A, model, ham, x, cnt):
+    from paper_2310_04166_gb300 import _lib
+    ere, eim = (torch.empty(x.numel(), dtype=torch.float64, device="cuda") for _ in range(2))
+    st = torch.empty(4, dtype=torch.float64, device="cuda")
+    _lib.check(_lib.load().anqs_local_energy_static(model._m, ham.handle, x.data_ptr(), cnt.data_ptr(), x.numel(),
+                                                    ere.data_ptr(), eim.data_ptr(), st.data_ptr(),
+                                                    C.c_void_p(torch.cuda.current_stream().cuda_stream)))
+    return ere, eim, st
+
+
+# (n, na, nb, samples): one orbital, full shells (no excitations), few samples of a larger sector (bitmap, samples
+# split over CTAs), most of a small sector (all prefixes), odd counts, several bitmap blocks
+SHAPES = [(1, 1, 0, 1), (3, 3, 0, 1), (4, 2, 2, 36), (5, 1, 4, 3), (7, 5, 2, 9), (9, 4, 5, 33), (10, 5, 5, 130)]
+
+
+@pytest.mark.parametrize("kind", ["mlp", "tf"])
+@pytest.mark.parametrize("n,na,nb,m", SHAPES)
+@pytest.mark.parametrize("z2,du", [(False, 0), (True, 0), (False, 1)])
+def test_fp32_equals_every_determinant_by_itself(A, kind, n, na, nb, m, z2, du):
+    model, ham = _problem(A, kind, "fp32", n, na, nb, 40 + n, z2, du)
+    par = None
+    if z2:
+        mask = sum(3 << (2 * p) for p in range(n) if p % 2)
+        ref = sum(1 << (2 * p) for p in range(na)) + sum(2 << (2 * p) for p in range(nb))
+        par = (mask, bin(ref & mask).count("1") % 2)
+    x = _dets(n, na, nb, m, n, par)
+    cnt = torch.arange(1, x.numel() + 1, dtype=torch.int64, device="cuda")
+    a, b = A.local_energy(model, ham, x, cnt), _static(A, model, ham, x, cnt)
+    assert all(torch.equal(u, v) for u, v in zip(a, b))
+    # a workspace sized for more samples, and rows counted on the device
+    ws = A._ws(A.local_energy_workspace_bytes(model, ham, 4 * x.numel() + 3), "cuda")
+    c = A.local_energy(model, ham, x, cnt, workspace=ws)
+    assert all(torch.equal(u, v) for u, v in zip(a, c))
+    nd = torch.tensor([x.numel()], dtype=torch.int64, device="cuda")
+    pad = torch.cat([x, x[:1].expand(5)])
+    d = A.local_energy(model, ham, pad, torch.cat([cnt, cnt[:1].expand(5)]), n_dev=nd)
+    assert all(torch.allclose(u[:v.numel()], v, rtol=1e-12, atol=1e-12) for u, v in zip(d, a))
+
+
+@pytest.mark.parametrize("kind,form", [("mlp", "bf16"), ("tf", "bf16"), ("nade", "fp32")])
+@pytest.mark.parametrize("n,na,nb,m", SHAPES + [(13, 6, 7, 40)])
+@pytest.mark.parametrize("du", [0, 2])
+def test_reuse_forms_match_amplitudes_of_the_connected_list(A, kind, form, n, na, nb, m, du):
+    model, ham = _problem(A, kind, form, n, na, nb, 60 + n, du=min(du, n))
+    x = _dets(n, na, nb, m, 3 * n)
+    ere, eim, _ = A.local_energy(model, ham, x, torch.ones_like(x))
+    if ham.n_connected == 0:  # the diagonal element alone (anqs_connected takes no empty list)
+        other, _ = _problem(A, "mlp", "fp32", n, na, nb, 60 + n)
+        ref = A.local_energy(other, ham, x)
+        assert torch.equal(ere, ref[0]) and torch.equal(eim, ref[1])
+        return
+    xp, hv, _, hd = A.connected(ham, x)
+    la, ph = A.logpsi(model, ham, x)
+    lp, pp = (t.view(xp.shape).double() for t in A.logpsi(model, ham, xp.reshape(-1)))
+    r = torch.exp(lp - la.double()[:, None])
+    dp = pp - ph.double()[:, None]
+    e = torch.complex(hd + (hv * r * torch.cos(dp)).sum(1), (hv * r * torch.sin(dp)).sum(1))
+    bound = 1e-9 + 4e-5 * (hv.abs() * r).sum(1)
+    assert torch.all((ere - e.real).abs() <= bound) and torch.all((eim - e.imag).abs() <= bound)
+
+
+@pytest.mark.parametrize("kind,form", [("mlp", "fp32"), ("mlp", "bf16"), ("tf", "bf16"), ("nade", "fp32")])
+def test_determinants_outside_the_sector(A, kind, form):
+    """NaN for rows with other electron counts or bits beyond the orbitals; the other rows as without them."""
+    model, ham = _problem(A, kind, form, 6, 3, 2, 7)
+    x = _dets(6, 3, 2, 20, 1)
+    ref = A.local_energy(model, ham, x)
+    bad = torch.cat([x[:7], torch.tensor([0, 1 << 12, (1 << 12) | int(x[0]), -1], device="cuda"), x[7:]])
+    ere, eim, _ = A.local_energy(model, ham, bad)
+    assert torch.isnan(ere[7:11]).all() and torch.isnan(eim[7:11]).all()
+    keep = torch.cat([torch.arange(7), torch.arange(11, bad.numel())]).cuda()
+    if form == "bf16" or kind == "nade":  # in the FP32 forms a row's last bits follow its place in the list
+        assert torch.allclose(ere[keep], ref[0], rtol=1e-12, atol=1e-12)
+        assert torch.allclose(eim[keep], ref[1], rtol=1e-12, atol=1e-12)
+    else:
+        assert torch.allclose(ere[keep], ref[0], rtol=0, atol=1e-3)
+
+
+def test_index_arithmetic_over_the_supported_range():
+    """Division by multiplication (FastDiv) for every divisor and the values it meets."""
+    for d in range(2, 513):
+        m = (0xFFFFFFFF + d) // d
+        v = np.unique(np.concatenate([np.arange(0, 512 * d, max(1, d // 3)), np.arange(1, 512) * d,
+                                      np.arange(1, 512) * d - 1])).astype(np.uint64)
+        assert np.array_equal((v * np.uint64(m)) >> np.uint64(32), v // np.uint64(d)), d
+    assert math.comb(31, 2) < 512 and 16 * 16 <= 256
