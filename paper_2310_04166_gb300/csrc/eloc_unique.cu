@@ -23,98 +23,10 @@
 // determinant by itself, so the amplitudes have its bits.
 #include <algorithm>
 
-#include "common.cuh"
+#include "excite.cuh"
 
 namespace anqs {
 namespace {
-
-constexpr int MAXS = 256;  // singles of one spin: at most 16 x 16
-constexpr int MAXP = 512;  // pairs of a list: at most C(31, 2) = 465
-
-// Per-sample tables in shared memory.  A single (i, a) of spin s has index
-// r_i * n_virt + r_a in the order of the occupied and virtual lists.
-struct Exc {
-  uint64_t x;
-  uint32_t str[2];
-  int ok;
-  uint8_t occ[2][32], vir[2][32];
-  uint8_t sgn[2][MAXS];   // parity of the electrons strictly between the two spin-orbitals
-  uint8_t si[2][MAXS], sa[2][MAXS];
-  uint32_t rank[2][MAXS]; // alpha: rank of the new string times nb_p[n]; beta: rank of the new string
-  uint32_t g[2][MAXS];    // alpha: (a n + i) n^2, beta: a n + i
-  uint16_t po[2][MAXP], pv[2][MAXP];  // pairs r1 | r2 << 8, lexicographic
-  uint32_t own[2];        // rank(alpha) * nb_p[n], rank(beta)
-};
-
-// q = v / d for v < 2^24, d <= 512 by multiplication with ceil(2^32 / d): the
-// product's excess over v / d is below v / 2^32 * 1 < 1 / d.
-struct FastDiv {
-  uint32_t d, m;
-};
-__host__ __device__ inline FastDiv fast_div(uint32_t d) {
-  return FastDiv{d, d > 1 ? uint32_t((0xffffffffull + d) / d) : 0u};
-}
-__device__ __forceinline__ uint32_t fdiv(const FastDiv& f, uint32_t v) { return f.d > 1 ? __umulhi(v, f.m) : v; }
-
-// pair lists of both spins (they depend on the electron counts only)
-__device__ __forceinline__ void build_pairs(const HamView& hv, Exc& E) {
-  for (int s = 0; s < 2; ++s) {
-    const int ne = s ? hv.nb : hv.na, nv = hv.n - ne;
-    for (int t = 0; t < 2; ++t) {
-      const int m = t ? nv : ne;
-      uint16_t* o = t ? E.pv[s] : E.po[s];
-      for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        if (i < j) o[i * (2 * m - i - 1) / 2 + j - i - 1] = uint16_t(i | j << 8);
-      }
-    }
-  }
-}
-
-// tables of sample x; begins and ends with the CTA synchronised
-template <bool RANK>
-__device__ __forceinline__ void build_exc(const HamView& hv, const SectorView& sv, uint64_t x, Exc& E) {
-  const int n = hv.n;
-  const uint32_t oa = even_bits(x), ob = even_bits(x >> 1);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    E.x = x;
-    E.str[0] = oa;
-    E.str[1] = ob;
-    E.ok = __popc(oa) == hv.na && __popc(ob) == hv.nb && (n == 32 || (x >> (2 * n)) == 0);
-  }
-  if (threadIdx.x < 64) {
-    const int s = threadIdx.x >> 5, p = threadIdx.x & 31;
-    if (p < n) {
-      const uint32_t o = s ? ob : oa, below = o & ((1u << p) - 1u);
-      const int k = __popc(below);
-      if ((o >> p) & 1u) E.occ[s][k] = uint8_t(p);
-      else E.vir[s][p - k] = uint8_t(p);
-    }
-  }
-  __syncthreads();
-  if (!E.ok) return;
-  for (int s = 0; s < 2; ++s) {
-    const int ne = s ? hv.nb : hv.na, nv = n - ne;
-    for (int e = threadIdx.x; e < ne * nv; e += blockDim.x) {
-      const int i = E.occ[s][e / nv], a = E.vir[s][e % nv];
-      const int lo = 2 * min(i, a) + s, hi = 2 * max(i, a) + s;
-      E.sgn[s][e] = uint8_t(__popcll(x & ((1ull << hi) - 1ull) & ~((2ull << lo) - 1ull)) & 1);
-      E.si[s][e] = uint8_t(i);
-      E.sa[s][e] = uint8_t(a);
-      E.g[s][e] = uint32_t(a * n + i) * (s ? 1u : uint32_t(n * n));
-      if constexpr (RANK) {
-        const uint32_t t = E.str[s] ^ (1u << i) ^ (1u << a);
-        E.rank[s][e] = s ? __ldg(sv.rkb + (1u << n) + t) : __ldg(sv.rka + (1u << n) + t) * sv.nb_p[n];
-      }
-    }
-  }
-  if constexpr (RANK) {
-    if (threadIdx.x == 0) E.own[0] = __ldg(sv.rka + (1u << n) + oa) * sv.nb_p[n];
-    if (threadIdx.x == 32) E.own[1] = __ldg(sv.rkb + (1u << n) + ob);
-  }
-  __syncthreads();
-}
 
 // whether a determinant of the right electron counts lies in the sector (its
 // last slot is allowed after its prefix): always, without Z2 symmetries
@@ -416,11 +328,6 @@ __global__ void chunk_counts_kernel(const uint64_t* __restrict__ total, uint64_t
 // ---- E_loc ------------------------------------------------------------------------
 constexpr int ET = 128;
 
-__device__ __forceinline__ double Gi(const HamView& hv, int p, int q, int r, int s) {
-  const int n = hv.n;
-  return __ldg(hv.g + ((size_t(p) * n + q) * n + r) * n + s);
-}
-
 template <AmpMode MODE>
 __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView sv, NodeView nv,
                                                          const uint64_t* __restrict__ xs, Count n_x_, int splits,
@@ -536,13 +443,11 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
       for (uint32_t k = max(k0, kd) + threadIdx.x; k < k1; k += ET) {
         const uint32_t r = k - kd, ea = fdiv(dsb, r), eb = r - ea * nsb;
         const int i = E.si[0][ea], a = E.sa[0][ea], j = E.si[1][eb], b = E.sa[1][eb];
-        const int lo = min(i, a), hi = max(i, a);
-        // the beta move changes the occupation of J and B, which lie between I and A when lo <= . < hi
-        const int sg = E.sgn[0][ea] ^ E.sgn[1][eb] ^ int(j >= lo && j < hi) ^ int(b >= lo && b < hi);
+        const int sg = sign_ab(E, ea, eb, i, a, j, b);
         const double v = __ldg(hv.g + E.g[0][ea] + E.g[1][eb]);
         uint32_t idx = 0;
         if constexpr (RANK) idx = E.rank[0][ea] + E.rank[1][eb];
-        add(k, idx, E.str[0] ^ (1u << i) ^ (1u << a), E.str[1] ^ (1u << j) ^ (1u << b), min(lo, min(j, b)),
+        add(k, idx, E.str[0] ^ (1u << i) ^ (1u << a), E.str[1] ^ (1u << j) ^ (1u << b), min(min(i, a), min(j, b)),
             sg ? -v : v);
       }
       // same-spin doubles I<J -> A<B: [AI|BJ] - [AJ|BI], as I -> A then J -> B
@@ -553,10 +458,8 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         const uint32_t q = fdiv(dp[s], r), po = E.po[s][q], pv = E.pv[s][r - q * dp[s].d];
         const uint32_t nv_ = s ? nvb : nva;
         const int i = E.occ[s][po & 255u], j = E.occ[s][po >> 8], a = E.vir[s][pv & 255u], b = E.vir[s][pv >> 8];
-        const int lo = min(j, b), hi = max(j, b);
-        const int sg = E.sgn[s][(po & 255u) * nv_ + (pv & 255u)] ^ E.sgn[s][(po >> 8) * nv_ + (pv >> 8)] ^
-                       int(i > lo && i < hi) ^ int(a > lo && a < hi);
-        const double v = Gi(hv, a, i, b, j) - Gi(hv, a, j, b, i);
+        const int sg = sign_ss(E, s, po, pv, nv_, i, j, a, b);
+        const double v = Gint(hv, a, i, b, j) - Gint(hv, a, j, b, i);
         const uint32_t flip = (1u << i) ^ (1u << j) ^ (1u << a) ^ (1u << b);
         const uint32_t sa = E.str[0] ^ (s ? 0u : flip), sb = E.str[1] ^ (s ? flip : 0u);
         uint32_t idx = 0;
@@ -569,15 +472,7 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         const int s = k < hv.nsa ? 0 : 1;
         const uint32_t e = s ? k - hv.nsa : k;
         const int i = E.si[s][e], a = E.sa[s][e];
-        double v = __ldg(hv.h + a * n + i);
-        for (int t2 = 0; t2 < 2; ++t2) {
-          const int ne = t2 ? hv.nb : hv.na;
-          for (int m = 0; m < ne; ++m) {
-            const int jj = E.occ[t2][m];
-            v += Gi(hv, a, i, jj, jj);
-            if (t2 == s) v -= Gi(hv, a, jj, jj, i);
-          }
-        }
+        const double v = single_value(hv, E, s, i, a);
         uint32_t idx = 0;
         if constexpr (RANK) idx = s ? E.own[0] + E.rank[1][e] : E.rank[0][e] + E.own[1];
         const uint32_t flip = (1u << i) ^ (1u << a);
@@ -590,8 +485,8 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
             const int I = t / ne, J = t - I * ne;
             const int si = I < hv.na ? 0 : 1, sj = J < hv.na ? 0 : 1;
             const int i = E.occ[si][si ? I - hv.na : I], j = E.occ[sj][sj ? J - hv.na : J];
-            dg += 0.5 * Gi(hv, i, i, j, j);
-            if (si == sj) dg -= 0.5 * Gi(hv, i, j, j, i);
+            dg += 0.5 * Gint(hv, i, i, j, j);
+            if (si == sj) dg -= 0.5 * Gint(hv, i, j, j, i);
           } else {
             const int I = t - ne * ne;
             const int i = I < hv.na ? E.occ[0][I] : E.occ[1][I - hv.na];
