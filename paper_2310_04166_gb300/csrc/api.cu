@@ -234,8 +234,8 @@ static int check_adjoint(const anqs_model* M) {
 // model-specific adjoint workspace (bytes) beyond the two cotangent arrays;
 // with `least`, the smallest the adjoint accepts (the transformer then
 // recomputes each block's activations from the block's input)
-static size_t vjp_ws_bytes(const anqs_model* M, uint64_t n_x, bool least = false) {
-  if (M->d.kind == ANQS_MODEL_TF) return tf_grad_workspace(M->tf, n_x, least);
+static size_t vjp_ws_bytes(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool least = false) {
+  if (M->d.kind == ANQS_MODEL_TF) return tf_grad_workspace(M->tf, H, n_x, least);
   if (M->d.kind == ANQS_MODEL_NADE) return nade_grad_partial_floats(M->nade, M->n_params, n_x) * sizeof(float);
   return 0;
 }
@@ -250,7 +250,7 @@ static int vjp_dispatch(const anqs_model* M, const anqs_ham* H, const uint64_t* 
       return launch_mlp_tc_grad(M, H->v, x, n_x, c, grad, part, s);
     return launch_mlp_fp32_grad(M->mlp, H->v, x, n_x, c, grad, part, s);
   }
-  if (M->d.kind == ANQS_MODEL_TF) return launch_tf_fp32_grad(M->tf, H->v, x, n_x, cl, cp, grad, ws, ws_bytes, s);
+  if (M->d.kind == ANQS_MODEL_TF) return launch_tf_fp32_grad(M->tf, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
   if (M->d.kind == ANQS_MODEL_NADE)
     return launch_nade_grad(M->nade, H->v, x, n_x, CotSrc{cl, cp, nullptr, nullptr, nullptr, nullptr}, grad,
                             M->n_params, static_cast<float*>(ws), s);
@@ -395,16 +395,22 @@ static int build_index(anqs_ham* H) {
   for (int s = 0; s < 2; ++s) {
     const int ne = s ? H->v.nb : H->v.na;
     tab[s].assign(size_t(2) << n, 0u);
-    for (int p = 0; p <= n; ++p) {
+    // level p + 1's strings from level p's, in the order of the slots (slot 0
+    // first), so that neighbours share prefixes
+    std::vector<uint32_t> cur{0u}, nxt;
+    for (int p = 0;; ++p) {
       (s ? sv.sob : sv.soa)[p] = uint32_t(str[s].size());
-      uint32_t r = 0;
-      for (uint32_t v = 0; v < (1u << p); ++v) {
-        const int e = __builtin_popcount(v);
-        if (e > ne || e + (n - p) < ne) continue;
-        tab[s][(size_t(1) << p) + v] = r++;
-        str[s].push_back(v);
-      }
-      (s ? sv.nb_p : sv.na_p)[p] = r;
+      (s ? sv.nb_p : sv.na_p)[p] = uint32_t(cur.size());
+      for (size_t r = 0; r < cur.size(); ++r) tab[s][(size_t(1) << p) + cur[r]] = uint32_t(r);
+      str[s].insert(str[s].end(), cur.begin(), cur.end());
+      if (p == n) break;
+      nxt.clear();
+      for (uint32_t v : cur)
+        for (uint32_t bit = 0; bit < 2; ++bit) {
+          const int e = __builtin_popcount(v) + int(bit);
+          if (e <= ne && e + (n - p - 1) >= ne) nxt.push_back(v | bit << p);
+        }
+      cur.swap(nxt);
     }
   }
   uint64_t words = 0, below = 0;
@@ -417,37 +423,45 @@ static int build_index(anqs_ham* H) {
   }
   sv.woff[n + 1] = uint32_t(words);
   const uint64_t leaves = uint64_t(sv.na_p[n]) * sv.nb_p[n];
-  std::vector<uint32_t> all;
+  const bool full = below <= kPrefixTable && leaves <= 4 * kPrefixTable;
+  std::vector<uint64_t> xs;
+  if (full) {
+    auto spread = [](uint64_t x) {
+      x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
+      x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
+      x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
+      x = (x | (x << 2)) & 0x3333333333333333ull;
+      return (x | (x << 1)) & 0x5555555555555555ull;
+    };
+    xs.reserve(below + leaves);
+    for (int p = 0; p <= n; ++p) {
+      H->full_off.push_back(uint32_t(xs.size()));
+      for (uint32_t a = 0; a < sv.na_p[p]; ++a) {
+        const uint64_t xa = spread(str[0][sv.soa[p] + a]);
+        for (uint32_t b = 0; b < sv.nb_p[p]; ++b) xs.push_back(xa | spread(str[1][sv.sob[p] + b]) << 1);
+      }
+    }
+    H->full_off.push_back(uint32_t(xs.size()));
+  }
+  // one allocation and copy: prefixes | rank tables | strings | level offsets
+  std::vector<uint32_t> all(2 * xs.size());
+  if (full) memcpy(all.data(), xs.data(), xs.size() * sizeof(uint64_t));
+  const size_t rk0 = all.size();
   for (int s = 0; s < 2; ++s) all.insert(all.end(), tab[s].begin(), tab[s].end());
   const size_t st0 = all.size();
   for (int s = 0; s < 2; ++s) all.insert(all.end(), str[s].begin(), str[s].end());
+  const size_t of0 = all.size();
+  all.insert(all.end(), H->full_off.begin(), H->full_off.end());
   ANQS_CUDA(cudaMalloc(&H->d_idx, all.size() * sizeof(uint32_t)));
   ANQS_CUDA(cudaMemcpy(H->d_idx, all.data(), all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  sv.rka = H->d_idx;
-  sv.rkb = H->d_idx + tab[0].size();
+  H->d_full_x = reinterpret_cast<uint64_t*>(H->d_idx);
+  H->d_full_off = H->d_idx + of0;
+  sv.rka = H->d_idx + rk0;
+  sv.rkb = sv.rka + tab[0].size();
   sv.sta = H->d_idx + st0;
   sv.stb = sv.sta + str[0].size();
   H->has_index = true;
-  if (below > kPrefixTable || leaves > 4 * kPrefixTable) return ANQS_OK;
-  auto spread = [](uint32_t v) {
-    uint64_t x = 0;
-    for (int i = 0; i < 32; ++i) x |= uint64_t((v >> i) & 1u) << (2 * i);
-    return x;
-  };
-  std::vector<uint64_t> xs;
-  for (int p = 0; p <= n; ++p) {
-    H->full_off.push_back(uint32_t(xs.size()));
-    for (uint32_t a = 0; a < sv.na_p[p]; ++a)
-      for (uint32_t b = 0; b < sv.nb_p[p]; ++b)
-        xs.push_back(spread(str[0][sv.soa[p] + a]) | spread(str[1][sv.sob[p] + b]) << 1);
-  }
-  H->full_off.push_back(uint32_t(xs.size()));
-  ANQS_CUDA(cudaMalloc(&H->d_full_x, xs.size() * sizeof(uint64_t)));
-  ANQS_CUDA(cudaMemcpy(H->d_full_x, xs.data(), xs.size() * sizeof(uint64_t), cudaMemcpyHostToDevice));
-  ANQS_CUDA(cudaMalloc(&H->d_full_off, H->full_off.size() * sizeof(uint32_t)));
-  ANQS_CUDA(cudaMemcpy(H->d_full_off, H->full_off.data(), H->full_off.size() * sizeof(uint32_t),
-                       cudaMemcpyHostToDevice));
-  H->has_full = true;
+  H->has_full = full;
   return ANQS_OK;
 }
 
@@ -574,8 +588,6 @@ int anqs_hamiltonian_destroy(anqs_ham* H) {
   cudaFree(H->d_pt_child);
   cudaFree(H->d_status);
   cudaFree(H->d_idx);
-  cudaFree(H->d_full_x);
-  cudaFree(H->d_full_off);
   delete H;
   return ANQS_OK;
 }
@@ -1181,26 +1193,26 @@ int anqs_batch_autotune(anqs_batch* b, const anqs_eloc_problem* q, int n, void* 
   return ANQS_OK;
 }
 
-static size_t grad_ws_bytes(const anqs_model* M, uint64_t n_x, bool least) {
+static size_t grad_ws_bytes(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool least) {
   Arena A(nullptr, 0);
   A.take<float>(n_x);
   A.take<float>(n_x);
   if (M->d.kind == ANQS_MODEL_MLP) A.take<float>(mlp_fp32_grad_partial_floats(M->mlp, n_x));
-  A.take<char>(vjp_ws_bytes(M, n_x, least));
+  A.take<char>(vjp_ws_bytes(M, H, n_x, least));
   return A.off;
 }
 
 int anqs_grad_workspace_size(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
   ANQS_TRY(check_pair(M, H));
   if (!bytes) return set_error(ANQS_ERR_ARG, "null output");
-  *bytes = grad_ws_bytes(M, n_x, false);
+  *bytes = grad_ws_bytes(M, H, n_x, false);
   return ANQS_OK;
 }
 
 int anqs_grad_workspace_size_min(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
   ANQS_TRY(check_pair(M, H));
   if (!bytes) return set_error(ANQS_ERR_ARG, "null output");
-  *bytes = grad_ws_bytes(M, n_x, true);
+  *bytes = grad_ws_bytes(M, H, n_x, true);
   return ANQS_OK;
 }
 
@@ -1215,12 +1227,12 @@ int anqs_grad(const anqs_model* M, const anqs_ham* H, const uint64_t* x, const u
   float* cl = A.take<float>(n_x);
   float* cp = A.take<float>(n_x);
   float* part = (M->d.kind == ANQS_MODEL_MLP) ? A.take<float>(mlp_fp32_grad_partial_floats(M->mlp, n_x)) : nullptr;
-  size_t tfb = vjp_ws_bytes(M, n_x);
+  size_t tfb = vjp_ws_bytes(M, H, n_x);
   const size_t off0 = A.off;
   void* tfws = tfb ? A.take<char>(tfb) : nullptr;
   if (!A.fits() && tfb) {  // too small for every activation: the recomputing adjoint
     A.off = off0;
-    tfb = vjp_ws_bytes(M, n_x, true);
+    tfb = vjp_ws_bytes(M, H, n_x, true);
     tfws = A.take<char>(tfb);
   }
   if (!A.fits() || !ws) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
@@ -1243,7 +1255,7 @@ int anqs_grad(const anqs_model* M, const anqs_ham* H, const uint64_t* x, const u
 int anqs_logpsi_vjp_workspace_size(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
   ANQS_TRY(check_pair(M, H));
   if (!bytes) return set_error(ANQS_ERR_ARG, "null output");
-  *bytes = vjp_ws_bytes(M, n_x);
+  *bytes = vjp_ws_bytes(M, H, n_x);
   return ANQS_OK;
 }
 
@@ -1253,7 +1265,7 @@ int anqs_logpsi_vjp(const anqs_model* M, const anqs_ham* H, const uint64_t* x, u
   if (!grad) return set_error(ANQS_ERR_ARG, "null gradient output");
   if (n_x && (!x || !cl || !cp)) return set_error(ANQS_ERR_ARG, "null array argument");
   ANQS_TRY(check_adjoint(M));
-  const size_t need = vjp_ws_bytes(M, n_x, true);  // with less than vjp_ws_bytes(M, n_x) the transformer recomputes
+  const size_t need = vjp_ws_bytes(M, H, n_x, true);  // with less than vjp_ws_bytes(M, H, n_x) the transformer recomputes
   if (ws_bytes < need || (need && !ws)) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
   cudaStream_t s = (cudaStream_t)stream;
   ANQS_CUDA(cudaMemsetAsync(grad, 0, M->n_params * sizeof(float), s));

@@ -392,9 +392,9 @@ struct anqs_ham {
   // small sectors, the list of all prefixes with its level offsets
   bool has_index = false, has_full = false;
   SectorView sv{};
-  uint32_t* d_idx = nullptr;        // rank and string tables
-  uint64_t* d_full_x = nullptr;     // all prefixes of levels 0..n
-  uint32_t* d_full_off = nullptr;   // [n + 2]
+  uint32_t* d_idx = nullptr;        // one allocation: rank and string tables and
+  uint64_t* d_full_x = nullptr;     // all prefixes of levels 0..n,
+  uint32_t* d_full_off = nullptr;   // their level offsets [n + 2]
   std::vector<uint32_t> full_off;
   unsigned* d_status;  // HamView::status
   double* d_h;
@@ -483,8 +483,8 @@ int launch_tf_fp32_variants(const TfView& m, const HamView& hv, const uint64_t* 
                             cudaStream_t s);
 int launch_tf_fp32_slot_logits(const TfView& m, int p, const uint64_t* pre, const uint64_t* nr, uint64_t max_rows,
                                float* out, cudaStream_t s);
-size_t tf_grad_workspace(const TfView& m, uint64_t n_x, bool recompute);  // recompute: block inputs only
-int launch_tf_fp32_grad(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, const float* cl,
+size_t tf_grad_workspace(const TfView& m, const anqs_ham* H, uint64_t n_x, bool recompute);  // recompute: block inputs only
+int launch_tf_fp32_grad(const TfView& m, const anqs_ham* H, const uint64_t* x, Count n_x, const float* cl,
                         const float* cp, float* grad, void* ws, size_t ws_bytes, cudaStream_t s);
 int launch_table_logpsi(const anqs_model* md, const HamView& hv, const uint64_t* x, Count n_x,
                         float* la, float* ph, cudaStream_t s);
@@ -547,6 +547,20 @@ struct AmpSrc {
   uint32_t variants = 1;
 };
 uint64_t eloc_partials(const anqs_ham* H, uint64_t n_x);  // doubles
+
+// The distinct prefixes of the samples themselves, levels 0..n-1 (off [n + 1])
+struct TreeWs {
+  NodeView nodes;
+  uint64_t max_rows;
+  uint64_t* n_rows;   // device count
+  size_t zero_bytes;  // n_rows and the bitmap
+  uint32_t *bits, *bsum, *off;
+  uint2* packed;
+  uint64_t* node_x;
+};
+bool tree_applies(const anqs_ham* H);
+void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w);
+int launch_tree(const anqs_ham* H, const uint64_t* x, Count n_x, const TreeWs& w, cudaStream_t s);
 // E_loc and (counts set) the statistics; the ticket must be zero
 int launch_eloc_direct(const anqs_ham* H, const uint64_t* x, Count n_x, const NodeView& nodes, const AmpSrc& amp,
                        double* ere, double* eim, double* part, const StatsOut& so, cudaStream_t s);

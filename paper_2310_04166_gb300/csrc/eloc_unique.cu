@@ -119,6 +119,23 @@ __global__ void __launch_bounds__(MT_) mark_kernel(HamView hv, SectorView sv, co
   }
 }
 
+// the prefixes of the samples alone (one thread per sample)
+__global__ void mark_samples_kernel(HamView hv, SectorView sv, const uint64_t* __restrict__ xs, Count n_x_,
+                                    uint32_t* __restrict__ bits) {
+  ANQS_PDL_ENTRY();
+  const uint64_t n_x = n_x_.get();
+  const int n = sv.n;
+  for (uint64_t l = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; l < n_x; l += uint64_t(gridDim.x) * blockDim.x) {
+    const uint64_t x = xs[l];
+    const uint32_t a = even_bits(x), b = even_bits(x >> 1);
+    if (__popc(a) != hv.na || __popc(b) != hv.nb || (x >> (2 * n)) != 0 || !in_sector(hv, a, b)) continue;
+    for (int p = n - 1; p >= 0; --p) {
+      const uint32_t i = prefix_index(sv, p, a, b);
+      if (!set_bit(bits + sv.woff[p] + (i >> 5), 1u << (i & 31u))) break;
+    }
+  }
+}
+
 constexpr int CT = 256;      // threads of the count and emit kernels
 constexpr uint32_t CW = 4096;  // bitmap words per CTA
 
@@ -152,12 +169,13 @@ __global__ void __launch_bounds__(CT) count_kernel(const uint32_t* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, const uint32_t* __restrict__ bits, uint32_t words,
+// words: those of the levels below `levels`; writes off[0 .. levels]
+__global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, int levels, const uint32_t* __restrict__ bits, uint32_t words,
                                                   const uint32_t* __restrict__ bsum, uint2* __restrict__ packed,
                                                   uint64_t* __restrict__ node_x, uint32_t* __restrict__ off) {
   ANQS_PDL_ENTRY();
   __shared__ uint32_t s_base, s_warp[CT / 32];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, n = sv.n;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_base = 0;
   __syncthreads();
   {  // nodes before this CTA's words
@@ -193,7 +211,7 @@ __global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, const uint32_t*
       int p = 0;
       while (w >= sv.woff[p + 1]) ++p;
       if (w == sv.woff[p]) off[p] = id;
-      if (w + 1 == words) off[n + 1] = id + c;
+      if (w + 1 == words) off[levels] = id + c;
       const uint32_t i0 = (w - sv.woff[p]) * 32u, nb = sv.nb_p[p];
       while (v) {
         const uint32_t idx = i0 + uint32_t(__ffs(v)) - 1u;
@@ -627,7 +645,7 @@ int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueW
   const uint32_t words = uint32_t(index_words(H));
   const unsigned blocks = (words + CW - 1) / CW;
   ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, H->sv.woff[H->v.n], w.bsum, reinterpret_cast<unsigned long long*>(w.n_leaves)));
-  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, w.bits, words, w.bsum, w.packed, w.node_x, w.off));
+  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n + 1, w.bits, words, w.bsum, w.packed, w.node_x, w.off));
   return ANQS_OK;
 }
 
@@ -657,6 +675,35 @@ const uint64_t* unique_leaf_x(const anqs_ham* H, const UniqueWs& w) {
 bool use_unique(const anqs_ham* H, bool preferred, size_t plain, size_t unique, size_t ws_bytes) {
   if (!H->has_index) return false;
   return preferred ? unique <= ws_bytes || plain > ws_bytes : plain > ws_bytes && unique <= ws_bytes;
+}
+
+// the samples' prefixes; 2^21 bitmap words cost about 20 us to clear and scan
+bool tree_applies(const anqs_ham* H) { return H->has_index && H->sv.woff[H->v.n] <= (1u << 21); }
+
+void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w) {
+  const int n = H->v.n;
+  const uint32_t words = H->sv.woff[n];
+  w = TreeWs{};
+  for (int p = 0; p < n; ++p) w.max_rows += std::min<uint64_t>(uint64_t(H->sv.na_p[p]) * H->sv.nb_p[p], n_x);
+  w.zero_bytes = 256 + words * sizeof(uint32_t);
+  char* z = A.take<char>(w.zero_bytes);
+  w.n_rows = reinterpret_cast<uint64_t*>(z);
+  w.bits = z ? reinterpret_cast<uint32_t*>(z + 256) : nullptr;
+  w.packed = A.take<uint2>(words);
+  w.bsum = A.take<uint32_t>((words + CW - 1) / CW);
+  w.node_x = A.take<uint64_t>(w.max_rows);
+  w.off = A.take<uint32_t>(n + 1);
+  w.nodes = NodeView{w.node_x, w.off, w.packed};
+}
+
+int launch_tree(const anqs_ham* H, const uint64_t* x, Count n_x, const TreeWs& w, cudaStream_t s) {
+  const uint32_t words = H->sv.woff[H->v.n];
+  const unsigned blocks = (words + CW - 1) / CW;
+  ANQS_CUDA(cudaMemsetAsync(w.n_rows, 0, w.zero_bytes, s));
+  ANQS_CUDA_LAUNCH("mark_samples_kernel", launch_k(mark_samples_kernel, dim3(unsigned(std::min<uint64_t>((n_x.n + 63) / 64, 152 * 16))), dim3(64), 0, s, H->v, H->sv, x, n_x, w.bits));
+  ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, 0u, w.bsum, reinterpret_cast<unsigned long long*>(w.n_rows)));
+  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n, w.bits, words, w.bsum, w.packed, w.node_x, w.off));
+  return ANQS_OK;
 }
 
 Count unique_leaves(const UniqueWs& w) {

@@ -3,9 +3,9 @@
 // product of sum_l [cot_la_l log|psi(x_l)| + cot_ph_l arg psi(x_l)] with the
 // cotangents 2 w_l Re(E_loc,l - E) and 2 w_l Im(E_loc,l - E).
 //
-// The unique samples are few (thousands) while each has n positions, so the
-// adjoint runs as batched passes over all R = n_x * n rows (sample,
-// position) with every activation of the forward stored in the workspace
+// The adjoint runs as batched passes over all rows (struct Rows: distinct
+// prefixes of the samples, or (sample, position) pairs) with every activation
+// of the forward stored in the workspace
 // (or, when the workspace is too small for that, only the block inputs, each
 // block's activations being recomputed from its input before its backward):
 // embedding; per block LN1, q|k|v, causal attention (probabilities kept),
@@ -22,126 +22,237 @@
 namespace anqs {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, GT = 256;
+// The rows of a pass, one per distinct prefix of the samples ("node", tree
+// form) or one per (sample, position) (flat form).  Positions see only the
+// tokens before them, so samples that share a prefix share its activations,
+// and the cotangents of its outputs add up: 10,816 samples x 10 positions of
+// the 20-qubit workload are 27,000 distinct prefixes.
+struct Rows {
+  const uint64_t* x;    // prefix bits (higher bits may be set)
+  const uint8_t* lv;    // position
+  const uint32_t* anc;  // [row][n]: rows of positions 0..lv of the same sequence (anc[lv] = row)
+  Count rows;
+  int n;
+};
+
+__global__ void flat_rows_kernel(const uint64_t* __restrict__ xs, Count rows_, int n, uint64_t* __restrict__ x,
+                                 uint8_t* __restrict__ lv, uint32_t* __restrict__ anc) {
+  ANQS_PDL_ENTRY();
+  const uint64_t rows = rows_.get();
+  for (uint64_t r = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; r < rows; r += uint64_t(gridDim.x) * blockDim.x) {
+    const uint64_t s = r / n;
+    const int t = int(r - s * n);
+    x[r] = xs[s];
+    lv[r] = uint8_t(t);
+    for (int u = 0; u <= t; ++u) anc[r * n + u] = uint32_t(s * n + u);
+  }
+}
+
+__global__ void tree_rows_kernel(SectorView sv, NodeView nv, uint8_t* __restrict__ lv, uint32_t* __restrict__ anc) {
+  ANQS_PDL_ENTRY();
+  const int n = sv.n;
+  const uint32_t rows = __ldcg(nv.off + n);
+  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
+    const uint64_t x = __ldcg(reinterpret_cast<const unsigned long long*>(nv.x) + r);
+    const uint32_t a = even_bits(x), b = even_bits(x >> 1);
+    int p = 0;
+    while (r >= __ldcg(nv.off + p + 1)) ++p;
+    lv[r] = uint8_t(p);
+    for (int u = 0; u < p; ++u) anc[size_t(r) * n + u] = node_id(sv, nv, u, prefix_index(sv, u, a, b));
+    anc[size_t(r) * n + p] = r;
+  }
+}
+
+constexpr int BM = 128, BN = 64, BK = 16, GT = 256;
+
+// A matrix whose rows come in segments (the q, k and v weights lie one
+// behind the other with their biases between): row i starts at
+// (i / seg) * stride + (i % seg) * ld.
+struct Seg {
+  int seg;
+  size_t stride;
+};
 
 struct Gm {
   const float* A;
   int lda;
   const float* B;
   int ldb;
+  Seg sb;            // segments of B's rows
   float* C;
   int ldc;
+  Seg sc;            // segments of C's rows (weight products)
   const float* Cin;  // residual input (may alias C), or null
   int ldcin;
-  const float* bias;  // per column, or null
+  const float* bias;  // per column (segments as B's), or null
   const float* mask;  // result zeroed where mask <= 0, or null
   int ldmask;
-  Count M, K;  // M (rows) and K may be device counts
+  float* colsum;      // += the sums of A's columns (weight products: the bias gradient; segments as C's), or null
+  Count M, K;         // M (rows) and K may be device counts
   int N;
   int relu_a, relu_b, atomic;
-  uint64_t k_chunk;  // split-K: K range per blockIdx.z
+  int b_vec;          // B and bias are 16-byte aligned (parameters may be any float tensor, say a slice)
+  uint64_t k_chunk;   // split-K: K range per blockIdx.z
 };
 
+__device__ __forceinline__ float4 ld4(const float* p, int vec) {
+  if (vec) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+
+__device__ __forceinline__ size_t seg_row(const Seg& s, int i, int ld) {
+  return s.seg ? size_t(i / s.seg) * s.stride + size_t(i % s.seg) * ld : size_t(i) * ld;
+}
+
 // C[m][n] = sum_k opA(m, k) opB(k, n), opA(m, k) = A[m][k] (TA: A[k][m]),
-// opB(k, n) = B[k][n] (TB: B[n][k]).  64 x 64 tile per CTA, 4 x 4 per thread.
+// opB(k, n) = B[k][n] (TB: B[n][k]).  128 x 64 tile per CTA, 8 x 4 per thread
+// (3 16-byte shared loads for 32 FMAs; a 4 x 4 tile is bound by its shared
+// loads), the next K step's operands loaded to registers while this one runs.
+// All leading dimensions, segments and widths are multiples of 4 floats.
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
   ANQS_PDL_ENTRY();
-  __shared__ __align__(16) float As[BK][BM + 4];
-  __shared__ __align__(16) float Bs[BK][BN + 4];
+  __shared__ __align__(16) float As[2][BK][BM + 4];
+  __shared__ __align__(16) float Bs[2][BK][BN + 4];
   const uint64_t M = g.M.get(), K = g.K.get();
   const uint64_t m0 = uint64_t(blockIdx.y) * BM;
-  const int n0 = blockIdx.x * BN;
+  const int n0 = blockIdx.x * BN, tid = threadIdx.x;
   if (m0 >= M) return;
   const uint64_t k_lo = uint64_t(blockIdx.z) * g.k_chunk;
   if (k_lo >= K && !(k_lo == 0)) return;
   const uint64_t k_hi = k_lo + g.k_chunk < K ? k_lo + g.k_chunk : K;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[4][4] = {};
+  const int tx = tid % 16, ty = tid / 16;
+  float4 ra[2], rb;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  // A: 128 x 16 elements, two 4-vectors per thread; B: 16 x 64, one
+  auto load = [&](uint64_t k0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = tid + GT * i;
+      ra[i] = zero;
+      if (TA) {  // [k][m]: vectors along m
+        const uint64_t m = m0 + uint64_t(e % 32) * 4, k = k0 + e / 32;
+        if (k < k_hi) {
+          const float* p = g.A + k * g.lda + m;
+          if (m + 4 <= M) ra[i] = *reinterpret_cast<const float4*>(p);
+          else {
+            if (m < M) ra[i].x = p[0];
+            if (m + 1 < M) ra[i].y = p[1];
+            if (m + 2 < M) ra[i].z = p[2];
+          }
+        }
+      } else {  // [m][k]: vectors along k
+        const uint64_t m = m0 + e / 4, k = k0 + uint64_t(e % 4) * 4;
+        if (m < M && k + 4 <= k_hi) ra[i] = *reinterpret_cast<const float4*>(g.A + m * g.lda + k);
+      }
+      if (g.relu_a) {
+        ra[i].x = fmaxf(ra[i].x, 0.f), ra[i].y = fmaxf(ra[i].y, 0.f);
+        ra[i].z = fmaxf(ra[i].z, 0.f), ra[i].w = fmaxf(ra[i].w, 0.f);
+      }
+    }
+    rb = zero;
+    if (TB) {  // [n][k]: vectors along k
+      const int n = n0 + tid / 4;
+      const uint64_t k = k0 + uint64_t(tid % 4) * 4;
+      if (n < g.N && k + 4 <= k_hi) rb = ld4(g.B + seg_row(g.sb, n, g.ldb) + k, g.b_vec);
+    } else {  // [k][n]: vectors along n
+      const int n = n0 + (tid % 16) * 4;
+      const uint64_t k = k0 + tid / 16;
+      if (k < k_hi && n < g.N) rb = ld4(g.B + (g.sb.seg ? seg_row(g.sb, int(k), g.ldb) : k * g.ldb) + n, g.b_vec);
+    }
+    if (g.relu_b) {
+      rb.x = fmaxf(rb.x, 0.f), rb.y = fmaxf(rb.y, 0.f);
+      rb.z = fmaxf(rb.z, 0.f), rb.w = fmaxf(rb.w, 0.f);
+    }
+  };
+  auto store = [&](int b) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = tid + GT * i;
+      if (TA) {
+        *reinterpret_cast<float4*>(&As[b][e / 32][(e % 32) * 4]) = ra[i];
+      } else {
+        const int m = e / 4, k = (e % 4) * 4;
+        As[b][k][m] = ra[i].x, As[b][k + 1][m] = ra[i].y, As[b][k + 2][m] = ra[i].z, As[b][k + 3][m] = ra[i].w;
+      }
+    }
+    if (TB) {
+      const int n = tid / 4, k = (tid % 4) * 4;
+      Bs[b][k][n] = rb.x, Bs[b][k + 1][n] = rb.y, Bs[b][k + 2][n] = rb.z, Bs[b][k + 3][n] = rb.w;
+    } else {
+      *reinterpret_cast<float4*>(&Bs[b][tid / 16][(tid % 16) * 4]) = rb;
+    }
+  };
+  float acc[8][4] = {}, cs = 0.f;
+  const bool sums = g.colsum && blockIdx.x == 0;
+  load(k_lo);
+  store(0);
+  __syncthreads();
+  int b = 0;
   for (uint64_t k0 = k_lo; k0 < k_hi; k0 += BK) {
-    // A tile: BM x BK elements, 4 per thread
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = threadIdx.x + GT * i;
-      int mm, kk;
-      if (TA) {  // consecutive threads along m
-        mm = e % BM;
-        kk = e / BM;
-      } else {  // consecutive threads along k
-        kk = e % BK;
-        mm = e / BK;
-      }
-      const uint64_t m = m0 + mm, k = k0 + kk;
-      float v = 0.f;
-      if (m < M && k < k_hi) v = TA ? g.A[k * g.lda + m] : g.A[m * g.lda + k];
-      if (g.relu_a) v = fmaxf(v, 0.f);
-      As[kk][mm] = v;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = threadIdx.x + GT * i;
-      int nn, kk;
-      if (TB) {  // B[n][k]: consecutive threads along k
-        kk = e % BK;
-        nn = e / BK;
-      } else {  // B[k][n]: consecutive threads along n
-        nn = e % BN;
-        kk = e / BN;
-      }
-      const int n = n0 + nn;
-      const uint64_t k = k0 + kk;
-      float v = 0.f;
-      if (n < g.N && k < k_hi) v = TB ? g.B[uint64_t(n) * g.ldb + k] : g.B[k * g.ldb + n];
-      if (g.relu_b) v = fmaxf(v, 0.f);
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
+    const bool more = k0 + BK < k_hi;
+    if (more) load(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8 + 4]);
+      const float4 bb = *reinterpret_cast<const float4*>(&Bs[b][kk][tx * 4]);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
+    if (sums && tid < BM)
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) cs += As[b][kk][tid];
+    if (more) store(b ^ 1);
     __syncthreads();
+    b ^= 1;
   }
+  if (sums && tid < BM && m0 + tid < M) atomicAdd(g.colsum + seg_row(g.sc, int(m0 + tid), 1), cs);
+  const int n = n0 + tx * 4;
+  if (n >= g.N) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint64_t m = m0 + ty * 4 + i;
-    if (m >= M) continue;
+  for (int i = 0; i < 8; ++i) {
+    const uint64_t m = m0 + ty * 8 + i;
+    if (m >= M) break;
+    float* c = g.C + (g.sc.seg ? seg_row(g.sc, int(m), g.ldc) : m * g.ldc) + n;
+    if (g.atomic) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= g.N) continue;
-      float v = acc[i][j];
-      if (g.atomic) {
-        atomicAdd(g.C + m * g.ldc + n, v);
-        continue;
-      }
-      if (g.bias) v += g.bias[n];
-      if (g.Cin) v += g.Cin[m * g.ldcin + n];
-      if (g.mask && !(g.mask[m * g.ldmask + n] > 0.f)) v = 0.f;
-      g.C[m * g.ldc + n] = v;
+      for (int j = 0; j < 4; ++j) atomicAdd(c + j, acc[i][j]);
+      continue;
     }
+    float4 v = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    if (g.bias) {
+      const float4 t = ld4(g.bias + seg_row(g.sb, n, 1), g.b_vec);
+      v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
+    }
+    if (g.Cin) {
+      const float4 t = *reinterpret_cast<const float4*>(g.Cin + m * g.ldcin + n);
+      v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
+    }
+    if (g.mask) {
+      const float4 t = *reinterpret_cast<const float4*>(g.mask + m * g.ldmask + n);
+      v.x = t.x > 0.f ? v.x : 0.f, v.y = t.y > 0.f ? v.y : 0.f;
+      v.z = t.z > 0.f ? v.z : 0.f, v.w = t.w > 0.f ? v.w : 0.f;
+    }
+    *reinterpret_cast<float4*>(c) = v;
   }
 }
 
-// h0[r] = tok[token(r)] + pos[t], r = s n + t
-__global__ void embed_kernel(TfView m, const uint64_t* __restrict__ x, Count rows_, float* __restrict__ h0) {
+// h0[r] = tok[token(r)] + pos[position of r]
+__global__ void embed_kernel(TfView m, Rows R, float* __restrict__ h0) {
   ANQS_PDL_ENTRY();
-  const uint64_t rows = rows_.get();
-  const int D = m.d, n = m.n;
+  const uint64_t rows = R.rows.get();
+  const int D = m.d;
   const float* tok = m.params;
   const float* pos = m.params + 5 * size_t(D);
   for (uint64_t idx = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; idx < rows * D;
        idx += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t r = idx / D;
-    const int c = int(idx % D), t = int(r % n);
-    const uint64_t s = r / n;
-    const int token = t == 0 ? 4 : int((x[s] >> (2 * (t - 1))) & 3ull);
+    const int c = int(idx % D), t = R.lv[r];
+    const int token = t == 0 ? 4 : int((R.x[r] >> (2 * (t - 1))) & 3ull);
     h0[idx] = tok[token * D + c] + pos[t * D + c];
   }
 }
@@ -241,40 +352,36 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(const float* __restrict__ d
   }
 }
 
-// out[c] += sum_r X[r][c] for c < N
-__global__ void __launch_bounds__(256) colsum_kernel(const float* __restrict__ X, int N, Count rows_,
-                                                     float* __restrict__ out) {
+// Causal attention of one (row, head) per thread over the row's ancestors;
+// keeps the probabilities P[r][h][u].  qkv [row][3 D].  V4: the head width is
+// a multiple of 4.  The heads of a row are neighbouring threads, so a warp
+// reads whole key and value rows.
+template <bool V4>
+__global__ void attn_fwd_kernel(const float* __restrict__ qkv, float* __restrict__ P, float* __restrict__ O, int D,
+                                int H, Rows R) {
   ANQS_PDL_ENTRY();
-  const uint64_t rows = rows_.get();
-  for (int c0 = 0; c0 < N; c0 += 256) {
-    const int c = c0 + threadIdx.x;
-    if (c >= N) break;
-    float s = 0.f;
-    for (uint64_t r = blockIdx.x; r < rows; r += gridDim.x) s += X[r * N + c];
-    atomicAdd(out + c, s);
-  }
-}
-
-// causal attention of one (sample, head, query t) per thread; keeps the
-// probabilities P[s][h][t][u] (zero for u > t)
-__global__ void attn_fwd_kernel(const float* __restrict__ Q, const float* __restrict__ Kt,
-                                const float* __restrict__ V, float* __restrict__ P, float* __restrict__ O, int n,
-                                int D, int H, Count nx_) {
-  ANQS_PDL_ENTRY();
-  const uint64_t nx = nx_.get();
-  const int dh = D / H;
+  const uint64_t rows = R.rows.get();
+  const int dh = D / H, n = R.n;
   const float scale = 1.0f / sqrtf(float(dh));
-  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < nx * H * n;
+  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < rows * H;
        task += uint64_t(gridDim.x) * blockDim.x) {
-    const int t = int(task % n), hd = int((task / n) % H);
-    const uint64_t s = task / (uint64_t(n) * H);
-    const float* q = Q + (s * n + t) * D + hd * dh;
+    const uint64_t r = task / H;
+    const int hd = int(task - r * H), t = R.lv[r];
+    const float* q = qkv + r * 3 * D + hd * dh;
+    const uint32_t* anc = R.anc + r * n;
     float* prow = P + task * n;
     float mx = -INFINITY;
     for (int u = 0; u <= t; ++u) {
-      const float* k = Kt + (s * n + u) * D + hd * dh;
+      const float* k = qkv + size_t(anc[u]) * 3 * D + D + hd * dh;
       float dot = 0.f;
-      for (int e = 0; e < dh; ++e) dot = fmaf(q[e], k[e], dot);
+      if constexpr (V4) {
+        for (int e = 0; e < dh; e += 4) {
+          const float4 a = *reinterpret_cast<const float4*>(q + e), b = *reinterpret_cast<const float4*>(k + e);
+          dot = fmaf(a.x, b.x, dot), dot = fmaf(a.y, b.y, dot), dot = fmaf(a.z, b.z, dot), dot = fmaf(a.w, b.w, dot);
+        }
+      } else {
+        for (int e = 0; e < dh; ++e) dot = fmaf(q[e], k[e], dot);
+      }
       prow[u] = dot * scale;
       mx = fmaxf(mx, dot * scale);
     }
@@ -285,121 +392,249 @@ __global__ void attn_fwd_kernel(const float* __restrict__ Q, const float* __rest
       sum += p;
     }
     const float inv = 1.0f / sum;
-    for (int u = 0; u < n; ++u) prow[u] = u <= t ? prow[u] * inv : 0.f;
-    float* o = O + (s * n + t) * D + hd * dh;
-    for (int e = 0; e < dh; ++e) {
-      float a = 0.f;
-      for (int u = 0; u <= t; ++u) a = fmaf(prow[u], V[(s * n + u) * D + hd * dh + e], a);
-      o[e] = a;
-    }
-  }
-}
-
-// backward of the attention of one (sample, head): dQ, dK, dV (written)
-__global__ void attn_bwd_kernel(const float* __restrict__ Q, const float* __restrict__ Kt,
-                                const float* __restrict__ V, const float* __restrict__ P,
-                                const float* __restrict__ dO, float* __restrict__ dQ, float* __restrict__ dK,
-                                float* __restrict__ dV, int n, int D, int H, Count nx_) {
-  ANQS_PDL_ENTRY();
-  const uint64_t nx = nx_.get();
-  const int dh = D / H;
-  const float scale = 1.0f / sqrtf(float(dh));
-  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < nx * H;
-       task += uint64_t(gridDim.x) * blockDim.x) {
-    const int hd = int(task % H);
-    const uint64_t s = task / H;
-    const uint64_t rb = s * n;
-    for (int u = 0; u < n; ++u)
-      for (int e = 0; e < dh; ++e) {
-        dK[(rb + u) * D + hd * dh + e] = 0.f;
-        dV[(rb + u) * D + hd * dh + e] = 0.f;
-      }
-    for (int t = 0; t < n; ++t) {
-      const float* prow = P + (task * n + t) * n;
-      const float* go = dO + (rb + t) * D + hd * dh;
-      // dP_u = dO_t . V_u ; dS_u = P_u (dP_u - sum_u' P_u' dP_u')
-      float dp[32];
-      float dot = 0.f;
+    for (int u = 0; u <= t; ++u) prow[u] *= inv;
+    float* o = O + r * D + hd * dh;
+    constexpr int S = V4 ? 4 : 1;
+    for (int e = 0; e < dh; e += S) {
+      float a[S] = {};
       for (int u = 0; u <= t; ++u) {
-        float a = 0.f;
-        for (int e = 0; e < dh; ++e) a = fmaf(go[e], V[(rb + u) * D + hd * dh + e], a);
-        dp[u] = a;
-        dot = fmaf(prow[u], a, dot);
-      }
-      const float* q = Q + (rb + t) * D + hd * dh;
-      float* gq = dQ + (rb + t) * D + hd * dh;
-      for (int e = 0; e < dh; ++e) gq[e] = 0.f;
-      for (int u = 0; u <= t; ++u) {
-        const float ds = prow[u] * (dp[u] - dot) * scale;
-        const float* k = Kt + (rb + u) * D + hd * dh;
-        float* gk = dK + (rb + u) * D + hd * dh;
-        float* gv = dV + (rb + u) * D + hd * dh;
-        for (int e = 0; e < dh; ++e) {
-          gq[e] = fmaf(ds, k[e], gq[e]);
-          gk[e] = fmaf(ds, q[e], gk[e]);
-          gv[e] = fmaf(prow[u], go[e], gv[e]);
+        const float p = prow[u];
+        const float* v = qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh + e;
+        if constexpr (V4) {
+          const float4 w = *reinterpret_cast<const float4*>(v);
+          a[0] = fmaf(p, w.x, a[0]), a[1] = fmaf(p, w.y, a[1]), a[2] = fmaf(p, w.z, a[2]), a[3] = fmaf(p, w.w, a[3]);
+        } else {
+          a[0] = fmaf(p, v[0], a[0]);
         }
       }
+#pragma unroll
+      for (int i = 0; i < S; ++i) o[e + i] = a[i];
     }
   }
 }
 
-// head cotangents: d out8[r] from the masked log-softmax of every slot
-__global__ void head_dout_kernel(HamView hv, const uint64_t* __restrict__ x, Count nx_,
-                                 const float* __restrict__ out8, const float* __restrict__ cl,
-                                 const float* __restrict__ cp, float* __restrict__ dout8, int n) {
+// Backward of the attention of one (row, head): dS[r][h][u] (with the score
+// scale) and dQ.  dP_u = dO . V_u; dS_u = P_u (dP_u - sum_u' P_u' dP_u') scale.
+// The row's dQ | dK | dV slots hold dQ after it; dK and dV are zeroed here for
+// attn_bwd_kv_kernel.
+template <bool V4>
+__global__ void attn_bwd_q_kernel(const float* __restrict__ qkv, const float* __restrict__ P,
+                                  const float* __restrict__ dO, float* __restrict__ dS, float* __restrict__ dqkv, int D,
+                                  int H, Rows R) {
+  ANQS_PDL_ENTRY();
+  const uint64_t rows = R.rows.get();
+  const int dh = D / H, n = R.n;
+  const float scale = 1.0f / sqrtf(float(dh));
+  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < rows * H;
+       task += uint64_t(gridDim.x) * blockDim.x) {
+    const uint64_t r = task / H;
+    const int hd = int(task - r * H), t = R.lv[r];
+    const uint32_t* anc = R.anc + r * n;
+    const float* prow = P + task * n;
+    float* srow = dS + task * n;
+    const float* go = dO + r * D + hd * dh;
+    float dot = 0.f;
+    for (int u = 0; u <= t; ++u) {
+      const float* v = qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh;
+      float a = 0.f;
+      if constexpr (V4) {
+        for (int e = 0; e < dh; e += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(go + e), y = *reinterpret_cast<const float4*>(v + e);
+          a = fmaf(x.x, y.x, a), a = fmaf(x.y, y.y, a), a = fmaf(x.z, y.z, a), a = fmaf(x.w, y.w, a);
+        }
+      } else {
+        for (int e = 0; e < dh; ++e) a = fmaf(go[e], v[e], a);
+      }
+      srow[u] = a;
+      dot = fmaf(prow[u], a, dot);
+    }
+    for (int u = 0; u <= t; ++u) srow[u] = prow[u] * (srow[u] - dot) * scale;
+    float* gq = dqkv + r * 3 * D + hd * dh;
+    constexpr int S = V4 ? 4 : 1;
+    for (int e = 0; e < dh; e += S) {
+      float a[S] = {};
+      for (int u = 0; u <= t; ++u) {
+        const float ds = srow[u];
+        const float* k = qkv + size_t(anc[u]) * 3 * D + D + hd * dh + e;
+        if constexpr (V4) {
+          const float4 w = *reinterpret_cast<const float4*>(k);
+          a[0] = fmaf(ds, w.x, a[0]), a[1] = fmaf(ds, w.y, a[1]), a[2] = fmaf(ds, w.z, a[2]), a[3] = fmaf(ds, w.w, a[3]);
+        } else {
+          a[0] = fmaf(ds, k[0], a[0]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < S; ++i) {
+        gq[e + i] = a[i];
+        gq[D + e + i] = 0.f;
+        gq[2 * D + e + i] = 0.f;
+      }
+    }
+  }
+}
+
+// dK_u = sum over the rows r below key u of dS[r][u] q_r, dV_u = the same of
+// P[r][u] dO_r.  A CTA takes KVR consecutive rows and one ancestor level;
+// thread = column (dK's, then dV's).  Rows of one level are ordered so that
+// neighbours mostly share their ancestors: the sums stay in a register while
+// the ancestor is the same and are added to its row when it changes (one add
+// per run instead of one per (row, key)).
+constexpr int KVR = 64;
+__global__ void attn_bwd_kv_kernel(const float* __restrict__ qkv, const float* __restrict__ P,
+                                   const float* __restrict__ dO, const float* __restrict__ dS,
+                                   float* __restrict__ dqkv, int D, int H, Rows R) {
+  ANQS_PDL_ENTRY();
+  const uint64_t rows = R.rows.get(), r0 = uint64_t(blockIdx.x) * KVR;
+  if (r0 >= rows) return;
+  const uint64_t r1 = r0 + KVR < rows ? r0 + KVR : rows;
+  const int n = R.n, u = blockIdx.y, dh = D / H;
+  __shared__ uint32_t key[KVR];
+  for (int i = threadIdx.x; i < KVR; i += blockDim.x) {
+    const uint64_t r = r0 + i;
+    key[i] = r < r1 && R.lv[r] >= u ? R.anc[r * n + u] : 0xffffffffu;
+  }
+  __syncthreads();
+  for (int col = threadIdx.x; col < 2 * D; col += blockDim.x) {
+    const int kv = col / D, c = col - kv * D, hd = c / dh;
+    const float* w = (kv ? P : dS) + hd * n + u;
+    const float* v = kv ? dO + c : qkv + c;
+    const size_t ldv = kv ? D : 3 * size_t(D);
+    uint32_t cur = 0xffffffffu;
+    float acc = 0.f;
+    for (int i = 0; i < int(r1 - r0); ++i) {
+      const uint32_t k = key[i];
+      if (k != cur) {
+        if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
+        cur = k;
+        acc = 0.f;
+      }
+      if (k != 0xffffffffu) acc = fmaf(w[(r0 + i) * H * n], v[(r0 + i) * ldv], acc);
+    }
+    if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
+  }
+}
+
+// Cotangents of every row's slot terms: cot[r][v] += cl, cot[r][4 + v] += cp
+// over the samples whose path takes outcome v at row r (FP64: a root row adds
+// up all samples).  Samples outside the sector add nothing.  nv.packed null:
+// flat rows.
+__global__ void cot_rows_kernel(HamView hv, SectorView sv, NodeView nv, const uint64_t* __restrict__ x, Count nx_,
+                                const float* __restrict__ cl, const float* __restrict__ cp, double* __restrict__ cot) {
   ANQS_PDL_ENTRY();
   const uint64_t nx = nx_.get();
-  for (uint64_t s = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; s < nx; s += uint64_t(gridDim.x) * blockDim.x) {
-    const uint64_t xs = x[s];
-    bool dead = hv.n < 32 && (xs >> (2 * hv.n)) != 0;
-    int ca = 0, cb = 0;
+  const int n = hv.n, lane = threadIdx.x & 31;
+  for (uint64_t s0 = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) - lane; s0 < nx;
+       s0 += uint64_t(gridDim.x) * blockDim.x) {
+    const uint64_t s = s0 + lane;
+    const uint64_t xs = s < nx ? x[s] : 0ull;
+    bool dead = s >= nx || (n < 32 && (xs >> (2 * n)) != 0);
     for (int p = 0; p < n; ++p) {
-      const int v = int((xs >> (2 * p)) & 3ull);
-      if (!((slot_mask(hv, p, ca, cb, xs) >> v) & 1u)) dead = true;
-      ca += v & 1;
-      cb += v >> 1;
+      const uint64_t below = xs & ((1ull << (2 * p)) - 1ull);
+      const unsigned pm = slot_mask(hv, p, __popcll(below & 0x5555555555555555ull),
+                                    __popcll(below & 0xAAAAAAAAAAAAAAAAull), xs);
+      if (!((pm >> ((xs >> (2 * p)) & 3ull)) & 1u)) dead = true;
     }
-    ca = cb = 0;
+    const double l = dead ? 0.0 : double(cl[s]), c = dead ? 0.0 : double(cp[s]);
+    const uint32_t a = even_bits(xs), b = even_bits(xs >> 1);
     for (int p = 0; p < n; ++p) {
       const int v = int((xs >> (2 * p)) & 3ull);
-      const unsigned mk = norm_mask(hv, p, slot_mask(hv, p, ca, cb, xs));
-      const float* o = out8 + (s * n + p) * 8;
-      float* d = dout8 + (s * n + p) * 8;
-      float mx = -INFINITY;
-      for (int u = 0; u < 4; ++u)
-        if ((mk >> u) & 1u) mx = fmaxf(mx, o[u]);
-      float e[4], sum = 0.f;
-      for (int u = 0; u < 4; ++u) {
-        e[u] = ((mk >> u) & 1u) ? expf(o[u] - mx) : 0.f;
-        sum += e[u];
+      uint32_t row = 0xffffffffu;
+      if (!dead) row = nv.packed ? node_id(sv, nv, p, prefix_index(sv, p, a, b)) : uint32_t(s * n + p);
+      if (p < 4 && nv.packed) {  // few rows take all samples: one add per warp and row
+        const unsigned peers = __match_any_sync(0xffffffffu, dead ? 0xffffffffu : row * 4 + v);
+        double tl = 0.0, tc = 0.0;
+        const int lead = __ffs(peers) - 1;
+        for (int o = 0; o < 32; ++o) {
+          const double ol = __shfl_sync(0xffffffffu, l, o), oc = __shfl_sync(0xffffffffu, c, o);
+          if ((peers >> o) & 1u) tl += ol, tc += oc;
+        }
+        if (lane == lead && !dead) {
+          atomicAdd(cot + size_t(row) * 8 + v, tl);
+          atomicAdd(cot + size_t(row) * 8 + 4 + v, tc);
+        }
+      } else if (!dead) {
+        atomicAdd(cot + size_t(row) * 8 + v, l);
+        atomicAdd(cot + size_t(row) * 8 + 4 + v, c);
       }
-      for (int u = 0; u < 4; ++u) {
-        const float pu = e[u] / sum;
-        d[u] = dead ? 0.f : 0.5f * cl[s] * ((u == v ? 1.f : 0.f) - pu);
-        d[4 + u] = (dead || u != v) ? 0.f : cp[s];
-      }
-      ca += v & 1;
-      cb += v >> 1;
     }
   }
 }
 
-// gtok[token(r)] += dH0[r], gpos[t] += dH0[r]
-__global__ void embed_bwd_kernel(TfView m, const uint64_t* __restrict__ x, Count rows_, const float* __restrict__ dh0,
-                                 float* __restrict__ gtok, float* __restrict__ gpos) {
+// head cotangents d out8[r] from the masked log-softmax of the row's slot:
+// d l_u = (sum of cl with outcome u - p_u sum of cl) / 2, d phi_u = sum of cp with outcome u
+__global__ void head_dout_kernel(HamView hv, Rows R, const float* __restrict__ out8, const double* __restrict__ cot,
+                                 float* __restrict__ dout8) {
+  ANQS_PDL_ENTRY();
+  const uint64_t rows = R.rows.get();
+  for (uint64_t r = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; r < rows; r += uint64_t(gridDim.x) * blockDim.x) {
+    const int p = R.lv[r];
+    const uint64_t x = R.x[r], below = x & ((1ull << (2 * p)) - 1ull);
+    const unsigned mk = norm_mask(hv, p, slot_mask(hv, p, __popcll(below & 0x5555555555555555ull),
+                                                   __popcll(below & 0xAAAAAAAAAAAAAAAAull), x));
+    const float* o = out8 + r * 8;
+    const double* c = cot + r * 8;
+    float* d = dout8 + r * 8;
+    float mx = -INFINITY;
+    for (int u = 0; u < 4; ++u)
+      if ((mk >> u) & 1u) mx = fmaxf(mx, o[u]);
+    float e[4], sum = 0.f;
+    double tot = 0.0;
+    for (int u = 0; u < 4; ++u) {
+      e[u] = ((mk >> u) & 1u) ? expf(o[u] - mx) : 0.f;
+      sum += e[u];
+      tot += c[u];
+    }
+    for (int u = 0; u < 4; ++u) {
+      // a row without an allowed outcome takes no samples
+      d[u] = sum > 0.f ? float(0.5 * (c[u] - double(e[u] / sum) * tot)) : 0.f;
+      d[4 + u] = float(c[4 + u]);
+    }
+  }
+}
+
+// gtok[token(r)] += dH0[r], gpos[position of r] += dH0[r]: thread = column,
+// a CTA's rows in order, one add per token and per run of equal positions
+constexpr int EBR = 128;
+__global__ void embed_bwd_kernel(TfView m, Rows R, const float* __restrict__ dh0, float* __restrict__ gtok,
+                                 float* __restrict__ gpos) {
+  ANQS_PDL_ENTRY();
+  const uint64_t rows = R.rows.get(), r0 = uint64_t(blockIdx.x) * EBR;
+  if (r0 >= rows) return;
+  const uint64_t r1 = r0 + EBR < rows ? r0 + EBR : rows;
+  const int D = m.d;
+  for (int c = threadIdx.x; c < D; c += blockDim.x) {
+    float tk[5] = {}, ps = 0.f;
+    int cur = -1;
+    for (uint64_t r = r0; r < r1; ++r) {
+      const int t = R.lv[r];
+      const int token = t == 0 ? 4 : int((R.x[r] >> (2 * (t - 1))) & 3ull);
+      const float v = dh0[r * D + c];
+      if (t != cur) {
+        if (cur >= 0) atomicAdd(gpos + cur * D + c, ps);
+        cur = t;
+        ps = 0.f;
+      }
+      ps += v;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) tk[k] += k == token ? v : 0.f;
+    }
+    atomicAdd(gpos + cur * D + c, ps);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) atomicAdd(gtok + k * D + c, tk[k]);
+  }
+}
+
+// out[c] += sum_r X[r][c] for c < 8
+__global__ void __launch_bounds__(256) colsum8_kernel(const float* __restrict__ X, Count rows_, float* __restrict__ out) {
   ANQS_PDL_ENTRY();
   const uint64_t rows = rows_.get();
-  const int D = m.d, n = m.n;
-  for (uint64_t idx = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; idx < rows * D;
-       idx += uint64_t(gridDim.x) * blockDim.x) {
-    const uint64_t r = idx / D;
-    const int c = int(idx % D), t = int(r % n);
-    const int token = t == 0 ? 4 : int((x[r / n] >> (2 * (t - 1))) & 3ull);
-    const float v = dh0[idx];
-    atomicAdd(gtok + token * D + c, v);
-    atomicAdd(gpos + t * D + c, v);
-  }
+  const int c = threadIdx.x & 7;
+  float s = 0.f;
+  for (uint64_t r = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 3; r < rows; r += (uint64_t(gridDim.x) * blockDim.x) >> 3)
+    s += X[r * 8 + c];
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  if ((threadIdx.x & 31) < 8) atomicAdd(out + c, s);
 }
 
 // ---- host side ----------------------------------------------------------------
@@ -431,25 +666,43 @@ LayerOff layer_off(const TfView& m, int l) {
 }
 
 struct Acts {
-  float *H[17], *Xh1[16], *A1[16], *RS1[16], *Q[16], *K[16], *V[16], *P[16], *O[16], *Hm[16], *Xh2[16],
-      *A2[16], *RS2[16], *F[16];
-  float *Xhf, *Af, *RSf, *out8, *dout8, *dH, *dA, *dHm, *dF, *dQ, *dK, *dV, *dO;
+  float *H[17], *Xh1[16], *A1[16], *RS1[16], *QKV[16], *P[16], *O[16], *Hm[16], *Xh2[16], *A2[16], *RS2[16], *F[16];
+  float *Xhf, *Af, *RSf, *out8, *dout8, *dH, *dA, *dHm, *dF, *dQKV, *dO, *dS;
+  double* cot;
+  // rows
+  bool tree;
+  uint64_t R;  // bound on the rows
+  uint64_t* x;
+  uint8_t* lv;
+  uint32_t* anc;
+  TreeWs t;
 };
 
 // Full storage keeps every block's activations; with `ckpt` (activation
 // recomputation) only the block inputs H[l] are kept and one set of block
 // activations is shared by all blocks: the backward recomputes block l's
 // forward from H[l] just before its own backward.
-size_t plan(const TfView& m, uint64_t nx, Arena& Ar, Acts& a, bool ckpt = false) {
-  const uint64_t R = nx * m.n, D = m.d;
+size_t plan(const TfView& m, const anqs_ham* Hm, uint64_t nx, Arena& Ar, Acts& a, bool ckpt = false) {
+  const uint64_t D = m.d;
+  a.tree = tree_applies(Hm);
+  a.x = nullptr;
+  if (a.tree) {
+    plan_tree(Hm, nx, Ar, a.t);
+    a.R = a.t.max_rows;
+  } else {
+    a.R = nx * m.n;
+    a.x = Ar.take<uint64_t>(a.R);
+  }
+  const uint64_t R = a.R;
+  a.lv = Ar.take<uint8_t>(R);
+  a.anc = Ar.take<uint32_t>(R * m.n);
+  a.cot = Ar.take<double>(R * 8);
   for (int l = 0; l <= m.L; ++l) a.H[l] = Ar.take<float>(R * D);
   for (int l = 0; l < (ckpt ? 1 : m.L); ++l) {
     a.Xh1[l] = Ar.take<float>(R * D);
     a.A1[l] = Ar.take<float>(R * D);
     a.RS1[l] = Ar.take<float>(R);
-    a.Q[l] = Ar.take<float>(R * D);
-    a.K[l] = Ar.take<float>(R * D);
-    a.V[l] = Ar.take<float>(R * D);
+    a.QKV[l] = Ar.take<float>(R * 3 * D);
     a.P[l] = Ar.take<float>(R * m.H * m.n);
     a.O[l] = Ar.take<float>(R * D);
     a.Hm[l] = Ar.take<float>(R * D);
@@ -459,8 +712,8 @@ size_t plan(const TfView& m, uint64_t nx, Arena& Ar, Acts& a, bool ckpt = false)
     a.F[l] = Ar.take<float>(R * 4 * D);
   }
   for (int l = 1; ckpt && l < m.L; ++l) {
-    a.Xh1[l] = a.Xh1[0], a.A1[l] = a.A1[0], a.RS1[l] = a.RS1[0], a.Q[l] = a.Q[0], a.K[l] = a.K[0];
-    a.V[l] = a.V[0], a.P[l] = a.P[0], a.O[l] = a.O[0], a.Hm[l] = a.Hm[0], a.Xh2[l] = a.Xh2[0];
+    a.Xh1[l] = a.Xh1[0], a.A1[l] = a.A1[0], a.RS1[l] = a.RS1[0], a.QKV[l] = a.QKV[0];
+    a.P[l] = a.P[0], a.O[l] = a.O[0], a.Hm[l] = a.Hm[0], a.Xh2[l] = a.Xh2[0];
     a.A2[l] = a.A2[0], a.RS2[l] = a.RS2[0], a.F[l] = a.F[0];
   }
   a.Xhf = Ar.take<float>(R * D);
@@ -472,10 +725,9 @@ size_t plan(const TfView& m, uint64_t nx, Arena& Ar, Acts& a, bool ckpt = false)
   a.dA = Ar.take<float>(R * D);
   a.dHm = Ar.take<float>(R * D);
   a.dF = Ar.take<float>(R * 4 * D);
-  a.dQ = Ar.take<float>(R * D);
-  a.dK = Ar.take<float>(R * D);
-  a.dV = Ar.take<float>(R * D);
+  a.dQKV = Ar.take<float>(R * 3 * D);
   a.dO = Ar.take<float>(R * D);
+  a.dS = Ar.take<float>(R * m.H * m.n);
   return Ar.off;
 }
 
@@ -489,20 +741,22 @@ unsigned grid_for(uint64_t work, int threads, uint64_t cap) {
 // host), K given by Kc.  Weight products (atomic) split K over CTAs.
 template <bool TA, bool TB>
 int gemm(Gm g, uint64_t M_host, uint64_t K_host, cudaStream_t s) {
-  const unsigned gx = unsigned((g.N + BN - 1) / BN), gy = unsigned((M_host + BM - 1) / BM);
+  const unsigned gx = unsigned((g.N + BN - 1) / BN);
+  const uint64_t gy = (M_host + BM - 1) / BM;
   unsigned gz = 1;
   g.k_chunk = K_host ? K_host : 1;
   if (g.atomic) {
     const uint64_t tiles = uint64_t(gx) * gy;
-    uint64_t want = (152 * 4 + tiles - 1) / tiles;
-    const uint64_t max_split = (K_host + 255) / 256;  // at least 256 rows per split
+    uint64_t want = (152 * 3 + tiles - 1) / tiles;
+    const uint64_t max_split = (K_host + 127) / 128;  // at least 128 rows per split
     if (want > max_split) want = max_split;
     if (want < 1) want = 1;
     gz = unsigned(want);
     g.k_chunk = ((K_host + gz - 1) / gz + BK - 1) / BK * BK;
   }
   if (gy > 65535u) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows for the transformer adjoint");
-  ANQS_CUDA_LAUNCH("tf sgemm_kernel", launch_k(sgemm_kernel<TA, TB>, dim3(gx, gy, gz), dim3(GT), 0, s, g));
+  g.b_vec = reinterpret_cast<uintptr_t>(g.B) % 16 == 0 && reinterpret_cast<uintptr_t>(g.bias) % 16 == 0;
+  ANQS_CUDA_LAUNCH("tf sgemm_kernel", launch_k(sgemm_kernel<TA, TB>, dim3(gx, unsigned(gy), gz), dim3(GT), 0, s, g));
   return ANQS_OK;
 }
 
@@ -525,45 +779,55 @@ Gm mk(const float* A, int lda, const float* B, int ldb, float* C, int ldc, Count
 }
 
 template <int D>
-int run(const TfView& m, const HamView& hv, const uint64_t* x, Count nx, const float* cl, const float* cp,
+int run(const TfView& m, const anqs_ham* Hm, const uint64_t* x, Count nx, const float* cl, const float* cp,
         float* grad, void* ws, size_t ws_bytes, cudaStream_t s) {
+  const HamView& hv = Hm->v;
   Arena Ar(ws, ws_bytes);
-  Acts a;
-  plan(m, nx.n, Ar, a);
+  Acts a{};
+  plan(m, Hm, nx.n, Ar, a);
   bool ckpt = false;
   if (!Ar.fits()) {  // too little workspace for every activation: recompute each block's
     Arena Ac(ws, ws_bytes);
-    plan(m, nx.n, Ac, a, true);
+    plan(m, Hm, nx.n, Ac, a, true);
     if (!Ac.fits())
       return set_error(ANQS_ERR_CAPACITY, "transformer adjoint workspace needs %zu bytes (%zu with recomputation)",
                        Ar.off, Ac.off);
     ckpt = true;
   }
   const int n = m.n, L = m.L, H = m.H;
-  const Count rows = scaled(nx, n);
-  const uint64_t R = rows.n;
-  const Count kD = host_count(D), k4D = host_count(4 * D), k8 = host_count(8);
+  const bool v4 = (D / H) % 4 == 0;
+  const uint64_t R = a.R;
+  const Count rows = a.tree ? Count{R, a.t.n_rows, 1} : scaled(nx, n);
+  const Count kD = host_count(D), k3D = host_count(3 * D), k4D = host_count(4 * D), k8 = host_count(8);
   const float* P = m.params;
   ProfScope ps(PROF_TF_GRAD, s);
   const unsigned eg = grid_for(R * D, 256, 152 * 16), lg = grid_for(R * 32, 256, 152 * 16);
-  ANQS_CUDA_LAUNCH("tf embed_kernel", launch_k(embed_kernel, dim3(eg), dim3(256), 0, s, m, x, rows, a.H[0]));
+  const unsigned ag = grid_for(R * H, 128, 152 * 16);
+  Rows rw{a.x, a.lv, a.anc, rows, n};
+  ANQS_CUDA(cudaMemsetAsync(a.cot, 0, R * 8 * sizeof(double), s));
+  if (a.tree) {
+    ANQS_TRY(launch_tree(Hm, x, nx, a.t, s));
+    rw.x = a.t.nodes.x;
+    ANQS_CUDA_LAUNCH("tf tree_rows_kernel", launch_k(tree_rows_kernel, dim3(grid_for(R, 64, 152 * 16)), dim3(64), 0, s, Hm->sv, a.t.nodes, a.lv, a.anc));
+  } else {
+    ANQS_CUDA_LAUNCH("tf flat_rows_kernel", launch_k(flat_rows_kernel, dim3(grid_for(R, 64, 152 * 16)), dim3(64), 0, s, x, rows, n, a.x, a.lv, a.anc));
+  }
+  ANQS_CUDA_LAUNCH("tf cot_rows_kernel", launch_k(cot_rows_kernel, dim3(grid_for(nx.n, 64, 152 * 16)), dim3(64), 0, s, hv, Hm->sv, a.t.nodes, x, nx, cl, cp, a.cot));
+  ANQS_CUDA_LAUNCH("tf embed_kernel", launch_k(embed_kernel, dim3(eg), dim3(256), 0, s, m, rw, a.H[0]));
+  const Seg qkv_seg{D, size_t(D) * D + D};  // wq, bq, wk, bk, wv, bv
   // forward of block l from H[l]: its activations and H[l + 1] (deterministic,
   // so a recomputation reproduces them bit for bit)
   auto fwd_block = [&](int l) -> int {
     const LayerOff o = layer_off(m, l);
     ANQS_CUDA_LAUNCH("tf ln_fwd_kernel", launch_k(ln_fwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.H[l], P + o.ln1_g,
                                                   P + o.ln1_b, a.Xh1[l], a.A1[l], a.RS1[l], rows));
-    const float* Wqkv[3] = {P + o.wq, P + o.wk, P + o.wv};
-    const float* bqkv[3] = {P + o.bq, P + o.bk, P + o.bv};
-    float* qkv[3] = {a.Q[l], a.K[l], a.V[l]};
-    for (int i = 0; i < 3; ++i) {
-      Gm g = mk(a.A1[l], D, Wqkv[i], D, qkv[i], D, rows, kD, D);
-      g.bias = bqkv[i];
+    {
+      Gm g = mk(a.A1[l], D, P + o.wq, D, a.QKV[l], 3 * D, rows, kD, 3 * D);
+      g.sb = qkv_seg;
+      g.bias = P + o.bq;
       ANQS_TRY(gemm_nt(g, R, D, s));
     }
-    ANQS_CUDA_LAUNCH("tf attn_fwd_kernel",
-                     launch_k(attn_fwd_kernel, dim3(grid_for(nx.n * H * n, 128, 152 * 16)), dim3(128), 0, s,
-                              a.Q[l], a.K[l], a.V[l], a.P[l], a.O[l], n, D, H, nx));
+    ANQS_CUDA_LAUNCH("tf attn_fwd_kernel", launch_k(v4 ? attn_fwd_kernel<true> : attn_fwd_kernel<false>, dim3(ag), dim3(128), 0, s, a.QKV[l], a.P[l], a.O[l], D, H, rw));
     {
       Gm g = mk(a.O[l], D, P + o.wo, D, a.Hm[l], D, rows, kD, D);
       g.bias = P + o.bo;
@@ -598,22 +862,21 @@ int run(const TfView& m, const HamView& hv, const uint64_t* x, Count nx, const f
     g.bias = P + head_b;
     ANQS_TRY(gemm_nt(g, R, D, s));
   }
-  ANQS_CUDA_LAUNCH("tf head_dout_kernel", launch_k(head_dout_kernel, dim3(grid_for(nx.n, 128, 152 * 8)), dim3(128), 0,
-                                                   s, hv, x, nx, a.out8, cl, cp, a.dout8, n));
+  ANQS_CUDA_LAUNCH("tf head_dout_kernel", launch_k(head_dout_kernel, dim3(grid_for(R, 128, 152 * 8)), dim3(128), 0, s,
+                                                   hv, rw, a.out8, a.cot, a.dout8));
   // ---- backward ----
-  const unsigned cg = grid_for(R, 64, 152 * 4);
-  auto wgrad = [&](const float* dY, int ldy, const float* X, int ldx, int Mo, int Ni, float* gW, int relu_x) -> int {
+  // weight gradient gW += dY^T X and bias gradient gb += the column sums of dY
+  auto wgrad = [&](const float* dY, int ldy, const float* X, int ldx, int Mo, int Ni, float* gW, float* gb, int relu_x,
+                   Seg seg = Seg{}) -> int {
     Gm g = mk(dY, ldy, X, ldx, gW, Ni, host_count(Mo), rows, Ni);
     g.relu_b = relu_x;
     g.atomic = 1;
+    g.sc = seg;
+    g.colsum = gb;
     return gemm_tn(g, Mo, R, s);
   };
-  auto colsum = [&](const float* X, int N, float* out) -> int {
-    ANQS_CUDA_LAUNCH("tf colsum_kernel", launch_k(colsum_kernel, dim3(cg), dim3(256), 0, s, X, N, rows, out));
-    return ANQS_OK;
-  };
-  ANQS_TRY(wgrad(a.dout8, 8, a.Af, D, 8, D, grad + head_w, 0));
-  ANQS_TRY(colsum(a.dout8, 8, grad + head_b));
+  ANQS_TRY(wgrad(a.dout8, 8, a.Af, D, 8, D, grad + head_w, nullptr, 0));
+  ANQS_CUDA_LAUNCH("tf colsum8_kernel", launch_k(colsum8_kernel, dim3(grid_for(R * 8, 256, 152)), dim3(256), 0, s, a.dout8, rows, grad + head_b));
   {
     Gm g = mk(a.dout8, 8, P + head_w, D, a.dA, D, rows, k8, D);
     ANQS_TRY(gemm_nn(g, R, 8, s));
@@ -624,16 +887,14 @@ int run(const TfView& m, const HamView& hv, const uint64_t* x, Count nx, const f
   for (int l = L - 1; l >= 0; --l) {
     const LayerOff o = layer_off(m, l);
     if (ckpt && l + 1 < L) ANQS_TRY(fwd_block(l));  // the shared activations hold block L-1's after the forward
-    ANQS_TRY(wgrad(a.dH, D, a.F[l], 4 * D, D, 4 * D, grad + o.w2, 1));
-    ANQS_TRY(colsum(a.dH, D, grad + o.b2));
+    ANQS_TRY(wgrad(a.dH, D, a.F[l], 4 * D, D, 4 * D, grad + o.w2, grad + o.b2, 1));
     {
       Gm g = mk(a.dH, D, P + o.w2, 4 * D, a.dF, 4 * D, rows, kD, 4 * D);
       g.mask = a.F[l];
       g.ldmask = 4 * D;
       ANQS_TRY(gemm_nn(g, R, D, s));
     }
-    ANQS_TRY(wgrad(a.dF, 4 * D, a.A2[l], D, 4 * D, D, grad + o.w1, 0));
-    ANQS_TRY(colsum(a.dF, 4 * D, grad + o.b1));
+    ANQS_TRY(wgrad(a.dF, 4 * D, a.A2[l], D, 4 * D, D, grad + o.w1, grad + o.b1, 0));
     {
       Gm g = mk(a.dF, 4 * D, P + o.w1, D, a.dA, D, rows, k4D, D);
       ANQS_TRY(gemm_nn(g, R, 4 * D, s));
@@ -641,53 +902,44 @@ int run(const TfView& m, const HamView& hv, const uint64_t* x, Count nx, const f
     ANQS_CUDA_LAUNCH("tf ln_bwd_kernel", launch_k(ln_bwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.dA, a.Xh2[l],
                                                   P + o.ln2_g, a.RS2[l], (const float*)a.dH, a.dHm, grad + o.ln2_g,
                                                   grad + o.ln2_b, rows));
-    ANQS_TRY(wgrad(a.dHm, D, a.O[l], D, D, D, grad + o.wo, 0));
-    ANQS_TRY(colsum(a.dHm, D, grad + o.bo));
+    ANQS_TRY(wgrad(a.dHm, D, a.O[l], D, D, D, grad + o.wo, grad + o.bo, 0));
     {
       Gm g = mk(a.dHm, D, P + o.wo, D, a.dO, D, rows, kD, D);
       ANQS_TRY(gemm_nn(g, R, D, s));
     }
-    ANQS_CUDA_LAUNCH("tf attn_bwd_kernel",
-                     launch_k(attn_bwd_kernel, dim3(grid_for(nx.n * H, 64, 152 * 16)), dim3(64), 0, s, a.Q[l], a.K[l],
-                              a.V[l], a.P[l], a.dO, a.dQ, a.dK, a.dV, n, D, H, nx));
-    const float* dqkv[3] = {a.dQ, a.dK, a.dV};
-    const size_t wo3[3] = {o.wq, o.wk, o.wv}, bo3[3] = {o.bq, o.bk, o.bv};
-    for (int i = 0; i < 3; ++i) {
-      ANQS_TRY(wgrad(dqkv[i], D, a.A1[l], D, D, D, grad + wo3[i], 0));
-      ANQS_TRY(colsum(dqkv[i], D, grad + bo3[i]));
-      Gm g = mk(dqkv[i], D, P + wo3[i], D, a.dA, D, rows, kD, D);
-      if (i) {
-        g.Cin = a.dA;
-        g.ldcin = D;
-      }
-      ANQS_TRY(gemm_nn(g, R, D, s));
+    ANQS_CUDA_LAUNCH("tf attn_bwd_q_kernel", launch_k(v4 ? attn_bwd_q_kernel<true> : attn_bwd_q_kernel<false>, dim3(ag), dim3(128), 0, s, a.QKV[l], a.P[l], a.dO, a.dS, a.dQKV, D, H, rw));
+    ANQS_CUDA_LAUNCH("tf attn_bwd_kv_kernel", launch_k(attn_bwd_kv_kernel, dim3(unsigned((R + KVR - 1) / KVR), unsigned(n)), dim3(2 * D < 256 ? 2 * D : 256), 0, s, a.QKV[l], a.P[l], a.dO, a.dS, a.dQKV, D, H, rw));
+    ANQS_TRY(wgrad(a.dQKV, 3 * D, a.A1[l], D, 3 * D, D, grad + o.wq, grad + o.bq, 0, qkv_seg));
+    {
+      Gm g = mk(a.dQKV, 3 * D, P + o.wq, D, a.dA, D, rows, k3D, D);
+      g.sb = qkv_seg;
+      ANQS_TRY(gemm_nn(g, R, 3 * D, s));
     }
     ANQS_CUDA_LAUNCH("tf ln_bwd_kernel", launch_k(ln_bwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.dA, a.Xh1[l],
                                                   P + o.ln1_g, a.RS1[l], (const float*)a.dHm, a.dH, grad + o.ln1_g,
                                                   grad + o.ln1_b, rows));
   }
-  ANQS_CUDA_LAUNCH("tf embed_bwd_kernel", launch_k(embed_bwd_kernel, dim3(eg), dim3(256), 0, s, m, x, rows, a.dH,
-                                                   grad, grad + 5 * size_t(D)));
+  ANQS_CUDA_LAUNCH("tf embed_bwd_kernel", launch_k(embed_bwd_kernel, dim3(unsigned((R + EBR - 1) / EBR)), dim3(D), 0, s, m, rw, a.dH, grad, grad + 5 * size_t(D)));
   return ANQS_OK;
 }
 
 }  // namespace
 
-size_t tf_grad_workspace(const TfView& m, uint64_t n_x, bool recompute) {
+size_t tf_grad_workspace(const TfView& m, const anqs_ham* H, uint64_t n_x, bool recompute) {
   Arena Ar(nullptr, 0);
-  Acts a;
-  return plan(m, n_x, Ar, a, recompute);
+  Acts a{};
+  return plan(m, H, n_x, Ar, a, recompute);
 }
 
-int launch_tf_fp32_grad(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, const float* cl,
+int launch_tf_fp32_grad(const TfView& m, const anqs_ham* H, const uint64_t* x, Count n_x, const float* cl,
                         const float* cp, float* grad, void* ws, size_t ws_bytes, cudaStream_t s) {
   if (n_x.n == 0) return ANQS_OK;
   if (m.n > 32) return set_error(ANQS_ERR_UNSUPPORTED, "n_orb %d", m.n);
   switch (m.d) {
-    case 32: return run<32>(m, hv, x, n_x, cl, cp, grad, ws, ws_bytes, s);
-    case 64: return run<64>(m, hv, x, n_x, cl, cp, grad, ws, ws_bytes, s);
-    case 128: return run<128>(m, hv, x, n_x, cl, cp, grad, ws, ws_bytes, s);
-    case 256: return run<256>(m, hv, x, n_x, cl, cp, grad, ws, ws_bytes, s);
+    case 32: return run<32>(m, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
+    case 64: return run<64>(m, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
+    case 128: return run<128>(m, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
+    case 256: return run<256>(m, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
   }
   return set_error(ANQS_ERR_UNSUPPORTED, "d_model %d", m.d);
 }

@@ -141,3 +141,36 @@ def test_index_arithmetic_over_the_supported_range():
                                       np.arange(1, 512) * d - 1])).astype(np.uint64)
         assert np.array_equal((v * np.uint64(m)) >> np.uint64(32), v // np.uint64(d)), d
     assert math.comb(31, 2) < 512 and 16 * 16 <= 256
+
+
+# Transformer adjoint over distinct prefixes: heads of width 2 and 16, one sample and a whole level, repeated samples
+# (their cotangents add up), rows outside the sector (no contribution), parameters at an odd float offset, and more
+# orbitals than the prefix index covers (one row per sample and position).  The same bar as the other adjoint tests.
+@pytest.mark.parametrize("n,na,nb,heads,m", [(1, 1, 0, 4, 1), (3, 1, 2, 32, 1), (6, 3, 3, 4, 90), (9, 2, 7, 32, 300),
+                                             (11, 5, 5, 4, 257), (20, 3, 2, 4, 40)])
+def test_transformer_adjoint_rows(A, n, na, nb, heads, m):
+    from oracle.anqs import TFAnsatz, log_psi
+    from oracle.sector import molecular_isphys
+    from synthetic import flatten_tf, integrals, tf_params
+    P = tf_params(n, n, 64, 2, bias_std=0.2)
+    flat = flatten_tf(P)
+    params = torch.zeros(flat.size + 1, device="cuda")[1:]
+    params.copy_(torch.tensor(flat))
+    h, g, e = integrals(n, n, 2)
+    ham = A.Hamiltonian(h, g, e, na, nb)
+    model = A.Model.transformer(n, 64, heads, 2, params)
+    x = _dets(n, na, nb, m, 5 * n)
+    rng = np.random.default_rng(n)
+    x = torch.cat([x, x[: max(1, x.numel() // 3)]])
+    ca, cp = rng.normal(size=x.numel()), rng.normal(size=x.numel())
+    om, ip = TFAnsatz(P, n, heads), molecular_isphys(n, na, nb)
+    ps = om.parameters()
+    for t in ps:
+        t.requires_grad_(True)
+    la, ph = log_psi(om, ip, x.cpu().numpy().astype(np.uint64))
+    ref = torch.autograd.grad((torch.tensor(ca) * la).sum() + (torch.tensor(cp) * ph).sum(), ps, allow_unused=True)
+    ref = np.concatenate([(torch.zeros_like(t) if r is None else r).reshape(-1).numpy() for r, t in zip(ref, ps)])
+    bad = torch.tensor([0 if na + nb else 1, (1 << 2 * n) | int(x[0])], device="cuda")
+    dev = lambda a: torch.tensor(np.concatenate([a, [3.0, -2.0]]), device="cuda", dtype=torch.float32)
+    got = A.logpsi_vjp(model, ham, torch.cat([x, bad]), dev(ca), dev(cp)).cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref)
