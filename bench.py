@@ -963,8 +963,8 @@ def _tf_work(A, ham, w, x):
     set x.  One (sequence, position t) row costs f(t) = L (24 d^2 + 4 (t+1) d)
     + 16 d: the q|k|v, output and FFN projections, the attention scores and
     weighted sum over the t+1 keys, and the head.  suffix = every position of
-    every distinct determinant (beyond INDEX_MAX_ORB orbitals: positions > j(x')
-    of every connected x'); parent = every position of every sample; slot
+    every distinct determinant (beyond INDEX_MAX_ORB orbitals: one position of
+    every distinct prefix of each sample's connected determinants); parent = every position of every sample; slot
     (sampler) = positions 0..p of every distinct prefix at level p; grad =
     3 x parent (forward plus the two products of the adjoint)."""
     n, d, L = w["n"], w["d_model"], w["n_layers"]
@@ -981,12 +981,16 @@ def _tf_work(A, ham, w, x):
         full = _distinct_prefixes(A, ham, x)[n] * cf[n]
         return dict(out, tf_tc_suffix_kernel=full, tf_fp32_kernel=full + slot,
                     eloc_assemble_kernel=_eloc_bytes(len(x), ham.n_connected))
-    xp, hv, js, hd = A.connected(ham, x)
-    j = js.reshape(-1).cpu().numpy().astype(np.int64)
-    return dict(out, tf_tc_suffix_kernel=float((cf[n] - cf[j + 1]).sum()),
-                tf_fp32_kernel=len(j) * cf[n] + parent + slot,
-                eloc_assemble_kernel=float((8 + 1 + 8 + 8 + 8 * (n - 1 - j)).sum()),
-                connected_kernel=float(len(j) * (8 + 8 + 1) + len(x) * 8))
+    nodes = np.zeros(n)  # each sample's own distinct prefixes
+    for xi, xp in zip(x, A.connected(ham, x)[0]):
+        u = torch.cat([xi[None], xp])
+        for p in range(n - 1, -1, -1):
+            u = torch.unique(u & ((1 << (2 * p)) - 1))
+            nodes[p] += u.numel()
+    m = len(x) * ham.n_connected
+    return dict(out, tf_tc_suffix_kernel=float((nodes * f).sum()), tf_fp32_kernel=m * cf[n] + parent + slot,
+                eloc_assemble_kernel=_eloc_bytes(len(x), ham.n_connected),
+                connected_kernel=float(m * (8 + 8 + 1) + len(x) * 8))
 
 
 def _tc_work(A, ham, model, w, x):

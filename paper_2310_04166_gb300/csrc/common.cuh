@@ -115,7 +115,10 @@ struct Count {
   const uint64_t* dev;
   uint64_t mult;
 #ifdef __CUDACC__
-  __device__ __forceinline__ uint64_t get() const { return dev ? *dev * mult : n; }
+  // through L2: the kernel just before may have written it, next to words it read
+  __device__ __forceinline__ uint64_t get() const {
+    return dev ? __ldcg(reinterpret_cast<const unsigned long long*>(dev)) * mult : n;
+  }
 #endif
 };
 inline Count host_count(uint64_t n) { return Count{n, nullptr, 1}; }
@@ -565,6 +568,39 @@ int launch_tree(const anqs_ham* H, const uint64_t* x, Count n_x, const TreeWs& w
 int launch_eloc_direct(const anqs_ham* H, const uint64_t* x, Count n_x, const NodeView& nodes, const AmpSrc& amp,
                        double* ere, double* eim, double* part, const StatsOut& so, cudaStream_t s);
 
+// trie.cu: the connected determinants of each sample as a prefix tree, for
+// sectors too large for a prefix index.  Samples are taken in groups; level p
+// of a group holds the distinct prefixes of p slots of each sample's own
+// connected determinants (and of the sample), sample by sample.
+constexpr int TRIE_ANC = 32;  // entries of a node's table of prefixes
+struct TrieLevel {
+  int p;
+  const uint64_t* x;    // prefixes
+  Count rows;
+  const uint32_t* anc;  // [row][TRIE_ANC] node ids of its prefixes of 0..p-1 slots
+  uint64_t node0;       // id of the first node
+};
+struct TrieWs {
+  uint64_t group;                     // samples per group
+  uint64_t cap[ANQS_MAX_ORB + 1];     // bounds on the nodes of a level; level n: the determinants
+  uint64_t node0[ANQS_MAX_ORB + 1];   // ids of level p start here
+  uint64_t *x[2], *cnt;               // prefixes (levels alternate), nodes of each level
+  uint32_t *src[2], *par[2], *anc[2], *bsum;
+  float2 *amp, *own;                  // per determinant of the group; per sample
+  double* part;                       // [n_x][TRIE_PARTS][2]
+  int parts;
+};
+// max_nodes: bound on the nodes below level n - 1 of a group (at least one sample)
+void plan_trie(const anqs_ham* H, uint64_t n_x, uint64_t max_nodes, Arena& A, TrieWs& w);
+// level p of group c, after level p - 1
+int launch_trie_level(const anqs_ham* H, const uint64_t* x, Count n_x, uint64_t c, int p, const TrieWs& w,
+                      TrieLevel& lv, cudaStream_t s);
+// after all levels: the determinants' amplitudes from the node terms, and the samples' local energies
+int launch_trie_eloc(const anqs_ham* H, const uint64_t* x, Count n_x, uint64_t c, const TrieWs& w, const float2* terms,
+                     cudaStream_t s);
+int launch_trie_finish(const anqs_ham* H, Count n_x, const TrieWs& w, double* ere, double* eim, const uint64_t* counts,
+                       double* stats, cudaStream_t s);
+
 // eloc.cu
 int launch_stats_combine(const double* in, int world, double* out, cudaStream_t s);
 int launch_grad_cotangents(const double* ere, const double* eim, const uint64_t* counts,
@@ -622,8 +658,7 @@ int launch_js_sort(const uint8_t* js, Count mc, int n, uint32_t* ctl, uint32_t* 
                    uint32_t* perm, cudaStream_t s);
 int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const uint8_t* js, const float* cache,
                          const float2* T, const double* hval, const double* hdiag, const float* la_x,
-                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s,
-                         bool tsum = false);
+                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s);
 // BF16 transformer form
 int tf_tc_pack_alloc(anqs_model* m);
 int tf_tc_pack(anqs_model* m, cudaStream_t s);

@@ -1,6 +1,7 @@
 // 16-bit tensor-core form of the causal-transformer ansatz (d = 64): tcgen05
-// MMAs with TMEM accumulators for every projection, with reuse of the parent
-// determinant's keys and values for its connected determinants.
+// MMAs with TMEM accumulators for every projection, over
+// whole sequences or over the distinct prefixes of one level with the stored
+// keys and values of the others.
 //
 // The GEMM operands (weights, LayerNorm outputs, attention outputs, FFN
 // hidden units) and the stored keys and values are fp16, not bf16: the same
@@ -28,14 +29,12 @@
 // Modes
 //   FULL    sequences x[s] (determinants or sampler prefixes), positions
 //           0..P-1: the 8 raw outputs of every position (or of the last one
-//           only), optionally the keys and values of every position and block
-//           (the parent cache).
-//   SUFFIX  connected determinants x', grouped by first differing slot j:
-//           positions t = j+1..n-1 only (positions <= j see the same tokens as
-//           in the parent x, Eq. anqs_def); keys and values of positions <= j
-//           come from the parent cache; writes the sum over those positions of
-//           the masked slot terms, one (log|psi|, phase) pair T[x'] per
-//           connected determinant (a sequence's positions are rows of one tile).
+//           only).
+//   NODES   the distinct prefixes of one level p (trie.cu), one row each:
+//           position p, attending to the stored keys and values of the row's
+//           own prefixes (levels < p, found through its table) and to itself;
+//           keeps its keys and values for the later levels and writes the
+//           masked half-log-probability and the phase of each outcome.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -52,10 +51,9 @@ size_t tf128_packed_bytes(const anqs_model* M);
 int tf128_pack(anqs_model* M, cudaStream_t s);
 int tf128_status_offset(const anqs_model* M);
 int launch_tf128_full(const anqs_model* M, const HamView& hv, const uint64_t* x, Count n_seq, int P, int last_only,
-                      float* raw, __half* kv_out, int prof, cudaStream_t s);
-int launch_tf128_suffix(const anqs_model* M, const HamView& hv, const uint64_t* xp, const uint32_t* perm,
-                        const uint32_t* offsets, uint32_t K, const __half* kv_in, float2* T, uint64_t m_max,
-                        int prof, cudaStream_t s);
+                      float* raw, int prof, cudaStream_t s);
+int launch_tf128_nodes(const anqs_model* M, const HamView& hv, const TrieLevel& lv, __half* kv, float2* terms,
+                       cudaStream_t s);
 
 namespace {
 
@@ -81,7 +79,7 @@ constexpr uint32_t OFF_LP = OFF_HEAD + (8 * D + 8) * 4;    // every block's, the
 constexpr uint32_t SMEM_BYTES = OFF_LP + (kMaxL * LP_FLOATS + 2 * D) * 4;
 constexpr uint32_t TMEM_WG = 256;  // columns per warpgroup: [0,192) qkv / o / f1 buffers, [192,256) acc2
 constexpr uint64_t kWaitNs = 2000000000ull;
-constexpr int MODE_FULL = 0, MODE_SUFFIX = 1;
+constexpr int MODE_FULL = 0, MODE_NODES = 1;
 static_assert(2 * A_BYTES <= KV_BYTES, "hidden chunks live in the k|v region");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
@@ -94,16 +92,14 @@ struct Args {
   // FULL
   const uint64_t* x;
   Count n_seq;
-  int P, last_only;
+  int P, last_only;  // NODES: P = the level
   float* raw;
-  __half* kv_out;
-  // SUFFIX
-  const uint64_t* xp;
-  const uint32_t* perm;
-  const uint32_t* offsets;
-  uint32_t K;
-  const __half* kv_in;
-  float2* T;
+  // NODES (x, n_seq: the level's prefixes)
+  const uint32_t* anc;  // [row][TRIE_ANC] node ids of the prefix's own prefixes, levels 0..P-1
+  __half* kv;           // [node][L][2 D]
+  uint64_t node0;       // id of the level's first node
+  int keep_kv;          // the level's keys and values are needed by a later one
+  float2* terms;        // [node][4]
   int* status;
 };
 
@@ -227,14 +223,6 @@ __device__ __forceinline__ void f16x8_to_f32(const uint4 u, float (&f)[8]) {
   }
 }
 
-// Row geometry of one tile
-struct Tile {
-  bool live;   // the tile has rows
-  int P, t0, S;
-  uint64_t first;  // FULL: first sequence; SUFFIX: first index into perm
-  uint64_t count;  // sequences available from `first`
-};
-
 template <int DH>
 __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
   constexpr int H = D / DH;
@@ -243,7 +231,6 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[4];  // 0: q|k|v|o weights, 1: FFN weights, 2: MMA chain, 3: FFN2 chain
   __shared__ uint32_t s_tmem;
-  __shared__ uint64_t s_tiles[ANQS_MAX_ORB + 1];
   const int wg = threadIdx.x / MT, t = threadIdx.x % MT;
   const int n = a.n, L = a.L;
   if (threadIdx.x == 0) {
@@ -282,28 +269,13 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
     }
     for (int i = threadIdx.x; i < 2 * D; i += NT) s_lp[kMaxL * LP_FLOATS + i] = a.params[tail + i];
   }
-  // work: FULL one group; SUFFIX the groups j = 0..n-2 (P = n-1-j positions)
-  uint64_t total = 0;
-  if (threadIdx.x == 0) {
-    if (a.mode == MODE_FULL) {
-      const uint64_t S = MT / a.P, ns = a.n_seq.get();
-      total = (ns + S - 1) / S;
-      s_tiles[0] = 0;
-      s_tiles[1] = total;
-    } else {
-      s_tiles[0] = 0;
-      for (int j = 0; j < n - 1; ++j) {
-        const uint64_t cnt = a.offsets[j + 1] - a.offsets[j], S = MT / (n - 1 - j);
-        total += (cnt + S - 1) / S;
-        s_tiles[j + 1] = total;
-      }
-    }
-  }
+  const int P = a.mode == MODE_FULL ? a.P : 1;     // rows per sequence
+  const int t0 = a.mode == MODE_FULL ? 0 : a.P;    // their first position
+  const int S = MT / P;                            // sequences per tile
+  const uint64_t n_seq = a.n_seq.get(), total = (n_seq + S - 1) / S;
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const int n_groups = a.mode == MODE_FULL ? 1 : n - 1;
-  total = s_tiles[n_groups];
   const uint32_t tmem = s_tmem + uint32_t(wg) * TMEM_WG;
   const uint32_t lane_base = uint32_t((t & ~31)) << 16;
   unsigned char* sA = smem + OFF_WG + wg * WG_BYTES;
@@ -325,41 +297,11 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
     const bool more = pair + gridDim.x < n_pairs;
     // ---- this warpgroup's tile and this thread's row ----
     const uint64_t tile = 2 * pair + wg;
-    Tile tl{};
-    if (tile < total) {
-      int g = 0;
-      while (s_tiles[g + 1] <= tile) ++g;
-      const uint64_t k = tile - s_tiles[g];
-      tl.live = true;
-      if (a.mode == MODE_FULL) {
-        tl.P = a.P;
-        tl.t0 = 0;
-        tl.S = MT / tl.P;
-        tl.first = k * tl.S;
-        tl.count = a.n_seq.get() - tl.first;
-      } else {
-        tl.P = n - 1 - g;
-        tl.t0 = g + 1;
-        tl.S = MT / tl.P;
-        tl.first = a.offsets[g] + k * tl.S;
-        tl.count = a.offsets[g + 1] - tl.first;
-      }
-    }
-    const int s_loc = tl.live ? t / tl.P : 0;
-    const bool valid = tl.live && s_loc < tl.S && uint64_t(s_loc) < tl.count;
-    const int pos = valid ? tl.t0 + t % tl.P : 0;
-    uint64_t x = 0, seq = 0, parent = 0;
-    if (valid) {
-      if (a.mode == MODE_FULL) {
-        seq = tl.first + s_loc;
-        x = a.x[seq];
-      } else {
-        seq = a.perm[tl.first + s_loc];  // row of the connected list
-        x = a.xp[seq];
-        parent = seq / a.K;
-      }
-    }
-    const int row0 = s_loc * (valid ? tl.P : 0);  // tile row of this sequence's first computed position
+    const uint64_t seq = tile * S + t / P;
+    const bool valid = t / P < S && seq < n_seq;
+    const int pos = valid ? t0 + t % P : 0;
+    const uint64_t x = valid ? a.x[seq] : 0;
+    const int row0 = t - t % P;  // tile row of this sequence's first position
     float h[D];
     {
       const int token = pos == 0 ? 4 : int((x >> (2 * (pos - 1))) & 3ull);
@@ -403,7 +345,7 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
       ph_m ^= 1;
       if (!ok) break;
       tc::fence_after_sync();
-      // k, v of this row (+ bias) -> shared memory (and the parent cache)
+      // k, v of this row (+ bias) -> shared memory (and the node store)
 #pragma unroll 1
       for (int c0 = D; c0 < 3 * D; c0 += 32) {
         float v[32];
@@ -415,15 +357,15 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
         uint4* dst = reinterpret_cast<uint4*>(sKV + t * KV_STRIDE + (c0 - D) * 2);
 #pragma unroll
         for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-        if (valid && a.kv_out) {
-          uint4* g = reinterpret_cast<uint4*>(a.kv_out + ((seq * L + l) * n + pos) * (2 * D) + (c0 - D));
+        if (valid && a.keep_kv) {
+          uint4* g = reinterpret_cast<uint4*>(a.kv + ((a.node0 + seq) * L + l) * (2 * D) + (c0 - D));
 #pragma unroll
           for (int q = 0; q < 4; ++q) g[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
         }
       }
       __syncthreads();
       // causal attention of this row over the keys 0..pos
-      const __half* pkv = a.kv_in ? a.kv_in + (parent * L + l) * size_t(n) * (2 * D) : nullptr;
+      const uint32_t* anc = a.anc + seq * TRIE_ANC;
 #pragma unroll 1
       for (int hd = 0; hd < H; ++hd) {
         float q[DH];
@@ -465,35 +407,33 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
           }
           m = mn;
         };
-        // keys of positions < t0 from the parent cache (global memory; the
-        // next key's words are loaded before this key's arithmetic), then
-        // the tile's own keys from shared memory
-        const int n_par = min(upto + 1, tl.t0);
-        if (n_par > 0) {
-          const uint4* gp = reinterpret_cast<const uint4*>(pkv);
+        // keys of positions < t0 (NODES) from the nodes' keys and values in
+        // global memory (the next key's words are loaded before this key's
+        // arithmetic), then the tile's own keys from shared memory
+        const int n_anc = min(upto + 1, t0);
+        if (n_anc > 0) {
+          const uint4* gp = reinterpret_cast<const uint4*>(a.kv) + size_t(l) * (2 * D / 8) + (hd * DH) / 8;
+          const size_t node = size_t(L) * (2 * D / 8);
+          uint32_t id = __ldcg(anc + (n_anc > 1 ? 1 : 0));
+          const uint4* p = gp + __ldcg(anc) * node;
           uint4 kw[DH / 8], vw[DH / 8];
 #pragma unroll
-          for (int e = 0; e < DH / 8; ++e) {
-            kw[e] = __ldg(gp + (hd * DH) / 8 + e);
-            vw[e] = __ldg(gp + (D + hd * DH) / 8 + e);
-          }
+          for (int e = 0; e < DH / 8; ++e) kw[e] = __ldg(p + e), vw[e] = __ldg(p + D / 8 + e);
 #pragma unroll 1
-          for (int u = 0; u < n_par; ++u) {
+          for (int u = 0; u < n_anc; ++u) {
             uint4 kn[DH / 8], vn[DH / 8];
-            const uint4* np = gp + size_t(u + 1 < n_par ? u + 1 : u) * (2 * D / 8);
+            p = gp + id * node;
+            id = __ldcg(anc + min(u + 2, n_anc - 1));
 #pragma unroll
-            for (int e = 0; e < DH / 8; ++e) {
-              kn[e] = __ldg(np + (hd * DH) / 8 + e);
-              vn[e] = __ldg(np + (D + hd * DH) / 8 + e);
-            }
+            for (int e = 0; e < DH / 8; ++e) kn[e] = __ldg(p + e), vn[e] = __ldg(p + D / 8 + e);
             step(kw, vw);
 #pragma unroll
             for (int e = 0; e < DH / 8; ++e) kw[e] = kn[e], vw[e] = vn[e];
           }
         }
 #pragma unroll 1
-        for (int u = tl.t0; u <= upto; ++u) {
-          const uint4* sp = reinterpret_cast<const uint4*>(sKV + (row0 + u - tl.t0) * KV_STRIDE);
+        for (int u = t0; u <= upto; ++u) {
+          const uint4* sp = reinterpret_cast<const uint4*>(sKV + (row0 + u - t0) * KV_STRIDE);
           uint4 kw[DH / 8], vw[DH / 8];
 #pragma unroll
           for (int e = 0; e < DH / 8; ++e) {
@@ -651,6 +591,7 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
             dst[1] = make_float4(out[4], out[5], out[6], out[7]);
           }
         } else {
+          // the masked half-log-probability and the phase of each outcome
           const uint64_t pm = (1ull << (2 * pos)) - 1ull;
           const unsigned pmk = slot_mask(a.hv, pos, __popcll(x & pm & 0x5555555555555555ull),
                                          __popcll(x & pm & 0xAAAAAAAAAAAAAAAAull), x);
@@ -663,27 +604,14 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             if ((mk >> u) & 1u) sum += __expf(out[u] - mx);
-          const int v = int((x >> (2 * pos)) & 3ull);
-          const float ov = (v == 0) ? out[0] : (v == 1) ? out[1] : (v == 2) ? out[2] : out[3];
-          const float pv = (v == 0) ? out[4] : (v == 1) ? out[5] : (v == 2) ? out[6] : out[7];
           const float lse = mx + __logf(sum);
-          // the row's term to shared memory (the k|v region is free now); the
-          // sequence's first row adds its positions' terms below
-          reinterpret_cast<float2*>(sKV)[t] = make_float2(((pmk >> v) & 1u) ? 0.5f * (ov - lse) : -INFINITY, pv);
+          float tm[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) tm[u] = ((pmk >> u) & 1u) ? 0.5f * (out[u] - lse) : -INFINITY;
+          float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
+          dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
+          dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
         }
-      }
-    }
-    if (a.mode == MODE_SUFFIX) {
-      // one sum per connected determinant, over its positions in order: T[x']
-      __syncthreads();
-      if (valid && pos == tl.t0) {
-        const float2* tr = reinterpret_cast<const float2*>(sKV) + t;
-        float sl = 0.f, sp = 0.f;
-        for (int i = 0; i < tl.P; ++i) {
-          sl += tr[i].x;
-          sp += tr[i].y;
-        }
-        a.T[seq] = make_float2(sl, sp);
       }
     }
     __syncthreads();  // shared k|v and hidden buffers are rewritten by the next tile
@@ -729,8 +657,7 @@ int launch(const anqs_model* M, Args a, uint64_t max_tiles, int prof, cudaStream
   return ANQS_OK;
 }
 
-Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw, __half* kv_out,
-               const HamView& hv) {
+Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw, const HamView& hv) {
   Args a{};
   a.mode = MODE_FULL;
   a.x = x;
@@ -738,39 +665,25 @@ Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw,
   a.P = P;
   a.last_only = last_only;
   a.raw = raw;
-  a.kv_out = kv_out;
   a.hv = hv;
   return a;
 }
 
-struct TfElocWs {
-  uint64_t* xp;
-  double* hv;
-  uint8_t* js;
-  double* hd;
-  float *la_x, *ph_x, *raw, *cache;
-  float2* T;
-  uint32_t *perm, *hist, *cursor, *offsets, *ticket;
-  __half* kv;
+// Scratch of the form over each sample's own prefix tree (trie.cu)
+struct TfTrieWs {
+  TrieWs t;
+  __half* kv;     // [nodes][L][2 d]
+  float2* terms;  // [nodes][4]
 };
 
-size_t plan(const anqs_model* M, const anqs_ham* H, uint64_t n_x, Arena& A, TfElocWs& w) {
-  const uint64_t n = H->v.n, m = n_x * H->v.K;
-  w.xp = A.take<uint64_t>(m);
-  w.hv = A.take<double>(m);
-  w.js = A.take<uint8_t>(m);
-  w.hd = A.take<double>(n_x);
-  w.la_x = A.take<float>(n_x);
-  w.ph_x = A.take<float>(n_x);
-  w.raw = A.take<float>(n_x * n * 8);
-  w.cache = A.take<float>(n_x * n * TC_CACHE_F);
-  w.T = A.take<float2>(m);  // one sum of the suffix positions' terms per connected determinant
-  w.perm = A.take<uint32_t>(m);
-  w.cursor = A.take<uint32_t>(ANQS_MAX_ORB);
-  w.offsets = A.take<uint32_t>(ANQS_MAX_ORB + 1);
-  w.hist = A.take<uint32_t>(TC_CTL_WORDS);
-  w.ticket = w.hist + TC_CTL_STATS_TICKET;
-  w.kv = A.take<__half>(n_x * uint64_t(M->d.n_layers) * n * 2 * uint64_t(M->d.d_model));
+// The keys and values of a group of samples take at most about this much
+constexpr uint64_t kTrieKvBytes = 8ull << 30;
+
+size_t plan_trie_tf(const anqs_model* M, const anqs_ham* H, uint64_t n_x, Arena& A, TfTrieWs& w) {
+  const uint64_t per = uint64_t(M->d.n_layers) * 2 * uint64_t(M->d.d_model);
+  plan_trie(H, n_x, kTrieKvBytes / (per * sizeof(__half)), A, w.t);
+  w.kv = A.take<__half>(w.t.node0[H->v.n - 1] * per);  // the last level's keys have no readers
+  w.terms = A.take<float2>(w.t.node0[H->v.n] * 4);
   return A.off;
 }
 
@@ -831,9 +744,9 @@ int launch_tf_tc_logpsi(const anqs_model* M, const HamView& hv, const uint64_t* 
   for (uint64_t off = 0; off < n_x; off += M->tc_raw_rows) {
     const uint64_t k = std::min<uint64_t>(M->tc_raw_rows, n_x - off);
     if (M->d.d_model == 128) {
-      ANQS_TRY(launch_tf128_full(M, hv, x + off, host_count(k), n, 0, M->tc_raw, nullptr, PROF_TF_TC_PARENT, s));
+      ANQS_TRY(launch_tf128_full(M, hv, x + off, host_count(k), n, 0, M->tc_raw, PROF_TF_TC_PARENT, s));
     } else {
-      Args a = full_args(x + off, host_count(k), n, 0, M->tc_raw, nullptr, hv);
+      Args a = full_args(x + off, host_count(k), n, 0, M->tc_raw, hv);
       ANQS_TRY(launch(M, a, (k + MT / n - 1) / (MT / n), PROF_TF_TC_PARENT, s));
     }
     ProfScope ps(PROF_TC_FINALIZE, s);
@@ -846,8 +759,8 @@ int launch_tf_tc_slot_logits(const anqs_model* M, int p, const uint64_t* pre, co
                              uint64_t max_rows, float* out8, cudaStream_t s) {
   HamView hv{};
   if (M->d.d_model == 128)
-    return launch_tf128_full(M, hv, pre, Count{max_rows, n_dev, 1}, p + 1, 1, out8, nullptr, PROF_TF_TC_SLOT, s);
-  Args a = full_args(pre, Count{max_rows, n_dev, 1}, p + 1, 1, out8, nullptr, hv);
+    return launch_tf128_full(M, hv, pre, Count{max_rows, n_dev, 1}, p + 1, 1, out8, PROF_TF_TC_SLOT, s);
+  Args a = full_args(pre, Count{max_rows, n_dev, 1}, p + 1, 1, out8, hv);
   const uint64_t S = MT / (p + 1);
   return launch(M, a, (max_rows + S - 1) / S, PROF_TF_TC_SLOT, s);
 }
@@ -858,8 +771,8 @@ size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x
     TfLeafWs v;
     return plan_leaves(H, n_x, A, v);
   }
-  TfElocWs w;
-  return plan(M, H, n_x, A, w);
+  TfTrieWs w;
+  return plan_trie_tf(M, H, n_x, A, w);
 }
 
 int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
@@ -882,9 +795,9 @@ int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Co
       const uint64_t lo = uint64_t(c) * kChunk, most = std::min<uint64_t>(kChunk, leaves.n - lo);
       const Count rows{most, leaves.dev ? (chunks > 1 ? v.counts + c : leaves.dev) : nullptr, 1};
       if (M->d.d_model == 128) {
-        ANQS_TRY(launch_tf128_full(M, H->v, lx + lo, rows, n, 0, v.raw, nullptr, PROF_TF_TC_SUFFIX, s));
+        ANQS_TRY(launch_tf128_full(M, H->v, lx + lo, rows, n, 0, v.raw, PROF_TF_TC_SUFFIX, s));
       } else {
-        const Args a = full_args(lx + lo, rows, n, 0, v.raw, nullptr, H->v);
+        const Args a = full_args(lx + lo, rows, n, 0, v.raw, H->v);
         ANQS_TRY(launch(M, a, (most + MT / n - 1) / (MT / n), PROF_TF_TC_SUFFIX, s));
       }
       ANQS_TRY(launch_byj(H->v, lx + lo, rows, v.raw, v.tab + lo * (n + 1), s));
@@ -894,51 +807,36 @@ int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Co
     amp.tab = v.tab;
     return launch_eloc_direct(H, x, n_x, v.u.nodes, amp, ere, eim, v.u.part, StatsOut{counts, stats, v.u.ticket}, s);
   }
-  TfElocWs w;
-  plan(M, H, n_x.n, A, w);
+  TfTrieWs w;
+  plan_trie_tf(M, H, n_x.n, A, w);
   if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+  if (n_x.n * H->v.K > 0xffffffffull)
+    return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
   const int n = H->v.n;
-  const uint64_t K = H->v.K;
-  const Count mc = scaled(n_x, K);
-  if (mc.n > 0xffffffffull) return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
-  ANQS_TRY(launch_connected(H->v, x, n_x, w.xp, w.hv, w.js, w.hd, s, w.hist));
-  {
-    if (M->d.d_model == 128) {
-      ANQS_TRY(launch_tf128_full(M, H->v, x, n_x, n, 0, w.raw, w.kv, PROF_TF_TC_PARENT, s));
-    } else {
-      Args a = full_args(x, n_x, n, 0, w.raw, w.kv, H->v);
-      ANQS_TRY(launch(M, a, (n_x.n + MT / n - 1) / (MT / n), PROF_TF_TC_PARENT, s));
+  for (uint64_t c = 0; c * w.t.group < n_x.n; ++c) {
+    for (int p = 0; p < n; ++p) {
+      TrieLevel lv;
+      ANQS_TRY(launch_trie_level(H, x, n_x, c, p, w.t, lv, s));
+      if (M->d.d_model == 128) {
+        ANQS_TRY(launch_tf128_nodes(M, H->v, lv, w.kv, w.terms, s));
+      } else {
+        Args a{};
+        a.mode = MODE_NODES;
+        a.hv = H->v;
+        a.x = lv.x;
+        a.n_seq = lv.rows;
+        a.P = p;
+        a.anc = lv.anc;
+        a.node0 = lv.node0;
+        a.kv = w.kv;
+        a.keep_kv = p + 1 < n;
+        a.terms = w.terms;
+        ANQS_TRY(launch(M, a, (lv.rows.n + MT - 1) / MT, PROF_TF_TC_SUFFIX, s));
+      }
     }
-    ProfScope ps(PROF_TC_FINALIZE, s);
-    ANQS_TRY(launch_tc_finalize(H->v, x, n_x, w.raw, w.la_x, w.ph_x, w.cache, s));
+    ANQS_TRY(launch_trie_eloc(H, x, n_x, c, w.t, w.terms, s));
   }
-  {
-    ProfScope ps(PROF_TC_SORT, s);
-    ANQS_TRY(launch_js_sort(w.js, mc, n, w.hist, w.cursor, w.offsets, w.perm, s));
-  }
-  if (M->d.d_model == 128) {
-    ANQS_TRY(launch_tf128_suffix(M, H->v, w.xp, w.perm, w.offsets, uint32_t(K), w.kv, w.T, mc.n, PROF_TF_TC_SUFFIX,
-                                 s));
-  } else {
-    Args a{};
-    a.mode = MODE_SUFFIX;
-    a.hv = H->v;
-    a.xp = w.xp;
-    a.perm = w.perm;
-    a.offsets = w.offsets;
-    a.K = uint32_t(K);
-    a.kv_in = w.kv;
-    a.T = w.T;
-    uint64_t tiles = 0;  // upper bound over the groups
-    for (int j = 0; j + 1 < n; ++j) tiles += mc.n / uint64_t(MT / (n - 1 - j)) + 1;
-    ANQS_TRY(launch(M, a, tiles, PROF_TF_TC_SUFFIX, s));
-  }
-  {
-    ProfScope ps(PROF_TC_ELOC, s);
-    ANQS_TRY(launch_eloc_assemble(n, uint32_t(K), n_x, w.xp, w.js, w.cache, w.T, w.hv, w.hd, w.la_x, w.ph_x, ere,
-                                  eim, StatsOut{counts, stats, w.ticket}, s, true));
-  }
-  return ANQS_OK;
+  return launch_trie_finish(H, n_x, w.t, ere, eim, counts, stats, s);
 }
 
 }  // namespace anqs

@@ -1,6 +1,6 @@
 // 16-bit tensor-core form of the causal-transformer ansatz at d_model = 128
-// (tcgen05 MMAs with TMEM accumulators), with reuse of the parent
-// determinant's keys and values for its connected determinants.  GEMM
+// (tcgen05 MMAs with TMEM accumulators), over whole sequences or over the
+// distinct prefixes of one level with the stored keys and values of the others.  GEMM
 // operands and stored keys and values are fp16 (see tf_tc.cu for why).
 //
 // The network is the one of the FP32 form (decoder-only, pre-LayerNorm, eps
@@ -28,7 +28,7 @@
 // accumulators at 128 and 256 (after k and v are consumed), the FFN output
 // accumulator at 384.  Per block:
 //   LN1 -> A (fp16)        MMA q, k, v = A W^T
-//   k, v (+ bias) -> shared memory and the parent cache; causal attention of
+//   k, v (+ bias) -> shared memory (FULL) or the node store; causal attention of
 //   each row over keys 0..t on the CUDA cores (online softmax, f32) -> A
 //   MMA o = A Wo^T         h += o + bo;  LN2 -> A
 //   FFN chunk c: MMA f1_c = A W1_c^T (issued one chunk ahead), ReLU -> H_c
@@ -38,11 +38,12 @@
 //
 // Modes (as for d_model 64)
 //   FULL    sequences x[s], positions 0..P-1: the 8 raw outputs of every
-//           position (or of the last one), optionally keys and values of
-//           every position and block (the parent cache).
-//   SUFFIX  connected determinants x' grouped by first differing slot j:
-//           positions j+1..n-1 only, keys and values of positions <= j from
-//           the parent cache; writes the masked slot terms T[x'][t].
+//           position (or of the last one).
+//   NODES   the distinct prefixes of one level p (trie.cu), one row each:
+//           position p, attending to the stored keys and values of the row's
+//           own prefixes (levels < p, found through its table) and to itself;
+//           keeps its keys and values for the later levels and writes the
+//           masked half-log-probability and the phase of each outcome.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -77,7 +78,7 @@ constexpr uint32_t OFF_LP = OFF_HX + MT * 8 * 4;              // the layer's Lay
 constexpr uint32_t LP_FLOATS = 14 * D;                         // ln1 g,b | bq bk bv bo | ln2 g,b | b1 (4D) | b2
 constexpr uint32_t SMEM_BYTES = OFF_LP + LP_FLOATS * 4;
 constexpr uint64_t kWaitNs = 2000000000ull;
-constexpr int MODE_FULL = 0, MODE_SUFFIX = 1;
+constexpr int MODE_FULL = 0, MODE_NODES = 1;
 // chunk indices within a layer
 enum { C_Q = 0, C_K, C_V, C_O, C_W1_0, C_W1_1, C_W2_0, C_W1_2, C_W2_1, C_W1_3, C_W2_2, C_W2_3 };
 static_assert(2 * A_BYTES <= KV_BYTES, "hidden chunks live in the k|v region");
@@ -92,16 +93,14 @@ struct Args {
   // FULL
   const uint64_t* x;
   Count n_seq;
-  int P, last_only;
+  int P, last_only;  // NODES: P = the level
   float* raw;
-  __half* kv_out;
-  // SUFFIX
-  const uint64_t* xp;
-  const uint32_t* perm;
-  const uint32_t* offsets;
-  uint32_t K;
-  const __half* kv_in;
-  float2* T;
+  // NODES (x, n_seq: the level's prefixes)
+  const uint32_t* anc;  // [row][TRIE_ANC] node ids of the prefix's own prefixes, levels 0..P-1
+  __half* kv;           // [node][L][2 D]
+  uint64_t node0;       // id of the level's first node
+  int keep_kv;          // the level's keys and values are needed by a later one
+  float2* terms;        // [node][4]
   int* status;
 };
 
@@ -272,14 +271,6 @@ __device__ __forceinline__ void f16x8_to_f32(const uint4 u, float (&f)[8]) {
   }
 }
 
-// Row geometry of one tile
-struct Tile {
-  bool live;
-  int P, t0, S;
-  uint64_t first;  // FULL: first sequence; SUFFIX: first index into perm
-  uint64_t count;  // sequences available from `first`
-};
-
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t phase) {
   uint32_t ok;
   asm volatile(
@@ -346,14 +337,13 @@ struct Ring {
   }
 };
 
-template <int DH>
+template <int DH, int MODE>
 __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
   constexpr int H = D / DH;        // heads
   constexpr int HPH = H / 2;       // heads per half
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2 * NS + 2];  // full[NS], empty[NS], MMA chain, FFN-output chain
   __shared__ uint32_t s_tmem;
-  __shared__ uint64_t s_tiles[ANQS_MAX_ORB + 1];
   __shared__ int s_abort;
   const int warp = threadIdx.x / 32;
   const int n = a.n, L = a.L;
@@ -373,26 +363,13 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
     const size_t tail = 5 * size_t(D) + size_t(n) * D + size_t(L) * layer_floats();
     for (int i = threadIdx.x; i < 8 * D + 8; i += NT) s_head[i] = a.params[tail + 2 * D + i];
   }
-  // work: FULL one group; SUFFIX the groups j = 0..n-2 (P = n-1-j positions)
-  if (threadIdx.x == 0) {
-    uint64_t total = 0;
-    s_tiles[0] = 0;
-    if (a.mode == MODE_FULL) {
-      const uint64_t S = MT / a.P, ns = a.n_seq.get();
-      s_tiles[1] = (ns + S - 1) / S;
-    } else {
-      for (int j = 0; j < n - 1; ++j) {
-        const uint64_t cnt = a.offsets[j + 1] - a.offsets[j], S = MT / (n - 1 - j);
-        total += (cnt + S - 1) / S;
-        s_tiles[j + 1] = total;
-      }
-    }
-  }
+  const int P = MODE == MODE_FULL ? a.P : 1;     // rows per sequence
+  const int t0 = MODE == MODE_FULL ? 0 : a.P;    // their first position
+  const int S = MT / P;                            // sequences per tile
+  const uint64_t n_seq = a.n_seq.get(), total = (n_seq + S - 1) / S;
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const int n_groups = a.mode == MODE_FULL ? 1 : n - 1;
-  const uint64_t total = s_tiles[n_groups];
   const uint32_t w_addr = tc::smem_u32(smem + OFF_W);
   const uint32_t bar_full = tc::smem_u32(&bars[0]), bar_empty = tc::smem_u32(&bars[NS]);
   const uint32_t bar_m = tc::smem_u32(&bars[2 * NS]), bar_2 = tc::smem_u32(&bars[2 * NS + 1]);
@@ -418,41 +395,11 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
     const int cb = h * HD;  // this half's first model dimension
     for (uint64_t tile = blockIdx.x; ok && tile < total; tile += gridDim.x) {
       // ---- this thread's row
-      Tile tl{};
-      {
-        int g = 0;
-        while (s_tiles[g + 1] <= tile) ++g;
-        const uint64_t k = tile - s_tiles[g];
-        tl.live = true;
-        if (a.mode == MODE_FULL) {
-          tl.P = a.P;
-          tl.t0 = 0;
-          tl.S = MT / tl.P;
-          tl.first = k * tl.S;
-          tl.count = a.n_seq.get() - tl.first;
-        } else {
-          tl.P = n - 1 - g;
-          tl.t0 = g + 1;
-          tl.S = MT / tl.P;
-          tl.first = a.offsets[g] + k * tl.S;
-          tl.count = a.offsets[g + 1] - tl.first;
-        }
-      }
-      const int s_loc = t / tl.P;
-      const bool valid = s_loc < tl.S && uint64_t(s_loc) < tl.count;
-      const int pos = valid ? tl.t0 + t % tl.P : 0;
-      uint64_t x = 0, seq = 0, parent = 0;
-      if (valid) {
-        if (a.mode == MODE_FULL) {
-          seq = tl.first + s_loc;
-          x = a.x[seq];
-        } else {
-          seq = a.perm[tl.first + s_loc];
-          x = a.xp[seq];
-          parent = seq / a.K;
-        }
-      }
-      const int row0 = s_loc * (valid ? tl.P : 0);
+      const uint64_t seq = tile * S + t / P;
+      const bool valid = t / P < S && seq < n_seq;
+      const int pos = valid ? t0 + t % P : 0;
+      const uint64_t x = valid ? a.x[seq] : 0;
+      const int row0 = t - t % P;  // tile row of this sequence's first position
       float hh[HD];
       {
         const int token = pos == 0 ? 4 : int((x >> (2 * (pos - 1))) & 3ull);
@@ -486,60 +433,73 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
         ph_m ^= 1;
         if (!ok) break;
         tc::fence_after_sync();
-        // k, v of this row and half (+ bias) -> shared memory (and the parent cache)
+        if constexpr (MODE == MODE_NODES) {
+          // 26 orbitals, 64 samples (1.29e7 rows of about 20 keys each, 4 blocks):
+          // 383 ms per call when every position after the first difference was
+          // evaluated (4.7e7 rows), 244 ms over the prefixes with the heads one
+          // after the other, 147 ms as below; what bounds it is still the wait
+          // for the keys' L2 sectors.
+          // The row's heads of this half side by side, one key after the other:
+          // a key's words of all heads are 256 contiguous bytes, all loaded
+          // before they are used (with the heads one after the other each
+          // 32-byte piece was waited for on its own, 80 waits per block).  The
+          // residual stream waits in the FFN output's columns meanwhile, so
+          // that the heads' queries and sums stay in registers.
+          tc::tmem_st32(tmem + lane_base + uint32_t(384 + cb), hh);
+          tc::tmem_st32(tmem + lane_base + uint32_t(384 + cb + 32), hh + 32);
+          tc::tmem_st_wait();
+          if (a.keep_kv) {  // k, v of this row and half (+ bias) for the later levels
+            uint4* gd = reinterpret_cast<uint4*>(a.kv + ((a.node0 + seq) * L + l) * (2 * D) + cb);
 #pragma unroll 1
-        for (int kv = 0; kv < 2; ++kv) {
-#pragma unroll 1
-          for (int c0 = 0; c0 < HD; c0 += 32) {
-            float v[32];
-            tc::tmem_ld32(tmem + lane_base + uint32_t(128 * (kv + 1) + cb + c0), v);
-            const float* bias = (kv == 0 ? lp.bk : lp.bv) + cb + c0;
-            uint32_t w[16];
+            for (int c = 0; c < 4; ++c) {
+              const int kv = c >> 1, c0 = (c & 1) * 32;
+              float v[32];
+              tc::tmem_ld32(tmem + lane_base + uint32_t(128 * (kv + 1) + cb + c0), v);
+              const float* bias = (kv == 0 ? lp.bk : lp.bv) + cb + c0;
+              if (valid) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) w[i / 2] = tc::pack_f16x2(v[i] + bias[i], v[i + 1] + bias[i + 1]);
-            const int off = kv * D + cb + c0;  // element offset within the k|v row
-            uint4* dst = reinterpret_cast<uint4*>(sKV + t * KV_STRIDE + off * 2);
+                for (int q8 = 0; q8 < 32; q8 += 8) {
+                  uint32_t w[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-            if (valid && a.kv_out) {
-              uint4* gd = reinterpret_cast<uint4*>(a.kv_out + ((seq * L + l) * n + pos) * (2 * D) + off);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) gd[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                  for (int e = 0; e < 4; ++e)
+                    w[e] = tc::pack_f16x2(v[q8 + 2 * e] + bias[q8 + 2 * e], v[q8 + 2 * e + 1] + bias[q8 + 2 * e + 1]);
+                  gd[(kv * D + c0 + q8) / 8] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+              }
+              __syncwarp();
             }
           }
-        }
-        csync();
-        // causal attention of this row over the keys 0..pos, this half's heads
-        const __half* pkv = a.kv_in ? a.kv_in + (parent * L + l) * size_t(n) * (2 * D) : nullptr;
-#pragma unroll 1
-        for (int hq = 0; hq < HPH; ++hq) {
-          const int hd = h * HPH + hq;
-          float q[DH];
-          if constexpr (DH == 16) {
-            tc::tmem_ld16(tmem + lane_base + uint32_t(hd * DH), q);
-          } else {
-            tc::tmem_ld32(tmem + lane_base + uint32_t(hd * DH), q);
+          float q[HPH][DH], acc[HPH][DH], m[HPH], ls[HPH];
+#pragma unroll
+          for (int hq = 0; hq < HPH; ++hq) {
+            if constexpr (DH == 16) {
+              tc::tmem_ld16(tmem + lane_base + uint32_t(cb + hq * DH), q[hq]);
+            } else {
+              tc::tmem_ld32(tmem + lane_base + uint32_t(cb + hq * DH), q[hq]);
+            }
+#pragma unroll
+            for (int e = 0; e < DH; ++e) {
+              q[hq][e] = (q[hq][e] + lp.bq[cb + hq * DH + e]) * scale;
+              acc[hq][e] = 0.f;
+            }
+            m[hq] = -INFINITY;
+            ls[hq] = 0.f;
           }
-#pragma unroll
-          for (int e = 0; e < DH; ++e) q[e] = (q[e] + lp.bq[hd * DH + e]) * scale;
-          float m = -INFINITY, lsum = 0.f, acc[DH];
-#pragma unroll
-          for (int e = 0; e < DH; ++e) acc[e] = 0.f;
-          const int upto = valid ? pos : -1;
-          // one key: score, online-softmax update of (m, lsum, acc)
-          auto step = [&](const uint4 (&kw)[DH / 8], const uint4 (&vw)[DH / 8]) {
+          // one key of one head: score, online-softmax update of (m, ls, acc)
+          auto step = [&](const int hq, const uint4* kw, const uint4* vw) {
             float s0 = 0.f, s1 = 0.f;
 #pragma unroll
             for (int e8 = 0; e8 < DH; e8 += 8) {
               float kf[8];
               f16x8_to_f32(kw[e8 / 8], kf);
 #pragma unroll
-              for (int e = 0; e < 8; e += 2) tc::fma_f32x2(q[e8 + e], q[e8 + e + 1], kf[e], kf[e + 1], s0, s1, s0, s1);
+              for (int e = 0; e < 8; e += 2)
+                tc::fma_f32x2(q[hq][e8 + e], q[hq][e8 + e + 1], kf[e], kf[e + 1], s0, s1, s0, s1);
             }
             const float sc = s0 + s1;
-            const float mn = fmaxf(m, sc);
-            const float corr = __expf(m - mn), p = __expf(sc - mn);
-            lsum = fmaf(lsum, corr, p);
+            const float mn = fmaxf(m[hq], sc);
+            const float corr = __expf(m[hq] - mn), p = __expf(sc - mn);
+            ls[hq] = fmaf(ls[hq], corr, p);
 #pragma unroll
             for (int e8 = 0; e8 < DH; e8 += 8) {
               float vf[8];
@@ -548,55 +508,151 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
               for (int e = 0; e < 8; e += 2) {
                 float p0, p1;
                 tc::fma_f32x2(p, p, vf[e], vf[e + 1], 0.f, 0.f, p0, p1);
-                tc::fma_f32x2(acc[e8 + e], acc[e8 + e + 1], corr, corr, p0, p1, acc[e8 + e], acc[e8 + e + 1]);
+                tc::fma_f32x2(acc[hq][e8 + e], acc[hq][e8 + e + 1], corr, corr, p0, p1, acc[hq][e8 + e],
+                              acc[hq][e8 + e + 1]);
               }
             }
-            m = mn;
+            m[hq] = mn;
           };
-          // keys of positions < t0 from the parent cache (global memory; the
-          // next key's words are loaded before this key's arithmetic), then
-          // the tile's own keys from shared memory
-          const int n_par = min(upto + 1, tl.t0);
-          if (n_par > 0) {
-            const uint4* gp = reinterpret_cast<const uint4*>(pkv);
-            uint4 kw[DH / 8], vw[DH / 8];
-#pragma unroll
-            for (int e = 0; e < DH / 8; ++e) {
-              kw[e] = __ldg(gp + (hd * DH) / 8 + e);
-              vw[e] = __ldg(gp + (D + hd * DH) / 8 + e);
-            }
+          const int n_anc = valid ? t0 : 0;
+          const uint32_t* anc = a.anc + seq * TRIE_ANC;
+          const uint4* gp = reinterpret_cast<const uint4*>(a.kv) + size_t(l) * (2 * D / 8) + cb / 8;
+          const size_t node = size_t(L) * (2 * D / 8);
+          uint32_t id = n_anc > 0 ? __ldg(anc) : 0u;
 #pragma unroll 1
-            for (int u = 0; u < n_par; ++u) {
-              uint4 kn[DH / 8], vn[DH / 8];
-              const uint4* np = gp + size_t(u + 1 < n_par ? u + 1 : u) * (2 * D / 8);
+          for (int u = 0; u < n_anc; ++u) {
+            const uint4* p = gp + id * node;
+            id = __ldg(anc + min(u + 1, n_anc - 1));
+            uint4 kw[HD / 8], vw[HD / 8];
+#pragma unroll
+            for (int e = 0; e < HD / 8; ++e) kw[e] = __ldg(p + e);
+#pragma unroll
+            for (int e = 0; e < HD / 8; ++e) vw[e] = __ldg(p + D / 8 + e);
+#pragma unroll
+            for (int hq = 0; hq < HPH; ++hq) step(hq, kw + hq * (DH / 8), vw + hq * (DH / 8));
+          }
+          __syncwarp();
+          // the row's own key, rounded as it is stored
+#pragma unroll
+          for (int hq = 0; hq < HPH; ++hq) {
+            uint4 kv[2][DH / 8];
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+              float v[DH];
+              if constexpr (DH == 16) {
+                tc::tmem_ld16(tmem + lane_base + uint32_t(128 * (w + 1) + cb + hq * DH), v);
+              } else {
+                tc::tmem_ld32(tmem + lane_base + uint32_t(128 * (w + 1) + cb + hq * DH), v);
+              }
+              const float* bias = (w == 0 ? lp.bk : lp.bv) + cb + hq * DH;
+#pragma unroll
+              for (int e8 = 0; e8 < DH; e8 += 8)
+                kv[w][e8 / 8] = make_uint4(tc::pack_f16x2(v[e8] + bias[e8], v[e8 + 1] + bias[e8 + 1]),
+                                           tc::pack_f16x2(v[e8 + 2] + bias[e8 + 2], v[e8 + 3] + bias[e8 + 3]),
+                                           tc::pack_f16x2(v[e8 + 4] + bias[e8 + 4], v[e8 + 5] + bias[e8 + 5]),
+                                           tc::pack_f16x2(v[e8 + 6] + bias[e8 + 6], v[e8 + 7] + bias[e8 + 7]));
+            }
+            if (valid) step(hq, kv[0], kv[1]);
+            __syncwarp();
+            const float inv = valid ? 1.0f / ls[hq] : 0.f;
+#pragma unroll
+            for (int e8 = 0; e8 < DH; e8 += 8) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                w[e] = tc::pack_f16x2(acc[hq][e8 + 2 * e] * inv, acc[hq][e8 + 2 * e + 1] * inv);
+              *reinterpret_cast<uint4*>(sA + tc::canon_off(t, cb + hq * DH + e8, D)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+#pragma unroll
+          for (int c0 = 0; c0 < HD; c0 += 32) {
+            float v[32];
+            tc::tmem_ld32(tmem + lane_base + uint32_t(384 + cb + c0), v);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) hh[c0 + i] = v[i];
+          }
+        } else {
+          // k, v of this row and half (+ bias) -> shared memory
+#pragma unroll 1
+          for (int kv = 0; kv < 2; ++kv) {
+#pragma unroll 1
+            for (int c0 = 0; c0 < HD; c0 += 32) {
+              float v[32];
+              tc::tmem_ld32(tmem + lane_base + uint32_t(128 * (kv + 1) + cb + c0), v);
+              const float* bias = (kv == 0 ? lp.bk : lp.bv) + cb + c0;
+              uint32_t w[16];
+#pragma unroll
+              for (int i = 0; i < 32; i += 2) w[i / 2] = tc::pack_f16x2(v[i] + bias[i], v[i + 1] + bias[i + 1]);
+              const int off = kv * D + cb + c0;  // element offset within the k|v row
+              uint4* dst = reinterpret_cast<uint4*>(sKV + t * KV_STRIDE + off * 2);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            }
+          }
+          csync();
+          // causal attention of this row over the keys 0..pos, this half's heads
+#pragma unroll 1
+          for (int hq = 0; hq < HPH; ++hq) {
+            const int hd = h * HPH + hq;
+            float q[DH];
+            if constexpr (DH == 16) {
+              tc::tmem_ld16(tmem + lane_base + uint32_t(hd * DH), q);
+            } else {
+              tc::tmem_ld32(tmem + lane_base + uint32_t(hd * DH), q);
+            }
+#pragma unroll
+            for (int e = 0; e < DH; ++e) q[e] = (q[e] + lp.bq[hd * DH + e]) * scale;
+            float m = -INFINITY, lsum = 0.f, acc[DH];
+#pragma unroll
+            for (int e = 0; e < DH; ++e) acc[e] = 0.f;
+            const int upto = valid ? pos : -1;
+            // one key: score, online-softmax update of (m, lsum, acc)
+            auto step = [&](const uint4 (&kw)[DH / 8], const uint4 (&vw)[DH / 8]) {
+              float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+              for (int e8 = 0; e8 < DH; e8 += 8) {
+                float kf[8];
+                f16x8_to_f32(kw[e8 / 8], kf);
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) tc::fma_f32x2(q[e8 + e], q[e8 + e + 1], kf[e], kf[e + 1], s0, s1, s0, s1);
+              }
+              const float sc = s0 + s1;
+              const float mn = fmaxf(m, sc);
+              const float corr = __expf(m - mn), p = __expf(sc - mn);
+              lsum = fmaf(lsum, corr, p);
+#pragma unroll
+              for (int e8 = 0; e8 < DH; e8 += 8) {
+                float vf[8];
+                f16x8_to_f32(vw[e8 / 8], vf);
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                  float p0, p1;
+                  tc::fma_f32x2(p, p, vf[e], vf[e + 1], 0.f, 0.f, p0, p1);
+                  tc::fma_f32x2(acc[e8 + e], acc[e8 + e + 1], corr, corr, p0, p1, acc[e8 + e], acc[e8 + e + 1]);
+                }
+              }
+              m = mn;
+            };
+            // the sequence's keys from shared memory
+#pragma unroll 1
+            for (int u = t0; u <= upto; ++u) {
+              const uint4* sp = reinterpret_cast<const uint4*>(sKV + (row0 + u - t0) * KV_STRIDE);
+              uint4 kw[DH / 8], vw[DH / 8];
 #pragma unroll
               for (int e = 0; e < DH / 8; ++e) {
-                kn[e] = __ldg(np + (hd * DH) / 8 + e);
-                vn[e] = __ldg(np + (D + hd * DH) / 8 + e);
+                kw[e] = sp[(hd * DH) / 8 + e];
+                vw[e] = sp[(D + hd * DH) / 8 + e];
               }
               step(kw, vw);
-#pragma unroll
-              for (int e = 0; e < DH / 8; ++e) kw[e] = kn[e], vw[e] = vn[e];
             }
-          }
-#pragma unroll 1
-          for (int u = tl.t0; u <= upto; ++u) {
-            const uint4* sp = reinterpret_cast<const uint4*>(sKV + (row0 + u - tl.t0) * KV_STRIDE);
-            uint4 kw[DH / 8], vw[DH / 8];
+            const float inv = valid ? 1.0f / lsum : 0.f;
 #pragma unroll
-            for (int e = 0; e < DH / 8; ++e) {
-              kw[e] = sp[(hd * DH) / 8 + e];
-              vw[e] = sp[(D + hd * DH) / 8 + e];
+            for (int e8 = 0; e8 < DH; e8 += 8) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) w[e] = tc::pack_f16x2(acc[e8 + 2 * e] * inv, acc[e8 + 2 * e + 1] * inv);
+              *reinterpret_cast<uint4*>(sA + tc::canon_off(t, hd * DH + e8, D)) = make_uint4(w[0], w[1], w[2], w[3]);
             }
-            step(kw, vw);
-          }
-          const float inv = valid ? 1.0f / lsum : 0.f;
-#pragma unroll
-          for (int e8 = 0; e8 < DH; e8 += 8) {
-            uint32_t w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) w[e] = tc::pack_f16x2(acc[e8 + 2 * e] * inv, acc[e8 + 2 * e + 1] * inv);
-            *reinterpret_cast<uint4*>(sA + tc::canon_off(t, hd * DH + e8, D)) = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
         tc::fence_async_smem();
@@ -717,13 +773,14 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
         if (h == 0 && valid) {
 #pragma unroll
           for (int o = 0; o < 8; ++o) out[o] += s_hx[t * 8 + o] + s_head[8 * D + o];
-          if (a.mode == MODE_FULL) {
+          if constexpr (MODE == MODE_FULL) {
             if (!a.last_only || pos == a.P - 1) {
               float4* dst = reinterpret_cast<float4*>(a.raw + (a.last_only ? seq : seq * a.P + pos) * 8);
               dst[0] = make_float4(out[0], out[1], out[2], out[3]);
               dst[1] = make_float4(out[4], out[5], out[6], out[7]);
             }
           } else {
+            // the masked half-log-probability and the phase of each outcome
             const uint64_t pm = (1ull << (2 * pos)) - 1ull;
             const unsigned pmk = slot_mask(a.hv, pos, __popcll(x & pm & 0x5555555555555555ull),
                                            __popcll(x & pm & 0xAAAAAAAAAAAAAAAAull), x);
@@ -736,28 +793,14 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
 #pragma unroll
             for (int u = 0; u < 4; ++u)
               if ((mk >> u) & 1u) sum += __expf(out[u] - mx);
-            const int v = int((x >> (2 * pos)) & 3ull);
-            const float ov = (v == 0) ? out[0] : (v == 1) ? out[1] : (v == 2) ? out[2] : out[3];
-            const float pv = (v == 0) ? out[4] : (v == 1) ? out[5] : (v == 2) ? out[6] : out[7];
             const float lse = mx + __logf(sum);
-            // the row's term to its own exchange slot (read above); the
-            // sequence's first row adds its positions' terms below
-            reinterpret_cast<float2*>(s_hx + t * 8)[0] =
-                make_float2(((pmk >> v) & 1u) ? 0.5f * (ov - lse) : -INFINITY, pv);
+            float tm[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) tm[u] = ((pmk >> u) & 1u) ? 0.5f * (out[u] - lse) : -INFINITY;
+            float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
+            dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
+            dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
           }
-        }
-      }
-      if (a.mode == MODE_SUFFIX) {
-        // one sum per connected determinant, over its positions in order: T[x']
-        csync();
-        if (h == 0 && valid && pos == tl.t0) {
-          float sl = 0.f, sp = 0.f;
-          for (int i = 0; i < tl.P; ++i) {
-            const float2 tv = reinterpret_cast<const float2*>(s_hx + (t + i) * 8)[0];
-            sl += tv.x;
-            sp += tv.y;
-          }
-          a.T[seq] = make_float2(sl, sp);
         }
       }
       csync();  // shared k|v, hidden buffers and exchange slots are rewritten by the next tile
@@ -792,18 +835,17 @@ int launch(const anqs_model* M, Args a, uint64_t max_tiles, int prof, cudaStream
   const unsigned grid = unsigned(std::max<uint64_t>(1, std::min<uint64_t>(max_tiles, uint64_t(sms()))));
   const int dh = D / M->d.n_heads;
   ProfScope ps(prof, s);
-  if (dh == 16) {
-    ANQS_CUDA(cudaFuncSetAttribute(tf128_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES)));
-    ANQS_CUDA_LAUNCH("tf128_kernel", launch_k(tf128_kernel<16>, dim3(grid), dim3(NT), SMEM_BYTES, s, a));
-  } else {
-    ANQS_CUDA(cudaFuncSetAttribute(tf128_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES)));
-    ANQS_CUDA_LAUNCH("tf128_kernel", launch_k(tf128_kernel<32>, dim3(grid), dim3(NT), SMEM_BYTES, s, a));
-  }
+  auto go = [&](auto kern) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES));
+    return e != cudaSuccess ? e : launch_k(kern, dim3(grid), dim3(NT), SMEM_BYTES, s, a);
+  };
+  ANQS_CUDA_LAUNCH("tf128_kernel", a.mode == MODE_NODES
+                                       ? (dh == 16 ? go(tf128_kernel<16, MODE_NODES>) : go(tf128_kernel<32, MODE_NODES>))
+                                       : (dh == 16 ? go(tf128_kernel<16, MODE_FULL>) : go(tf128_kernel<32, MODE_FULL>)));
   return ANQS_OK;
 }
 
-Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw, __half* kv_out,
-               const HamView& hv) {
+Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw, const HamView& hv) {
   Args a{};
   a.mode = MODE_FULL;
   a.x = x;
@@ -811,7 +853,6 @@ Args full_args(const uint64_t* x, Count n_seq, int P, int last_only, float* raw,
   a.P = P;
   a.last_only = last_only;
   a.raw = raw;
-  a.kv_out = kv_out;
   a.hv = hv;
   return a;
 }
@@ -834,28 +875,26 @@ int tf128_pack(anqs_model* M, cudaStream_t s) {
 int tf128_status_offset(const anqs_model* M) { return int(size_t(M->d.n_layers) * LAYER_BYTES); }
 
 int launch_tf128_full(const anqs_model* M, const HamView& hv, const uint64_t* x, Count n_seq, int P, int last_only,
-                      float* raw, __half* kv_out, int prof, cudaStream_t s) {
-  Args a = full_args(x, n_seq, P, last_only, raw, kv_out, hv);
+                      float* raw, int prof, cudaStream_t s) {
+  Args a = full_args(x, n_seq, P, last_only, raw, hv);
   const uint64_t S = MT / P;
   return launch(M, a, (n_seq.n + S - 1) / S, prof, s);
 }
 
-int launch_tf128_suffix(const anqs_model* M, const HamView& hv, const uint64_t* xp, const uint32_t* perm,
-                        const uint32_t* offsets, uint32_t K, const __half* kv_in, float2* T, uint64_t m_max,
-                        int prof, cudaStream_t s) {
+int launch_tf128_nodes(const anqs_model* M, const HamView& hv, const TrieLevel& lv, __half* kv, float2* terms,
+                       cudaStream_t s) {
   Args a{};
-  a.mode = MODE_SUFFIX;
+  a.mode = MODE_NODES;
   a.hv = hv;
-  a.xp = xp;
-  a.perm = perm;
-  a.offsets = offsets;
-  a.K = K;
-  a.kv_in = kv_in;
-  a.T = T;
-  const int n = hv.n;
-  uint64_t tiles = 0;  // upper bound over the groups
-  for (int j = 0; j + 1 < n; ++j) tiles += m_max / uint64_t(MT / (n - 1 - j)) + 1;
-  return launch(M, a, tiles, prof, s);
+  a.x = lv.x;
+  a.n_seq = lv.rows;
+  a.P = lv.p;
+  a.anc = lv.anc;
+  a.node0 = lv.node0;
+  a.kv = kv;
+  a.keep_kv = lv.p + 1 < hv.n;
+  a.terms = terms;
+  return launch(M, a, (lv.rows.n + MT - 1) / MT, PROF_TF_TC_SUFFIX, s);
 }
 
 }  // namespace anqs

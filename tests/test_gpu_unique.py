@@ -49,7 +49,7 @@ def _dets(n, na, nb, m, seed, parity=None):
         x = sum(1 << (2 * int(p)) for p in rng.choice(n, na, replace=False))
         x += sum(1 << (2 * int(p) + 1) for p in rng.choice(n, nb, replace=False))
         if parity is None or bin(x & parity[0]).count("1") % 2 == parity[1]:
-            out.add(x)
+            out.add(x - ((x >> 63) << 64))  # as int64
         if len(out) == m:
             break
     return torch.tensor(sorted(out), dtype=torch.int64, device="cuda")
@@ -116,13 +116,49 @@ def test_reuse_forms_match_amplitudes_of_the_connected_list(A, kind, form, n, na
     assert torch.all((ere - e.real).abs() <= bound) and torch.all((eim - e.imag).abs() <= bound)
 
 
-@pytest.mark.parametrize("kind,form", [("mlp", "fp32"), ("mlp", "bf16"), ("tf", "bf16"), ("nade", "fp32")])
-def test_determinants_outside_the_sector(A, kind, form):
+# sectors without a prefix index (csrc/trie.cu): few and many electrons, full shells of one spin, and pruning
+@pytest.mark.parametrize("n,na,nb,m,du", [(19, 1, 1, 5, 0), (20, 2, 1, 40, 0), (21, 21, 2, 7, 1), (24, 0, 2, 3, 0),
+                                          (32, 2, 30, 6, 2)])
+def test_prefix_trees_match_amplitudes_of_the_connected_list(A, n, na, nb, m, du):
+    test_reuse_forms_match_amplitudes_of_the_connected_list(A, "tf", "bf16", n, na, nb, m, du)
+
+
+def test_prefix_trees_in_groups(A):
+    """24 samples of 26 orbitals (more than one group of keys and values) against two calls of 12, bit for bit, and
+    the excitations' order against anqs_connected's elements through a sum rule: for a constant amplitude E_loc is
+    the row sum of the Hamiltonian."""
+    from synthetic import flatten_tf, integrals, tf_params
+    n, ne = 26, 9
+    h, g, e = integrals(5, n, 8)
+    ham = A.Hamiltonian(h, g, e, ne, ne)
+    P = tf_params(5, n, 128, 4, bias_std=0.1)
+    model = A.Model.transformer(n, 128, 8, 4, torch.tensor(flatten_tf(P), device="cuda"), "bf16")
+    x = _dets(n, ne, ne, 24, 8)
+    cnt = torch.ones_like(x)
+    a = A.local_energy(model, ham, x, cnt)
+    halves = [A.local_energy(model, ham, x[k:k + 12].contiguous(), cnt[:12]) for k in (0, 12)]
+    for i in range(2):
+        assert torch.equal(a[i], torch.cat([v[i] for v in halves]))
+    P["head_w"][:] = 0  # all logits and phases equal: |psi|^2 uniform over each slot's allowed outcomes, phase zero
+    P["head_b"][:] = 0
+    flat = A.Model.transformer(n, 128, 8, 4, torch.tensor(flatten_tf(P), device="cuda"), "bf16")
+    xp, hv, _, hd = A.connected(ham, x[:4].contiguous())
+    la = A.logpsi(flat, ham, x[:4].contiguous())[0].double()
+    lp = A.logpsi(flat, ham, xp.reshape(-1))[0].view(xp.shape).double()
+    w = hv * torch.exp(lp - la[:, None])
+    ere, eim, _ = A.local_energy(flat, ham, x[:4].contiguous())
+    assert torch.all((ere - hd - w.sum(1)).abs() <= 1e-9 + 4e-5 * w.abs().sum(1)) and torch.all(eim == 0)
+
+
+@pytest.mark.parametrize("kind,form,n", [("mlp", "fp32", 6), ("mlp", "bf16", 6), ("tf", "bf16", 6), ("nade", "fp32", 6),
+                                         ("tf", "bf16", 20)])
+def test_determinants_outside_the_sector(A, kind, form, n):
     """NaN for rows with other electron counts or bits beyond the orbitals; the other rows as without them."""
-    model, ham = _problem(A, kind, form, 6, 3, 2, 7)
-    x = _dets(6, 3, 2, 20, 1)
+    model, ham = _problem(A, kind, form, n, 3, 2, 7)
+    x = _dets(n, 3, 2, 20, 1)
     ref = A.local_energy(model, ham, x)
-    bad = torch.cat([x[:7], torch.tensor([0, 1 << 12, (1 << 12) | int(x[0]), -1], device="cuda"), x[7:]])
+    high = 1 << (2 * n)
+    bad = torch.cat([x[:7], torch.tensor([0, high, high | int(x[0]), -1], device="cuda"), x[7:]])
     ere, eim, _ = A.local_energy(model, ham, bad)
     assert torch.isnan(ere[7:11]).all() and torch.isnan(eim[7:11]).all()
     keep = torch.cat([torch.arange(7), torch.arange(11, bad.numel())]).cuda()
