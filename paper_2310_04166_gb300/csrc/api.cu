@@ -244,10 +244,7 @@ static int vjp_dispatch(const anqs_model* M, const anqs_ham* H, const uint64_t* 
                         const float* cp, float* grad, float* part, void* ws, size_t ws_bytes, cudaStream_t s) {
   if (M->d.kind == ANQS_MODEL_MLP) {
     const CotSrc c{cl, cp, nullptr, nullptr, nullptr, nullptr};
-    // the tensor-core adjoint writes per-tile partial gradients (anqs_grad's
-    // workspace); anqs_logpsi_vjp, which has none for the MLP, stays in FP32
-    if (part && M->d.form == ANQS_FORM_BF16 && mlp_tc_grad_supported(M))
-      return launch_mlp_tc_grad(M, H->v, x, n_x, c, grad, part, s);
+    // anqs_logpsi_vjp stays in FP32 (the tensor-core adjoint needs anqs_grad's workspace)
     return launch_mlp_fp32_grad(M->mlp, H->v, x, n_x, c, grad, part, s);
   }
   if (M->d.kind == ANQS_MODEL_TF) return launch_tf_fp32_grad(M->tf, H, x, n_x, cl, cp, grad, ws, ws_bytes, s);
@@ -1243,7 +1240,7 @@ int anqs_grad(const anqs_model* M, const anqs_ham* H, const uint64_t* x, const u
   const CotSrc vmc{nullptr, nullptr, ere, eim, stats, counts};
   if (M->d.kind == ANQS_MODEL_MLP) {
     if (M->d.form == ANQS_FORM_BF16 && mlp_tc_grad_supported(M))  // 16-bit forward and adjoint on the tensor cores
-      return launch_mlp_tc_grad(M, H->v, x, nc, vmc, grad, part, s);
+      return launch_mlp_tc_grad(M, H->v, x, nc, vmc, cl, cp, grad, part, s);
     return launch_mlp_fp32_grad(M->mlp, H->v, x, nc, vmc, grad, part, s);
   }
   if (M->d.kind == ANQS_MODEL_NADE)

@@ -549,11 +549,13 @@ __global__ void __launch_bounds__(NT) grad_kernel(MlpView m, HamView hv, const u
   }
 }
 
-// grad[i] = sum over the tiles of the per-tile copies (only tiles holding rows)
-__global__ void partial_sum_kernel(const float* __restrict__ part, Count n_x_, uint64_t n_params, int rg,
+// grad[i] = sum over the copies: one per tile of rg rows (only tiles holding
+// rows), at most `most`
+__global__ void partial_sum_kernel(const float* __restrict__ part, Count n_x_, uint64_t n_params, int rg, uint64_t most,
                                    float* __restrict__ grad) {
   ANQS_PDL_ENTRY();
-  const uint64_t tiles = (n_x_.get() + rg - 1) / rg;
+  uint64_t tiles = (n_x_.get() + rg - 1) / rg;
+  if (tiles > most) tiles = most;
   for (uint64_t i = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; i < n_params;
        i += uint64_t(gridDim.x) * blockDim.x) {
     // four tiles' loads in flight at a time, added in tile order
@@ -632,7 +634,7 @@ int grad_launch(const MlpView& m, const HamView& hv, const uint64_t* x, Count n_
     ProfScope ps(PROF_GRAD_REDUCE, s);
     ANQS_CUDA_LAUNCH("mlp partial_sum_kernel",
                      launch_k(partial_sum_kernel, dim3(unsigned(std::min<uint64_t>((n_params + 255) / 256, 152 * 8))),
-                              dim3(256), 0, s, part, n_x, n_params, RG, g));
+                              dim3(256), 0, s, part, n_x, n_params, RG, ~0ull, g));
   } else {
     ANQS_TRY(set_smem(grad_kernel<W, RG, false, RES>, sm));
     ProfScope ps(PROF_MLP_FP32_GRAD, s);
@@ -699,12 +701,12 @@ int launch_mlp_fp32_slot_logits(const MlpView& m, int p, const uint64_t* pre, co
   return set_error(ANQS_ERR_UNSUPPORTED, "width %d", m.width);
 }
 
-int launch_grad_partial_sum(const float* part, Count n_x, uint64_t n_params, int rows_per_tile, float* g,
+int launch_grad_partial_sum(const float* part, Count n_x, uint64_t n_params, int rows_per_tile, uint64_t most, float* g,
                             cudaStream_t s) {
   ProfScope ps(PROF_GRAD_REDUCE, s);
   ANQS_CUDA_LAUNCH("mlp partial_sum_kernel",
                    launch_k(partial_sum_kernel, dim3(unsigned(std::min<uint64_t>((n_params + 255) / 256, 152 * 8))),
-                            dim3(256), 0, s, part, n_x, n_params, rows_per_tile, g));
+                            dim3(256), 0, s, part, n_x, n_params, rows_per_tile, most, g));
   return ANQS_OK;
 }
 

@@ -901,22 +901,30 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_multi_kernel(const __grid_consta
 
 // ---- the adjoint (Eq. grad_def) on the tensor cores ------------------------
 //
-// One CTA of 128 threads per (128-row tile of the samples, slot p); thread t
-// owns sample row t and TMEM lane t.  It recomputes slot p's forward pass in
-// the 16-bit form (layer 1 from the hi part of W1), turns the cotangents of
-// log|psi| and arg psi into the head's adjoint, and runs the backward pass:
+// CTA (g, p) of 256 threads takes the 128-row tiles g, g + G, ... of slot p
+// with the slot's weights resident in shared memory; thread (h, t) owns half
+// h of the columns of sample row t (TMEM lane t).  A tile recomputes slot p's
+// forward pass in the 16-bit form (layer 1 from the hi part of W1), turns the
+// cotangents of log|psi| and arg psi into the head's adjoint, and runs the
+// backward pass:
 //   data GEMMs    dh_{k-1} = dz_k W_k           (A: dz_k per row, B: W_k)
 //   weight GEMMs  dW_k = dz_k^T h_{k-1}, dW_1 = dz_1^T u, dW_h = dout^T h_L
 // The weight GEMMs reduce over the tile's rows, so their operands are the
 // same per-row tiles read as MN-major matrices (K = rows), and the data GEMMs
 // read the forward weight image as an MN-major B operand: no transposed copy
-// of anything is made.  Operands are fp16; the cotangents of each tile are
-// scaled by a power of two that puts their largest magnitude at 2^8 (the
-// gradient is linear in them; the scale is divided out, exactly, when the
-// tile's partial gradient is written).  Biases' gradients are the column sums
-// of the dz tiles, one more small MMA per layer against the dout tile, whose
-// column 8 holds ones.  Each tile writes its slot's block of a per-tile
-// partial gradient; a reduction over the tiles follows.
+// of anything is made.  Biases' gradients are the column sums of the dz
+// tiles, one more small MMA per layer against the dout tile, whose column 8
+// holds ones.  Operands are fp16; the cotangents are scaled by a power of two
+// that puts their largest magnitude at 2^8 (the gradient is linear in them;
+// the scale is divided out, exactly, when the sums are written).
+//
+// The weight gradients stay in tensor memory over kFlush tiles, so a CTA
+// writes its slot's block of partial gradients (f32, one slab per g) once per
+// kFlush tiles instead of once per tile; a reduction over the slabs follows.
+// One tile is a serial chain of MMA, wait and epilogue; what a tile cost
+// beyond it before was reading and writing its 150 KB of partial gradients,
+// fetching its 84 KB of weights and 128 instead of 256 threads in each
+// epilogue.
 __device__ __forceinline__ int popc_alpha_tc(uint64_t x, int p) {
   return __popcll(x & ((1ull << (2 * p)) - 1ull) & 0x5555555555555555ull);
 }
@@ -949,7 +957,34 @@ struct GradArgs {
   float* part;  // [tiles][n_params]
   uint64_t n_params;
   uint32_t img_bytes, kmax1;  // image region (without W1's lo part), widest layer-1 input
+  const float* maxes;  // [kMaxes] maxima of the cotangents' magnitudes, or null: each CTA has one tile, its own scale
 };
+constexpr int kMaxes = 152;
+constexpr uint32_t kFlush = 16;  // 128 MMAs in a row onto one accumulator
+
+// Cotangents to arrays (cl, cp) and the maximum of their magnitudes per CTA
+__global__ void __launch_bounds__(256) cot_max_kernel(CotSrc cot, Count n_x_, float* cl, float* cp, float* maxes) {
+  ANQS_PDL_ENTRY();
+  __shared__ float s_max[8];
+  const uint64_t n_x = n_x_.get();
+  float mx = 0.f;
+  for (uint64_t l = blockIdx.x * 256ull + threadIdx.x; l < n_x; l += gridDim.x * 256ull) {
+    float a, b;
+    cot_of(cot, l, a, b);
+    if (cot.stats) {
+      cl[l] = a;
+      cp[l] = b;
+    }
+    mx = fmaxf(mx, fmaxf(fabsf(a), fabsf(b)));
+  }
+  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, s_max[w]);
+    maxes[blockIdx.x] = mx;
+  }
+}
 
 // MN-major view of a tile stored per row in the canonical K-major layout with
 // `cols` columns: the MMA's K runs over the rows (16 per step), M or N over
@@ -962,19 +997,22 @@ __host__ __device__ constexpr uint32_t idesc_f16_mn(int M, int N, bool a_mn, boo
   return tc::idesc_f16_f32(M, N) | (a_mn ? (1u << 15) : 0u) | (b_mn ? (1u << 16) : 0u);
 }
 
+constexpr int GNT = 2 * MT;
+
 template <int W>
-__global__ void __launch_bounds__(MT, 1) mlp_tc_grad_kernel(const __grid_constant__ GradArgs a) {
+__global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_constant__ GradArgs a) {
   static_assert(W == 128, "the weight GEMMs put the layer width on the MMA's M = 128");
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t s_tmem;
-  __shared__ float s_max[4], s_bh[4][8];
-  __shared__ int s_abort;
+  __shared__ float s_max[8], s_bh[4][8];
   constexpr uint32_t TILE = MT * W * 2u;
-  constexpr uint32_t C_ACC = 0, C_DW = W, C_DWH = 2 * W, C_DB = 2 * W + 16, C_DW1 = 2 * W + 32,
-                     NCOL = W == 128 ? 512 : 256;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  constexpr int HW = W / 2;  // columns per half
+  const int h = threadIdx.x / MT, t = threadIdx.x % MT, warp = t >> 5, lane = t & 31;
   const int p = blockIdx.y, L = a.m.n_hidden;
+  // TMEM columns: data accumulator | dW_L..dW_2 | dW_1 (64) | dW_h (16) | db_1..db_L (16 each)
+  const uint32_t C_ACC = 0, C_DW1 = uint32_t(L) * W, C_DWH = C_DW1 + 64, C_DB = C_DWH + 16;
+  constexpr uint32_t NCOL = 512;
   const SlotLayout S = slot_layout(p, W, L, a.tv.lo);
   const uint32_t k1 = S.k1, lo_bytes = S.wk - S.w1lo;
   // shared memory: image (W1 hi | hidden | bias | f32 head) | H_1..H_{L-1} | P1 | P2 | U | dout (and ones)
@@ -986,18 +1024,17 @@ __global__ void __launch_bounds__(MT, 1) mlp_tc_grad_kernel(const __grid_constan
   unsigned char* U = P2 + TILE;
   unsigned char* DO = U + MT * a.kmax1 * 2u;
   const uint32_t bar_w = tc::smem_u32(&bars[0]), bar_m = tc::smem_u32(&bars[1]);
-  if (t == 0) {
+  if (threadIdx.x == 0) {
     tc::mbar_init(bar_w, 1);
     tc::mbar_init(bar_m, 1);
     tc::fence_mbar_init();
-    s_abort = 0;
     // the image, written by the packing kernel several launches back
     const unsigned char* src = a.tv.img + a.tv.img_off[p];
     tc::mbar_arrive_expect_tx(bar_w, S.w1lo + (S.head16 - S.wk));
     if (S.w1lo) tc::bulk_g2s(tc::smem_u32(img), src, S.w1lo, bar_w);
     tc::bulk_g2s(tc::smem_u32(img + o_wk), src + S.wk, S.head16 - S.wk, bar_w);
   }
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     tc::tmem_alloc(tc::smem_u32(&s_tmem), NCOL);
     tc::tmem_relinquish();
   }
@@ -1008,40 +1045,9 @@ __global__ void __launch_bounds__(MT, 1) mlp_tc_grad_kernel(const __grid_constan
   ANQS_PDL_TRIGGER();
   const uint32_t tm = s_tmem, lb = uint32_t(t & ~31) << 16;
   const uint64_t n_x = a.n_x.get();
-  const uint64_t row = uint64_t(blockIdx.x) * MT + t;
-  const bool valid = row < n_x;
-  const uint64_t x = valid ? a.xs[row] : 0ull;
-  float cla = 0.f, cph = 0.f;
-  if (valid) cot_of(a.cot, row, cla, cph);
-  // scale of the tile's cotangents: a power of two, largest magnitude -> 2^8
-  {
-    float mx = fmaxf(fabsf(cla), fabsf(cph));
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) s_max[warp] = mx;
-  }
-  // one-hot input of v_<p (layer 1's A operand and dW_1's B operand)
-  for (uint32_t k = 0; k < k1; k += 8) {
-    uint32_t w4[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      uint32_t lo = 0, hi = 0;
-      const uint32_t k0 = k + 2 * e, kk = k0 + 1;
-      if (k0 < 4u * p && ((x >> (2 * (k0 >> 2))) & 3ull) == (k0 & 3u)) lo = 0x3C00u;
-      if (kk < 4u * p && ((x >> (2 * (kk >> 2))) & 3ull) == (kk & 3u)) hi = 0x3C00u;
-      w4[e] = lo | (hi << 16);
-    }
-    *reinterpret_cast<uint4*>(U + tc::canon_off(t, k, k1)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-  }
-  tc::fence_async_smem();
-  tc::fence_before_sync();
-  __syncthreads();
-  float mx = fmaxf(fmaxf(s_max[0], s_max[1]), fmaxf(s_max[2], s_max[3]));
-  int e2 = 0;
-  if (mx > 0.f) {
-    frexpf(mx, &e2);  // mx in [2^(e2-1), 2^e2)
-    e2 = 8 - e2;
-  }
-  const float sc = ldexpf(1.f, e2), inv_sc = ldexpf(1.f, -e2);
+  const uint32_t tiles = uint32_t((n_x + MT - 1) / MT);
+  const MlpPtrTc P = slot_ptrs_tc(a.m, p);
+  float* gbase = a.part + uint64_t(blockIdx.x) * a.n_params;
   bool ok = __syncthreads_and(wait_bar(bar_w, 0));
   uint32_t ph = 0;
   auto mma_wait = [&]() -> bool {
@@ -1050,224 +1056,53 @@ __global__ void __launch_bounds__(MT, 1) mlp_tc_grad_kernel(const __grid_constan
     tc::fence_after_sync();
     return r;
   };
+  auto sync_tiles = [&]() {  // operand tiles written: visible to the MMAs issued next
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+  };
   const float* bias = reinterpret_cast<const float*>(img + o_bias);
   const float4* head = reinterpret_cast<const float4*>(img + o_head);
   const float* hbias = reinterpret_cast<const float*>(img + o_hb);
   const uint32_t img_a = tc::smem_u32(img);
-  // ---- forward: h_1 .. h_{L-1} to their tiles, z_L left in TMEM ----
-  for (int layer = 0; ok && layer < L; ++layer) {
-    const uint32_t K = layer == 0 ? k1 : uint32_t(W);
-    if (K > 0) {
-      if (t == 0) {
-        tc::fence_after_sync();
-        const uint32_t a_addr = layer == 0 ? tc::smem_u32(U) : tc::smem_u32(Hb + uint32_t(layer - 1) * TILE);
-        const uint32_t b_addr = img_a + (layer == 0 ? 0u : o_wk + uint32_t(layer - 1) * W * W * 2u);
-        for (uint32_t ks = 0; ks < K / 16; ++ks)
-          tc::mma_f16(tm + C_ACC, tc::sdesc(a_addr + ks * 256u, 128u, K * 16u),
-                      tc::sdesc(b_addr + ks * 256u, 128u, K * 16u), tc::idesc_f16_f32(MT, W), ks > 0 ? 1u : 0u);
-        tc::mma_commit(bar_m);
-      }
-      ok = mma_wait();
-    }
-    if (!ok || layer == L - 1) break;
-    unsigned char* dst = Hb + uint32_t(layer) * TILE;
-    for (int c0 = 0; c0 < W; c0 += 32) {
-      float v[32];
-      if (K > 0) {
-        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(c0), v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t u4[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int i = 8 * q + 2 * e;
-          u4[e] = tc::pack_f16x2(tc::tanh_fast(v[i] + bias[layer * W + c0 + i]),
-                                 tc::tanh_fast(v[i + 1] + bias[layer * W + c0 + i + 1]));
-        }
-        *reinterpret_cast<uint4*>(dst + tc::canon_off(t, c0 + 8 * q, W)) = make_uint4(u4[0], u4[1], u4[2], u4[3]);
-      }
-    }
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-  }
   const bool kL = (L == 1 ? k1 : uint32_t(W)) > 0;  // z_L is in TMEM (else it is zero)
-  // ---- head (f32) and the adjoint of its 8 outputs ----
-  float dout[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (ok) {
-    float out[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) out[o] = 0.f;
-    for (int c0 = 0; c0 < W; c0 += 32) {
-      float v[32];
-      if (kL) {
-        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(c0), v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float h = tc::tanh_fast(v[i] + bias[(L - 1) * W + c0 + i]);
-        const float4 w0 = head[(c0 + i) * 2], w1 = head[(c0 + i) * 2 + 1];
-        out[0] = fmaf(w0.x, h, out[0]);
-        out[1] = fmaf(w0.y, h, out[1]);
-        out[2] = fmaf(w0.z, h, out[2]);
-        out[3] = fmaf(w0.w, h, out[3]);
-        out[4] = fmaf(w1.x, h, out[4]);
-        out[5] = fmaf(w1.y, h, out[5]);
-        out[6] = fmaf(w1.z, h, out[6]);
-        out[7] = fmaf(w1.w, h, out[7]);
-      }
+  const int cb = h * HW;
+  float sc = 1.f, inv_sc = 1.f, bh[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // scale from the largest magnitude of mx over the CTA: largest magnitude -> 2^8
+  auto set_scale = [&](float mx) {
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_max[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_max[w]);
+    int e2 = 0;
+    if (mx > 0.f) {
+      frexpf(mx, &e2);  // mx in [2^(e2-1), 2^e2)
+      e2 = 8 - e2;
     }
-#pragma unroll
-    for (int o = 0; o < 8; ++o) out[o] += hbias[o];
-    // d l_u = cot_la 1/2 (delta_uv - p~_u) over the allowed u; d phi_u = cot_ph delta_uv
-    if (valid) {
-      const unsigned pm = slot_mask(a.hv, p, popc_alpha_tc(x, p), popc_beta_tc(x, p), x), mk = norm_mask(a.hv, p, pm);
-      const int v = int((x >> (2 * p)) & 3ull);
-      if ((pm >> v) & 1u) {
-        float m = -INFINITY;
-        for (int u = 0; u < 4; ++u)
-          if ((mk >> u) & 1u) m = fmaxf(m, out[u]);
-        float ex[4], sum = 0.f;
-        for (int u = 0; u < 4; ++u) {
-          ex[u] = ((mk >> u) & 1u) ? __expf(out[u] - m) : 0.f;
-          sum += ex[u];
-        }
-        const float c = 0.5f * cla * sc;
-        for (int u = 0; u < 4; ++u) dout[u] = ((mk >> u) & 1u) ? c * ((u == v ? 1.f : 0.f) - ex[u] / sum) : 0.f;
-        dout[4 + v] = cph * sc;
-      }
-    }
-    // dout tile (fp16, 16 columns: dout, then a one in column 8): B operand of
-    // dW_h and of the bias sums
-    uint32_t d4[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) d4[e] = tc::pack_f16x2(dout[2 * e], dout[2 * e + 1]);
-    *reinterpret_cast<uint4*>(DO + tc::canon_off(t, 0, 16)) = make_uint4(d4[0], d4[1], d4[2], d4[3]);
-    *reinterpret_cast<uint4*>(DO + tc::canon_off(t, 8, 16)) = make_uint4(0x3C00u, 0u, 0u, 0u);
-    // h_L (fp16) to P1, dz_L = (W_h^T dout) (1 - h_L^2) to P2
-    for (int c0 = 0; c0 < W; c0 += 32) {
-      float v[32];
-      if (kL) {
-        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(c0), v);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t hu[4], zu[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float hh[2], zz[2];
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int i = 8 * q + 2 * e + j, k = c0 + i;
-            const float h = tc::tanh_fast(v[i] + bias[(L - 1) * W + k]);
-            const float4 w0 = head[k * 2], w1 = head[k * 2 + 1];
-            float dh = w0.x * dout[0];
-            dh = fmaf(w0.y, dout[1], dh);
-            dh = fmaf(w0.z, dout[2], dh);
-            dh = fmaf(w0.w, dout[3], dh);
-            dh = fmaf(w1.x, dout[4], dh);
-            dh = fmaf(w1.y, dout[5], dh);
-            dh = fmaf(w1.z, dout[6], dh);
-            dh = fmaf(w1.w, dout[7], dh);
-            hh[j] = h;
-            zz[j] = dh * (1.f - h * h);
-          }
-          hu[e] = tc::pack_f16x2(hh[0], hh[1]);
-          zu[e] = tc::pack_f16x2(zz[0], zz[1]);
-        }
-        *reinterpret_cast<uint4*>(P1 + tc::canon_off(t, c0 + 8 * q, W)) = make_uint4(hu[0], hu[1], hu[2], hu[3]);
-        *reinterpret_cast<uint4*>(P2 + tc::canon_off(t, c0 + 8 * q, W)) = make_uint4(zu[0], zu[1], zu[2], zu[3]);
-      }
-    }
-  }
-  // d b_h: column sums of dout over the rows (f32, warp shuffles)
-#pragma unroll
-  for (int o = 0; o < 8; ++o) {
-    float sum = dout[o];
-    for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-    if (lane == 0) s_bh[warp][o] = sum;
-  }
-  tc::fence_async_smem();
-  tc::fence_before_sync();
-  __syncthreads();
-  const MlpPtrTc P = slot_ptrs_tc(a.m, p);
-  float* gbase = a.part + uint64_t(blockIdx.x) * a.n_params;
-  if (t < 8) gbase[P.bh + t] = (s_bh[0][t] + s_bh[1][t] + s_bh[2][t] + s_bh[3][t]) * inv_sc;
-  // ---- backward: step k = L .. 1; dz_k in Z, the next dz into the other buffer ----
-  unsigned char* Z = P2;
-  unsigned char* Zn = P1;
-  for (int k = L; ok && k >= 1; --k) {
-    const bool first = (k == L);
-    // dW_k's B operand: h_{k-1} (U for k = 1); it has k1 columns at k = 1
-    const uint32_t hprev = k == 1 ? tc::smem_u32(U) : tc::smem_u32(Hb + uint32_t(k - 2) * TILE);
-    const uint32_t ncols = k == 1 ? k1 : uint32_t(W);
-    if (t == 0) {
-      tc::fence_after_sync();
-      const uint32_t z = tc::smem_u32(Z);
-      if (first)  // dW_h^T[k][o] = sum_r h_L[r][k] dout[r][o]
-        for (uint32_t ks = 0; ks < MT / 16; ++ks)
-          tc::mma_f16(tm + C_DWH, mn_desc(tc::smem_u32(P1), W, ks), mn_desc(tc::smem_u32(DO), 16, ks),
-                      idesc_f16_mn(MT, 16, true, true), ks > 0 ? 1u : 0u);
-      if (k >= 2)  // dh_{k-1} = dz_k W_k
-        for (uint32_t ks = 0; ks < W / 16; ++ks)
-          tc::mma_f16(tm + C_ACC, tc::sdesc(z + ks * 256u, 128u, W * 16u),
-                      mn_desc(img_a + o_wk + uint32_t(k - 2) * W * W * 2u, W, ks),
-                      idesc_f16_mn(MT, W, false, true), ks > 0 ? 1u : 0u);
-      if (ncols > 0)  // dW_k = dz_k^T h_{k-1}
-        for (uint32_t ks = 0; ks < MT / 16; ++ks)
-          tc::mma_f16(tm + (k == 1 ? C_DW1 : C_DW), mn_desc(z, W, ks), mn_desc(hprev, ncols, ks),
-                      idesc_f16_mn(MT, int(ncols), true, true), ks > 0 ? 1u : 0u);
-      for (uint32_t ks = 0; ks < MT / 16; ++ks)  // db_k = dz_k^T 1 (column 8)
-        tc::mma_f16(tm + C_DB, mn_desc(z, W, ks), mn_desc(tc::smem_u32(DO), 16, ks), idesc_f16_mn(MT, 16, true, true),
-                    ks > 0 ? 1u : 0u);
-      tc::mma_commit(bar_m);
-    }
-    ok = mma_wait();
-    if (!ok) break;
-    // dz_{k-1} = dh_{k-1} (1 - h_{k-1}^2), h_{k-1} from its tile
-    if (k >= 2) {
-      const unsigned char* hp = Hb + uint32_t(k - 2) * TILE;
-      for (int c0 = 0; c0 < W; c0 += 32) {
-        float v[32];
-        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(c0), v);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 h4 = *reinterpret_cast<const uint4*>(hp + tc::canon_off(t, c0 + 8 * q, W));
-          const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w};
-          uint32_t zu[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 h2 = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
-            zu[e] = tc::pack_f16x2(v[8 * q + 2 * e] * (1.f - h2.x * h2.x), v[8 * q + 2 * e + 1] * (1.f - h2.y * h2.y));
-          }
-          *reinterpret_cast<uint4*>(Zn + tc::canon_off(t, c0 + 8 * q, W)) = make_uint4(zu[0], zu[1], zu[2], zu[3]);
-        }
-      }
-    }
-    // dW_k (lane t = output unit t), unscaled, to the tile's partial gradient:
-    // 32 columns at a time through shared memory (dz_k's tile, free now), so
-    // that each warp store covers 32 consecutive columns of one row
-    if (ncols > 0) {
+    sc = ldexpf(1.f, e2);
+    inv_sc = ldexpf(1.f, -e2);
+  };
+  if (a.maxes) set_scale(threadIdx.x < kMaxes ? __ldcg(a.maxes + threadIdx.x) : 0.f);
+
+  // The sums of the last tiles to the slab (the first flush of a CTA writes
+  // it, later ones add): 32 columns at a time through shared memory, so that
+  // each warp's access covers 32 consecutive columns of one row.  The halves
+  // take alternate chunks.
+  uint32_t flushes = 0;
+  auto put = [&](float* d, float v) { *d = flushes ? *d + v * inv_sc : v * inv_sc; };
+  auto flush = [&]() {
+    float* stage = reinterpret_cast<float*>(h ? P2 : P1);  // [128][33]
+    for (int k = 1; k <= L; ++k) {
+      const uint32_t ncols = k == 1 ? k1 : uint32_t(W), col = k == 1 ? C_DW1 : uint32_t(k - 1) * W;
       float* gw = gbase + (k == 1 ? P.W1 : P.Wk + uint64_t(k - 2) * (uint64_t(W) * W + W));
-      const uint32_t ld = k == 1 ? 4u * p : uint32_t(W), nvalid = ld;
-      float* stage = reinterpret_cast<float*>(Z);  // [128][33]
-      for (uint32_t c0 = 0; c0 < ncols; c0 += 32) {
+      const uint32_t ld = k == 1 ? 4u * p : uint32_t(W);
+      for (uint32_t c0 = 32u * h; c0 < ncols; c0 += 64) {
         float v[32];
         if (c0 + 32 <= ncols) {
-          tc::tmem_ld32(tm + lb + (k == 1 ? C_DW1 : C_DW) + c0, v);
+          tc::tmem_ld32(tm + lb + col + c0, v);
         } else {
           float v16[16];
-          tc::tmem_ld16(tm + lb + (k == 1 ? C_DW1 : C_DW) + c0, v16);
+          tc::tmem_ld16(tm + lb + col + c0, v16);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             v[i] = v16[i];
@@ -1276,36 +1111,278 @@ __global__ void __launch_bounds__(MT, 1) mlp_tc_grad_kernel(const __grid_constan
         }
 #pragma unroll
         for (int i = 0; i < 32; ++i) stage[t * 33 + i] = v[i];
-        __syncthreads();
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + h) : "memory");
         const uint32_t c = c0 + uint32_t(lane);
-        if (c < nvalid)
-          for (int r = warp; r < MT; r += 4) gw[uint64_t(r) * ld + c] = stage[r * 33 + lane] * inv_sc;
-        __syncthreads();
+        if (c < ld)
+          for (int r = warp; r < MT; r += 4) put(gw + uint64_t(r) * ld + c, stage[r * 33 + lane]);
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + h) : "memory");
+      }
+      if (h == 0) {  // d b_k[t]
+        float v[8];
+        tc::tmem_ld8(tm + lb + C_DB + 16u * uint32_t(k - 1) + 8u, v);
+        put(gbase + (k == 1 ? P.b1 : P.Wk + uint64_t(k - 2) * (uint64_t(W) * W + W) + uint64_t(W) * W) + t, v[0]);
       }
     }
-    if (first) {  // dW_h[o][t]
+    if (h == 1) {  // dW_h[o][t]
       float v[8];
       tc::tmem_ld8(tm + lb + C_DWH, v);
 #pragma unroll
-      for (int o = 0; o < 8; ++o) gbase[P.Wh + uint64_t(o) * W + t] = v[o] * inv_sc;
+      for (int o = 0; o < 8; ++o) put(gbase + P.Wh + uint64_t(o) * W + t, v[o]);
+    } else {  // d b_h: sums of dout over the rows (f32, warp shuffles)
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        float sum = bh[o];
+        for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        if (lane == 0) s_bh[warp][o] = sum;
+        bh[o] = 0.f;
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (t < 8) put(gbase + P.bh + t, s_bh[0][t] + s_bh[1][t] + s_bh[2][t] + s_bh[3][t]);
     }
-    {  // d b_k[t]
-      float v[8];
-      tc::tmem_ld8(tm + lb + C_DB + 8u, v);
-      gbase[(k == 1 ? P.b1 : P.Wk + uint64_t(k - 2) * (uint64_t(W) * W + W) + uint64_t(W) * W) + t] = v[0] * inv_sc;
-    }
-    tc::fence_async_smem();
+    ++flushes;
     tc::fence_before_sync();
     __syncthreads();
-    unsigned char* tmp = Z;
-    Z = Zn;
-    Zn = tmp;
+    tc::fence_after_sync();
+  };
+
+  uint32_t in_tmem = 0;  // tiles summed in tensor memory
+  for (uint32_t tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
+    const uint64_t row = uint64_t(tile) * MT + t;
+    const bool valid = row < n_x;
+    const uint64_t x = valid ? a.xs[row] : 0ull;
+    float cla = 0.f, cph = 0.f;
+    if (valid) cot_of(a.cot, row, cla, cph);
+    if (!a.maxes) set_scale(fmaxf(fabsf(cla), fabsf(cph)));
+    const uint32_t acc = in_tmem ? 1u : 0u;
+    // one-hot input of v_<p (layer 1's A operand and dW_1's B operand)
+    for (uint32_t k = 8u * h; k < k1; k += 16) {
+      uint32_t w4[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t lo = 0, hi = 0;
+        const uint32_t k0 = k + 2 * e, kk = k0 + 1;
+        if (k0 < 4u * p && ((x >> (2 * (k0 >> 2))) & 3ull) == (k0 & 3u)) lo = 0x3C00u;
+        if (kk < 4u * p && ((x >> (2 * (kk >> 2))) & 3ull) == (kk & 3u)) hi = 0x3C00u;
+        w4[e] = lo | (hi << 16);
+      }
+      *reinterpret_cast<uint4*>(U + tc::canon_off(t, k, k1)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    }
+    sync_tiles();
+    // ---- forward: h_1 .. h_{L-1} to their tiles, z_L left in TMEM ----
+    for (int layer = 0; ok && layer < L; ++layer) {
+      const uint32_t K = layer == 0 ? k1 : uint32_t(W);
+      if (K > 0) {
+        if (threadIdx.x == 0) {
+          tc::fence_after_sync();
+          const uint32_t a_addr = layer == 0 ? tc::smem_u32(U) : tc::smem_u32(Hb + uint32_t(layer - 1) * TILE);
+          const uint32_t b_addr = img_a + (layer == 0 ? 0u : o_wk + uint32_t(layer - 1) * W * W * 2u);
+          for (uint32_t ks = 0; ks < K / 16; ++ks)
+            tc::mma_f16(tm + C_ACC, tc::sdesc(a_addr + ks * 256u, 128u, K * 16u),
+                        tc::sdesc(b_addr + ks * 256u, 128u, K * 16u), tc::idesc_f16_f32(MT, W), ks > 0 ? 1u : 0u);
+          tc::mma_commit(bar_m);
+        }
+        ok = mma_wait();
+      }
+      if (!ok || layer == L - 1) break;
+      unsigned char* dst = Hb + uint32_t(layer) * TILE;
+#pragma unroll
+      for (int c0 = 0; c0 < HW; c0 += 32) {
+        float v[32];
+        if (K > 0) {
+          tc::tmem_ld32(tm + lb + C_ACC + uint32_t(cb + c0), v);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = 0.f;
+        }
+        const float* b = bias + layer * W + cb + c0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t u4[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int i = 8 * q + 2 * e;
+            u4[e] = tc::pack_f16x2(tc::tanh_fast(v[i] + b[i]), tc::tanh_fast(v[i + 1] + b[i + 1]));
+          }
+          *reinterpret_cast<uint4*>(dst + tc::canon_off(t, cb + c0 + 8 * q, W)) = make_uint4(u4[0], u4[1], u4[2], u4[3]);
+        }
+      }
+      sync_tiles();
+    }
+    if (!ok) break;
+    // ---- head (f32; each half its columns' part of the sums) and the adjoint of its 8 outputs ----
+    float hl[HW], out[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) out[o] = 0.f;
+#pragma unroll
+    for (int c0 = 0; c0 < HW; c0 += 32) {
+      float v[32];
+      if (kL) {
+        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(cb + c0), v);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int c = cb + c0 + i;
+        const float y = tc::tanh_fast(v[i] + bias[(L - 1) * W + c]);
+        const float4 w0 = head[c * 2], w1 = head[c * 2 + 1];
+        out[0] = fmaf(w0.x, y, out[0]);
+        out[1] = fmaf(w0.y, y, out[1]);
+        out[2] = fmaf(w0.z, y, out[2]);
+        out[3] = fmaf(w0.w, y, out[3]);
+        out[4] = fmaf(w1.x, y, out[4]);
+        out[5] = fmaf(w1.y, y, out[5]);
+        out[6] = fmaf(w1.z, y, out[6]);
+        out[7] = fmaf(w1.w, y, out[7]);
+        hl[c0 + i] = y;
+      }
+    }
+    {
+      float4* xo = reinterpret_cast<float4*>(P1) + (h * MT + t) * 2;
+      xo[0] = make_float4(out[0], out[1], out[2], out[3]);
+      xo[1] = make_float4(out[4], out[5], out[6], out[7]);
+      __syncthreads();
+      const float4* xi = reinterpret_cast<const float4*>(P1) + ((1 - h) * MT + t) * 2;
+      const float4 q0 = xi[0], q1 = xi[1];
+      const float other[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+      for (int o = 0; o < 8; ++o) out[o] = out[o] + other[o] + hbias[o];
+      __syncthreads();  // P1 takes h_L next
+    }
+    float dout[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    // d l_u = cot_la 1/2 (delta_uv - p~_u) over the allowed u; d phi_u = cot_ph delta_uv
+    if (valid) {
+      const unsigned pm = slot_mask(a.hv, p, popc_alpha_tc(x, p), popc_beta_tc(x, p), x), mk = norm_mask(a.hv, p, pm);
+      const unsigned v = unsigned((x >> (2 * p)) & 3ull);
+      if ((pm >> v) & 1u) {
+        float m = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if ((mk >> u) & 1u) m = fmaxf(m, out[u]);
+        float ex[4], sum = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          ex[u] = ((mk >> u) & 1u) ? __expf(out[u] - m) : 0.f;
+          sum += ex[u];
+        }
+        const float c = 0.5f * cla * sc;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          dout[u] = ((mk >> u) & 1u) ? c * ((unsigned(u) == v ? 1.f : 0.f) - ex[u] / sum) : 0.f;
+          dout[4 + u] = unsigned(u) == v ? cph * sc : 0.f;
+        }
+      }
+    }
+    if (h == 0) {
+      // dout tile (fp16, 16 columns: dout, then a one in column 8): B operand of
+      // dW_h and of the bias sums
+      uint32_t d4[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) d4[e] = tc::pack_f16x2(dout[2 * e], dout[2 * e + 1]);
+      *reinterpret_cast<uint4*>(DO + tc::canon_off(t, 0, 16)) = make_uint4(d4[0], d4[1], d4[2], d4[3]);
+      *reinterpret_cast<uint4*>(DO + tc::canon_off(t, 8, 16)) = make_uint4(0x3C00u, 0u, 0u, 0u);
+#pragma unroll
+      for (int o = 0; o < 8; ++o) bh[o] += dout[o];
+    }
+    // h_L (fp16) to P1, dz_L = (W_h^T dout) (1 - h_L^2) to P2
+#pragma unroll
+    for (int q = 0; q < HW / 8; ++q) {
+      uint32_t hu[4], zu[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float zz[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int k = cb + 8 * q + 2 * e + j;
+          const float y = hl[8 * q + 2 * e + j];
+          const float4 w0 = head[k * 2], w1 = head[k * 2 + 1];
+          float dh = w0.x * dout[0];
+          dh = fmaf(w0.y, dout[1], dh);
+          dh = fmaf(w0.z, dout[2], dh);
+          dh = fmaf(w0.w, dout[3], dh);
+          dh = fmaf(w1.x, dout[4], dh);
+          dh = fmaf(w1.y, dout[5], dh);
+          dh = fmaf(w1.z, dout[6], dh);
+          dh = fmaf(w1.w, dout[7], dh);
+          zz[j] = dh * (1.f - y * y);
+        }
+        hu[e] = tc::pack_f16x2(hl[8 * q + 2 * e], hl[8 * q + 2 * e + 1]);
+        zu[e] = tc::pack_f16x2(zz[0], zz[1]);
+      }
+      *reinterpret_cast<uint4*>(P1 + tc::canon_off(t, cb + 8 * q, W)) = make_uint4(hu[0], hu[1], hu[2], hu[3]);
+      *reinterpret_cast<uint4*>(P2 + tc::canon_off(t, cb + 8 * q, W)) = make_uint4(zu[0], zu[1], zu[2], zu[3]);
+    }
+    sync_tiles();
+    // ---- backward: step k = L .. 1; dz_k in Z, the next dz into the other
+    // buffer.  dh_{k-1} is committed by itself: the weight GEMMs of step k run
+    // while the next dz is formed, and are done before step k - 1's dh is (MMAs
+    // complete in order), so before anything overwrites their operands ----
+    unsigned char* Z = P2;
+    unsigned char* Zn = P1;
+    for (int k = L; ok && k >= 1; --k) {
+      const uint32_t hprev = k == 1 ? tc::smem_u32(U) : tc::smem_u32(Hb + uint32_t(k - 2) * TILE);
+      const uint32_t ncols = k == 1 ? k1 : uint32_t(W);
+      if (threadIdx.x == 0) {
+        tc::fence_after_sync();
+        const uint32_t z = tc::smem_u32(Z);
+        if (k == L)  // dW_h^T[k][o] = sum_r h_L[r][k] dout[r][o]; the next dz overwrites h_L
+          for (uint32_t ks = 0; ks < MT / 16; ++ks)
+            tc::mma_f16(tm + C_DWH, mn_desc(tc::smem_u32(P1), W, ks), mn_desc(tc::smem_u32(DO), 16, ks),
+                        idesc_f16_mn(MT, 16, true, true), ks > 0 ? 1u : acc);
+        if (k >= 2) {  // dh_{k-1} = dz_k W_k
+          for (uint32_t ks = 0; ks < W / 16; ++ks)
+            tc::mma_f16(tm + C_ACC, tc::sdesc(z + ks * 256u, 128u, W * 16u),
+                        mn_desc(img_a + o_wk + uint32_t(k - 2) * W * W * 2u, W, ks),
+                        idesc_f16_mn(MT, W, false, true), ks > 0 ? 1u : 0u);
+          tc::mma_commit(bar_m);
+        }
+        if (ncols > 0)  // dW_k = dz_k^T h_{k-1}
+          for (uint32_t ks = 0; ks < MT / 16; ++ks)
+            tc::mma_f16(tm + (k == 1 ? C_DW1 : uint32_t(k - 1) * W), mn_desc(z, W, ks), mn_desc(hprev, ncols, ks),
+                        idesc_f16_mn(MT, int(ncols), true, true), ks > 0 ? 1u : acc);
+        for (uint32_t ks = 0; ks < MT / 16; ++ks)  // db_k = dz_k^T 1 (column 8)
+          tc::mma_f16(tm + C_DB + 16u * uint32_t(k - 1), mn_desc(z, W, ks), mn_desc(tc::smem_u32(DO), 16, ks),
+                      idesc_f16_mn(MT, 16, true, true), ks > 0 ? 1u : acc);
+        if (k == 1) tc::mma_commit(bar_m);
+      }
+      ok = mma_wait();
+      if (!ok || k == 1) break;
+      // dz_{k-1} = dh_{k-1} (1 - h_{k-1}^2), h_{k-1} from its tile
+      const unsigned char* hp = Hb + uint32_t(k - 2) * TILE;
+#pragma unroll
+      for (int c0 = 0; c0 < HW; c0 += 32) {
+        float v[32];
+        tc::tmem_ld32(tm + lb + C_ACC + uint32_t(cb + c0), v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 h4 = *reinterpret_cast<const uint4*>(hp + tc::canon_off(t, cb + c0 + 8 * q, W));
+          const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w};
+          uint32_t zu[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 h2 = __half22float2(*reinterpret_cast<const __half2*>(&hw[e]));
+            zu[e] = tc::pack_f16x2(v[8 * q + 2 * e] * (1.f - h2.x * h2.x), v[8 * q + 2 * e + 1] * (1.f - h2.y * h2.y));
+          }
+          *reinterpret_cast<uint4*>(Zn + tc::canon_off(t, cb + c0 + 8 * q, W)) = make_uint4(zu[0], zu[1], zu[2], zu[3]);
+        }
+      }
+      sync_tiles();
+      unsigned char* tmp = Z;
+      Z = Zn;
+      Zn = tmp;
+    }
+    if (!ok) break;
+    if (++in_tmem == kFlush || tile + gridDim.x >= tiles) {
+      flush();
+      in_tmem = 0;
+    }
   }
-  if (!ok && t == 0) atomicExch(a.tv.status, ST_TIMEOUT);
+  if (!ok && threadIdx.x == 0) atomicExch(a.tv.status, ST_TIMEOUT);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tm, NCOL);
+  if (threadIdx.x < 32) tc::tmem_dealloc(tm, NCOL);
 }
 
 // One CTA of AT threads per parent x (grid-stride over the parents), its
@@ -1964,15 +2041,16 @@ static size_t tc_grad_smem(const anqs_model* M, uint32_t* img_bytes, uint32_t* k
   if (kmax1) *kmax1 = k1;
   const size_t tile = size_t(MT) * W * 2;
   const size_t sm = size_t(img) + size_t(L - 1) * tile + 2 * tile + size_t(MT) * k1 * 2 + size_t(MT) * 16 * 2;
-  return sm <= kSmemLimit ? sm : 0;
+  return sm <= kSmemLimit && k1 <= 64 ? sm : 0;  // (dW_1 has 64 tensor-memory columns)
 }
 
 bool mlp_tc_grad_supported(const anqs_model* M) { return tc_grad_smem(M, nullptr, nullptr) > 0; }
 
-// The VMC gradient of a 16-bit MLP on the tensor cores: per-tile partial
-// gradients in `part` ([tiles][n_params], tiles of 128 rows), then their sum.
+// The VMC gradient of a 16-bit MLP on the tensor cores: a slab of partial
+// gradients per CTA of a slot in `part` ([slabs][n_params]), then their sum.
+// cl, cp: n_x floats each, for the cotangents when a CTA has several tiles.
 int launch_mlp_tc_grad(const anqs_model* M, const HamView& hv, const uint64_t* x, Count n_x, const CotSrc& cot,
-                       float* grad, float* part, cudaStream_t s) {
+                       float* cl, float* cp, float* grad, float* part, cudaStream_t s) {
   GradArgs a{};
   const size_t sm = tc_grad_smem(M, &a.img_bytes, &a.kmax1);
   if (!sm) return set_error(ANQS_ERR_UNSUPPORTED, "tensor-core adjoint does not apply to this model");
@@ -1987,13 +2065,22 @@ int launch_mlp_tc_grad(const anqs_model* M, const HamView& hv, const uint64_t* x
   a.n_params = M->mlp.slot_off[M->mlp.n];
   const uint64_t tiles = std::max<uint64_t>((n_x.n + MT - 1) / MT, 1);
   if (tiles > 0x7fffffffull) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows");
+  // one CTA per SM over all slots
+  const unsigned slabs = unsigned(std::min<uint64_t>(tiles, std::max<uint64_t>(1, uint64_t(num_sms()) / uint64_t(M->d.n_orb))));
+  if (tiles > slabs) {  // several tiles per CTA: one scale for all; `part` holds at least one slab per tile
+    float* maxes = part + uint64_t(slabs) * a.n_params;
+    ProfScope ps(PROF_COTANGENT, s);
+    ANQS_CUDA_LAUNCH("cot_max_kernel", launch_k(cot_max_kernel, dim3(kMaxes), dim3(256), 0, s, cot, n_x, cl, cp, maxes));
+    a.maxes = maxes;
+    if (cot.stats) a.cot = CotSrc{cl, cp, nullptr, nullptr, nullptr, nullptr};
+  }
   ANQS_CUDA(cudaFuncSetAttribute(mlp_tc_grad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
   {
     ProfScope ps(PROF_MLP_TC_GRAD, s);
-    ANQS_CUDA_LAUNCH("mlp_tc_grad_kernel", launch_k(mlp_tc_grad_kernel<128>, dim3(unsigned(tiles), unsigned(M->d.n_orb)),
-                                                    dim3(MT), sm, s, a));
+    ANQS_CUDA_LAUNCH("mlp_tc_grad_kernel", launch_k(mlp_tc_grad_kernel<128>, dim3(slabs, unsigned(M->d.n_orb)),
+                                                    dim3(GNT), sm, s, a));
   }
-  return launch_grad_partial_sum(part, n_x, a.n_params, MT, grad, s);
+  return launch_grad_partial_sum(part, n_x, a.n_params, MT, slabs, grad, s);
 }
 
 int mlp_tc_multi_max() { return kMaxBatch; }
