@@ -511,8 +511,8 @@ int anqs_hamiltonian_create(anqs_ham** out, int n, int na, int nb, const double*
   }
 
   size_t hn = size_t(n) * n, gn = hn * hn;
-  if (cudaMalloc(&H->d_h, hn * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&H->d_g, gn * sizeof(double)) != cudaSuccess ||
+  if (cudaMalloc(&H->d_h, 3 * hn * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&H->d_g, 2 * gn * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&H->d_mask, H->mask_host.size()) != cudaSuccess ||
       cudaMalloc(&H->d_status, sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
@@ -526,6 +526,13 @@ int anqs_hamiltonian_create(anqs_ham** out, int n, int na, int nb, const double*
   v.status = H->d_status;
   v.h = H->d_h;
   v.g = H->d_g;
+  v.ga = H->d_g + gn;
+  v.pair = H->d_h + hn;
+  if (launch_integral_tables(n, H->d_g, H->d_g + gn, H->d_h + hn, cudaStreamLegacy) != ANQS_OK ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    anqs_hamiltonian_destroy(H);
+    return set_error(ANQS_ERR_CUDA, "integral tables could not be built");
+  }
   v.mask = H->d_mask;
   v.mu_lv = n;
   if (build_prefix_table(H) != ANQS_OK || build_index(H) != ANQS_OK) {

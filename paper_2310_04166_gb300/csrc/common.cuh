@@ -222,6 +222,8 @@ struct HamView {
   double e_nuc;
   const double* h;     // [n][n]
   const double* g;     // [n][n][n][n] chemist notation
+  const double* ga;    // [n][n][n][n]: [pq|rs] - [ps|rq]
+  const double* pair;  // [2][n][n]: J_ij - K_ij of one spin, J_ij of two (each averaged over ij and ji)
   const uint8_t* mask; // [n][na+1][nb+1] allowed-outcome bits per slot and prefix counts
   int mu_lv;           // slots p < mu_lv are masked (MU), slots p >= mu_lv discard (DU): MU-d, d = n - mu_lv
   int nz;              // Z2 symmetries (Pauli-Z strings commuting with H), 0..ANQS_MAX_Z2
@@ -450,6 +452,7 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 
 // connect.cu
 // ctl (optional): a tensor-core local energy's control words, set to zero
+int launch_integral_tables(int n, const double* g, double* ga, double* pair, cudaStream_t s);
 int launch_connected(const HamView& hv, const uint64_t* x, Count n_x, uint64_t* xp, double* hval,
                      uint8_t* first_slot, double* hdiag, cudaStream_t s, uint32_t* ctl = nullptr);
 

@@ -65,7 +65,7 @@ __device__ __forceinline__ void connected_body(const HamView& hv, const uint64_t
       const uint32_t e = s ? k - hv.nsa : k;
       const int i = E.si[s][e], a = E.sa[s][e];
       const double v = single_value(hv, E, s, i, a);
-      put(k, x ^ (1ull << (2 * i + s)) ^ (1ull << (2 * a + s)), E.sgn[s][e] ? -v : v, min(i, a));
+      put(k, x ^ (1ull << (2 * i + s)) ^ (1ull << (2 * a + s)), flip_sign(v, E.sgn[s][e]), min(i, a));
     }
     // same-spin doubles I<J -> A<B: [AI|BJ] - [AJ|BI]
     for (uint32_t k = max(k0, ks) + threadIdx.x; k < min(k1, kd); k += blockDim.x) {
@@ -75,9 +75,9 @@ __device__ __forceinline__ void connected_body(const HamView& hv, const uint64_t
       const FastDiv d = s ? dp[1] : dp[0];
       const uint32_t q = fdiv(d, r), po = E.po[s][q], pv = E.pv[s][r - q * d.d];
       const int i = E.occ[s][po & 255u], j = E.occ[s][po >> 8], a = E.vir[s][pv & 255u], b = E.vir[s][pv >> 8];
-      const double v = Gint(hv, a, i, b, j) - Gint(hv, a, j, b, i);
+      const double v = __ldg(hv.ga + ((a * n + i) * n + b) * n + j);
       put(k, x ^ (1ull << (2 * i + s)) ^ (1ull << (2 * j + s)) ^ (1ull << (2 * a + s)) ^ (1ull << (2 * b + s)),
-          sign_ss(E, s, po, pv, s ? nvirt[1] : nvirt[0], i, j, a, b) ? -v : v, min(min(i, j), min(a, b)));
+          flip_sign(v, sign_ss(E, s, po, pv, s ? nvirt[1] : nvirt[0], i, j, a, b)), min(min(i, j), min(a, b)));
     }
     // opposite-spin doubles (I_a, A_a, I_b, A_b): [AI|BJ] (exchange term vanishes by spin)
     for (uint32_t k = max(k0, kd) + threadIdx.x; k < k1; k += blockDim.x) {
@@ -85,7 +85,7 @@ __device__ __forceinline__ void connected_body(const HamView& hv, const uint64_t
       const int i = E.si[0][ea], a = E.sa[0][ea], j = E.si[1][eb], b = E.sa[1][eb];
       const double v = __ldg(hv.g + E.g[0][ea] + E.g[1][eb]);
       put(k, x ^ (1ull << (2 * i)) ^ (1ull << (2 * a)) ^ (2ull << (2 * j)) ^ (2ull << (2 * b)),
-          sign_ab(E, ea, eb, i, a, j, b) ? -v : v, min(min(i, a), min(j, b)));
+          flip_sign(v, sign_ab(E, ea, eb, i, a, j, b)), min(min(i, a), min(j, b)));
     }
   }
 }
@@ -152,6 +152,23 @@ __global__ void diagonal_kernel(HamView hv, const uint64_t* __restrict__ xs, Cou
   diagonal_body(hv, xs, n_x, hdiag, blockIdx.x, gridDim.x);
 }
 
+// [pq|rs] - [ps|rq] for the same-spin doubles and the pair energies of the
+// diagonal, once per Hamiltonian
+__global__ void integral_tables_kernel(int n, const double* __restrict__ g, double* __restrict__ ga,
+                                       double* __restrict__ pair) {
+  const uint32_t n1 = uint32_t(n), n2 = n1 * n1, all = n2 * n2;
+  auto G = [&](uint32_t p, uint32_t q, uint32_t r, uint32_t s) { return g[(p * n1 + q) * n2 + r * n1 + s]; };
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < all; t += gridDim.x * blockDim.x) {
+    const uint32_t p = t / (n2 * n1), q = t / n2 % n1, r = t / n1 % n1, s = t % n1;
+    ga[t] = g[t] - G(p, s, r, q);
+    if (t < n2) {
+      const double J = 0.5 * G(r, r, s, s) + 0.5 * G(s, s, r, r);
+      pair[t] = J - (0.5 * G(r, s, s, r) + 0.5 * G(s, r, r, s));
+      pair[n2 + t] = J;
+    }
+  }
+}
+
 // the connected set on blocks [0, nb_c) and the diagonal on the rest, in one
 // launch
 __global__ void connected_diag_kernel(HamView hv, const uint64_t* __restrict__ xs, Count n_x,
@@ -165,6 +182,13 @@ __global__ void connected_diag_kernel(HamView hv, const uint64_t* __restrict__ x
 }
 
 }  // namespace
+
+int launch_integral_tables(int n, const double* g, double* ga, double* pair, cudaStream_t s) {
+  const unsigned all = unsigned(n) * unsigned(n) * unsigned(n) * unsigned(n);
+  const unsigned grid = std::min(152u * 8u, (all + 255u) / 256u);
+  ANQS_CUDA_LAUNCH("integral_tables_kernel", launch_k(integral_tables_kernel, dim3(grid), dim3(256), 0, s, n, g, ga, pair));
+  return ANQS_OK;
+}
 
 int launch_connected(const HamView& hv, const uint64_t* x, Count n_x, uint64_t* xp, double* hval,
                      uint8_t* first_slot, double* hdiag, cudaStream_t s, uint32_t* ctl) {

@@ -18,6 +18,8 @@
 //           looked up; nothing of the connected set is written to memory.
 //           Statistics in the last CTA.
 // Sectors of few prefixes skip mark, count and emit: every prefix is a node.
+// Where the connected determinants outnumber a larger sector's, all bits are
+// set without looking at them (covers_sector).
 //
 // All float32 sums run in the order of an evaluation of each connected
 // determinant by itself, so the amplitudes have its bits.
@@ -58,6 +60,16 @@ __device__ __forceinline__ void mark_det(const HamView& hv, const SectorView& sv
   }
 }
 
+// Whether a call's connected determinants outnumber the sector's so far that
+// all its prefixes are taken as marked: hardly any is left out then, and one
+// word is written per 32 determinants instead of an atomic or a load per
+// connected one (1.1e7 of a 14,400-determinant sector: 126 us).  From the
+// device's count: a buffer may hold fewer samples than it has room for.
+// Not with Z2 symmetries, where the index also holds other sectors' prefixes.
+__device__ __forceinline__ bool covers_sector(const HamView& hv, const SectorView& sv, uint64_t n_x) {
+  return hv.nz == 0 && n_x * uint64_t(hv.K) >= 4ull * sv.na_p[sv.n] * sv.nb_p[sv.n];
+}
+
 constexpr int MT_ = 128;
 
 __global__ void __launch_bounds__(MT_) mark_kernel(HamView hv, SectorView sv, const uint64_t* __restrict__ xs,
@@ -66,6 +78,14 @@ __global__ void __launch_bounds__(MT_) mark_kernel(HamView hv, SectorView sv, co
   __shared__ Exc E;
   const uint64_t items = n_x_.get() * uint64_t(splits);
   const uint32_t K = hv.K;
+  if (covers_sector(hv, sv, n_x_.get())) {
+    for (int p = levels ? 0 : sv.n; p <= sv.n; ++p) {
+      const uint32_t all = sv.na_p[p] * sv.nb_p[p], words = (all + 31u) / 32u;
+      for (uint32_t w = blockIdx.x * MT_ + threadIdx.x; w < words; w += gridDim.x * MT_)
+        bits[sv.woff[p] + w] = w + 1 < words || !(all & 31u) ? ~0u : (1u << (all & 31u)) - 1u;
+    }
+    return;
+  }
   build_pairs(hv, E);
   const uint32_t nvb = hv.n - hv.nb, nsb = hv.nb * nvb;
   const FastDiv dsb = fast_div(nsb);
@@ -136,12 +156,18 @@ __global__ void mark_samples_kernel(HamView hv, SectorView sv, const uint64_t* _
   }
 }
 
-constexpr int CT = 256;      // threads of the count and emit kernels
-constexpr uint32_t CW = 4096;  // bitmap words per CTA
+constexpr int CT = 256;  // threads of the count and emit kernels
 
-// nodes of each CTA's words, and the total of the determinants' level (words from leaf_w on)
-__global__ void __launch_bounds__(CT) count_kernel(const uint32_t* __restrict__ bits, uint32_t words, uint32_t leaf_w,
-                                                   uint32_t* __restrict__ bsum,
+// Bitmap words per CTA: one per thread, so that the 450 words of a 20-qubit
+// sector occupy two SMs for a microsecond (with 4,096 words per CTA one CTA
+// expanded them all, 27 us), and more where the CTAs, each of which sums the
+// counts of all CTAs before it, would number above 4,096.
+constexpr uint32_t CW_MAX = 4096;
+uint32_t words_per_cta(uint32_t words) { return std::min(CW_MAX, std::max<uint32_t>(1, (words + 4096 * CT - 1) / (4096 * CT)) * CT); }
+
+// nodes of each CTA's CW words, and the total of the determinants' level (words from leaf_w on)
+__global__ void __launch_bounds__(CT) count_kernel(const uint32_t* __restrict__ bits, uint32_t words, uint32_t CW,
+                                                   uint32_t leaf_w, uint32_t* __restrict__ bsum,
                                                    unsigned long long* __restrict__ n_leaves) {
   ANQS_PDL_ENTRY();
   __shared__ uint32_t s_sum, s_leaf;
@@ -171,7 +197,7 @@ __global__ void __launch_bounds__(CT) count_kernel(const uint32_t* __restrict__ 
 
 // words: those of the levels below `levels`; writes off[0 .. levels]
 __global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, int levels, const uint32_t* __restrict__ bits, uint32_t words,
-                                                  const uint32_t* __restrict__ bsum, uint2* __restrict__ packed,
+                                                  uint32_t CW, const uint32_t* __restrict__ bsum, uint2* __restrict__ packed,
                                                   uint64_t* __restrict__ node_x, uint32_t* __restrict__ off) {
   ANQS_PDL_ENTRY();
   __shared__ uint32_t s_base, s_warp[CT / 32];
@@ -205,19 +231,29 @@ __global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, int levels, con
       if (q < wp) before += s_warp[q];
       total += s_warp[q];
     }
-    uint32_t id = base + before + inc - c;
+    const uint32_t id = base + before + inc - c;
+    int p = 0;
+    uint32_t i0 = 0;
     if (w < w_end) {
       packed[w] = make_uint2(v, id);
-      int p = 0;
       while (w >= sv.woff[p + 1]) ++p;
       if (w == sv.woff[p]) off[p] = id;
       if (w + 1 == words) off[levels] = id + c;
-      const uint32_t i0 = (w - sv.woff[p]) * 32u, nb = sv.nb_p[p];
-      while (v) {
-        const uint32_t idx = i0 + uint32_t(__ffs(v)) - 1u;
-        v &= v - 1u;
-        const uint32_t ra = idx / nb, rb = idx - ra * nb;
-        node_x[id++] = spread_bits(__ldg(sv.sta + sv.soa[p] + ra)) | spread_bits(__ldg(sv.stb + sv.sob[p] + rb)) << 1;
+      i0 = (w - sv.woff[p]) * 32u;
+    }
+    // the warp's words one after the other, a lane per bit: the lookups of one
+    // word are in flight together and its nodes are written side by side
+    uint32_t some = __ballot_sync(0xffffffffu, v != 0u);
+    while (some) {
+      const int q = __ffs(some) - 1;
+      some &= some - 1u;
+      const uint32_t vq = __shfl_sync(0xffffffffu, v, q), idq = __shfl_sync(0xffffffffu, id, q),
+                     idx = __shfl_sync(0xffffffffu, i0, q) + uint32_t(lane);
+      const int pq = __shfl_sync(0xffffffffu, p, q);
+      if ((vq >> lane) & 1u) {
+        const uint32_t nb = sv.nb_p[pq], ra = idx / nb, rb = idx - ra * nb;
+        node_x[idq + __popc(vq & ((1u << lane) - 1u))] =
+            spread_bits(__ldg(sv.sta + sv.soa[pq] + ra)) | spread_bits(__ldg(sv.stb + sv.sob[pq] + rb)) << 1;
       }
     }
     base += total;
@@ -345,7 +381,43 @@ __global__ void chunk_counts_kernel(const uint64_t* __restrict__ total, uint64_t
 
 // ---- E_loc ------------------------------------------------------------------------
 constexpr int ET = 128;
+constexpr uint64_t kTailStats = 1024;  // samples up to which eloc_direct_kernel's last CTA reduces the statistics
 
+// a * b with the sign flipped if odd, exactly: the 48-bit product of two float
+// significands fits into a double, and multiplying and packing them as
+// integers keeps three conversions and a multiplication off the FP64 pipe.
+__device__ __forceinline__ double exact_product(float a, float b, int odd) {
+  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+  const uint32_t ea = (ua >> 23) & 255u, eb = (ub >> 23) & 255u;
+  if (ea - 1u < 254u && eb - 1u < 254u) {  // both normal
+    // significands scaled by 2^3 each: the product has bit 52 or 53 set
+    const uint64_t m = uint64_t((ua << 3 & 0x03fffff8u) | 0x04000000u) * ((ub << 3 & 0x03fffff8u) | 0x04000000u);
+    const uint32_t top = uint32_t(m >> 53);
+    const uint64_t r = m >> top;  // bit 52 set; a bit shifted out is zero
+    const uint32_t hi = uint32_t(r >> 32) + ((ea + eb + 768u + top) << 20);
+    return __hiloint2double(int(hi | (((ua ^ ub) & 0x80000000u) ^ (uint32_t(odd) << 31))), int(uint32_t(r)));
+  }
+  return flip_sign(double(a) * double(b), odd);
+}
+
+// h_ai + sum_{J occ} ([AI|JJ] - [AJ|JI]) of the single I -> A of spin s, one
+// table entry per occupied orbital
+__device__ __forceinline__ double single_sum(const HamView& hv, const Exc& E, int s, int i, int a) {
+  const int n = hv.n, row = (a * n + i) * n * n;
+  double v = __ldg(hv.h + a * n + i);
+  for (int t = 0; t < 2; ++t) {
+    const double* src = (t == s ? hv.ga : hv.g) + row;
+    const int ne = t ? hv.nb : hv.na;
+    for (int m = 0; m < ne; ++m) v += __ldg(src + E.occ[t][m] * (n + 1));
+  }
+  return v;
+}
+
+// One CTA per (sample, part).  The FP64 pipe bounds it: it takes two lanes per
+// clock and SM, so a term costs two FP64 operations, the accumulations of its
+// real and imaginary part (7 when the amplitude ratio was converted and
+// multiplied there: the pipe was 80% busy), the diagonal comes from pair
+// energies and one warp adds up the CTA's 128 partial sums.
 template <AmpMode MODE>
 __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView sv, NodeView nv,
                                                          const uint64_t* __restrict__ xs, Count n_x_, int splits,
@@ -354,7 +426,7 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
   ANQS_PDL_ENTRY();
   constexpr bool RANK = MODE != AMP_ARRAY;
   __shared__ Exc E;
-  __shared__ double red[3][ET / 32];
+  __shared__ double red[2][ET];
   __shared__ int s_last;
   const uint64_t n_x = n_x_.get();
   const int n = hv.n, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -372,9 +444,10 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
   const FastDiv dvar = fast_div(var);
   uint32_t leaf0 = 0;
   if constexpr (RANK) leaf0 = __ldcg(nv.off + n);
+  const bool all = !nv.packed || covers_sector(hv, sv, n_x);  // every determinant of the sector has a row
   // row of determinant index idx in the amplitude tables; false if it is not there
   auto leaf = [&](uint32_t idx, uint32_t& r) -> bool {
-    if (!nv.packed) {
+    if (all) {
       r = idx;
       return true;
     }
@@ -409,7 +482,7 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         px = __ldcg(A.ph_x + l);
       }
       // log|psi(x')| and phase of excitation k (determinant index idx, strings a and b, first differing slot j)
-      auto add = [&](uint32_t k, uint32_t idx, uint32_t a, uint32_t b, int j, double h) {
+      auto add = [&](uint32_t k, uint32_t idx, uint32_t a, uint32_t b, int j, double h, int odd) {
         float la, ph;
         if constexpr (MODE == AMP_ARRAY) {
           la = __ldcg(A.la + l * K + k);
@@ -450,9 +523,8 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         const float r = expf(la - lx);
         float s, co;
         sincosf(ph - px, &s, &co);
-        const double hr = h * double(r);
-        re = fma(hr, double(co), re);
-        im = fma(hr, double(s), im);
+        re = fma(h, exact_product(r, co, odd), re);
+        im = fma(h, exact_product(r, s, odd), im);
       };
       const uint32_t k0 = uint32_t(uint64_t(K) * pt / uint32_t(splits)),
                      k1 = uint32_t(uint64_t(K) * (pt + 1) / uint32_t(splits));
@@ -465,8 +537,7 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         const double v = __ldg(hv.g + E.g[0][ea] + E.g[1][eb]);
         uint32_t idx = 0;
         if constexpr (RANK) idx = E.rank[0][ea] + E.rank[1][eb];
-        add(k, idx, E.str[0] ^ (1u << i) ^ (1u << a), E.str[1] ^ (1u << j) ^ (1u << b), min(min(i, a), min(j, b)),
-            sg ? -v : v);
+        add(k, idx, E.str[0] ^ (1u << i) ^ (1u << a), E.str[1] ^ (1u << j) ^ (1u << b), min(min(i, a), min(j, b)), v, sg);
       }
       // same-spin doubles I<J -> A<B: [AI|BJ] - [AJ|BI], as I -> A then J -> B
       for (uint32_t k = max(k0, ks) + threadIdx.x; k < min(k1, kd); k += ET) {
@@ -477,39 +548,41 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
         const uint32_t nv_ = s ? nvb : nva;
         const int i = E.occ[s][po & 255u], j = E.occ[s][po >> 8], a = E.vir[s][pv & 255u], b = E.vir[s][pv >> 8];
         const int sg = sign_ss(E, s, po, pv, nv_, i, j, a, b);
-        const double v = Gint(hv, a, i, b, j) - Gint(hv, a, j, b, i);
+        const double v = __ldg(hv.ga + ((a * n + i) * n + b) * n + j);
         const uint32_t flip = (1u << i) ^ (1u << j) ^ (1u << a) ^ (1u << b);
         const uint32_t sa = E.str[0] ^ (s ? 0u : flip), sb = E.str[1] ^ (s ? flip : 0u);
         uint32_t idx = 0;
         if constexpr (RANK)
           idx = s ? E.own[0] + __ldg(sv.rkb + (1u << n) + sb) : __ldg(sv.rka + (1u << n) + sa) * sv.nb_p[n] + E.own[1];
-        add(k, idx, sa, sb, min(min(i, j), min(a, b)), sg ? -v : v);
+        add(k, idx, sa, sb, min(min(i, j), min(a, b)), v, sg);
       }
       // singles I -> A of spin s: h_ai + sum_{J occ} ([AI|JJ] - [AJ|JI])
       for (uint32_t k = k0 + threadIdx.x; k < min(k1, ks); k += ET) {
         const int s = k < hv.nsa ? 0 : 1;
         const uint32_t e = s ? k - hv.nsa : k;
         const int i = E.si[s][e], a = E.sa[s][e];
-        const double v = single_value(hv, E, s, i, a);
+        const double v = single_sum(hv, E, s, i, a);
         uint32_t idx = 0;
         if constexpr (RANK) idx = s ? E.own[0] + E.rank[1][e] : E.rank[0][e] + E.own[1];
         const uint32_t flip = (1u << i) ^ (1u << a);
-        add(k, idx, E.str[0] ^ (s ? 0u : flip), E.str[1] ^ (s ? flip : 0u), min(i, a), E.sgn[s][e] ? -v : v);
+        add(k, idx, E.str[0] ^ (s ? 0u : flip), E.str[1] ^ (s ? flip : 0u), min(i, a), v, E.sgn[s][e]);
       }
-      if (pt == 0) {  // <x|H|x> = E_nuc + sum_I h_ii + 1/2 sum_{I,J occ} ([II|JJ] - [IJ|JI])
-        const int ne = hv.na + hv.nb;
-        for (int t = threadIdx.x; t < ne * ne + ne; t += ET) {
-          if (t < ne * ne) {
-            const int I = t / ne, J = t - I * ne;
-            const int si = I < hv.na ? 0 : 1, sj = J < hv.na ? 0 : 1;
-            const int i = E.occ[si][si ? I - hv.na : I], j = E.occ[sj][sj ? J - hv.na : J];
-            dg += 0.5 * Gint(hv, i, i, j, j);
-            if (si == sj) dg -= 0.5 * Gint(hv, i, j, j, i);
+      if (pt == 0) {  // <x|H|x> = E_nuc + sum_I h_ii + sum_{I<J occ} ([II|JJ] - [IJ|JI])
+        const int ca = hv.na * (hv.na - 1) / 2, cs = ca + hv.nb * (hv.nb - 1) / 2, cd = cs + hv.na * hv.nb;
+        for (int t = threadIdx.x; t < cd + hv.na + hv.nb; t += ET) {
+          const double* src;
+          if (t < cs) {
+            const int s = t >= ca ? 1 : 0;
+            const uint32_t po = E.po[s][s ? t - ca : t];
+            src = hv.pair + E.occ[s][po & 255u] * n + E.occ[s][po >> 8];
+          } else if (t < cd) {
+            const int q = (t - cs) / hv.nb;
+            src = hv.pair + n * n + E.occ[0][q] * n + E.occ[1][t - cs - q * hv.nb];
           } else {
-            const int I = t - ne * ne;
-            const int i = I < hv.na ? E.occ[0][I] : E.occ[1][I - hv.na];
-            dg += __ldg(hv.h + i * n + i);
+            const int I = t - cd;
+            src = hv.h + (I < hv.na ? E.occ[0][I] : E.occ[1][I - hv.na]) * (n + 1);
           }
+          dg += __ldg(src);
         }
         if (threadIdx.x == 0) dg += hv.e_nuc;
       }
@@ -518,30 +591,25 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
       re = nan;
       im = K ? nan : 0.0;
     }
-    re += dg;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      re += __shfl_xor_sync(0xffffffffu, re, o);
-      im += __shfl_xor_sync(0xffffffffu, im, o);
-    }
-    if (lane == 0) {
-      red[0][wp] = re;
-      red[1][wp] = im;
-    }
+    red[0][threadIdx.x] = re + dg;
+    red[1][threadIdx.x] = im;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double sr = 0.0, si = 0.0;
+    if (wp == 0) {  // lanes 0..15 the real parts, 16..31 the imaginary ones
+      const double* r = red[lane >> 4] + (lane & 15);
+      double v = 0.0;
 #pragma unroll
-      for (int q = 0; q < ET / 32; ++q) {
-        sr += red[0][q];
-        si += red[1][q];
-      }
-      if (splits == 1) {
-        ere[l] = sr;
-        eim[l] = si;
-      } else {
-        part[2 * it] = sr;
-        part[2 * it + 1] = si;
+      for (int q = 0; q < ET; q += 16) v += r[q];
+#pragma unroll
+      for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const double vi = __shfl_sync(0xffffffffu, v, 16);
+      if (lane == 0) {
+        if (splits == 1) {
+          ere[l] = v;
+          eim[l] = vi;
+        } else {
+          part[2 * it] = v;
+          part[2 * it + 1] = vi;
+        }
       }
     }
   }
@@ -567,6 +635,62 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
     __syncthreads();
   }
   if (so.counts) cta_energy_stats<ET>(ere, eim, so.counts, n_x, so.stats);
+}
+
+// Statistics of more than kTailStats samples: a CTA per 512 of them, the last
+// one adds up the partial sums in order.  One CTA alone, bound by its SM's FP64
+// pipe, takes 2 ns per sample.
+constexpr int SB = 152;  // CTAs at most
+__global__ void __launch_bounds__(ET) stats_kernel(const double* ere, const double* eim,
+                                                   const uint64_t* __restrict__ counts, Count n_x_, double* part,
+                                                   uint32_t* ticket, double* stats) {
+  ANQS_PDL_ENTRY();
+  __shared__ double red[4][ET / 32];
+  __shared__ int s_last;
+  const uint64_t n_x = n_x_.get();
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const double kr = n_x ? __ldcg(ere) : 0.0, ki = n_x ? __ldcg(eim) : 0.0;
+  double t[4] = {0.0, 0.0, 0.0, 0.0};  // sums of n, n d, n |d|^2 with d the distance from the first sample's energy
+  for (uint64_t l = blockIdx.x * uint64_t(ET) + threadIdx.x; l < n_x; l += uint64_t(gridDim.x) * ET) {
+    const double c = double(__ldcg(reinterpret_cast<const unsigned long long*>(counts) + l));
+    const double dr = __ldcg(ere + l) - kr, di = __ldcg(eim + l) - ki;
+    t[0] += c;
+    t[1] = fma(c, dr, t[1]);
+    t[2] = fma(c, di, t[2]);
+    t[3] = fma(c, fma(dr, dr, di * di), t[3]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+    if (lane == 0) red[k][wp] = t[k];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < 4; ++k) {
+      double v = 0.0;
+      for (int q = 0; q < ET / 32; ++q) v += red[k][q];
+      part[4 * blockIdx.x + k] = v;
+    }
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last || wp) return;
+  __threadfence();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    t[k] = 0.0;
+    for (uint32_t b = lane; b < gridDim.x; b += 32) t[k] += __ldcg(part + 4 * b + k);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+  }
+  if (lane) return;
+  const double mr = t[1] / t[0], mi = t[2] / t[0];
+  stats[0] = kr + mr;
+  stats[1] = ki + mi;
+  stats[2] = fmax(0.0, t[3] / t[0] - fma(mr, mr, mi * mi));
+  stats[3] = t[0];
 }
 
 // CTAs per sample: a whole sample each when there are enough to fill the GPU
@@ -624,7 +748,7 @@ void plan_unique(const anqs_ham* H, uint64_t n_x, bool levels, Arena& A, UniqueW
   w.part = A.take<double>(eloc_partials(H, n_x));
   w.bits = z ? reinterpret_cast<uint32_t*>(z + 256) : nullptr;
   w.packed = A.take<uint2>(words);
-  w.bsum = A.take<uint32_t>((words + CW - 1) / CW);
+  w.bsum = A.take<uint32_t>((words + words_per_cta(uint32_t(words)) - 1) / words_per_cta(uint32_t(words)));
   w.n_leaves = z ? reinterpret_cast<uint64_t*>(z + 8) : nullptr;
   w.node_x = A.take<uint64_t>(w.max_nodes);
   w.leaf_x = w.node_x;  // without levels, the determinants are the only nodes
@@ -642,10 +766,10 @@ int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueW
     ANQS_CUDA_LAUNCH("mark_kernel", launch_k(mark_kernel, dim3(grid), dim3(MT_), 0, s, H->v, H->sv, x, n_x, splits, w.bits, w.levels ? 1 : 0));
   }
   ProfScope ps(PROF_TC_SORT, s);
-  const uint32_t words = uint32_t(index_words(H));
-  const unsigned blocks = (words + CW - 1) / CW;
-  ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, H->sv.woff[H->v.n], w.bsum, reinterpret_cast<unsigned long long*>(w.n_leaves)));
-  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n + 1, w.bits, words, w.bsum, w.packed, w.node_x, w.off));
+  const uint32_t words = uint32_t(index_words(H)), cw = words_per_cta(words);
+  const unsigned blocks = (words + cw - 1) / cw;
+  ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, cw, H->sv.woff[H->v.n], w.bsum, reinterpret_cast<unsigned long long*>(w.n_leaves)));
+  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n + 1, w.bits, words, cw, w.bsum, w.packed, w.node_x, w.off));
   return ANQS_OK;
 }
 
@@ -690,7 +814,7 @@ void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w) {
   w.n_rows = reinterpret_cast<uint64_t*>(z);
   w.bits = z ? reinterpret_cast<uint32_t*>(z + 256) : nullptr;
   w.packed = A.take<uint2>(words);
-  w.bsum = A.take<uint32_t>((words + CW - 1) / CW);
+  w.bsum = A.take<uint32_t>((words + words_per_cta(uint32_t(words)) - 1) / words_per_cta(uint32_t(words)));
   w.node_x = A.take<uint64_t>(w.max_rows);
   w.off = A.take<uint32_t>(n + 1);
   w.nodes = NodeView{w.node_x, w.off, w.packed};
@@ -698,11 +822,12 @@ void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w) {
 
 int launch_tree(const anqs_ham* H, const uint64_t* x, Count n_x, const TreeWs& w, cudaStream_t s) {
   const uint32_t words = H->sv.woff[H->v.n];
-  const unsigned blocks = (words + CW - 1) / CW;
+  const uint32_t cw = words_per_cta(words);
+  const unsigned blocks = (words + cw - 1) / cw;
   ANQS_CUDA(cudaMemsetAsync(w.n_rows, 0, w.zero_bytes, s));
   ANQS_CUDA_LAUNCH("mark_samples_kernel", launch_k(mark_samples_kernel, dim3(unsigned(std::min<uint64_t>((n_x.n + 63) / 64, 152 * 16))), dim3(64), 0, s, H->v, H->sv, x, n_x, w.bits));
-  ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, 0u, w.bsum, reinterpret_cast<unsigned long long*>(w.n_rows)));
-  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n, w.bits, words, w.bsum, w.packed, w.node_x, w.off));
+  ANQS_CUDA_LAUNCH("count_kernel", launch_k(count_kernel, dim3(blocks), dim3(CT), 0, s, w.bits, words, cw, 0u, w.bsum, reinterpret_cast<unsigned long long*>(w.n_rows)));
+  ANQS_CUDA_LAUNCH("emit_kernel", launch_k(emit_kernel, dim3(blocks), dim3(CT), 0, s, H->sv, H->v.n, w.bits, words, cw, w.bsum, w.packed, w.node_x, w.off));
   return ANQS_OK;
 }
 
@@ -726,24 +851,32 @@ int launch_path_sums(const anqs_ham* H, const UniqueWs& w, const float2* terms, 
   return ANQS_OK;
 }
 
-// n_x * split_of(n_x) stays below 1216 + n_x; never less for more samples
+// n_x * split_of(n_x) stays below 1216 + n_x; never less for more samples.
+// A call of more samples that is not split keeps its statistics' sums there.
 uint64_t eloc_partials(const anqs_ham* H, uint64_t n_x) {
-  return H->v.K >= 1024 ? 2 * (kFillCtas + std::min<uint64_t>(n_x, kFillCtas)) : 0;
+  return std::max<uint64_t>(H->v.K >= 1024 ? 2 * (kFillCtas + std::min<uint64_t>(n_x, kFillCtas)) : 0,
+                            n_x > kTailStats ? 4 * SB : 0);
 }
 
 int launch_eloc_direct(const anqs_ham* H, const uint64_t* x, Count n_x, const NodeView& nodes, const AmpSrc& amp,
                        double* ere, double* eim, double* part, const StatsOut& so, cudaStream_t s) {
   const int splits = split_of(n_x.n, H->v.K);
   const unsigned grid = unsigned(std::min<uint64_t>(n_x.n * splits, 152 * 16));
+  const bool tail = splits > 1 || n_x.n <= kTailStats;  // else the statistics are a launch of their own
+  const StatsOut in_kernel = tail ? so : StatsOut{};
   ProfScope ps(PROF_TC_ELOC, s);
   auto go = [&](auto kern) {
-    return launch_k(kern, dim3(grid), dim3(ET), 0, s, H->v, H->sv, nodes, x, n_x, splits, amp, ere, eim, part, so);
+    return launch_k(kern, dim3(grid), dim3(ET), 0, s, H->v, H->sv, nodes, x, n_x, splits, amp, ere, eim, part, in_kernel);
   };
   switch (amp.mode) {
     case AMP_SUM: ANQS_CUDA_LAUNCH("eloc_direct_kernel", go(eloc_direct_kernel<AMP_SUM>)); break;
     case AMP_BYJ: ANQS_CUDA_LAUNCH("eloc_direct_kernel", go(eloc_direct_kernel<AMP_BYJ>)); break;
     case AMP_TERMS: ANQS_CUDA_LAUNCH("eloc_direct_kernel", go(eloc_direct_kernel<AMP_TERMS>)); break;
     case AMP_ARRAY: ANQS_CUDA_LAUNCH("eloc_direct_kernel", go(eloc_direct_kernel<AMP_ARRAY>)); break;
+  }
+  if (!tail && so.counts) {
+    const unsigned blocks = unsigned(std::min<uint64_t>((n_x.n + 511) / 512, SB));
+    ANQS_CUDA_LAUNCH("stats_kernel", launch_k(stats_kernel, dim3(blocks), dim3(ET), 0, s, ere, eim, so.counts, n_x, part, so.ticket, so.stats));
   }
   return ANQS_OK;
 }

@@ -114,6 +114,13 @@ __device__ __forceinline__ int sign_ss(const Exc& E, int s, uint32_t po, uint32_
          int(i > lo && i < hi) ^ int(a > lo && a < hi);
 }
 
+// v with its sign flipped if odd: on the integer pipe (the FP64 pipe takes two
+// lanes per clock and SM on this GPU, and a conditional negation is an FP64
+// instruction)
+__device__ __forceinline__ double flip_sign(double v, int odd) {
+  return __hiloint2double(__double2hiint(v) ^ (odd << 31), __double2loint(v));
+}
+
 // two-electron integral (pq|rs)
 __device__ __forceinline__ double Gint(const HamView& hv, int p, int q, int r, int s) {
   const int n = hv.n;
