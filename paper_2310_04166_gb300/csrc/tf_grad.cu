@@ -11,10 +11,11 @@
 // embedding; per block LN1, q|k|v, causal attention (probabilities kept),
 // output projection + residual, LN2, FFN (pre-activation kept) + residual;
 // final LN and head.  The backward walks the same steps in reverse.  Matrix
-// products go through one tiled SGEMM kernel (operands normal or transposed,
-// optional bias, residual input, ReLU on an operand, ReLU'-mask of the
-// result); weight gradients are products over the R rows, split along R
-// across CTAs and accumulated with atomics into the flat gradient.
+// products go through one SGEMM tile (operands normal or transposed, optional
+// bias, residual input, ReLU on an operand, ReLU'-mask of the result); weight
+// gradients are products over the R rows, split along R across CTAs and
+// accumulated with atomics into the flat gradient.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -63,7 +64,7 @@ __global__ void tree_rows_kernel(SectorView sv, NodeView nv, uint8_t* __restrict
   }
 }
 
-constexpr int BM = 128, BN = 64, BK = 16, GT = 256;
+constexpr int BM = 64, BN = 64, BK = 16, GT = 128;
 
 // A matrix whose rows come in segments (the q, k and v weights lie one
 // behind the other with their biases between): row i starts at
@@ -92,6 +93,7 @@ struct Gm {
   int N;
   int relu_a, relu_b, atomic;
   int b_vec;          // B and bias are 16-byte aligned (parameters may be any float tensor, say a slice)
+  int c_vec;          // C is
   uint64_t k_chunk;   // split-K: K range per blockIdx.z
 };
 
@@ -104,34 +106,49 @@ __device__ __forceinline__ size_t seg_row(const Seg& s, int i, int ld) {
   return s.seg ? size_t(i / s.seg) * s.stride + size_t(i % s.seg) * ld : size_t(i) * ld;
 }
 
+// c += a b of two floats each (one instruction, the rounding of two fmaf)
+__device__ __forceinline__ void fma2(uint64_t a, uint64_t b, uint64_t& c) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t both(float v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
+
+struct GmSmem {
+  float A[2][BK][BM + 4], B[2][BK][BN + 4];
+};
+
 // C[m][n] = sum_k opA(m, k) opB(k, n), opA(m, k) = A[m][k] (TA: A[k][m]),
-// opB(k, n) = B[k][n] (TB: B[n][k]).  128 x 64 tile per CTA, 8 x 4 per thread
-// (3 16-byte shared loads for 32 FMAs; a 4 x 4 tile is bound by its shared
-// loads), the next K step's operands loaded to registers while this one runs.
+// opB(k, n) = B[k][n] (TB: B[n][k]); tile (bx, by), K part bz.  64 x 64 tile
+// per CTA of 128 threads, 8 x 4 per thread (3 16-byte shared loads for 32
+// FMAs, paired along the rows; a 4 x 4 tile is bound by its shared loads), the
+// next K step's operands loaded to registers while this one runs.  A CTA waits
+// for those loads in every step, so what counts is how many share an SM: with
+// 128 x 64 tiles the 26,000 rows of the 20-qubit workload were 205 CTAs of a
+// 64-column product, and half of every tile of a 64-row weight product empty.
 // All leading dimensions, segments and widths are multiples of 4 floats.
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
-  ANQS_PDL_ENTRY();
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
+__device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by, unsigned bz, GmSmem& sm) {
   const uint64_t M = g.M.get(), K = g.K.get();
-  const uint64_t m0 = uint64_t(blockIdx.y) * BM;
-  const int n0 = blockIdx.x * BN, tid = threadIdx.x;
+  const uint64_t m0 = uint64_t(by) * BM;
+  const int n0 = bx * BN, tid = threadIdx.x;
   if (m0 >= M) return;
-  const uint64_t k_lo = uint64_t(blockIdx.z) * g.k_chunk;
+  const uint64_t k_lo = uint64_t(bz) * g.k_chunk;
   if (k_lo >= K && !(k_lo == 0)) return;
   const uint64_t k_hi = k_lo + g.k_chunk < K ? k_lo + g.k_chunk : K;
   const int tx = tid % 16, ty = tid / 16;
-  float4 ra[2], rb;
+  float4 ra[2], rb[2];
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  // A: 128 x 16 elements, two 4-vectors per thread; B: 16 x 64, one
+  // A: 64 x 16 elements, B: 16 x 64: two 4-vectors per thread each
   auto load = [&](uint64_t k0) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int e = tid + GT * i;
-      ra[i] = zero;
+      ra[i] = rb[i] = zero;
       if (TA) {  // [k][m]: vectors along m
-        const uint64_t m = m0 + uint64_t(e % 32) * 4, k = k0 + e / 32;
+        const uint64_t m = m0 + uint64_t(e % 16) * 4, k = k0 + e / 16;
         if (k < k_hi) {
           const float* p = g.A + k * g.lda + m;
           if (m + 4 <= M) ra[i] = *reinterpret_cast<const float4*>(p);
@@ -149,42 +166,34 @@ __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
         ra[i].x = fmaxf(ra[i].x, 0.f), ra[i].y = fmaxf(ra[i].y, 0.f);
         ra[i].z = fmaxf(ra[i].z, 0.f), ra[i].w = fmaxf(ra[i].w, 0.f);
       }
-    }
-    rb = zero;
-    if (TB) {  // [n][k]: vectors along k
-      const int n = n0 + tid / 4;
-      const uint64_t k = k0 + uint64_t(tid % 4) * 4;
-      if (n < g.N && k + 4 <= k_hi) rb = ld4(g.B + seg_row(g.sb, n, g.ldb) + k, g.b_vec);
-    } else {  // [k][n]: vectors along n
-      const int n = n0 + (tid % 16) * 4;
-      const uint64_t k = k0 + tid / 16;
-      if (k < k_hi && n < g.N) rb = ld4(g.B + (g.sb.seg ? seg_row(g.sb, int(k), g.ldb) : k * g.ldb) + n, g.b_vec);
-    }
-    if (g.relu_b) {
-      rb.x = fmaxf(rb.x, 0.f), rb.y = fmaxf(rb.y, 0.f);
-      rb.z = fmaxf(rb.z, 0.f), rb.w = fmaxf(rb.w, 0.f);
+      if (TB) {  // [n][k]: vectors along k
+        const int n = n0 + e / 4;
+        const uint64_t k = k0 + uint64_t(e % 4) * 4;
+        if (n < g.N && k + 4 <= k_hi) rb[i] = ld4(g.B + seg_row(g.sb, n, g.ldb) + k, g.b_vec);
+      } else {  // [k][n]: vectors along n
+        const int n = n0 + (e % 16) * 4;
+        const uint64_t k = k0 + e / 16;
+        if (k < k_hi && n < g.N) rb[i] = ld4(g.B + (g.sb.seg ? seg_row(g.sb, int(k), g.ldb) : k * g.ldb) + n, g.b_vec);
+      }
+      if (g.relu_b) {
+        rb[i].x = fmaxf(rb[i].x, 0.f), rb[i].y = fmaxf(rb[i].y, 0.f);
+        rb[i].z = fmaxf(rb[i].z, 0.f), rb[i].w = fmaxf(rb[i].w, 0.f);
+      }
     }
   };
   auto store = [&](int b) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int e = tid + GT * i;
-      if (TA) {
-        *reinterpret_cast<float4*>(&As[b][e / 32][(e % 32) * 4]) = ra[i];
-      } else {
-        const int m = e / 4, k = (e % 4) * 4;
-        As[b][k][m] = ra[i].x, As[b][k + 1][m] = ra[i].y, As[b][k + 2][m] = ra[i].z, As[b][k + 3][m] = ra[i].w;
-      }
-    }
-    if (TB) {
-      const int n = tid / 4, k = (tid % 4) * 4;
-      Bs[b][k][n] = rb.x, Bs[b][k + 1][n] = rb.y, Bs[b][k + 2][n] = rb.z, Bs[b][k + 3][n] = rb.w;
-    } else {
-      *reinterpret_cast<float4*>(&Bs[b][tid / 16][(tid % 16) * 4]) = rb;
+      const int e = tid + GT * i, r = e / 4, k = (e % 4) * 4;
+      if (TA) *reinterpret_cast<float4*>(&sm.A[b][e / 16][(e % 16) * 4]) = ra[i];
+      else sm.A[b][k][r] = ra[i].x, sm.A[b][k + 1][r] = ra[i].y, sm.A[b][k + 2][r] = ra[i].z, sm.A[b][k + 3][r] = ra[i].w;
+      if (TB) sm.B[b][k][r] = rb[i].x, sm.B[b][k + 1][r] = rb[i].y, sm.B[b][k + 2][r] = rb[i].z, sm.B[b][k + 3][r] = rb[i].w;
+      else *reinterpret_cast<float4*>(&sm.B[b][e / 16][(e % 16) * 4]) = rb[i];
     }
   };
-  float acc[8][4] = {}, cs = 0.f;
-  const bool sums = g.colsum && blockIdx.x == 0;
+  uint64_t acc2[4][4] = {};  // rows 2 i and 2 i + 1 of the thread's eight
+  float cs = 0.f;
+  const bool sums = g.colsum && bx == 0;
   load(k_lo);
   store(0);
   __syncthreads();
@@ -194,18 +203,18 @@ __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
     if (more) load(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[b][kk][ty * 8 + 4]);
-      const float4 bb = *reinterpret_cast<const float4*>(&Bs[b][kk][tx * 4]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {bb.x, bb.y, bb.z, bb.w};
+      const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&sm.A[b][kk][ty * 8]);
+      const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&sm.A[b][kk][ty * 8 + 4]);
+      const float4 bb = *reinterpret_cast<const float4*>(&sm.B[b][kk][tx * 4]);
+      const uint64_t av[4] = {a0.x, a0.y, a1.x, a1.y}, bv[4] = {both(bb.x), both(bb.y), both(bb.z), both(bb.w)};
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) fma2(av[i], bv[j], acc2[i][j]);
     }
     if (sums && tid < BM)
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) cs += As[b][kk][tid];
+      for (int kk = 0; kk < BK; ++kk) cs += sm.A[b][kk][tid];
     if (more) store(b ^ 1);
     __syncthreads();
     b ^= 1;
@@ -217,13 +226,20 @@ __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
   for (int i = 0; i < 8; ++i) {
     const uint64_t m = m0 + ty * 8 + i;
     if (m >= M) break;
+    float a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] = __uint_as_float(uint32_t(acc2[i / 2][j] >> (32 * (i & 1))));
+    float4 v = make_float4(a[0], a[1], a[2], a[3]);
     float* c = g.C + (g.sc.seg ? seg_row(g.sc, int(m), g.ldc) : m * g.ldc) + n;
     if (g.atomic) {
+      if (g.c_vec) {
+        atomicAdd(reinterpret_cast<float4*>(c), v);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) atomicAdd(c + j, acc[i][j]);
+        for (int j = 0; j < 4; ++j) atomicAdd(c + j, a[j]);
+      }
       continue;
     }
-    float4 v = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
     if (g.bias) {
       const float4 t = ld4(g.bias + seg_row(g.sb, n, 1), g.b_vec);
       v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
@@ -238,6 +254,30 @@ __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
       v.z = t.z > 0.f ? v.z : 0.f, v.w = t.w > 0.f ? v.w : 0.f;
     }
     *reinterpret_cast<float4*>(c) = v;
+  }
+}
+
+// one product with a transposed B (the forward pass)
+__global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
+  ANQS_PDL_ENTRY();
+  __shared__ __align__(16) GmSmem sm;
+  gemm_tile<false, true>(g, blockIdx.x, blockIdx.y, 0, sm);
+}
+
+// A layer's two products of the backward pass, both from the cotangents of its
+// outputs: the input's cotangents d = dY W (CTAs from nw on, dx tiles wide) and
+// the weight gradient w += dY^T X (CTAs below nw: wx tiles wide, wy high, parts
+// of the rows).  In one launch, because neither fills the GPU by itself; the
+// weight product's CTAs run longest and come first.
+__global__ void __launch_bounds__(GT) sgemm_bwd_kernel(Gm w, Gm d, unsigned nw, unsigned wx, unsigned wy, unsigned dx) {
+  ANQS_PDL_ENTRY();
+  __shared__ __align__(16) GmSmem sm;
+  if (blockIdx.x < nw) {
+    const unsigned t = blockIdx.x % (wx * wy);
+    gemm_tile<true, false>(w, t % wx, t / wx, blockIdx.x / (wx * wy), sm);
+  } else {
+    const unsigned t = blockIdx.x - nw;
+    gemm_tile<false, false>(d, t % dx, t / dx, 0, sm);
   }
 }
 
@@ -353,28 +393,42 @@ __global__ void __launch_bounds__(256) ln_bwd_kernel(const float* __restrict__ d
 }
 
 // Causal attention of one (row, head) per thread over the row's ancestors;
-// keeps the probabilities P[r][h][u].  qkv [row][3 D].  V4: the head width is
-// a multiple of 4.  The heads of a row are neighbouring threads, so a warp
-// reads whole key and value rows.
-template <bool V4>
-__global__ void attn_fwd_kernel(const float* __restrict__ qkv, float* __restrict__ P, float* __restrict__ O, int D,
-                                int H, Rows R) {
+// keeps the probabilities P[r][h][u].  qkv [row][3 D].  The heads of a row are
+// neighbouring threads, so a warp reads whole key and value rows.  E4: the
+// head width in 4-vectors, held in registers (0: any width, one element or
+// 4-vector at a time).  Scores wait in shared memory: through global memory
+// (P itself) every one was written and read back three times, and the kernel
+// waited for that (26,000 rows x 4 heads: 30 us).
+constexpr int AT = 128;  // threads of the attention kernels
+template <int E4>
+__global__ void __launch_bounds__(AT) attn_fwd_kernel(const float* __restrict__ qkv, float* __restrict__ P,
+                                                      float* __restrict__ O, int D, int H, Rows R) {
   ANQS_PDL_ENTRY();
+  __shared__ float sp[32][AT];
   const uint64_t rows = R.rows.get();
-  const int dh = D / H, n = R.n;
+  const int dh = D / H, n = R.n, tid = threadIdx.x;
   const float scale = 1.0f / sqrtf(float(dh));
-  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < rows * H;
-       task += uint64_t(gridDim.x) * blockDim.x) {
+  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + tid; task < rows * H; task += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t r = task / H;
     const int hd = int(task - r * H), t = R.lv[r];
     const float* q = qkv + r * 3 * D + hd * dh;
     const uint32_t* anc = R.anc + r * n;
     float* prow = P + task * n;
     float mx = -INFINITY;
+    float4 qv[E4 ? E4 : 1];
+#pragma unroll
+    for (int e = 0; e < E4; ++e) qv[e] = *reinterpret_cast<const float4*>(q + 4 * e);
+#pragma unroll 2
     for (int u = 0; u <= t; ++u) {
       const float* k = qkv + size_t(anc[u]) * 3 * D + D + hd * dh;
       float dot = 0.f;
-      if constexpr (V4) {
+      if constexpr (E4 > 0) {
+#pragma unroll
+        for (int e = 0; e < E4; ++e) {
+          const float4 a = qv[e], b = *reinterpret_cast<const float4*>(k + 4 * e);
+          dot = fmaf(a.x, b.x, dot), dot = fmaf(a.y, b.y, dot), dot = fmaf(a.z, b.z, dot), dot = fmaf(a.w, b.w, dot);
+        }
+      } else if (dh % 4 == 0) {
         for (int e = 0; e < dh; e += 4) {
           const float4 a = *reinterpret_cast<const float4*>(q + e), b = *reinterpret_cast<const float4*>(k + e);
           dot = fmaf(a.x, b.x, dot), dot = fmaf(a.y, b.y, dot), dot = fmaf(a.z, b.z, dot), dot = fmaf(a.w, b.w, dot);
@@ -382,33 +436,52 @@ __global__ void attn_fwd_kernel(const float* __restrict__ qkv, float* __restrict
       } else {
         for (int e = 0; e < dh; ++e) dot = fmaf(q[e], k[e], dot);
       }
-      prow[u] = dot * scale;
+      sp[u][tid] = dot * scale;
       mx = fmaxf(mx, dot * scale);
     }
     float sum = 0.f;
     for (int u = 0; u <= t; ++u) {
-      const float p = expf(prow[u] - mx);
-      prow[u] = p;
+      const float p = expf(sp[u][tid] - mx);
+      sp[u][tid] = p;
       sum += p;
     }
     const float inv = 1.0f / sum;
-    for (int u = 0; u <= t; ++u) prow[u] *= inv;
     float* o = O + r * D + hd * dh;
-    constexpr int S = V4 ? 4 : 1;
-    for (int e = 0; e < dh; e += S) {
-      float a[S] = {};
+    if constexpr (E4 > 0) {
+      float4 acc[E4] = {};
+#pragma unroll 2
       for (int u = 0; u <= t; ++u) {
-        const float p = prow[u];
-        const float* v = qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh + e;
-        if constexpr (V4) {
-          const float4 w = *reinterpret_cast<const float4*>(v);
-          a[0] = fmaf(p, w.x, a[0]), a[1] = fmaf(p, w.y, a[1]), a[2] = fmaf(p, w.z, a[2]), a[3] = fmaf(p, w.w, a[3]);
-        } else {
-          a[0] = fmaf(p, v[0], a[0]);
+        const float p = sp[u][tid] * inv;
+        prow[u] = p;
+        const float* v = qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh;
+#pragma unroll
+        for (int e = 0; e < E4; ++e) {
+          const float4 w = *reinterpret_cast<const float4*>(v + 4 * e);
+          acc[e].x = fmaf(p, w.x, acc[e].x), acc[e].y = fmaf(p, w.y, acc[e].y);
+          acc[e].z = fmaf(p, w.z, acc[e].z), acc[e].w = fmaf(p, w.w, acc[e].w);
         }
       }
 #pragma unroll
-      for (int i = 0; i < S; ++i) o[e + i] = a[i];
+      for (int e = 0; e < E4; ++e) *reinterpret_cast<float4*>(o + 4 * e) = acc[e];
+    } else {
+      for (int u = 0; u <= t; ++u) prow[u] = sp[u][tid] = sp[u][tid] * inv;
+      if (dh % 4 == 0) {
+        for (int e = 0; e < dh; e += 4) {
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int u = 0; u <= t; ++u) {
+            const float p = sp[u][tid];
+            const float4 w = *reinterpret_cast<const float4*>(qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh + e);
+            a.x = fmaf(p, w.x, a.x), a.y = fmaf(p, w.y, a.y), a.z = fmaf(p, w.z, a.z), a.w = fmaf(p, w.w, a.w);
+          }
+          *reinterpret_cast<float4*>(o + e) = a;
+        }
+        continue;
+      }
+      for (int e = 0; e < dh; ++e) {
+        float a = 0.f;
+        for (int u = 0; u <= t; ++u) a = fmaf(sp[u][tid], qkv[size_t(anc[u]) * 3 * D + 2 * D + hd * dh + e], a);
+        o[e] = a;
+      }
     }
   }
 }
@@ -417,16 +490,16 @@ __global__ void attn_fwd_kernel(const float* __restrict__ qkv, float* __restrict
 // scale) and dQ.  dP_u = dO . V_u; dS_u = P_u (dP_u - sum_u' P_u' dP_u') scale.
 // The row's dQ | dK | dV slots hold dQ after it; dK and dV are zeroed here for
 // attn_bwd_kv_kernel.
-template <bool V4>
-__global__ void attn_bwd_q_kernel(const float* __restrict__ qkv, const float* __restrict__ P,
-                                  const float* __restrict__ dO, float* __restrict__ dS, float* __restrict__ dqkv, int D,
-                                  int H, Rows R) {
+template <int E4>
+__global__ void __launch_bounds__(AT) attn_bwd_q_kernel(const float* __restrict__ qkv, const float* __restrict__ P,
+                                                        const float* __restrict__ dO, float* __restrict__ dS,
+                                                        float* __restrict__ dqkv, int D, int H, Rows R) {
   ANQS_PDL_ENTRY();
+  __shared__ float sp[32][AT];
   const uint64_t rows = R.rows.get();
-  const int dh = D / H, n = R.n;
+  const int dh = D / H, n = R.n, tid = threadIdx.x;
   const float scale = 1.0f / sqrtf(float(dh));
-  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; task < rows * H;
-       task += uint64_t(gridDim.x) * blockDim.x) {
+  for (uint64_t task = blockIdx.x * uint64_t(blockDim.x) + tid; task < rows * H; task += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t r = task / H;
     const int hd = int(task - r * H), t = R.lv[r];
     const uint32_t* anc = R.anc + r * n;
@@ -434,10 +507,20 @@ __global__ void attn_bwd_q_kernel(const float* __restrict__ qkv, const float* __
     float* srow = dS + task * n;
     const float* go = dO + r * D + hd * dh;
     float dot = 0.f;
+    float4 gv[E4 ? E4 : 1];
+#pragma unroll
+    for (int e = 0; e < E4; ++e) gv[e] = *reinterpret_cast<const float4*>(go + 4 * e);
+#pragma unroll 2
     for (int u = 0; u <= t; ++u) {
       const float* v = qkv + size_t(anc[u]) * 3 * D + 2 * D + hd * dh;
       float a = 0.f;
-      if constexpr (V4) {
+      if constexpr (E4 > 0) {
+#pragma unroll
+        for (int e = 0; e < E4; ++e) {
+          const float4 x = gv[e], y = *reinterpret_cast<const float4*>(v + 4 * e);
+          a = fmaf(x.x, y.x, a), a = fmaf(x.y, y.y, a), a = fmaf(x.z, y.z, a), a = fmaf(x.w, y.w, a);
+        }
+      } else if (dh % 4 == 0) {
         for (int e = 0; e < dh; e += 4) {
           const float4 x = *reinterpret_cast<const float4*>(go + e), y = *reinterpret_cast<const float4*>(v + e);
           a = fmaf(x.x, y.x, a), a = fmaf(x.y, y.y, a), a = fmaf(x.z, y.z, a), a = fmaf(x.w, y.w, a);
@@ -445,29 +528,53 @@ __global__ void attn_bwd_q_kernel(const float* __restrict__ qkv, const float* __
       } else {
         for (int e = 0; e < dh; ++e) a = fmaf(go[e], v[e], a);
       }
-      srow[u] = a;
+      sp[u][tid] = a;
       dot = fmaf(prow[u], a, dot);
     }
-    for (int u = 0; u <= t; ++u) srow[u] = prow[u] * (srow[u] - dot) * scale;
     float* gq = dqkv + r * 3 * D + hd * dh;
-    constexpr int S = V4 ? 4 : 1;
-    for (int e = 0; e < dh; e += S) {
-      float a[S] = {};
+    if constexpr (E4 > 0) {
+      float4 acc[E4] = {};
+#pragma unroll 2
       for (int u = 0; u <= t; ++u) {
-        const float ds = srow[u];
-        const float* k = qkv + size_t(anc[u]) * 3 * D + D + hd * dh + e;
-        if constexpr (V4) {
-          const float4 w = *reinterpret_cast<const float4*>(k);
-          a[0] = fmaf(ds, w.x, a[0]), a[1] = fmaf(ds, w.y, a[1]), a[2] = fmaf(ds, w.z, a[2]), a[3] = fmaf(ds, w.w, a[3]);
-        } else {
-          a[0] = fmaf(ds, k[0], a[0]);
+        const float ds = prow[u] * (sp[u][tid] - dot) * scale;
+        srow[u] = ds;
+        const float* k = qkv + size_t(anc[u]) * 3 * D + D + hd * dh;
+#pragma unroll
+        for (int e = 0; e < E4; ++e) {
+          const float4 w = *reinterpret_cast<const float4*>(k + 4 * e);
+          acc[e].x = fmaf(ds, w.x, acc[e].x), acc[e].y = fmaf(ds, w.y, acc[e].y);
+          acc[e].z = fmaf(ds, w.z, acc[e].z), acc[e].w = fmaf(ds, w.w, acc[e].w);
         }
       }
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < S; ++i) {
-        gq[e + i] = a[i];
-        gq[D + e + i] = 0.f;
-        gq[2 * D + e + i] = 0.f;
+      for (int e = 0; e < E4; ++e) {
+        *reinterpret_cast<float4*>(gq + 4 * e) = acc[e];
+        *reinterpret_cast<float4*>(gq + D + 4 * e) = zero;
+        *reinterpret_cast<float4*>(gq + 2 * D + 4 * e) = zero;
+      }
+    } else {
+      for (int u = 0; u <= t; ++u) srow[u] = sp[u][tid] = prow[u] * (sp[u][tid] - dot) * scale;
+      if (dh % 4 == 0) {
+        for (int e = 0; e < dh; e += 4) {
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int u = 0; u <= t; ++u) {
+            const float p = sp[u][tid];
+            const float4 w = *reinterpret_cast<const float4*>(qkv + size_t(anc[u]) * 3 * D + D + hd * dh + e);
+            a.x = fmaf(p, w.x, a.x), a.y = fmaf(p, w.y, a.y), a.z = fmaf(p, w.z, a.z), a.w = fmaf(p, w.w, a.w);
+          }
+          *reinterpret_cast<float4*>(gq + e) = a;
+          *reinterpret_cast<float4*>(gq + D + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+          *reinterpret_cast<float4*>(gq + 2 * D + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        continue;
+      }
+      for (int e = 0; e < dh; ++e) {
+        float a = 0.f;
+        for (int u = 0; u <= t; ++u) a = fmaf(sp[u][tid], qkv[size_t(anc[u]) * 3 * D + D + hd * dh + e], a);
+        gq[e] = a;
+        gq[D + e] = 0.f;
+        gq[2 * D + e] = 0.f;
       }
     }
   }
@@ -501,14 +608,24 @@ __global__ void attn_bwd_kv_kernel(const float* __restrict__ qkv, const float* _
     const size_t ldv = kv ? D : 3 * size_t(D);
     uint32_t cur = 0xffffffffu;
     float acc = 0.f;
-    for (int i = 0; i < int(r1 - r0); ++i) {
-      const uint32_t k = key[i];
-      if (k != cur) {
-        if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
-        cur = k;
-        acc = 0.f;
+    for (int i0 = 0; i0 < int(r1 - r0); i0 += 8) {  // eight rows' loads in flight (rows beyond have no key)
+      float wr[8], vr[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const bool on = key[i0 + e] != 0xffffffffu;
+        wr[e] = on ? w[(r0 + i0 + e) * H * n] : 0.f;
+        vr[e] = on ? v[(r0 + i0 + e) * ldv] : 0.f;
       }
-      if (k != 0xffffffffu) acc = fmaf(w[(r0 + i) * H * n], v[(r0 + i) * ldv], acc);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t k = key[i0 + e];
+        if (k != cur) {
+          if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
+          cur = k;
+          acc = 0.f;
+        }
+        if (k != 0xffffffffu) acc = fmaf(wr[e], vr[e], acc);
+      }
     }
     if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
   }
@@ -593,34 +710,49 @@ __global__ void head_dout_kernel(HamView hv, Rows R, const float* __restrict__ o
 }
 
 // gtok[token(r)] += dH0[r], gpos[position of r] += dH0[r]: thread = column,
-// a CTA's rows in order, one add per token and per run of equal positions
-constexpr int EBR = 128;
+// a CTA's rows in order, one add per token and per run of equal positions.
+// The rows' positions and tokens come first, so that eight rows' loads are in
+// flight (a row at a time, waiting for its position, its token and its value
+// in turn, took 60 us for 26,000 rows).
+constexpr int EBR = 64;
 __global__ void embed_bwd_kernel(TfView m, Rows R, const float* __restrict__ dh0, float* __restrict__ gtok,
                                  float* __restrict__ gpos) {
   ANQS_PDL_ENTRY();
+  __shared__ uint8_t s_pos[EBR], s_tok[EBR];
   const uint64_t rows = R.rows.get(), r0 = uint64_t(blockIdx.x) * EBR;
   if (r0 >= rows) return;
-  const uint64_t r1 = r0 + EBR < rows ? r0 + EBR : rows;
-  const int D = m.d;
+  const int D = m.d, cnt = int(r0 + EBR < rows ? EBR : rows - r0);
+  for (int i = threadIdx.x; i < EBR; i += blockDim.x) {
+    const int t = i < cnt ? R.lv[r0 + i] : 255;
+    s_pos[i] = uint8_t(t);
+    s_tok[i] = uint8_t(i >= cnt ? 5 : t == 0 ? 4 : int((R.x[r0 + i] >> (2 * (t - 1))) & 3ull));
+  }
+  __syncthreads();
   for (int c = threadIdx.x; c < D; c += blockDim.x) {
     float tk[5] = {}, ps = 0.f;
-    int cur = -1;
-    for (uint64_t r = r0; r < r1; ++r) {
-      const int t = R.lv[r];
-      const int token = t == 0 ? 4 : int((R.x[r] >> (2 * (t - 1))) & 3ull);
-      const float v = dh0[r * D + c];
-      if (t != cur) {
-        if (cur >= 0) atomicAdd(gpos + cur * D + c, ps);
-        cur = t;
-        ps = 0.f;
-      }
-      ps += v;
+    int cur = s_pos[0];
+    for (int i0 = 0; i0 < cnt; i0 += 8) {
+      float v[8];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) tk[k] += k == token ? v : 0.f;
+      for (int e = 0; e < 8; ++e) v[e] = i0 + e < cnt ? dh0[(r0 + i0 + e) * D + c] : 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        if (i0 + e >= cnt) break;
+        const int t = s_pos[i0 + e], token = s_tok[i0 + e];
+        if (t != cur) {
+          atomicAdd(gpos + cur * D + c, ps);
+          cur = t;
+          ps = 0.f;
+        }
+        ps += v[e];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) tk[k] += k == token ? v[e] : 0.f;
+      }
     }
     atomicAdd(gpos + cur * D + c, ps);
 #pragma unroll
-    for (int k = 0; k < 5; ++k) atomicAdd(gtok + k * D + c, tk[k]);
+    for (int k = 0; k < 5; ++k)
+      if (tk[k] != 0.f) atomicAdd(gtok + k * D + c, tk[k]);
   }
 }
 
@@ -737,32 +869,38 @@ unsigned grid_for(uint64_t work, int threads, uint64_t cap) {
   return unsigned(b ? b : 1);
 }
 
-// C (M x N) = op(A) op(B) with the options of Gm; M a row count (device or
-// host), K given by Kc.  Weight products (atomic) split K over CTAs.
-template <bool TA, bool TB>
-int gemm(Gm g, uint64_t M_host, uint64_t K_host, cudaStream_t s) {
-  const unsigned gx = unsigned((g.N + BN - 1) / BN);
-  const uint64_t gy = (M_host + BM - 1) / BM;
-  unsigned gz = 1;
-  g.k_chunk = K_host ? K_host : 1;
-  if (g.atomic) {
-    const uint64_t tiles = uint64_t(gx) * gy;
-    uint64_t want = (152 * 3 + tiles - 1) / tiles;
-    const uint64_t max_split = (K_host + 127) / 128;  // at least 128 rows per split
-    if (want > max_split) want = max_split;
-    if (want < 1) want = 1;
-    gz = unsigned(want);
-    g.k_chunk = ((K_host + gz - 1) / gz + BK - 1) / BK * BK;
-  }
-  if (gy > 65535u) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows for the transformer adjoint");
+void set_vec(Gm& g) {
   g.b_vec = reinterpret_cast<uintptr_t>(g.B) % 16 == 0 && reinterpret_cast<uintptr_t>(g.bias) % 16 == 0;
-  ANQS_CUDA_LAUNCH("tf sgemm_kernel", launch_k(sgemm_kernel<TA, TB>, dim3(gx, unsigned(gy), gz), dim3(GT), 0, s, g));
+  g.c_vec = reinterpret_cast<uintptr_t>(g.C) % 16 == 0;
+}
+
+// C = A B^T with the options of Gm, M rows (device or host count)
+int gemm_nt(Gm g, uint64_t M_host, uint64_t K_host, cudaStream_t s) {
+  const uint64_t gy = (M_host + BM - 1) / BM;
+  if (gy > 65535u) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows for the transformer adjoint");
+  g.k_chunk = K_host ? K_host : 1;
+  set_vec(g);
+  ANQS_CUDA_LAUNCH("tf sgemm_kernel", launch_k(sgemm_kernel, dim3(unsigned((g.N + BN - 1) / BN), unsigned(gy)), dim3(GT), 0, s, g));
   return ANQS_OK;
 }
 
-int gemm_nt(const Gm& g, uint64_t M, uint64_t K, cudaStream_t s) { return gemm<false, true>(g, M, K, s); }
-int gemm_nn(const Gm& g, uint64_t M, uint64_t K, cudaStream_t s) { return gemm<false, false>(g, M, K, s); }
-int gemm_tn(const Gm& g, uint64_t M, uint64_t K, cudaStream_t s) { return gemm<true, false>(g, M, K, s); }
+// The weight product w (Mw x N, over R rows, split over CTAs) and the data
+// product d (R x N) of one layer
+int gemm_bwd(Gm w, uint64_t Mw, Gm d, uint64_t Kd, uint64_t R, cudaStream_t s) {
+  const unsigned wx = unsigned((w.N + BN - 1) / BN), wy = unsigned((Mw + BM - 1) / BM), dx = unsigned((d.N + BN - 1) / BN);
+  const uint64_t dy = (R + BM - 1) / BM;
+  uint64_t parts = (152 * 4 + wx * wy - 1) / (wx * wy);
+  parts = std::max<uint64_t>(1, std::min(parts, (R + 127) / 128));  // at least 128 rows each
+  w.k_chunk = ((R + parts - 1) / parts + BK - 1) / BK * BK;
+  d.k_chunk = Kd ? Kd : 1;
+  if (!w.k_chunk) w.k_chunk = BK;
+  if (dy * dx > (1ull << 30)) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows for the transformer adjoint");
+  set_vec(w);
+  set_vec(d);
+  const unsigned nw = unsigned(parts) * wx * wy;
+  ANQS_CUDA_LAUNCH("tf sgemm_bwd_kernel", launch_k(sgemm_bwd_kernel, dim3(nw + unsigned(dy) * dx), dim3(GT), 0, s, w, d, nw, wx, wy, dx));
+  return ANQS_OK;
+}
 
 Gm mk(const float* A, int lda, const float* B, int ldb, float* C, int ldc, Count M, Count K, int N) {
   Gm g = {};
@@ -795,14 +933,19 @@ int run(const TfView& m, const anqs_ham* Hm, const uint64_t* x, Count nx, const 
     ckpt = true;
   }
   const int n = m.n, L = m.L, H = m.H;
-  const bool v4 = (D / H) % 4 == 0;
+  // attention kernels with the head in registers for widths 4 to 32 in powers of two
+  const int e4 = D / H == 4 ? 1 : D / H == 8 ? 2 : D / H == 16 ? 4 : D / H == 32 ? 8 : 0;
+  const auto attn_fwd = e4 == 1 ? attn_fwd_kernel<1> : e4 == 2 ? attn_fwd_kernel<2> : e4 == 4 ? attn_fwd_kernel<4>
+                        : e4 == 8 ? attn_fwd_kernel<8> : attn_fwd_kernel<0>;
+  const auto attn_bwd_q = e4 == 1 ? attn_bwd_q_kernel<1> : e4 == 2 ? attn_bwd_q_kernel<2> : e4 == 4 ? attn_bwd_q_kernel<4>
+                          : e4 == 8 ? attn_bwd_q_kernel<8> : attn_bwd_q_kernel<0>;
   const uint64_t R = a.R;
   const Count rows = a.tree ? Count{R, a.t.n_rows, 1} : scaled(nx, n);
   const Count kD = host_count(D), k3D = host_count(3 * D), k4D = host_count(4 * D), k8 = host_count(8);
   const float* P = m.params;
   ProfScope ps(PROF_TF_GRAD, s);
   const unsigned eg = grid_for(R * D, 256, 152 * 16), lg = grid_for(R * 32, 256, 152 * 16);
-  const unsigned ag = grid_for(R * H, 128, 152 * 16);
+  const unsigned ag = grid_for(R * H, AT, 152 * 16);
   Rows rw{a.x, a.lv, a.anc, rows, n};
   ANQS_CUDA(cudaMemsetAsync(a.cot, 0, R * 8 * sizeof(double), s));
   if (a.tree) {
@@ -827,7 +970,7 @@ int run(const TfView& m, const anqs_ham* Hm, const uint64_t* x, Count nx, const 
       g.bias = P + o.bq;
       ANQS_TRY(gemm_nt(g, R, D, s));
     }
-    ANQS_CUDA_LAUNCH("tf attn_fwd_kernel", launch_k(v4 ? attn_fwd_kernel<true> : attn_fwd_kernel<false>, dim3(ag), dim3(128), 0, s, a.QKV[l], a.P[l], a.O[l], D, H, rw));
+    ANQS_CUDA_LAUNCH("tf attn_fwd_kernel", launch_k(attn_fwd, dim3(ag), dim3(AT), 0, s, a.QKV[l], a.P[l], a.O[l], D, H, rw));
     {
       Gm g = mk(a.O[l], D, P + o.wo, D, a.Hm[l], D, rows, kD, D);
       g.bias = P + o.bo;
@@ -867,19 +1010,18 @@ int run(const TfView& m, const anqs_ham* Hm, const uint64_t* x, Count nx, const 
   // ---- backward ----
   // weight gradient gW += dY^T X and bias gradient gb += the column sums of dY
   auto wgrad = [&](const float* dY, int ldy, const float* X, int ldx, int Mo, int Ni, float* gW, float* gb, int relu_x,
-                   Seg seg = Seg{}) -> int {
+                   Seg seg = Seg{}) -> Gm {
     Gm g = mk(dY, ldy, X, ldx, gW, Ni, host_count(Mo), rows, Ni);
     g.relu_b = relu_x;
     g.atomic = 1;
     g.sc = seg;
     g.colsum = gb;
-    return gemm_tn(g, Mo, R, s);
+    return g;
   };
-  ANQS_TRY(wgrad(a.dout8, 8, a.Af, D, 8, D, grad + head_w, nullptr, 0));
   ANQS_CUDA_LAUNCH("tf colsum8_kernel", launch_k(colsum8_kernel, dim3(grid_for(R * 8, 256, 152)), dim3(256), 0, s, a.dout8, rows, grad + head_b));
   {
-    Gm g = mk(a.dout8, 8, P + head_w, D, a.dA, D, rows, k8, D);
-    ANQS_TRY(gemm_nn(g, R, 8, s));
+    const Gm g = mk(a.dout8, 8, P + head_w, D, a.dA, D, rows, k8, D);
+    ANQS_TRY(gemm_bwd(wgrad(a.dout8, 8, a.Af, D, 8, D, grad + head_w, nullptr, 0), 8, g, 8, R, s));
   }
   ANQS_CUDA_LAUNCH("tf ln_bwd_kernel",
                    launch_k(ln_bwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.dA, a.Xhf, P + lnf_g, a.RSf,
@@ -887,33 +1029,29 @@ int run(const TfView& m, const anqs_ham* Hm, const uint64_t* x, Count nx, const 
   for (int l = L - 1; l >= 0; --l) {
     const LayerOff o = layer_off(m, l);
     if (ckpt && l + 1 < L) ANQS_TRY(fwd_block(l));  // the shared activations hold block L-1's after the forward
-    ANQS_TRY(wgrad(a.dH, D, a.F[l], 4 * D, D, 4 * D, grad + o.w2, grad + o.b2, 1));
     {
       Gm g = mk(a.dH, D, P + o.w2, 4 * D, a.dF, 4 * D, rows, kD, 4 * D);
       g.mask = a.F[l];
       g.ldmask = 4 * D;
-      ANQS_TRY(gemm_nn(g, R, D, s));
+      ANQS_TRY(gemm_bwd(wgrad(a.dH, D, a.F[l], 4 * D, D, 4 * D, grad + o.w2, grad + o.b2, 1), D, g, D, R, s));
     }
-    ANQS_TRY(wgrad(a.dF, 4 * D, a.A2[l], D, 4 * D, D, grad + o.w1, grad + o.b1, 0));
     {
-      Gm g = mk(a.dF, 4 * D, P + o.w1, D, a.dA, D, rows, k4D, D);
-      ANQS_TRY(gemm_nn(g, R, 4 * D, s));
+      const Gm g = mk(a.dF, 4 * D, P + o.w1, D, a.dA, D, rows, k4D, D);
+      ANQS_TRY(gemm_bwd(wgrad(a.dF, 4 * D, a.A2[l], D, 4 * D, D, grad + o.w1, grad + o.b1, 0), 4 * D, g, 4 * D, R, s));
     }
     ANQS_CUDA_LAUNCH("tf ln_bwd_kernel", launch_k(ln_bwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.dA, a.Xh2[l],
                                                   P + o.ln2_g, a.RS2[l], (const float*)a.dH, a.dHm, grad + o.ln2_g,
                                                   grad + o.ln2_b, rows));
-    ANQS_TRY(wgrad(a.dHm, D, a.O[l], D, D, D, grad + o.wo, grad + o.bo, 0));
     {
-      Gm g = mk(a.dHm, D, P + o.wo, D, a.dO, D, rows, kD, D);
-      ANQS_TRY(gemm_nn(g, R, D, s));
+      const Gm g = mk(a.dHm, D, P + o.wo, D, a.dO, D, rows, kD, D);
+      ANQS_TRY(gemm_bwd(wgrad(a.dHm, D, a.O[l], D, D, D, grad + o.wo, grad + o.bo, 0), D, g, D, R, s));
     }
-    ANQS_CUDA_LAUNCH("tf attn_bwd_q_kernel", launch_k(v4 ? attn_bwd_q_kernel<true> : attn_bwd_q_kernel<false>, dim3(ag), dim3(128), 0, s, a.QKV[l], a.P[l], a.dO, a.dS, a.dQKV, D, H, rw));
+    ANQS_CUDA_LAUNCH("tf attn_bwd_q_kernel", launch_k(attn_bwd_q, dim3(ag), dim3(AT), 0, s, a.QKV[l], a.P[l], a.dO, a.dS, a.dQKV, D, H, rw));
     ANQS_CUDA_LAUNCH("tf attn_bwd_kv_kernel", launch_k(attn_bwd_kv_kernel, dim3(unsigned((R + KVR - 1) / KVR), unsigned(n)), dim3(2 * D < 256 ? 2 * D : 256), 0, s, a.QKV[l], a.P[l], a.dO, a.dS, a.dQKV, D, H, rw));
-    ANQS_TRY(wgrad(a.dQKV, 3 * D, a.A1[l], D, 3 * D, D, grad + o.wq, grad + o.bq, 0, qkv_seg));
     {
       Gm g = mk(a.dQKV, 3 * D, P + o.wq, D, a.dA, D, rows, k3D, D);
       g.sb = qkv_seg;
-      ANQS_TRY(gemm_nn(g, R, 3 * D, s));
+      ANQS_TRY(gemm_bwd(wgrad(a.dQKV, 3 * D, a.A1[l], D, 3 * D, D, grad + o.wq, grad + o.bq, 0, qkv_seg), 3 * D, g, 3 * D, R, s));
     }
     ANQS_CUDA_LAUNCH("tf ln_bwd_kernel", launch_k(ln_bwd_kernel<D>, dim3(lg), dim3(256), 0, s, a.dA, a.Xh1[l],
                                                   P + o.ln1_g, a.RS1[l], (const float*)a.dHm, a.dH, grad + o.ln1_g,
