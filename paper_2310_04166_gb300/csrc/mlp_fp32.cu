@@ -109,28 +109,110 @@ __device__ __forceinline__ void tile_gemm(const float* in, const float* __restri
 
 template <int W, int RR = R>
 struct Smem {
-  static constexpr size_t ws_floats = KC * (W + 1);
+  static constexpr size_t ws_floats = KC * (W + 4);
   static size_t bytes(int n_act) { return (size_t(n_act) * RR * W + ws_floats + RR * 8) * sizeof(float); }
 };
+
+// o[r][c] = tanh(bk[c] + sum_k in[r][k] Wk[c][k]): tile_gemm's sums (k
+// ascending) with 16-byte shared loads of four columns' weights and of four of
+// a row's inputs, 5 passes of the shared memory for 16 FMAs of a warp instead
+// of 8.  Begins with the CTA synchronised.
+template <int W, int RR>
+__device__ __forceinline__ void hidden_layer(const float* in, const float* __restrict__ Wk, const float* __restrict__ bk,
+                                             float* ws, float* o) {
+  constexpr int RPT = RR / 8, CPT = W / 32, V = CPT < 4 ? CPT : 4, NJ = CPT / V, WS = W + 4;
+  const int lane = threadIdx.x & 31, wg = threadIdx.x >> 5;
+  float acc[RPT][CPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i)
+#pragma unroll
+    for (int j = 0; j < CPT; ++j) acc[i][j] = 0.f;
+  for (int k0 = 0; k0 < W; k0 += KC) {
+    __syncthreads();
+#pragma unroll 8
+    for (int idx = threadIdx.x; idx < KC * W; idx += NT) {
+      const int c = idx / KC, kk = idx % KC;
+      ws[kk * WS + c] = __ldg(Wk + size_t(c) * W + k0 + kk);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int kk = 0; kk < KC; kk += 4) {
+      float a[RPT][4];
+#pragma unroll
+      for (int i = 0; i < RPT; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(in + (wg * RPT + i) * W + k0 + kk);
+        a[i][0] = v.x, a[i][1] = v.y, a[i][2] = v.z, a[i][3] = v.w;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float b[CPT];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const float* src = ws + (kk + e) * WS + lane * V + 32 * V * j;
+          if constexpr (V == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(src);
+            b[4 * j] = v.x, b[4 * j + 1] = v.y, b[4 * j + 2] = v.z, b[4 * j + 3] = v.w;
+          } else {
+            const float2 v = *reinterpret_cast<const float2*>(src);
+            b[2 * j] = v.x, b[2 * j + 1] = v.y;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+#pragma unroll
+          for (int j = 0; j < CPT; ++j) acc[i][j] = fmaf(a[i][e], b[j], acc[i][j]);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < CPT; ++j) {
+    const int c = lane * V + 32 * V * (j / V) + j % V;
+    const float bias = __ldg(bk + c);
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) o[(wg * RPT + i) * W + c] = tanhf(acc[i][j] + bias);
+  }
+}
 
 // Forward of slot p for the R rows whose determinants are xs[0..R) (rows
 // >= nrows are computed on garbage-free zeros and ignored).  act holds
 // n_keep activation buffers [R][W]: with n_keep == L every layer's output is
 // kept (for the adjoint), with n_keep == 2 they ping-pong.  Leaves the head
 // outputs in out8[R][8] and returns the index of the last hidden buffer.
+// The layer-1 weights pass through ws eight slots at a time: gathered from
+// global memory, each of a warp's lanes met another row of W1, and those
+// loads took most of the time of a node (12,400 prefixes of 9 orbitals, width
+// 128, 3 layers: 200 us).
 template <int W, int RR = R>
 __device__ int slot_forward(const MlpView& m, int p, const uint64_t* xs, int nrows, float* act, int n_keep,
                             float* ws, float* out8, const float* wres = nullptr) {
   const MlpPtr P = slot_ptrs(m, p);
-  for (int idx = threadIdx.x; idx < RR * W; idx += NT) {
-    int r = idx / W, o = idx % W;
-    float acc = __ldg(P.b1 + o);
-    if (r < nrows) {
-      uint64_t x = xs[r];
-      const float* wrow = P.W1 + size_t(o) * 4 * p;
-      for (int q = 0; q < p; ++q) acc += __ldg(wrow + 4 * q + int((x >> (2 * q)) & 3ull));
+  {
+    constexpr int E = RR * W / NT, WS = W + 4;  // thread: column o of rows r0 + (NT / W) e
+    static_assert(NT % W == 0 && RR * W % NT == 0, "tile shape");
+    const int o = threadIdx.x % W, r0 = threadIdx.x / W;
+    float acc[E];
+    const float b = __ldg(P.b1 + o);
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = b;
+    for (int q0 = 0; q0 < p; q0 += 8) {
+      const int nq = p - q0 < 8 ? p - q0 : 8;
+      __syncthreads();
+#pragma unroll 4
+      for (int idx = threadIdx.x; idx < 32 * W; idx += NT) {
+        const int c = idx / 32, kk = idx % 32;
+        if (kk < 4 * nq) ws[kk * WS + c] = __ldg(P.W1 + size_t(c) * 4 * p + 4 * q0 + kk);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int r = r0 + NT / W * e;
+        if (r >= nrows) continue;
+        const uint64_t x = xs[r] >> (2 * q0);
+        for (int q = 0; q < nq; ++q) acc[e] += ws[(4 * q + int((x >> (2 * q)) & 3ull)) * WS + o];
+      }
     }
-    act[idx] = tanhf(acc);
+#pragma unroll
+    for (int e = 0; e < E; ++e) act[(r0 + NT / W * e) * W + o] = tanhf(acc[e]);
   }
   int cur = 0;
   const float* Wk = P.Wk;
@@ -138,11 +220,16 @@ __device__ int slot_forward(const MlpView& m, int p, const uint64_t* xs, int nro
   const int lane = threadIdx.x & 31, wg = threadIdx.x >> 5;
   for (int k = 2; k <= m.n_hidden; ++k) {
     const float* bk = Wk + size_t(W) * W;
-    float acc[RPT][CPT];
-    tile_gemm<W, false, RR>(act + size_t(cur) * RR * W, Wk, ws, acc,
-                            wres ? wres + size_t(k - 2) * W * (W + 1) : nullptr);
     int nxt = (n_keep == 2) ? (cur ^ 1) : (cur + 1);
     float* o = act + size_t(nxt) * RR * W;
+    if (!wres) {
+      hidden_layer<W, RR>(act + size_t(cur) * RR * W, Wk, bk, ws, o);
+      cur = nxt;
+      Wk = bk + W;
+      continue;
+    }
+    float acc[RPT][CPT];
+    tile_gemm<W, false, RR>(act + size_t(cur) * RR * W, Wk, ws, acc, wres + size_t(k - 2) * W * (W + 1));
 #pragma unroll
     for (int i = 0; i < RPT; ++i)
 #pragma unroll
