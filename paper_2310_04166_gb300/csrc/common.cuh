@@ -525,6 +525,7 @@ void plan_unique(const anqs_ham* H, uint64_t n_x, bool levels, Arena& A, UniqueW
 int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueWs& w, cudaStream_t s);
 Count unique_leaves(const UniqueWs& w);
 const uint64_t* unique_leaf_x(const anqs_ham* H, const UniqueWs& w);  // full, or planned without levels
+// per: float2 [2][w.max_nodes]
 int launch_path_terms(const anqs_ham* H, const UniqueWs& w, const float2* per, float2* out, cudaStream_t s);
 int launch_byj(const HamView& hv, const uint64_t* x, Count rows, const float* raw, float2* tab, cudaStream_t s);
 int launch_chunk_counts(const uint64_t* total, uint64_t chunk, int n, uint64_t* out, cudaStream_t s);

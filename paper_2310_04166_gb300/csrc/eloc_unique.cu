@@ -300,8 +300,8 @@ __global__ void path_sum_kernel(SectorView sv, NodeView nv, const float2* __rest
   }
 }
 
-// out[leaf][p] = per[node of the leaf's level p + 1 prefix]
-__global__ void path_terms_kernel(SectorView sv, NodeView nv, const float2* __restrict__ per,
+// out[leaf][p] = per[id] + per[stride + id], id the node of the leaf's level p + 1 prefix
+__global__ void path_terms_kernel(SectorView sv, NodeView nv, const float2* __restrict__ per, uint64_t stride,
                                   float2* __restrict__ out) {
   ANQS_PDL_ENTRY();
   const int n = sv.n;
@@ -311,7 +311,9 @@ __global__ void path_terms_kernel(SectorView sv, NodeView nv, const float2* __re
     const uint32_t r = uint32_t(t / uint32_t(n));
     const int p = int(t - uint64_t(r) * uint32_t(n)) + 1;
     const uint64_t x = __ldcg(reinterpret_cast<const unsigned long long*>(nv.x) + i0 + r);
-    out[t] = __ldcg(per + node_id(sv, nv, p, prefix_index(sv, p, even_bits(x), even_bits(x >> 1))));
+    const float2* at = per + node_id(sv, nv, p, prefix_index(sv, p, even_bits(x), even_bits(x >> 1)));
+    const float2 u = __ldcg(at), v = __ldcg(at + stride);
+    out[t] = make_float2(u.x + v.x, u.y + v.y);
   }
 }
 
@@ -776,7 +778,7 @@ int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueW
 int launch_path_terms(const anqs_ham* H, const UniqueWs& w, const float2* per, float2* out, cudaStream_t s) {
   ProfScope ps(PROF_TC_FINALIZE, s);
   const unsigned grid = unsigned(std::min<uint64_t>((w.max_leaves * H->v.n + 255) / 256, 152 * 8));
-  ANQS_CUDA_LAUNCH("path_terms_kernel", launch_k(path_terms_kernel, dim3(grid ? grid : 1), dim3(256), 0, s, H->sv, w.nodes, per, out));
+  ANQS_CUDA_LAUNCH("path_terms_kernel", launch_k(path_terms_kernel, dim3(grid ? grid : 1), dim3(256), 0, s, H->sv, w.nodes, per, w.max_nodes, out));
   return ANQS_OK;
 }
 

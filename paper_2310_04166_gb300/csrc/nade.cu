@@ -31,7 +31,7 @@
 // (for each connected x', sorted by its first differing slot j, the path terms
 // of the slots p > j: prefix reuse, the slots <= j come from the parent), and
 // LOGITS (slot p's 8 values for the sampler's prefixes), NODES (each distinct
-// prefix of p + 1 slots: the path term of its slot p).
+// prefix of p + 1 slots: the path terms of its slot p's two qubits).
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -140,14 +140,15 @@ __device__ __forceinline__ float2 input_layer(const float2* __restrict__ w1, flo
 // ---------------------------------------------------------------------------
 // Tile engine
 // ---------------------------------------------------------------------------
-template <int W, int RJ>
+// PARTS: parts of the head's sums, if not the tile's own
+template <int W, int RJ, int PARTS = 0>
 struct Tile {
   static constexpr int NTX = W / 4;      // GEMM thread grid: NTX x NTY threads, 4 units x RJ rows each
   static constexpr int NTY = NT / NTX;
   static constexpr int TR = NTY * RJ;    // rows per tile
   static constexpr int WS = W + 1;       // W2 row stride (float2)
   static constexpr int HS = TR + 4;      // h row stride (floats; real and imaginary planes)
-  static constexpr int KP = 128 / TR;    // k-parts of the head reduction
+  static constexpr int KP = PARTS ? PARTS : 128 / TR;  // k-parts of the head reduction
   static constexpr int NZ = 1;           // z3 tiles kept (one evaluation per CTA)
   static constexpr size_t w2_bytes = size_t(W) * WS * sizeof(float2);
   static constexpr size_t h_bytes = 2 * size_t(W) * HS * sizeof(float);
@@ -169,9 +170,9 @@ struct TileSmem {
   float2 *Z3p, *Z3;
 };
 
-template <int W, int RJ>
+template <int W, int RJ, int PARTS>
 __device__ __forceinline__ TileSmem tile_smem(float2* base) {
-  using T = Tile<W, RJ>;
+  using T = Tile<W, RJ, PARTS>;
   TileSmem s;
   char* p = reinterpret_cast<char*>(base);
   s.W2 = reinterpret_cast<float2*>(p);
@@ -190,10 +191,10 @@ __device__ __forceinline__ TileSmem tile_smem(float2* base) {
 // evaluation's GEMM is done with the buffer, so the copy overlaps the head,
 // the caller's row work and the next evaluation's input layer.
 // Starts and ends with the CTA synchronised.
-template <int W, int RJ>
+template <int W, int RJ, int PARTS>
 __device__ void eval_qubit(const NadeView& m, int i, int kx, int a, const uint64_t* xt, const TileSmem& S,
                            float2* z3out, int& staged, bool& pending, int next) {
-  using T = Tile<W, RJ>;
+  using T = Tile<W, RJ, PARTS>;
   constexpr int TR = T::TR, WS = T::WS, HS = T::HS, NTX = T::NTX;
   const int tid = threadIdx.x;
   const QubitPtr q = qubit_ptrs(m, i);
@@ -270,10 +271,13 @@ __device__ void eval_qubit(const NadeView& m, int i, int kx, int a, const uint64
   {  // head: z3[r][o] = b3[o] + sum_k W3[o][k] h2[r][k], the k range in KP parts
     constexpr int KL = W / T::KP;
     const int r = tid % TR, g = tid / TR, o = g & 1, part = g >> 1;
-    float2 z = make_float2(0.f, 0.f);
-    for (int k = part * KL; k < (part + 1) * KL; ++k)
-      cmac(z, __ldg(q.W3 + o * W + k), make_float2(S.Hr[k * HS + r], S.Hi[k * HS + r]));
-    S.Z3p[(part * TR + r) * 2 + o] = z;
+    if (part < T::KP) {
+      float2 z = make_float2(0.f, 0.f);
+#pragma unroll 8
+      for (int k = part * KL; k < (part + 1) * KL; ++k)
+        cmac(z, __ldg(q.W3 + o * W + k), make_float2(S.Hr[k * HS + r], S.Hi[k * HS + r]));
+      S.Z3p[(part * TR + r) * 2 + o] = z;
+    }
   }
   __syncthreads();
   if (tid < 2 * TR) {
@@ -344,15 +348,16 @@ struct FwdArgs {
   const uint8_t* js;        // SUFFIX: first differing slot of each connected row
   const uint32_t* perm;     // SUFFIX: connected rows in ascending js
   const uint32_t* offsets;  // SUFFIX: offsets[p] = rows with js < p
-  float2* T;                // SUFFIX: [row][n] path terms of the slots > js; NODES: [node]
+  float2* T;                // SUFFIX: [row][n] path terms of the slots > js; NODES: [2][stride] per qubit and node
+  uint64_t stride;
 };
 
-template <int W, int RJ, int MODE>
+template <int W, int RJ, int MODE, int PARTS>
 __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, FwdArgs A) {
   ANQS_PDL_ENTRY();
   constexpr int TR = Tile<W, RJ>::TR;
   extern __shared__ float2 dsm[];
-  const TileSmem S = tile_smem<W, RJ>(dsm);
+  const TileSmem S = tile_smem<W, RJ, PARTS>(dsm);
   __shared__ uint64_t xt[TR];
   __shared__ float la[TR], ph[TR], t0r[TR], t0i[TR];
   __shared__ int dead[TR], jr[TR];
@@ -361,13 +366,16 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
   int staged = -1;
   bool pending = false;
   if constexpr (MODE == MODE_NODES) {
-    // tiles of the levels 1..n in order; offsets[q] = first node of level q
+    // (tile, qubit) items, the tiles of the levels 1..n in order; offsets[q] =
+    // first node of level q.  The grid is even: a CTA serves one of the two
+    // qubits, and its W2 stays in shared memory within a level.
     __shared__ uint32_t off[2 * ANQS_MAX_ORB];
     if (tid <= n + 1) off[tid] = __ldcg(A.offsets + tid);
     __syncthreads();
     uint32_t first = 0;  // first tile of slot p's level
     int p = 0;
-    for (uint32_t tile = blockIdx.x;; tile += gridDim.x) {
+    for (uint32_t item = blockIdx.x;; item += gridDim.x) {
+      const uint32_t tile = item >> 1;
       uint32_t nt;
       while (p < n && tile >= first + (nt = (off[p + 2] - off[p + 1] + TR - 1) / TR)) {
         first += nt;
@@ -378,17 +386,15 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
       const bool valid = tid < TR && row < off[p + 2];
       if (tid < TR) xt[tid] = valid ? __ldcg(reinterpret_cast<const unsigned long long*>(A.x) + row) : 0ull;
       __syncthreads();
-      float tr[2] = {0.f, 0.f}, ti[2];
-      bool ok[2];
-      for (int e = 0; e < 2; ++e) {
-        const int i = 2 * p + e;
-        eval_qubit<W, RJ>(m, i, i, 0, xt, S, S.Z3, staged, pending, e == 0 ? i + 1 : -1);
-        if (valid) ok[e] = path_term(hv, i, xt[tid], S.Z3[tid * 2], S.Z3[tid * 2 + 1], tr[e], ti[e]);
+      const int i = 2 * p + int(item & 1u);
+      eval_qubit<W, RJ, PARTS>(m, i, i, 0, xt, S, S.Z3, staged, pending, -1);
+      if (valid) {
+        float tr = 0.f, ti;
+        const bool ok = path_term(hv, i, xt[tid], S.Z3[tid * 2], S.Z3[tid * 2 + 1], tr, ti);
+        A.T[(item & 1u) * A.stride + row] = make_float2(ok ? tr : -INFINITY, ti);
       }
-      if (valid) A.T[row] = make_float2(ok[1] ? (ok[0] ? tr[0] : -INFINITY) + tr[1] : -INFINITY, ti[0] + ti[1]);
       __syncthreads();
     }
-    if (pending) cp_async_wait_all();
     return;
   }
   const uint64_t rows = MODE == MODE_SUFFIX ? uint64_t(A.offsets[n - 1]) : A.rows.get();
@@ -411,7 +417,7 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
     __syncthreads();
     if (MODE == MODE_LOGPSI) {
       for (int i = 0; i < 2 * n; ++i) {
-        eval_qubit<W, RJ>(m, i, i, 0, xt, S, S.Z3, staged, pending, i + 1 < 2 * n ? i + 1 : -1);
+        eval_qubit<W, RJ, PARTS>(m, i, i, 0, xt, S, S.Z3, staged, pending, i + 1 < 2 * n ? i + 1 : -1);
         if (tid < TR) {
           float tr = 0.f, ti;
           if (path_term(hv, i, xt[tid], S.Z3[tid * 2], S.Z3[tid * 2 + 1], tr, ti)) la[tid] += tr;
@@ -430,7 +436,7 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
       // rows are in ascending j: the tile's first row has the smallest, and
       // every row needs the slots above its own j only
       for (int i = 2 * (jr[0] + 1); i < 2 * n; ++i) {
-        eval_qubit<W, RJ>(m, i, i, 0, xt, S, S.Z3, staged, pending, i + 1 < 2 * n ? i + 1 : -1);
+        eval_qubit<W, RJ, PARTS>(m, i, i, 0, xt, S, S.Z3, staged, pending, i + 1 < 2 * n ? i + 1 : -1);
         const int p = i >> 1;
         if (tid < TR && p > jr[tid]) {
           float tr = 0.f, ti;
@@ -451,7 +457,7 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
       cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
       const int e = int(blockIdx.y % 3);
       const int p = MODE == MODE_RAW ? int(blockIdx.y / 3) : A.p;
-      eval_qubit<W, RJ>(m, e == 0 ? 2 * p : 2 * p + 1, 2 * p, e == 2 ? 1 : 0, xt, S, S.Z3, staged, pending, -1);
+      eval_qubit<W, RJ, PARTS>(m, e == 0 ? 2 * p : 2 * p + 1, 2 * p, e == 2 ? 1 : 0, xt, S, S.Z3, staged, pending, -1);
       cl.sync();
       if (e == 0 && tid < TR && base + tid < rows) {
         const float2* const z[3] = {S.Z3, cl.map_shared_rank(S.Z3, cl.block_rank() + 1),
@@ -476,11 +482,11 @@ __global__ void __launch_bounds__(NT) nade_fwd_kernel(NadeView m, HamView hv, Fw
 template <int MODE>
 constexpr bool clustered() { return MODE == MODE_RAW || MODE == MODE_LOGITS; }
 
-template <int W, int RJ, int MODE>
+template <int W, int RJ, int MODE, int PARTS = 0>
 int fwd_launch(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t max_rows, int prof, cudaStream_t s) {
   constexpr int TR = Tile<W, RJ>::TR;
-  const size_t smem = Tile<W, RJ>::smem_bytes;
-  auto kern = nade_fwd_kernel<W, RJ, MODE>;
+  const size_t smem = Tile<W, RJ, PARTS>::smem_bytes;
+  auto kern = nade_fwd_kernel<W, RJ, MODE, PARTS>;
   ANQS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
   int occ = 0;
   ANQS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem));
@@ -489,7 +495,8 @@ int fwd_launch(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t 
   if (cap < 1) cap = 1;
   uint64_t blocks = (max_rows + TR - 1) / TR;
   if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
+  if (MODE == MODE_NODES) blocks &= ~1ull;  // (tile, qubit) items: see the kernel
+  if (blocks < 1) blocks = MODE == MODE_NODES ? 2 : 1;
   ProfScope ps(prof, s);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(blocks), unsigned(ny));
@@ -510,15 +517,19 @@ int fwd_launch(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t 
   return ANQS_OK;
 }
 
-// NODES: the register tile that the suffix launch over all `rows` connected
-// determinants would take (the head's partial sums, hence the terms' last
-// bits, depend on it)
+// NODES: the head's sums in the parts that the suffix launch over all `rows`
+// connected determinants would take (the terms' last bits depend on them).
+// Two items (qubits) per tile; small tiles while the large ones would number
+// fewer than two per SM (7 orbitals, 441 samples, width 64: 28 large tiles of
+// both qubits took 55 us).
 template <int W>
 int nodes_w(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t rows, uint64_t max_nodes, cudaStream_t s) {
-  const uint64_t big_tiles = (rows + Tile<W, 4>::TR - 1) / Tile<W, 4>::TR;
-  max_nodes += uint64_t(m.n) * Tile<W, 4>::TR;  // a level's last tile may be partial
-  if (big_tiles >= 152) return fwd_launch<W, 4, MODE_NODES>(m, hv, a, max_nodes, PROF_NADE_SUFFIX, s);
-  return fwd_launch<W, 1, MODE_NODES>(m, hv, a, max_nodes, PROF_NADE_SUFFIX, s);
+  constexpr int TR4 = Tile<W, 4>::TR, KP4 = Tile<W, 4>::KP;
+  const uint64_t big_tiles = (rows + TR4 - 1) / TR4;
+  const uint64_t items = 2 * (max_nodes + uint64_t(m.n) * TR4);  // rows of two qubits; a level's last tile may be partial
+  if (big_tiles < 152) return fwd_launch<W, 1, MODE_NODES>(m, hv, a, items, PROF_NADE_SUFFIX, s);
+  if (2 * max_nodes < 304 * TR4) return fwd_launch<W, 1, MODE_NODES, KP4>(m, hv, a, items, PROF_NADE_SUFFIX, s);
+  return fwd_launch<W, 4, MODE_NODES>(m, hv, a, items, PROF_NADE_SUFFIX, s);
 }
 
 int nodes(const NadeView& m, const HamView& hv, const FwdArgs& a, uint64_t rows, uint64_t max_nodes, cudaStream_t s) {
@@ -581,7 +592,7 @@ size_t plan_eloc(const anqs_ham* H, uint64_t n_x, Arena& A, NadeElocWs& w) {
 struct NadeNodeWs {
   UniqueWs u;
   float *la_x, *ph_x, *raw, *cache;
-  float2 *per, *T;  // per node, per determinant and slot
+  float2 *per, *T;  // per qubit and node, per determinant and slot
 };
 
 size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NadeNodeWs& w) {
@@ -591,7 +602,7 @@ size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NadeNodeWs& w) {
   w.ph_x = A.take<float>(n_x);
   w.raw = A.take<float>(n_x * n * 8);
   w.cache = A.take<float>(n_x * n * TC_CACHE_F);
-  w.per = A.take<float2>(w.u.max_nodes);
+  w.per = A.take<float2>(2 * w.u.max_nodes);
   w.T = A.take<float2>(w.u.max_leaves * n);
   return A.off;
 }
@@ -659,6 +670,7 @@ int run_eloc_nade(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Cou
     b.x = v.u.nodes.x;
     b.offsets = v.u.nodes.off;
     b.T = v.per;
+    b.stride = v.u.max_nodes;
     ANQS_TRY(nodes(M->nade, H->v, b, n_x.n * H->v.K, v.u.max_nodes, s));
     ANQS_TRY(launch_path_terms(H, v.u, v.per, v.T, s));
     AmpSrc amp{};
