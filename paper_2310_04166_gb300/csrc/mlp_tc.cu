@@ -1209,10 +1209,8 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
       sync_tiles();
     }
     if (!ok) break;
-    // ---- head (f32; each half its columns' part of the sums) and the adjoint of its 8 outputs ----
+    // ---- head (f32) and the adjoint of its 8 outputs ----
     float hl[HW], out[8];
-#pragma unroll
-    for (int o = 0; o < 8; ++o) out[o] = 0.f;
 #pragma unroll
     for (int c0 = 0; c0 < HW; c0 += 32) {
       float v[32];
@@ -1223,33 +1221,38 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
         for (int i = 0; i < 32; ++i) v[i] = 0.f;
       }
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int c = cb + c0 + i;
-        const float y = tc::tanh_fast(v[i] + bias[(L - 1) * W + c]);
-        const float4 w0 = head[c * 2], w1 = head[c * 2 + 1];
-        out[0] = fmaf(w0.x, y, out[0]);
-        out[1] = fmaf(w0.y, y, out[1]);
-        out[2] = fmaf(w0.z, y, out[2]);
-        out[3] = fmaf(w0.w, y, out[3]);
-        out[4] = fmaf(w1.x, y, out[4]);
-        out[5] = fmaf(w1.y, y, out[5]);
-        out[6] = fmaf(w1.z, y, out[6]);
-        out[7] = fmaf(w1.w, y, out[7]);
-        hl[c0 + i] = y;
-      }
+      for (int i = 0; i < 32; ++i) hl[c0 + i] = tc::tanh_fast(v[i] + bias[(L - 1) * W + cb + c0 + i]);
     }
-    {
-      float4* xo = reinterpret_cast<float4*>(P1) + (h * MT + t) * 2;
-      xo[0] = make_float4(out[0], out[1], out[2], out[3]);
-      xo[1] = make_float4(out[4], out[5], out[6], out[7]);
-      __syncthreads();
-      const float4* xi = reinterpret_cast<const float4*>(P1) + ((1 - h) * MT + t) * 2;
-      const float4 q0 = xi[0], q1 = xi[1];
-      const float other[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+    // The second half goes on with the first one's sums, so that they have one
+    // order: dout and dz are rounded to fp16, and a last bit of the outputs
+    // that differs moves a row's whole contribution by up to 2^-11.  The logits
+    // first: while the second half adds to them, the first one does the phases.
+    float4* xo = reinterpret_cast<float4*>(P1) + t * 4;  // logits and phases of the first half, then of both
+    auto head_sums = [&](int q, const float4 from) {
+      float4 r = from;
 #pragma unroll
-      for (int o = 0; o < 8; ++o) out[o] = out[o] + other[o] + hbias[o];
-      __syncthreads();  // P1 takes h_L next
+      for (int i = 0; i < HW; ++i) {
+        const float4 w = head[(cb + i) * 2 + q];
+        r.x = fmaf(w.x, hl[i], r.x), r.y = fmaf(w.y, hl[i], r.y), r.z = fmaf(w.z, hl[i], r.z), r.w = fmaf(w.w, hl[i], r.w);
+      }
+      xo[2 * h + q] = r;
+    };
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (h == 0) head_sums(0, zero);
+    __syncthreads();
+    if (h == 0) head_sums(1, zero);
+    else head_sums(0, xo[0]);
+    __syncthreads();
+    if (h == 1) head_sums(1, xo[1]);
+    __syncthreads();
+    {
+      const float4 q0 = xo[2], q1 = xo[3];
+      out[0] = q0.x, out[1] = q0.y, out[2] = q0.z, out[3] = q0.w;
+      out[4] = q1.x, out[5] = q1.y, out[6] = q1.z, out[7] = q1.w;
     }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) out[o] += hbias[o];
+    __syncthreads();  // P1 takes h_L next
     float dout[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     // d l_u = cot_la 1/2 (delta_uv - p~_u) over the allowed u; d phi_u = cot_ph delta_uv
     if (valid) {
