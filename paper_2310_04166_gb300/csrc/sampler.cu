@@ -1222,7 +1222,7 @@ int run_sampler(const anqs_model* M, const anqs_ham* H, uint64_t n_samples, uint
     if (small) {
       const uint64_t blocks = ((n_samples + 3) / 4 + Fp + SMALL_T - 1) / SMALL_T;
       ANQS_CUDA(cudaFuncSetAttribute(draw_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMALL_DYN)));
-      ANQS_CUDA_LAUNCH("sampler draw_small_kernel", launch_k(draw_small_kernel, dim3(blocks_for(blocks, 1, 152)), dim3(SMALL_T), SMALL_DYN, s, H->v, p, seed, counter, counter_dev, P.pre[cur], P.cnt[cur], nf, table ? P.plog : P.logits, P.child, P.done, last ? x_out : P.pre[nxt], last ? n_out : P.cnt[nxt], last ? n_unique : P.n_front + nxt, table ? P.idx[cur] : nullptr, table && !last ? P.idx[nxt] : nullptr, H->d_pt_child, (table && p > 0) ? 0 : 1));
+      ANQS_CUDA_LAUNCH("sampler draw_small_kernel", launch_k(draw_small_kernel, dim3(blocks_for(blocks, 1, 152 * 6)), dim3(SMALL_T), SMALL_DYN, s, H->v, p, seed, counter, counter_dev, P.pre[cur], P.cnt[cur], nf, table ? P.plog : P.logits, P.child, P.done, last ? x_out : P.pre[nxt], last ? n_out : P.cnt[nxt], last ? n_unique : P.n_front + nxt, table ? P.idx[cur] : nullptr, table && !last ? P.idx[nxt] : nullptr, H->d_pt_child, (table && p > 0) ? 0 : 1));
       continue;
     }
     ANQS_CUDA_LAUNCH("sampler prep_kernel", launch_k(prep_kernel, dim3(blocks_for(Fp, 256, 152 * 8)), dim3(256), 0, s, H->v, p, P.pre[cur], P.cnt[cur], nf, P.logits, P.thr, P.allowed, P.nblk, P.child));
