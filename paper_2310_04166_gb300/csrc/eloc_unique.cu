@@ -241,20 +241,28 @@ __global__ void __launch_bounds__(CT) emit_kernel(SectorView sv, int levels, con
       if (w + 1 == words) off[levels] = id + c;
       i0 = (w - sv.woff[p]) * 32u;
     }
-    // the warp's words one after the other, a lane per bit: the lookups of one
-    // word are in flight together and its nodes are written side by side
-    uint32_t some = __ballot_sync(0xffffffffu, v != 0u);
-    while (some) {
-      const int q = __ffs(some) - 1;
-      some &= some - 1u;
-      const uint32_t vq = __shfl_sync(0xffffffffu, v, q), idq = __shfl_sync(0xffffffffu, id, q),
-                     idx = __shfl_sync(0xffffffffu, i0, q) + uint32_t(lane);
-      const int pq = __shfl_sync(0xffffffffu, p, q);
-      if ((vq >> lane) & 1u) {
+    // the warp's words, a lane per bit, four words' lookups in flight (one word
+    // at a time waited for its two loads 32 times: 14 us for any sector); a
+    // word's nodes are written side by side
+    const uint32_t some = __ballot_sync(0xffffffffu, v != 0u);
+#pragma unroll 1
+    for (int q0 = 0; q0 < 32; q0 += 4) {
+      if (!((some >> q0) & 15u)) continue;
+      uint32_t sa[4], sb[4], at[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint32_t vq = __shfl_sync(0xffffffffu, v, q0 + e), idq = __shfl_sync(0xffffffffu, id, q0 + e),
+                       idx = __shfl_sync(0xffffffffu, i0, q0 + e) + uint32_t(lane);
+        const int pq = __shfl_sync(0xffffffffu, p, q0 + e);
+        const bool on = (vq >> lane) & 1u;
         const uint32_t nb = sv.nb_p[pq], ra = idx / nb, rb = idx - ra * nb;
-        node_x[idq + __popc(vq & ((1u << lane) - 1u))] =
-            spread_bits(__ldg(sv.sta + sv.soa[pq] + ra)) | spread_bits(__ldg(sv.stb + sv.sob[pq] + rb)) << 1;
+        sa[e] = on ? __ldg(sv.sta + sv.soa[pq] + ra) : 0u;
+        sb[e] = on ? __ldg(sv.stb + sv.sob[pq] + rb) : 0u;
+        at[e] = on ? idq + __popc(vq & ((1u << lane) - 1u)) : 0xffffffffu;
       }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (at[e] != 0xffffffffu) node_x[at[e]] = spread_bits(sa[e]) | spread_bits(sb[e]) << 1;
     }
     base += total;
     __syncthreads();
