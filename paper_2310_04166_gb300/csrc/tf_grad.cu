@@ -64,7 +64,9 @@ __global__ void tree_rows_kernel(SectorView sv, NodeView nv, uint8_t* __restrict
   }
 }
 
-constexpr int BM = 64, BN = 64, BK = 16, GT = 128;
+constexpr int BM = 64, BN = 64, BK = 32, GT = 128;
+constexpr int LV = BM * BK / 4 / GT;  // 4-vectors of A, and of B, that a thread loads per K step
+static_assert(BM == BN, "one index for both operands");
 
 // A matrix whose rows come in segments (the q, k and v weights lie one
 // behind the other with their biases between): row i starts at
@@ -125,7 +127,8 @@ struct GmSmem {
 // per CTA of 128 threads, 8 x 4 per thread (3 16-byte shared loads for 32
 // FMAs, paired along the rows; a 4 x 4 tile is bound by its shared loads), the
 // next K step's operands loaded to registers while this one runs.  A CTA waits
-// for those loads in every step, so what counts is how many share an SM: with
+// for those loads in every step (so the steps are 32 deep), and what counts is
+// how many share an SM: with
 // 128 x 64 tiles the 26,000 rows of the 20-qubit workload were 205 CTAs of a
 // 64-column product, and half of every tile of a 64-row weight product empty.
 // All leading dimensions, segments and widths are multiples of 4 floats.
@@ -139,12 +142,11 @@ __device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by,
   if (k_lo >= K && !(k_lo == 0)) return;
   const uint64_t k_hi = k_lo + g.k_chunk < K ? k_lo + g.k_chunk : K;
   const int tx = tid % 16, ty = tid / 16;
-  float4 ra[2], rb[2];
+  float4 ra[LV], rb[LV];
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  // A: 64 x 16 elements, B: 16 x 64: two 4-vectors per thread each
   auto load = [&](uint64_t k0) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < LV; ++i) {
       const int e = tid + GT * i;
       ra[i] = rb[i] = zero;
       if (TA) {  // [k][m]: vectors along m
@@ -159,7 +161,7 @@ __device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by,
           }
         }
       } else {  // [m][k]: vectors along k
-        const uint64_t m = m0 + e / 4, k = k0 + uint64_t(e % 4) * 4;
+        const uint64_t m = m0 + e / (BK / 4), k = k0 + uint64_t(e % (BK / 4)) * 4;
         if (m < M && k + 4 <= k_hi) ra[i] = *reinterpret_cast<const float4*>(g.A + m * g.lda + k);
       }
       if (g.relu_a) {
@@ -167,8 +169,8 @@ __device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by,
         ra[i].z = fmaxf(ra[i].z, 0.f), ra[i].w = fmaxf(ra[i].w, 0.f);
       }
       if (TB) {  // [n][k]: vectors along k
-        const int n = n0 + e / 4;
-        const uint64_t k = k0 + uint64_t(e % 4) * 4;
+        const int n = n0 + e / (BK / 4);
+        const uint64_t k = k0 + uint64_t(e % (BK / 4)) * 4;
         if (n < g.N && k + 4 <= k_hi) rb[i] = ld4(g.B + seg_row(g.sb, n, g.ldb) + k, g.b_vec);
       } else {  // [k][n]: vectors along n
         const int n = n0 + (e % 16) * 4;
@@ -183,8 +185,8 @@ __device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by,
   };
   auto store = [&](int b) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int e = tid + GT * i, r = e / 4, k = (e % 4) * 4;
+    for (int i = 0; i < LV; ++i) {
+      const int e = tid + GT * i, r = e / (BK / 4), k = (e % (BK / 4)) * 4;
       if (TA) *reinterpret_cast<float4*>(&sm.A[b][e / 16][(e % 16) * 4]) = ra[i];
       else sm.A[b][k][r] = ra[i].x, sm.A[b][k + 1][r] = ra[i].y, sm.A[b][k + 2][r] = ra[i].z, sm.A[b][k + 3][r] = ra[i].w;
       if (TB) sm.B[b][k][r] = rb[i].x, sm.B[b][k + 1][r] = rb[i].y, sm.B[b][k + 2][r] = rb[i].z, sm.B[b][k + 3][r] = rb[i].w;
@@ -258,7 +260,7 @@ __device__ __forceinline__ void gemm_tile(const Gm& g, unsigned bx, unsigned by,
 }
 
 // one product with a transposed B (the forward pass)
-__global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
+__global__ void __launch_bounds__(GT, 4) sgemm_kernel(Gm g) {
   ANQS_PDL_ENTRY();
   __shared__ __align__(16) GmSmem sm;
   gemm_tile<false, true>(g, blockIdx.x, blockIdx.y, 0, sm);
@@ -269,7 +271,7 @@ __global__ void __launch_bounds__(GT) sgemm_kernel(Gm g) {
 // the weight gradient w += dY^T X (CTAs below nw: wx tiles wide, wy high, parts
 // of the rows).  In one launch, because neither fills the GPU by itself; the
 // weight product's CTAs run longest and come first.
-__global__ void __launch_bounds__(GT) sgemm_bwd_kernel(Gm w, Gm d, unsigned nw, unsigned wx, unsigned wy, unsigned dx) {
+__global__ void __launch_bounds__(GT, 4) sgemm_bwd_kernel(Gm w, Gm d, unsigned nw, unsigned wx, unsigned wy, unsigned dx) {
   ANQS_PDL_ENTRY();
   __shared__ __align__(16) GmSmem sm;
   if (blockIdx.x < nw) {
@@ -603,9 +605,9 @@ __global__ void attn_bwd_kv_kernel(const float* __restrict__ qkv, const float* _
   __syncthreads();
   for (int col = threadIdx.x; col < 2 * D; col += blockDim.x) {
     const int kv = col / D, c = col - kv * D, hd = c / dh;
-    const float* w = (kv ? P : dS) + hd * n + u;
-    const float* v = kv ? dO + c : qkv + c;
-    const size_t ldv = kv ? D : 3 * size_t(D);
+    const int ldw = H * n, ldv = kv ? D : 3 * D;
+    const float* w = (kv ? P : dS) + hd * n + u + r0 * ldw;
+    const float* v = (kv ? dO + c : qkv + c) + r0 * ldv;
     uint32_t cur = 0xffffffffu;
     float acc = 0.f;
     for (int i0 = 0; i0 < int(r1 - r0); i0 += 8) {  // eight rows' loads in flight (rows beyond have no key)
@@ -613,8 +615,8 @@ __global__ void attn_bwd_kv_kernel(const float* __restrict__ qkv, const float* _
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const bool on = key[i0 + e] != 0xffffffffu;
-        wr[e] = on ? w[(r0 + i0 + e) * H * n] : 0.f;
-        vr[e] = on ? v[(r0 + i0 + e) * ldv] : 0.f;
+        wr[e] = on ? w[e * ldw] : 0.f;
+        vr[e] = on ? v[e * ldv] : 0.f;
       }
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -626,6 +628,8 @@ __global__ void attn_bwd_kv_kernel(const float* __restrict__ qkv, const float* _
         }
         if (k != 0xffffffffu) acc = fmaf(wr[e], vr[e], acc);
       }
+      w += 8 * ldw;
+      v += 8 * ldv;
     }
     if (cur != 0xffffffffu) atomicAdd(dqkv + size_t(cur) * 3 * D + (1 + kv) * D + c, acc);
   }
