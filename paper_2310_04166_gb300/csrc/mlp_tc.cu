@@ -207,6 +207,17 @@ __device__ __forceinline__ bool wg_all(int wg, bool v) {
   return r != 0;
 }
 
+// Columns k..k+7 (k a multiple of 8) of the one-hot input of v_<p as fp16: a
+// slot's four columns are 1.0 shifted to its outcome.  (Comparing every column
+// with its slot's outcome took as many integer instructions as a hidden layer's
+// whole epilogue.)
+__device__ __forceinline__ uint4 onehot8(uint64_t x, int p, uint32_t k) {
+  const uint32_t q = k >> 2, v = uint32_t(x >> (2 * q));
+  const uint64_t a = q < uint32_t(p) ? 0x3C00ull << (16u * (v & 3u)) : 0ull,
+                 b = q + 1u < uint32_t(p) ? 0x3C00ull << (16u * ((v >> 2) & 3u)) : 0ull;
+  return make_uint4(uint32_t(a), uint32_t(a >> 32), uint32_t(b), uint32_t(b >> 32));
+}
+
 // All layers of slot p for the 128 rows of one tile (one warpgroup; row t =
 // thread t).  Returns false if a wait timed out.
 template <int W>
@@ -216,16 +227,7 @@ __device__ bool tile_slot(const Ctx& c, uint32_t& ph_m, int p, uint64_t x, const
   const int L = c.tv->L;
   // layer-1 input: one-hot of v_<p (K = k1 columns)
   for (uint32_t k = 0; k < S.k1; k += 8) {
-    uint32_t w4[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      uint32_t lo = 0, hi = 0;
-      const uint32_t k0 = k + 2 * e, k1 = k0 + 1;
-      if (k0 < 4u * p && ((x >> (2 * (k0 >> 2))) & 3ull) == (k0 & 3u)) lo = 0x3C00u;  // fp16 1.0
-      if (k1 < 4u * p && ((x >> (2 * (k1 >> 2))) & 3ull) == (k1 & 3u)) hi = 0x3C00u;
-      w4[e] = lo | (hi << 16);
-    }
-    *reinterpret_cast<uint4*>(c.s_a + tc::canon_off(c.t, k, S.k1)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    *reinterpret_cast<uint4*>(c.s_a + tc::canon_off(c.t, k, S.k1)) = onehot8(x, p, k);
   }
   tc::fence_async_smem();
   tc::fence_before_sync();
@@ -1156,16 +1158,7 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
     const uint32_t acc = in_tmem ? 1u : 0u;
     // one-hot input of v_<p (layer 1's A operand and dW_1's B operand)
     for (uint32_t k = 8u * h; k < k1; k += 16) {
-      uint32_t w4[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t lo = 0, hi = 0;
-        const uint32_t k0 = k + 2 * e, kk = k0 + 1;
-        if (k0 < 4u * p && ((x >> (2 * (k0 >> 2))) & 3ull) == (k0 & 3u)) lo = 0x3C00u;
-        if (kk < 4u * p && ((x >> (2 * (kk >> 2))) & 3ull) == (kk & 3u)) hi = 0x3C00u;
-        w4[e] = lo | (hi << 16);
-      }
-      *reinterpret_cast<uint4*>(U + tc::canon_off(t, k, k1)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+      *reinterpret_cast<uint4*>(U + tc::canon_off(t, k, k1)) = onehot8(x, p, k);
     }
     sync_tiles();
     // ---- forward: h_1 .. h_{L-1} to their tiles, z_L left in TMEM ----
