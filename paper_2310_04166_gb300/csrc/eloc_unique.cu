@@ -1,7 +1,7 @@
 // Local energies over the distinct connected determinants of a sample set.
 //
 // The connected sets of different samples overlap: 10,816 samples of the
-// 20-qubit workload have 1.1e7 connected determinants, but the sector holds
+// 20-qubit workload have 6.6e6 connected determinants, but the sector holds
 // 14,400.  So the amplitudes are evaluated once per distinct determinant (for
 // the slot networks once per distinct prefix) and the local energies look
 // them up.  The steps of a call:
@@ -63,7 +63,7 @@ __device__ __forceinline__ void mark_det(const HamView& hv, const SectorView& sv
 // Whether a call's connected determinants outnumber the sector's so far that
 // all its prefixes are taken as marked: hardly any is left out then, and one
 // word is written per 32 determinants instead of an atomic or a load per
-// connected one (1.1e7 of a 14,400-determinant sector: 126 us).  From the
+// connected one (6.6e6 of a 14,400-determinant sector: 126 us).  From the
 // device's count: a buffer may hold fewer samples than it has room for.
 // Not with Z2 symmetries, where the index also holds other sectors' prefixes.
 __device__ __forceinline__ bool covers_sector(const HamView& hv, const SectorView& sv, uint64_t n_x) {
