@@ -956,7 +956,7 @@ struct GradArgs {
   const uint64_t* xs;
   Count n_x;
   CotSrc cot;
-  float* part;  // [tiles][n_params]
+  float* part;  // [slabs][n_params], a slab per CTA of a slot
   uint64_t n_params;
   uint32_t img_bytes, kmax1;  // image region (without W1's lo part), widest layer-1 input
   const float* maxes;  // [kMaxes] maxima of the cotangents' magnitudes, or null: each CTA has one tile, its own scale
@@ -1012,8 +1012,8 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   constexpr int HW = W / 2;  // columns per half
   const int h = threadIdx.x / MT, t = threadIdx.x % MT, warp = t >> 5, lane = t & 31;
   const int p = blockIdx.y, L = a.m.n_hidden;
-  // TMEM columns: data accumulator | dW_L..dW_2 | dW_1 (64) | dW_h (16) | db_1..db_L (16 each)
-  const uint32_t C_ACC = 0, C_DW1 = uint32_t(L) * W, C_DWH = C_DW1 + 64, C_DB = C_DWH + 16;
+  // TMEM columns (grad_tmem_cols): data accumulator | dW_L..dW_2 | dW_1 (kmax1) | dW_h (16) | db_1..db_L (16 each)
+  const uint32_t C_ACC = 0, C_DW1 = uint32_t(L) * W, C_DWH = C_DW1 + a.kmax1, C_DB = C_DWH + 16;
   constexpr uint32_t NCOL = 512;
   const SlotLayout S = slot_layout(p, W, L, a.tv.lo);
   const uint32_t k1 = S.k1, lo_bytes = S.wk - S.w1lo;
@@ -2020,6 +2020,11 @@ int run_eloc_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count
   return eloc_tc_post(H, x, n_x, ere, eim, counts, stats, ws, ws_bytes, s);
 }
 
+// Tensor-memory columns of the adjoint at width 128: dW_1 takes what its widest
+// layer-1 input needs, so that three hidden layers reach 17 orbitals (shared
+// memory ends before that) and one or two all 32.
+static uint32_t grad_tmem_cols(int L, uint32_t k1) { return uint32_t(L) * 128u + k1 + 16u + 16u * uint32_t(L); }
+
 // Shared memory of the tensor-core adjoint of model M (0 when it does not
 // apply: width other than 128, more than 3 hidden layers, or too large).
 static size_t tc_grad_smem(const anqs_model* M, uint32_t* img_bytes, uint32_t* kmax1) {
@@ -2037,7 +2042,7 @@ static size_t tc_grad_smem(const anqs_model* M, uint32_t* img_bytes, uint32_t* k
   if (kmax1) *kmax1 = k1;
   const size_t tile = size_t(MT) * W * 2;
   const size_t sm = size_t(img) + size_t(L - 1) * tile + 2 * tile + size_t(MT) * k1 * 2 + size_t(MT) * 16 * 2;
-  return sm <= kSmemLimit && k1 <= 64 ? sm : 0;  // (dW_1 has 64 tensor-memory columns)
+  return sm <= kSmemLimit && grad_tmem_cols(L, k1) <= 512 ? sm : 0;
 }
 
 bool mlp_tc_grad_supported(const anqs_model* M) { return tc_grad_smem(M, nullptr, nullptr) > 0; }

@@ -155,3 +155,59 @@ def test_tensor_core_adjoint_directly_after_a_repack(A):
     torch.cuda.synchronize()
     assert model.status() == 0
     assert torch.equal(g1, g2)
+
+
+def _adjoint_problem(A, n, na, nb, hidden, m, seed, width=128, form="bf16"):
+    """A 16-bit MLP, m random determinants of the sector and random local energies."""
+    from synthetic import flatten_mlp, integrals, mlp_params
+    h, g, e = integrals(seed, n, 2)
+    ham = A.Hamiltonian(h, g, e, na, nb)
+    P = mlp_params(seed, n, width, hidden, 0.2)
+    model = A.Model.mlp(n, width, hidden, torch.tensor(flatten_mlp(P), device="cuda"), form)
+    rng = np.random.default_rng(seed)
+    occ = lambda k: (np.argsort(rng.random((m, n)), axis=1)[:, :k]).astype(np.uint64)
+    x = (np.uint64(1) << (np.uint64(2) * occ(na))).sum(1, dtype=np.uint64)
+    x = x + (np.uint64(2) << (np.uint64(2) * occ(nb))).sum(1, dtype=np.uint64)
+    return ham, P, model, x, rng
+
+
+def _grad_and_kernels(A, model, ham, x, cnt, e, stats):
+    """The gradient, and how often the tensor-core adjoint's kernel ran."""
+    import ctypes as C
+    from paper_2310_04166_gb300 import _lib
+    lib = _lib.load()
+    t = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")
+    _lib.check(lib.anqs_profile_enable(1))
+    g = A.grad(model, ham, t(x.astype(np.int64)), t(cnt.astype(np.int64)), t(e.real), t(e.imag), t(stats))
+    torch.cuda.synchronize()
+    ran, k = {}, 0
+    while True:
+        name, c, ms = C.c_char_p(), C.c_uint64(), C.c_double()
+        if lib.anqs_profile_read(k, C.byref(name), C.byref(c), C.byref(ms)) != 0:
+            break
+        ran[name.value.decode()] = c.value
+        k += 1
+    _lib.check(lib.anqs_profile_enable(0))
+    return g.cpu().numpy().astype(np.float64), ran["mlp_tc_grad_kernel"]
+
+
+def _adjoint_reference(P, n, na, nb, x, cnt, e, stats):
+    """The FP64 oracle's gradient for given local energies and statistics."""
+    g = gradient(MLPAnsatz(P, n), molecular_isphys(n, na, nb), x, cnt, e, stats)
+    return np.concatenate([t.reshape(-1).numpy() for t in g])
+
+
+@pytest.mark.parametrize("n,na,nb", [(17, 3, 2), (18, 3, 3), (26, 2, 3), (32, 2, 1)])
+@pytest.mark.parametrize("hidden", [1, 2])
+def test_tensor_core_adjoint_of_wide_inputs(A, n, na, nb, hidden):
+    """Layer-1 inputs of 64 to 128 columns (17 to 32 orbitals) run on the
+    tensor cores with one and two hidden layers, two tiles, the last one
+    partial; the module's bar."""
+    ham, P, model, x, rng = _adjoint_problem(A, n, na, nb, hidden, 200, 11 * n + hidden)
+    cnt = rng.integers(1, 50, size=x.size)
+    e = rng.normal(size=x.size) + 1j * rng.normal(size=x.size)
+    stats = energy_stats(e, cnt)
+    g, ran = _grad_and_kernels(A, model, ham, x, cnt, e, stats)
+    ref = _adjoint_reference(P, n, na, nb, x, cnt, e, stats)
+    assert ran == 1 and model.status() == 0
+    assert np.linalg.norm(g - ref) < BAR * np.linalg.norm(ref)
