@@ -916,13 +916,19 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_multi_kernel(const __grid_consta
 // read the forward weight image as an MN-major B operand: no transposed copy
 // of anything is made.  Biases' gradients are the column sums of the dz
 // tiles, one more small MMA per layer against the dout tile, whose column 8
-// holds ones.  Operands are fp16; the cotangents are scaled by a power of two
-// that puts their largest magnitude at 2^8 (the gradient is linear in them;
-// the scale is divided out, exactly, when the sums are written).
+// holds ones.  Operands are fp16; each tile's cotangents are scaled by a power
+// of two that puts their largest magnitude at 2^8 (the gradient is linear in
+// them; the scale is divided out, exactly, when the sums are written).  One
+// scale for the whole sample set would put the cotangents of rows with 1e-5 of
+// the largest weight into fp16's subnormals, and with them the gradients of the
+// parameters that only such rows reach.
 //
 // The weight gradients stay in tensor memory over kFlush tiles, so a CTA
 // writes its slot's block of partial gradients (f32, one slab per g) once per
 // kFlush tiles instead of once per tile; a reduction over the slabs follows.
+// Where a tile's scale is another than the sums', these are multiplied by the
+// quotient, a power of two, while the first layer's MMAs run (24 qubits, 20,000
+// samples: 200 us, 185 with one scale, 334 with a slab per tile).
 // One tile is a serial chain of MMA, wait and epilogue; what a tile cost
 // beyond it before was reading and writing its 150 KB of partial gradients,
 // fetching its 84 KB of weights and 128 instead of 256 threads in each
@@ -959,34 +965,11 @@ struct GradArgs {
   float* part;  // [slabs][n_params], a slab per CTA of a slot
   uint64_t n_params;
   uint32_t img_bytes, kmax1;  // image region (without W1's lo part), widest layer-1 input
-  const float* maxes;  // [kMaxes] maxima of the cotangents' magnitudes, or null: each CTA has one tile, its own scale
 };
-constexpr int kMaxes = 152;
-constexpr uint32_t kFlush = 16;  // 128 MMAs in a row onto one accumulator
-
-// Cotangents to arrays (cl, cp) and the maximum of their magnitudes per CTA
-__global__ void __launch_bounds__(256) cot_max_kernel(CotSrc cot, Count n_x_, float* cl, float* cp, float* maxes) {
-  ANQS_PDL_ENTRY();
-  __shared__ float s_max[8];
-  const uint64_t n_x = n_x_.get();
-  float mx = 0.f;
-  for (uint64_t l = blockIdx.x * 256ull + threadIdx.x; l < n_x; l += gridDim.x * 256ull) {
-    float a, b;
-    cot_of(cot, l, a, b);
-    if (cot.stats) {
-      cl[l] = a;
-      cp[l] = b;
-    }
-    mx = fmaxf(mx, fmaxf(fabsf(a), fabsf(b)));
-  }
-  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, s_max[w]);
-    maxes[blockIdx.x] = mx;
-  }
-}
+// 128 MMAs in a row onto one accumulator: 2e-6 of the gradient (24 qubits,
+// 20,000 samples, against the FP64 sum of one-tile calls), where the rounding of
+// the operands takes 5e-4
+constexpr uint32_t kFlush = 16;
 
 // MN-major view of a tile stored per row in the canonical K-major layout with
 // `cols` columns: the MMA's K runs over the rows (16 per step), M or N over
@@ -1069,22 +1052,19 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   const uint32_t img_a = tc::smem_u32(img);
   const bool kL = (L == 1 ? k1 : uint32_t(W)) > 0;  // z_L is in TMEM (else it is zero)
   const int cb = h * HW;
+  int e_sum = 0;  // the sums are scaled by 2^e_sum
   float sc = 1.f, inv_sc = 1.f, bh[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  // scale from the largest magnitude of mx over the CTA: largest magnitude -> 2^8
-  auto set_scale = [&](float mx) {
+  // exponent that takes the largest magnitude of mx over the CTA to 2^8 (`none` if all are zero)
+  auto scale_exponent = [&](float mx, int none) -> int {
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) s_max[threadIdx.x >> 5] = mx;
     __syncthreads();
     for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_max[w]);
-    int e2 = 0;
-    if (mx > 0.f) {
-      frexpf(mx, &e2);  // mx in [2^(e2-1), 2^e2)
-      e2 = 8 - e2;
-    }
-    sc = ldexpf(1.f, e2);
-    inv_sc = ldexpf(1.f, -e2);
+    if (!(mx > 0.f)) return none;
+    int e2;
+    frexpf(mx, &e2);  // mx in [2^(e2-1), 2^e2)
+    return min(8 - e2, 120);
   };
-  if (a.maxes) set_scale(threadIdx.x < kMaxes ? __ldcg(a.maxes + threadIdx.x) : 0.f);
 
   // The sums of the last tiles to the slab (the first flush of a CTA writes
   // it, later ones add): 32 columns at a time through shared memory, so that
@@ -1154,8 +1134,30 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
     const uint64_t x = valid ? a.xs[row] : 0ull;
     float cla = 0.f, cph = 0.f;
     if (valid) cot_of(a.cot, row, cla, cph);
-    if (!a.maxes) set_scale(fmaxf(fabsf(cla), fabsf(cph)));
+    const int e2 = scale_exponent(fmaxf(fabsf(cla), fabsf(cph)), e_sum);
+    if (in_tmem && abs(e2 - e_sum) > 64) {  // beyond what the sums can follow exactly
+      flush();
+      in_tmem = 0;
+    }
+    const float follow = in_tmem ? ldexpf(1.f, e2 - e_sum) : 1.f;
+    e_sum = e2;
+    sc = ldexpf(1.f, e2);
+    inv_sc = ldexpf(1.f, -e2);
     const uint32_t acc = in_tmem ? 1u : 0u;
+    // the sums to this tile's scale; every MMA on them is done, and the next ones come after a barrier
+    auto rescale = [&]() {
+      __syncwarp();
+      for (uint32_t c0 = W + 32u * h; c0 < C_DB + 16u * L; c0 += 64) {
+        float v[32];
+        tc::tmem_ld32(tm + lb + c0, v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] *= follow;
+        tc::tmem_st32(tm + lb + c0, v);
+      }
+      tc::tmem_st_wait();
+#pragma unroll
+      for (int o = 0; o < 8; ++o) bh[o] *= follow;
+    };
     // one-hot input of v_<p (layer 1's A operand and dW_1's B operand)
     for (uint32_t k = 8u * h; k < k1; k += 16) {
       *reinterpret_cast<uint4*>(U + tc::canon_off(t, k, k1)) = onehot8(x, p, k);
@@ -1174,8 +1176,9 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
                         tc::sdesc(b_addr + ks * 256u, 128u, K * 16u), tc::idesc_f16_f32(MT, W), ks > 0 ? 1u : 0u);
           tc::mma_commit(bar_m);
         }
-        ok = mma_wait();
       }
+      if (layer == 0 && follow != 1.f) rescale();
+      if (K > 0) ok = mma_wait();
       if (!ok || layer == L - 1) break;
       unsigned char* dst = Hb + uint32_t(layer) * TILE;
 #pragma unroll
@@ -2068,12 +2071,9 @@ int launch_mlp_tc_grad(const anqs_model* M, const HamView& hv, const uint64_t* x
   if (tiles > 0x7fffffffull) return set_error(ANQS_ERR_UNSUPPORTED, "too many rows");
   // one CTA per SM over all slots
   const unsigned slabs = unsigned(std::min<uint64_t>(tiles, std::max<uint64_t>(1, uint64_t(num_sms()) / uint64_t(M->d.n_orb))));
-  if (tiles > slabs) {  // several tiles per CTA: one scale for all; `part` holds at least one slab per tile
-    float* maxes = part + uint64_t(slabs) * a.n_params;
-    ProfScope ps(PROF_COTANGENT, s);
-    ANQS_CUDA_LAUNCH("cot_max_kernel", launch_k(cot_max_kernel, dim3(kMaxes), dim3(256), 0, s, cot, n_x, cl, cp, maxes));
-    a.maxes = maxes;
-    if (cot.stats) a.cot = CotSrc{cl, cp, nullptr, nullptr, nullptr, nullptr};
+  if (tiles > slabs && cot.stats) {  // FP64 divisions once per row instead of once per row and slot
+    ANQS_TRY(launch_grad_cotangents(cot.ere, cot.eim, cot.counts, cot.stats, n_x, cl, cp, s));
+    a.cot = CotSrc{cl, cp, nullptr, nullptr, nullptr, nullptr};
   }
   ANQS_CUDA(cudaFuncSetAttribute(mlp_tc_grad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
   {

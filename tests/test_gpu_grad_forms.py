@@ -211,3 +211,73 @@ def test_tensor_core_adjoint_of_wide_inputs(A, n, na, nb, hidden):
     ref = _adjoint_reference(P, n, na, nb, x, cnt, e, stats)
     assert ran == 1 and model.status() == 0
     assert np.linalg.norm(g - ref) < BAR * np.linalg.norm(ref)
+
+
+def _tensors(x, cnt, e):
+    t = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")
+    return t(x.astype(np.int64)), t(cnt.astype(np.int64)), t(e.real), t(e.imag)
+
+
+@pytest.mark.parametrize("hidden", [2, 3])
+def test_tensor_core_adjoint_keeps_small_rows_beside_a_large_one(A, hidden):
+    """One sample holds nearly all draws (1e7 of them, alone in its tile), 29
+    tiles of samples drawn once follow, several tiles per CTA.  The columns of
+    W_1 of outcomes that the large sample does not take get their gradient
+    from the others alone: as without it, up to the order of float32 sums
+    (3,712 rows: some 1e-6 of a column block's norm; the bar is 1e-5)."""
+    n, na, nb = 12, 6, 6
+    ham, P, model, x, rng = _adjoint_problem(A, n, na, nb, hidden, 30 * 128, 5 + hidden)
+    cnt = np.ones(x.size, dtype=np.int64)
+    cnt[1:128] = 0
+    cnt[0] = 10_000_000
+    e = rng.normal(size=x.size) + 1j * rng.normal(size=x.size)
+    stats = np.array([0.3, -0.2, 1.0, float(cnt.sum())])
+    st = torch.tensor(stats, device="cuda")
+    without = cnt.copy()
+    without[0] = 0
+    g, g0 = (A.grad(model, ham, *_tensors(x, c, e), st).cpu().numpy().astype(np.float64) for c in (cnt, without))
+    assert model.status() == 0
+    off = 0
+    for p, layers in enumerate(P):
+        for k, (w, b) in enumerate(layers):
+            if k == 0 and p:
+                v = (int(x[0]) >> (2 * np.arange(p))) & 3
+                others = np.ones(4 * p, dtype=bool)
+                others[4 * np.arange(p) + v] = False
+                a, r = (u[off:off + w.size].reshape(w.shape)[:, others] for u in (g, g0))
+                assert np.linalg.norm(a - r) <= 1e-5 * np.linalg.norm(r), p
+            off += (w.size if w is not None else 0) + b.size
+
+
+@pytest.mark.parametrize("hidden,tiles", [(2, 26), (3, 26), (2, 200), (3, 200)])
+def test_tensor_core_adjoint_with_several_tiles_per_cta(A, hidden, tiles):
+    """2 to 3 tiles per CTA, and more than the 16 after which a CTA writes its
+    sums (12 CTAs per slot at 12 orbitals), the last tile partial: against the
+    oracle at the module's bar, and against the FP64 sum of calls of one tile
+    each (float32 sums of at most 150 terms in another order: 150 / 2^24 =
+    9e-6 at worst, the bar is twice that).  Then the same buffers with a device
+    row count that leaves some CTAs without a tile: as a call of those rows."""
+    n, na, nb = 12, 6, 6
+    ham, P, model, x, rng = _adjoint_problem(A, n, na, nb, hidden, 390, 17 + hidden)
+    cnt = rng.integers(1, 40, size=x.size)
+    e = rng.normal(size=x.size) + 1j * rng.normal(size=x.size)
+    rep = tiles * 128 // x.size
+    stats = energy_stats(e, cnt)
+    stats[3] *= rep
+    X, N, R, I = _tensors(np.tile(x, rep), np.tile(cnt, rep), np.tile(e, rep))
+    assert X.numel() % 128 and -(-X.numel() // 128) > 2 * 12
+    st = torch.tensor(stats, device="cuda")
+    g = A.grad(model, ham, X, N, R, I, st)
+    ref = _adjoint_reference(P, n, na, nb, x, cnt * rep, e, stats)
+    assert np.linalg.norm(g.cpu().numpy() - ref) < BAR * np.linalg.norm(ref)
+    parts = torch.zeros(model.n_params, dtype=torch.float64, device="cuda")
+    for k in range(0, X.numel(), 128):
+        s = slice(k, k + 128)
+        parts += A.grad(model, ham, X[s].contiguous(), N[s].contiguous(), R[s].contiguous(), I[s].contiguous(),
+                        st).double()
+    assert torch.linalg.norm(g.double() - parts) <= 1.8e-5 * torch.linalg.norm(parts)
+    few = 700  # six tiles for twelve CTAs
+    nd = torch.tensor([few], dtype=torch.int64, device="cuda")
+    a = A.grad(model, ham, X, N, R, I, st, n_dev=nd)
+    b = A.grad(model, ham, *(t[:few].contiguous() for t in (X, N, R, I)), st)
+    assert torch.equal(a, b) and model.status() == 0
