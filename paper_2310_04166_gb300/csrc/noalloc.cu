@@ -131,8 +131,11 @@ extern "C" int anqs_local_energy_static(const anqs_model* M, const anqs_ham* H, 
   float* la_p = S.take<float>(m);
   float* ph_p = S.take<float>(m);
   cudaStream_t s = (cudaStream_t)stream;
-  // the parts of samples split over CTAs go where the matrix elements were (at
-  // most one part per 512 excitations), the ticket where the diagonal would be
-  return run_eloc_array(M, H, x, host_count(n_x), xp, hv, la_x, ph_x, la_p, ph_p, hv, reinterpret_cast<uint32_t*>(hd),
+  // The ticket goes where the diagonal would be, the partial sums where the
+  // matrix elements were (at most two per excitation; of more than 1,024 samples
+  // 608).  Without excitations xp, hv and hd begin at one address: the partial
+  // sums then follow the ticket.
+  double* part = K ? hv : hd + 32;
+  return run_eloc_array(M, H, x, host_count(n_x), xp, hv, la_x, ph_x, la_p, ph_p, part, reinterpret_cast<uint32_t*>(hd),
                         ere, eim, counts, stats, s);
 }

@@ -230,3 +230,18 @@ def test_transformer_adjoint_rows(A, n, na, nb, heads, m):
     dev = lambda a: torch.tensor(np.concatenate([a, [3.0, -2.0]]), device="cuda", dtype=torch.float32)
     got = A.logpsi_vjp(model, ham, torch.cat([x, bad]), dev(ca), dev(cp)).cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("m", [3, 1025, 1500, 5000])
+def test_static_scratch_without_excitations(A, m):
+    """Full and empty shells: no connected determinants, so that the static form's arrays of them are empty; repeated
+    rows, also more than one CTA's statistics take.  All energies are the diagonal element: variance zero."""
+    model, ham = _problem(A, "mlp", "fp32", 3, 3, 0, 43)
+    assert ham.n_connected == 0
+    x = torch.full((m,), 21, dtype=torch.int64, device="cuda")
+    cnt = torch.arange(1, m + 1, dtype=torch.int64, device="cuda")
+    ref = A.local_energy(model, ham, x[:1])[0]
+    for _ in range(20):
+        ere, eim, st = _static(A, model, ham, x, cnt)
+        assert torch.equal(ere, ref.expand(m)) and not eim.any()
+        assert st.tolist() == [ref.item(), 0.0, 0.0, float(m * (m + 1) // 2)]
