@@ -706,8 +706,8 @@ __global__ void head_dout_kernel(HamView hv, Rows R, const float* __restrict__ o
       tot += c[u];
     }
     for (int u = 0; u < 4; ++u) {
-      // a row without an allowed outcome takes no samples
-      d[u] = sum > 0.f ? float(0.5 * (c[u] - double(e[u] / sum) * tot)) : 0.f;
+      // a row without an allowed outcome takes no samples (outputs that are not finite give NaN)
+      d[u] = mk ? float(0.5 * (c[u] - double(e[u] / sum) * tot)) : 0.f;
       d[4 + u] = float(c[4 + u]);
     }
   }

@@ -245,3 +245,22 @@ def test_static_scratch_without_excitations(A, m):
         ere, eim, st = _static(A, model, ham, x, cnt)
         assert torch.equal(ere, ref.expand(m)) and not eim.any()
         assert st.tolist() == [ref.item(), 0.0, 0.0, float(m * (m + 1) // 2)]
+
+
+@pytest.mark.parametrize("n,value", [(6, math.nan), (6, math.inf), (20, math.nan)])
+def test_transformer_adjoint_passes_nan_on(A, n, value):
+    """A logit bias that is not finite makes the softmax, and so the gradient of every logit bias, NaN; the phases'
+    biases keep theirs, the sum of the phase cotangents by outcome."""
+    from synthetic import flatten_tf, integrals, tf_params
+    P = tf_params(n, n, 64, 1, bias_std=0.2)
+    P["head_b"][:] = 0
+    P["head_b"][0] = value
+    h, g, e = integrals(n, n, 2)
+    ham = A.Hamiltonian(h, g, e, 3, 2)
+    model = A.Model.transformer(n, 64, 4, 1, torch.tensor(flatten_tf(P), device="cuda"))
+    x = _dets(n, 3, 2, 9, n)
+    one = torch.ones(9, device="cuda")
+    got = A.logpsi_vjp(model, ham, x, one, one)[-8:]
+    assert torch.isnan(got[:4]).all()
+    v = torch.stack([(x >> (2 * p)) & 3 for p in range(n)])
+    assert torch.equal(got[4:], torch.bincount(v.flatten(), minlength=4).float())
