@@ -181,12 +181,27 @@ __device__ __forceinline__ void hidden_layer(const float* in, const float* __res
 // The layer-1 weights pass through ws eight slots at a time: gathered from
 // global memory, each of a warp's lanes met another row of W1, and those
 // loads took most of the time of a node (12,400 prefixes of 9 orbitals, width
-// 128, 3 layers: 200 us).
-template <int W, int RR = R>
+// 128, 3 layers: 200 us).  The adjoint (STAGED false) gathers them: its CTAs
+// have one tile each and little of their time there, and waiting for the staged
+// slots cost more (16 orbitals, 500 samples, width 128, 2 layers: 108 us
+// gathered, 127 staged).  The sums and their order are the same.
+template <int W, int RR = R, bool STAGED = true>
 __device__ int slot_forward(const MlpView& m, int p, const uint64_t* xs, int nrows, float* act, int n_keep,
                             float* ws, float* out8, const float* wres = nullptr) {
   const MlpPtr P = slot_ptrs(m, p);
-  {
+  if constexpr (!STAGED) {
+    for (int idx = threadIdx.x; idx < RR * W; idx += NT) {
+      const int r = idx / W, o = idx % W;
+      float acc = __ldg(P.b1 + o);
+      if (r < nrows) {
+        const uint64_t x = xs[r];
+        const float* wrow = P.W1 + size_t(o) * 4 * p;
+#pragma unroll 4
+        for (int q = 0; q < p; ++q) acc += __ldg(wrow + 4 * q + int((x >> (2 * q)) & 3ull));
+      }
+      act[idx] = tanhf(acc);
+    }
+  } else {
     constexpr int E = RR * W / NT, WS = W + 4;  // thread: column o of rows r0 + (NT / W) e
     static_assert(NT % W == 0 && RR * W % NT == 0, "tile shape");
     const int o = threadIdx.x % W, r0 = threadIdx.x / W;
@@ -222,14 +237,15 @@ __device__ int slot_forward(const MlpView& m, int p, const uint64_t* xs, int nro
     const float* bk = Wk + size_t(W) * W;
     int nxt = (n_keep == 2) ? (cur ^ 1) : (cur + 1);
     float* o = act + size_t(nxt) * RR * W;
-    if (!wres) {
+    if constexpr (STAGED) {
       hidden_layer<W, RR>(act + size_t(cur) * RR * W, Wk, bk, ws, o);
       cur = nxt;
       Wk = bk + W;
       continue;
     }
     float acc[RPT][CPT];
-    tile_gemm<W, false, RR>(act + size_t(cur) * RR * W, Wk, ws, acc, wres + size_t(k - 2) * W * (W + 1));
+    tile_gemm<W, false, RR>(act + size_t(cur) * RR * W, Wk, ws, acc,
+                            wres ? wres + size_t(k - 2) * W * (W + 1) : nullptr);
 #pragma unroll
     for (int i = 0; i < RPT; ++i)
 #pragma unroll
@@ -253,6 +269,21 @@ __device__ int slot_forward(const MlpView& m, int p, const uint64_t* xs, int nro
   }
   __syncthreads();
   return cur;
+}
+
+// the adjoint's forward pass: a call at widths 64 and 256, inlined at 128 (the
+// other way round costs 5 to 8% of the kernel at 64, 3% at 128, and at 256 up to
+// 15% with few rows)
+template <int W, int RR>
+__device__ __noinline__ int forward_call(const MlpView& m, int p, const uint64_t* xs, int nrows, float* act, int n_keep,
+                                         float* ws, float* out8, const float* wres) {
+  return slot_forward<W, RR, false>(m, p, xs, nrows, act, n_keep, ws, out8, wres);
+}
+template <int W, int RR>
+__device__ __forceinline__ int adjoint_forward(const MlpView& m, int p, const uint64_t* xs, int nrows, float* act,
+                                               int n_keep, float* ws, float* out8, const float* wres) {
+  if constexpr (W == 128) return slot_forward<W, RR, false>(m, p, xs, nrows, act, n_keep, ws, out8, wres);
+  else return forward_call<W, RR>(m, p, xs, nrows, act, n_keep, ws, out8, wres);
 }
 
 // log-softmax term of the chosen outcome (FP32): normalised over nm, zero
@@ -531,7 +562,7 @@ __global__ void __launch_bounds__(NT) grad_kernel(MlpView m, HamView hv, const u
     cp[threadIdx.x] = b;
   }
   __syncthreads();
-  const int last = slot_forward<W, RG>(m, p, xt, nrows, act, L, ws, out8, wres);
+  const int last = adjoint_forward<W, RG>(m, p, xt, nrows, act, L, ws, out8, wres);
   const MlpPtr P = slot_ptrs(m, p);
   float* gbase = grad + (P.W1 - m.params) + (PARTIAL ? uint64_t(blockIdx.x) * n_params : 0ull);
   // d out: d l_u = cot_la * 1/2 (delta_uv - p~_u) over allowed u, d phi_u = cot_ph delta_uv
