@@ -1411,7 +1411,7 @@ __global__ void __launch_bounds__(AT) eloc_assemble_kernel(int n, uint32_t K, Co
     double re = 0.0, im = 0.0;
     for (uint32_t k = threadIdx.x; k < K; k += AT) {
       const uint64_t row = l * K + k;
-      const int j = js[row];
+      const int j = min(int(js[row]), n - 1);  // 255 for a parent outside the sector (h is NaN)
       const uint64_t x = xp[row];
       const float* cc = cache + (l * n + j) * CACHE_F;
       const int vj = int((x >> (2 * j)) & 3ull);
@@ -1548,7 +1548,11 @@ __global__ void finalize_kernel(HamView hv, const uint64_t* __restrict__ xs, Cou
 // ---- sort of connected rows by first differing slot ---------------------------
 // Histogram of the first slots into ctl[0, n) (zero on entry); the last CTA
 // to finish then writes cursor[i] = offsets[i] = rows with first slot < i
-// (exclusive prefix sums) and offsets[n] = rows.
+// (exclusive prefix sums) and offsets[n] = rows.  Rows of a determinant outside
+// the sector (first slot 255) go with the last slot, which has no suffix: their
+// matrix elements are NaN.
+__device__ __forceinline__ int sort_key(uint8_t j, int n) { return min(int(j), n - 1); }
+
 __global__ void js_hist_kernel(const uint8_t* __restrict__ js, Count m_, int n, uint32_t* __restrict__ ctl,
                                uint32_t* __restrict__ cursor, uint32_t* __restrict__ offsets) {
   ANQS_PDL_ENTRY();
@@ -1558,7 +1562,7 @@ __global__ void js_hist_kernel(const uint8_t* __restrict__ js, Count m_, int n, 
   for (int i = threadIdx.x; i < n; i += blockDim.x) h[i] = 0;
   __syncthreads();
   for (uint64_t t = blockIdx.x * uint64_t(blockDim.x) + threadIdx.x; t < m; t += uint64_t(gridDim.x) * blockDim.x)
-    atomicAdd(&h[js[t]], 1u);
+    atomicAdd(&h[sort_key(js[t], n)], 1u);
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x)
     if (h[i]) atomicAdd(&ctl[i], h[i]);
@@ -1584,14 +1588,14 @@ __global__ void js_hist_kernel(const uint8_t* __restrict__ js, Count m_, int n, 
   }
 }
 
-__global__ void js_scatter_kernel(const uint8_t* __restrict__ js, Count m_, uint32_t* __restrict__ cursor,
+__global__ void js_scatter_kernel(const uint8_t* __restrict__ js, Count m_, int n, uint32_t* __restrict__ cursor,
                                   uint32_t* __restrict__ perm) {
   ANQS_PDL_ENTRY();
   const uint64_t m = m_.get();
   const int lane = threadIdx.x & 31;
   for (uint64_t t0 = blockIdx.x * uint64_t(blockDim.x); t0 < m; t0 += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t t = t0 + threadIdx.x;
-    const int key = t < m ? int(js[t]) : -1;
+    const int key = t < m ? sort_key(js[t], n) : -1;
     // lanes with the same key reserve their slots with one atomic
     const unsigned peers = __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(peers) - 1;
@@ -1616,7 +1620,7 @@ __global__ void __launch_bounds__(1024) js_sort_small_kernel(const uint8_t* __re
   const int lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < n; i += blockDim.x) h[i] = 0;
   __syncthreads();
-  for (uint64_t t = threadIdx.x; t < m; t += blockDim.x) atomicAdd(&h[js[t]], 1u);
+  for (uint64_t t = threadIdx.x; t < m; t += blockDim.x) atomicAdd(&h[sort_key(js[t], n)], 1u);
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t acc = 0;
@@ -1630,7 +1634,7 @@ __global__ void __launch_bounds__(1024) js_sort_small_kernel(const uint8_t* __re
   __syncthreads();
   for (uint64_t t0 = 0; t0 < m; t0 += blockDim.x) {
     const uint64_t t = t0 + threadIdx.x;
-    const int key = t < m ? int(js[t]) : -1;
+    const int key = t < m ? sort_key(js[t], n) : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(peers) - 1;
     const int rank = __popc(peers & ((1u << lane) - 1u));
@@ -1882,7 +1886,7 @@ int launch_js_sort(const uint8_t* js, Count mc, int n, uint32_t* ctl, uint32_t* 
   }
   const unsigned g = unsigned(std::min<uint64_t>((mc.n + 255) / 256, 152 * 4));
   ANQS_CUDA_LAUNCH("js_hist_kernel", launch_k(js_hist_kernel, dim3(g ? g : 1), dim3(256), 0, s, js, mc, n, ctl, cursor, offsets));
-  ANQS_CUDA_LAUNCH("js_scatter_kernel", launch_k(js_scatter_kernel, dim3(g ? g : 1), dim3(256), 0, s, js, mc, cursor, perm));
+  ANQS_CUDA_LAUNCH("js_scatter_kernel", launch_k(js_scatter_kernel, dim3(g ? g : 1), dim3(256), 0, s, js, mc, n, cursor, perm));
   return ANQS_OK;
 }
 

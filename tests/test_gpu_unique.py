@@ -264,3 +264,132 @@ def test_transformer_adjoint_passes_nan_on(A, n, value):
     assert torch.isnan(got[:4]).all()
     v = torch.stack([(x >> (2 * p)) & 3 for p in range(n)])
     assert torch.equal(got[4:], torch.bincount(v.flatten(), minlength=4).float())
+
+
+def _reference(A, model, ham, x):
+    """E_loc from anqs_connected's list and anqs_logpsi's amplitudes, and the bound of this file's docstring."""
+    xp, hv, _, hd = A.connected(ham, x)
+    la, ph = A.logpsi(model, ham, x)
+    lp, pp = (t.view(xp.shape).double() for t in A.logpsi(model, ham, xp.reshape(-1)))
+    r = torch.exp(lp - la.double()[:, None])
+    dp = pp - ph.double()[:, None]
+    e = torch.complex(hd + (hv * r * torch.cos(dp)).sum(1), (hv * r * torch.sin(dp)).sum(1))
+    return e, 1e-9 + 4e-5 * (hv.abs() * r).sum(1)
+
+
+def _launches(A, name, call):
+    """What the call returns, and the timed launches of one kernel family in it."""
+    from paper_2310_04166_gb300 import _lib
+    lib = _lib.load()
+    _lib.check(lib.anqs_profile_enable(1))
+    out = call()
+    torch.cuda.synchronize()
+    k, ran = 0, {}
+    s, c, ms = C.c_char_p(), C.c_uint64(), C.c_double()
+    while lib.anqs_profile_read(k, C.byref(s), C.byref(c), C.byref(ms)) == 0:
+        ran[s.value.decode()] = c.value
+        k += 1
+    _lib.check(lib.anqs_profile_enable(0))
+    return out, ran[name]
+
+
+def _agrees(A, model, ham, x, e, bound, **kw):
+    ere, eim, _ = A.local_energy(model, ham, x, **kw)
+    assert torch.all((ere - e.real).abs() <= bound) and torch.all((eim - e.imag).abs() <= bound)
+
+
+def _tf16(A, n, na, nb, d, blocks, seed):
+    from synthetic import flatten_tf, integrals, tf_params
+    h, g, e = integrals(seed, n, 2 * n)
+    P = tf_params(seed, n, d, blocks, bias_std=0.1)
+    model = A.Model.transformer(n, d, d // 16, blocks, torch.tensor(flatten_tf(P), device="cuda"), "bf16")
+    return model, A.Hamiltonian(h, g, e, na, nb)
+
+
+# Enough samples (repeated where the sector has fewer) that a transformer's local energy takes the samples' prefix
+# trees, one network launch per orbital: few and many electrons, full and empty shells, and a workspace that only
+# holds the form over the suffixes of every connected determinant, in one launch.
+@pytest.mark.parametrize("n,na,nb,m", [(19, 1, 1, 900), (20, 2, 1, 300), (21, 21, 2, 900), (24, 0, 2, 900),
+                                       (32, 2, 30, 150), (32, 1, 0, 2500)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_transformer_forms_without_an_index(A, n, na, nb, m, d):
+    blocks = 2
+    model, ham = _tf16(A, n, na, nb, d, blocks, 90 + n)
+    x = _dets(n, na, nb, m, n)
+    x = x[torch.arange(m, device="cuda") % x.numel()].contiguous()
+    e, bound = _reference(A, model, ham, x)
+    need = A.local_energy_workspace_bytes(model, ham, m)
+    # the suffixes' scratch: 29 bytes per connected determinant, the samples' outputs, caches, keys and values
+    small = m * (29 * ham.n_connected + 16 + n * (32 + 40 + 4 * blocks * d)) + 8192
+    for ws, launches in ((need, n if d == 128 else None), (small, 1)):
+        buf = torch.empty(ws, dtype=torch.uint8, device="cuda")
+        _, ran = _launches(A, "tf_tc_suffix_kernel", lambda: _agrees(A, model, ham, x, e, bound, workspace=buf))
+        assert launches is None or ran == launches, (ws, ran)
+    with pytest.raises(A.AnqsError):
+        A.local_energy(model, ham, x, workspace=buf[:small // 2])
+    assert model.status() == 0
+
+
+@pytest.mark.parametrize("d,blocks", [(64, 1), (64, 2), (128, 2)])
+@pytest.mark.parametrize("n,na,nb,m", [(6, 3, 2, 5), (10, 5, 5, 4), (10, 5, 5, 40), (12, 6, 6, 10), (18, 2, 2, 9)])
+def test_transformer_forms_with_an_index(A, d, blocks, n, na, nb, m):
+    """The preferred form and the suffixes of every connected determinant (few samples, or a small workspace)."""
+    model, ham = _tf16(A, n, na, nb, d, blocks, 30 + n)
+    x = _dets(n, na, nb, m, n + 1)
+    e, bound = _reference(A, model, ham, x)
+    _agrees(A, model, ham, x, e, bound)
+    small = x.numel() * (29 * ham.n_connected + 16 + n * (32 + 40 + 4 * blocks * d)) + 8192
+    _agrees(A, model, ham, x, e, bound, workspace=torch.empty(small, dtype=torch.uint8, device="cuda"))
+    nd = torch.tensor([x.numel()], dtype=torch.int64, device="cuda")
+    pad = torch.cat([x, x[:1].expand(50)])  # room for more samples than there are, in the form of more
+    ere, eim, _ = A.local_energy(model, ham, pad, n_dev=nd)
+    assert torch.all((ere[:x.numel()] - e.real).abs() <= bound) and torch.all((eim[:x.numel()] - e.imag).abs() <= bound)
+
+
+@pytest.mark.parametrize("kind,form", [("mlp", "bf16"), ("tf", "bf16"), ("nade", "fp32"), ("mlp", "fp32"), ("tf", "fp32")])
+@pytest.mark.parametrize("n,na,nb,m", [(7, 4, 3, 3), (7, 4, 3, 100), (11, 5, 4, 2), (11, 5, 4, 150), (20, 2, 1, 60)])
+def test_z2_and_workspaces_of_more_samples(A, kind, form, n, na, nb, m):
+    """Z2 symmetries (determinants of the other parities have no amplitude) in the forms of few and of many samples,
+    with the workspace of a call of this and of twenty times as many samples."""
+    model, ham = _problem(A, kind, form, n, na, nb, 40 + n, z2=True)
+    mask = sum(3 << (2 * p) for p in range(n) if p % 2)
+    ref = sum(1 << (2 * p) for p in range(na)) + sum(2 << (2 * p) for p in range(nb))
+    x = _dets(n, na, nb, m, n, (mask, bin(ref & mask).count("1") % 2))
+    e, bound = _reference(A, model, ham, x)
+    for k in (1, 20):
+        ws = A._ws(A.local_energy_workspace_bytes(model, ham, k * x.numel()), "cuda")
+        _agrees(A, model, ham, x, e, bound, workspace=ws)
+
+
+def test_batch_of_few_and_many_samples(A):
+    """One persistent launch over problems by prefixes and problems by suffixes (few samples, and more orbitals than
+    the index covers): as one call each, bit for bit."""
+    items = []
+    for n, na, nb, m in [(10, 5, 5, 3), (10, 5, 5, 300), (20, 2, 2, 12), (7, 5, 5, 200), (12, 6, 6, 2), (1, 1, 0, 1)]:
+        model, ham = _problem(A, "mlp", "bf16", n, na, nb, 20 + n)
+        x = _dets(n, na, nb, m, m)
+        items.append(dict(model=model, ham=ham, x=x, counts=torch.arange(1, x.numel() + 1, dtype=torch.int64, device="cuda")))
+    batch = A.EnergyBatch(len(items))
+    for it, got in zip(items, batch.local_energy(items)):
+        one = A.local_energy(it["model"], it["ham"], it["x"], it["counts"])
+        assert all(torch.equal(u, v) for u, v in zip(got, one))
+
+
+# The forms that sort the connected list by its first differing slot: few samples, or no prefix index.
+@pytest.mark.parametrize("kind,form,n", [("mlp", "bf16", 10), ("mlp", "bf16", 20), ("nade", "fp32", 20), ("tf", "bf16", 12)])
+def test_determinants_outside_the_sector_in_the_list_forms(A, kind, form, n):
+    test_determinants_outside_the_sector(A, kind, form, n)
+
+
+@pytest.mark.parametrize("kind,form", [("mlp", "bf16"), ("tf", "bf16"), ("nade", "fp32"), ("mlp", "fp32"), ("tf", "fp32")])
+@pytest.mark.parametrize("n,na,nb,m", [(5, 5, 0, 3), (20, 20, 0, 1), (20, 20, 20, 1500)])
+def test_without_excitations(A, kind, form, n, na, nb, m):
+    """One determinant and no connected one: E_loc is the diagonal element, which the FP32 MLP's form also gives."""
+    model, ham = _problem(A, kind, form, n, na, nb, 5)
+    assert ham.n_connected == 0
+    x = _dets(n, na, nb, 1, 1).expand(m).contiguous()
+    other, _ = _problem(A, "mlp", "fp32", n, na, nb, 5)
+    ref = A.local_energy(other, ham, x[:1])[0]
+    ere, eim, st = A.local_energy(model, ham, x, torch.ones_like(x))
+    assert torch.allclose(ere, ref.expand(m), rtol=1e-13) and not eim.any()
+    assert torch.allclose(st, torch.tensor([ref.item(), 0.0, 0.0, m], dtype=torch.float64, device="cuda"), rtol=1e-13)
