@@ -693,7 +693,7 @@ int logpsi_dispatch(const anqs_model* M, const anqs_ham* H, const uint64_t* x, C
                     float* ph, cudaStream_t s);
 
 // the local energy from the amplitude of every connected determinant; part:
-// 2 n_x K / 512 doubles at most (eloc_partials), may alias hv
+// eloc_partials, at most n_x K / 64 or 608 doubles, may alias hv
 int run_eloc_array(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, uint64_t* xp, double* hv,
                    float* la_x, float* ph_x, float* la, float* ph, double* part, uint32_t* ticket, double* ere,
                    double* eim, const uint64_t* counts, double* stats, cudaStream_t s);

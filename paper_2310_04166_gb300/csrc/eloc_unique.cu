@@ -705,12 +705,14 @@ __global__ void __launch_bounds__(ET) stats_kernel(const double* ere, const doub
 
 // CTAs per sample: a whole sample each when there are enough to fill the GPU
 // (16 CTAs of 128 threads per SM are resident at most), else parts of at
-// least 512 excitations
-constexpr uint64_t kFillCtas = 152 * 8;
+// least one excitation per thread.  (With parts of 512 one sample of 10 orbitals,
+// 875 excitations, was one CTA: 70 us of marking, seven chains of dependent
+// loads and atomics one after the other, and 33 us of assembly.)
+constexpr uint64_t kFillCtas = 152 * 8, kPart = 128;
 
 int split_of(uint64_t n_x, uint32_t K) {
   if (n_x == 0) return 1;
-  const uint64_t want = (kFillCtas + n_x - 1) / n_x, most = std::max<uint64_t>(1, K / 512);
+  const uint64_t want = (kFillCtas + n_x - 1) / n_x, most = std::max<uint64_t>(1, K / kPart);
   return int(std::max<uint64_t>(1, std::min<uint64_t>(std::min(want, most), 128)));
 }
 
@@ -864,7 +866,7 @@ int launch_path_sums(const anqs_ham* H, const UniqueWs& w, const float2* terms, 
 // n_x * split_of(n_x) stays below 1216 + n_x; never less for more samples.
 // A call of more samples that is not split keeps its statistics' sums there.
 uint64_t eloc_partials(const anqs_ham* H, uint64_t n_x) {
-  return std::max<uint64_t>(H->v.K >= 1024 ? 2 * (kFillCtas + std::min<uint64_t>(n_x, kFillCtas)) : 0,
+  return std::max<uint64_t>(H->v.K >= 2 * kPart ? 2 * (kFillCtas + std::min<uint64_t>(n_x, kFillCtas)) : 0,
                             n_x > kTailStats ? 4 * SB : 0);
 }
 
