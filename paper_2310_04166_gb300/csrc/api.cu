@@ -172,7 +172,9 @@ static size_t plain_ws_bytes(const anqs_model* M, const anqs_ham* H, uint64_t n_
 // The variants' tables take up to 1 KB per prefix (MLP): they may use twice
 // the memory of the form without them, or 1 GiB.
 static bool plain_prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
-  return unique_applies(H, n_x) && plain_ws_bytes(M, H, n_x, true) <=
+  if (!unique_applies(H, n_x)) return false;
+  if (M->d.kind == ANQS_MODEL_TF && !tf_fp32_prefers_variants(M->tf, n_x, n_x * H->v.K, unique_expected(H, n_x))) return false;
+  return plain_ws_bytes(M, H, n_x, true) <=
                                        std::max<size_t>(size_t(1) << 30, 2 * plain_ws_bytes(M, H, n_x, false));
 }
 

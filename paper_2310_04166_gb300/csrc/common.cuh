@@ -485,6 +485,8 @@ int launch_tf_fp32_logpsi(const TfView& m, const HamView& hv, const uint64_t* x,
 // out [determinant][tf_fp32_variants(m)]: (log|psi|, phase) as each sequence
 // of a tile would have it
 uint32_t tf_fp32_variants(const TfView& m);
+// whether evaluating `distinct` determinants for every variant takes less than the connected ones of n_x samples
+bool tf_fp32_prefers_variants(const TfView& m, uint64_t n_x, uint64_t connected, double distinct);
 int launch_tf_fp32_variants(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float2* out,
                             cudaStream_t s);
 int launch_tf_fp32_slot_logits(const TfView& m, int p, const uint64_t* pre, const uint64_t* nr, uint64_t max_rows,
@@ -515,6 +517,8 @@ struct UniqueWs {
   double* part;        // partial sums when a sample is split over CTAs
 };
 bool unique_applies(const anqs_ham* H, uint64_t n_x);
+bool unique_full(const anqs_ham* H, uint64_t n_x);       // every prefix of the sector would be a node
+double unique_expected(const anqs_ham* H, uint64_t n_x); // distinct determinants to be expected
 // Which form a call takes: the preferred one if its scratch fits into the
 // workspace, else the other if that fits (a workspace may have been sized for
 // more samples, in the other form).

@@ -24,6 +24,7 @@
 // All float32 sums run in the order of an evaluation of each connected
 // determinant by itself, so the amplitudes have its bits.
 #include <algorithm>
+#include <cmath>
 
 #include "excite.cuh"
 
@@ -744,6 +745,17 @@ bool unique_applies(const anqs_ham* H, uint64_t n_x) {
   if (use_full(H, n_x)) return true;
   const uint64_t m = n_x * (uint64_t(H->v.K) + 1);
   return index_words(H) <= (1ull << 20) || index_words(H) <= 8 * m;
+}
+
+bool unique_full(const anqs_ham* H, uint64_t n_x) { return use_full(H, n_x); }
+
+// As if the connected sets fell into the sector at random, times 0.7: sets of
+// samples that follow a network's distribution overlap more (16 to 95 samples
+// of 11 to 18 orbitals: 0.3 to 0.7 of a random set's determinants).
+double unique_expected(const anqs_ham* H, uint64_t n_x) {
+  const double all = double(H->sv.na_p[H->v.n]) * double(H->sv.nb_p[H->v.n]);
+  if (use_full(H, n_x)) return all;
+  return std::max(0.7 * all * -std::expm1(-double(n_x) * (double(H->v.K) + 1.0) / all), std::min(all, double(H->v.K) + 1.0));
 }
 
 void plan_unique(const anqs_ham* H, uint64_t n_x, bool levels, Arena& A, UniqueWs& w) {

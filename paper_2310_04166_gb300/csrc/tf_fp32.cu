@@ -146,15 +146,15 @@ __device__ __forceinline__ void layer_norm(const float* x, float* y, const float
   __syncthreads();
 }
 
-// The 8 outputs of every row from the final LayerNorm's output a.  Row r's sums
-// start at input rot + r (the rows' different starts spread the shared-memory
-// banks).
+// The 8 outputs of the rows r0 <= r < r1 from the final LayerNorm's output a.
+// Row r's sums start at input rot + r (the rows' different starts spread the
+// shared-memory banks).
 template <int D>
-__device__ __forceinline__ void head(const TfView& m, const float* a, float* out8, int rot) {
-  constexpr int MT = Cfg<D>::MT;
+__device__ __forceinline__ void head(const TfView& m, const float* a, float* out8, int rot, int r0 = 0,
+                                     int r1 = Cfg<D>::MT) {
   const float* hw = tf_tail(m) + 2 * D;
   const float* hb = hw + 8 * D;
-  for (int task = threadIdx.x; task < MT * 8; task += NT) {
+  for (int task = r0 * 8 + threadIdx.x; task < r1 * 8; task += NT) {
     const int r = task >> 3, o = task & 7;
     float acc = __ldg(hb + o);
     const float* wr = hw + o * D;
@@ -307,46 +307,65 @@ __global__ void __launch_bounds__(NT, 1) tf_logpsi_kernel(TfView m, HamView hv, 
 // log psi of the distinct determinants of a call (eloc_unique.cu), as each of
 // the S sequences of a tile would have it: sequence s's row of position t is
 // s T + t, so for variant q the sums of sequence s start (q - s) T further on
-// (D a power of two: the start counts modulo D).
+// (D a power of two: the start counts modulo D).  The slot terms of a shift are
+// taken a row per thread and then added in order per sequence (a thread per
+// sequence that went through its slots held the CTA up for longer than a shift's
+// sums take).
 template <int D>
 __global__ void __launch_bounds__(NT, 1) tf_variants_kernel(TfView m, HamView hv, const uint64_t* __restrict__ xs,
                                                             Count n_x_, float2* __restrict__ out) {
   ANQS_PDL_ENTRY();
   extern __shared__ float smem[];
   constexpr int MT = Cfg<D>::MT;
+  static_assert(MT <= NT, "a row per thread");
   __shared__ uint64_t xt[MT];
+  __shared__ float2 term[MT];
+  __shared__ int dead[MT];
   float* out8 = smem + Cfg<D>::floats - MT * 8;
   const uint64_t n_x = n_x_.get();
-  const int T = m.n, S = MT / T;
+  const int T = m.n, S = MT / T, row = threadIdx.x, rp = row % T;
   const uint64_t n_tiles = (n_x + S - 1) / S;
   for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const uint64_t base = tile * S;
     const int ns = int(n_x - base < uint64_t(S) ? n_x - base : uint64_t(S));
-    if (threadIdx.x < S)
-      xt[threadIdx.x] = threadIdx.x < ns ? __ldcg(reinterpret_cast<const unsigned long long*>(xs) + base + threadIdx.x) : 0ull;
+    if (row < S) {
+      xt[row] = row < ns ? __ldcg(reinterpret_cast<const unsigned long long*>(xs) + base + row) : 0ull;
+      dead[row] = 0;
+    }
     __syncthreads();
     tile_forward<D>(m, xt, ns, T, smem);
-    // shift d = q - s mod S' over all (sequence, variant) pairs: with the sums
-    // shifted by d rows, sequence s holds variant s + d (for d < 0 too)
+    unsigned pm = 0, nm = 0;
+    int v = 0;
+    if (row < ns * T) {
+      const uint64_t x = xt[row / T], below = x & ((1ull << (2 * rp)) - 1ull);
+      pm = slot_mask(hv, rp, __popcll(below & 0x5555555555555555ull), __popcll(below & 0xAAAAAAAAAAAAAAAAull), x);
+      nm = norm_mask(hv, rp, pm);
+      v = int((x >> (2 * rp)) & 3ull);
+      if (!((pm >> v) & 1u)) dead[row / T] = 1;
+    }
+    // shift d = q - s over all (sequence, variant) pairs: with the sums shifted
+    // by d rows, sequence s holds variant s + d
     for (int d = 1 - S; d < S; ++d) {
-      head<D>(m, smem + MT * D, out8, ((d * T) % D + D) & (D - 1));
-      const int s = threadIdx.x, q = s + d;
-      if (s < ns && q >= 0 && q < S) {
-        const uint64_t x = xt[s];
+      const int s_lo = d < 0 ? -d : 0, s_hi = d < 0 ? ns : (S - d < ns ? S - d : ns);  // sequences that have it
+      if (s_lo >= s_hi) continue;
+      head<D>(m, smem + MT * D, out8, ((d * T) % D + D) & (D - 1), s_lo * T, s_hi * T);
+      if (row >= s_lo * T && row < s_hi * T) {
         float la = 0.f, ph = 0.f;
-        bool dead = false;
-        int ca = 0, cb = 0;
-        for (int p = 0; p < T; ++p) {
-          const int v = int((x >> (2 * p)) & 3ull);
-          const unsigned pm = slot_mask(hv, p, ca, cb, x);
-          slot_term(out8 + (s * T + p) * 8, norm_mask(hv, p, pm), pm, v, la, ph, dead);
-          ca += v & 1;
-          cb += v >> 1;
-        }
-        out[(base + s) * S + q] = make_float2(dead ? -INFINITY : la, ph);
+        bool off = false;
+        slot_term(out8 + row * 8, nm, pm, v, la, ph, off);
+        term[row] = make_float2(la, ph);
       }
       __syncthreads();
+      if (row >= s_lo && row < s_hi) {
+        float la = 0.f, ph = 0.f;
+        for (int p = 0; p < T; ++p) {
+          la += term[row * T + p].x;
+          ph += term[row * T + p].y;
+        }
+        out[(base + row) * S + row + d] = make_float2(dead[row] ? -INFINITY : la, ph);
+      }
     }
+    __syncthreads();
   }
 }
 
@@ -432,6 +451,20 @@ int launch_tf_fp32_logpsi(const TfView& m, const HamView& hv, const uint64_t* x,
 uint32_t tf_fp32_variants(const TfView& m) {
   const int mt = m.d <= 64 ? Cfg<64>::MT : m.d == 128 ? Cfg<128>::MT : Cfg<256>::MT;
   return uint32_t(mt / m.n);
+}
+
+// Tiles run in waves of 152 CTAs, and a wave with the head for every variant
+// takes f times one without.  Measured at 2 blocks (us per wave): d 64, 5
+// orbitals (25 sequences a tile) 490 of 213, 10 orbitals 366 of 215, 18 orbitals
+// 307 of 214; d 32, 10 orbitals 186 of 105; d 128, 10 orbitals 447 of 350, 18
+// orbitals 403 of 356.  Of 14 orbitals, 7 + 7 electrons, 35 samples have 118,335
+// connected determinants, some 70,000 distinct: 18.7 ms one by one, 16.0 ms
+// distinct; 4 samples 2.4 and 2.7 ms.
+bool tf_fp32_prefers_variants(const TfView& m, uint64_t n_x, uint64_t connected, double distinct) {
+  const uint64_t S = tf_fp32_variants(m);
+  auto waves = [&](double rows) { return std::ceil(std::ceil(rows / double(S)) / 152.0); };
+  const double f = m.d <= 64 ? 1.1 + 0.055 * double(S) : 1.05 + 0.03 * double(S);
+  return f * waves(distinct) <= waves(double(n_x)) + waves(double(connected));
 }
 
 int launch_tf_fp32_variants(const TfView& m, const HamView& hv, const uint64_t* x, Count n_x, float2* out,
