@@ -906,7 +906,8 @@ static size_t eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_
 }
 
 static bool prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
-  return uses_tc_eloc(M) ? unique_applies(H, n_x) : plain_prefers_unique(M, H, n_x);
+  if (!uses_tc_eloc(M)) return plain_prefers_unique(M, H, n_x);
+  return M->d.kind == ANQS_MODEL_MLP ? mlp_tc_prefers_unique(M, H, n_x) : unique_applies(H, n_x);
 }
 
 int anqs_local_energy_workspace_size(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
@@ -1120,7 +1121,7 @@ int anqs_batched_local_energy(anqs_batch* b, const anqs_eloc_problem* q, int n, 
           break;
         }
         const Count nc{q[k].n_x, q[k].n_x_dev, 1};
-        r = eloc_tc_post(q[k].ham, q[k].x_dev, nc, q[k].eloc_re_dev, q[k].eloc_im_dev, q[k].counts_dev, q[k].stats_dev,
+        r = eloc_tc_post(q[k].model, q[k].ham, q[k].x_dev, nc, q[k].eloc_re_dev, q[k].eloc_im_dev, q[k].counts_dev, q[k].stats_dev,
                          q[k].workspace_dev, q[k].workspace_bytes, sk);
         if (cudaEventRecord(b->done[k], sk) == cudaSuccess) join[k] = 2;
         else fail("event record");

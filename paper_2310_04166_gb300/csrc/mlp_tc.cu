@@ -1764,8 +1764,8 @@ size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NodeWs& w) {
   return A.off;
 }
 
-bool nodes_form(const anqs_ham* H, uint64_t n_x, size_t ws_bytes) {
-  return use_unique(H, unique_applies(H, n_x), eloc_tc_workspace(H, n_x, false), H->has_index ? eloc_tc_workspace(H, n_x, true) : 0,
+bool nodes_form(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t ws_bytes) {
+  return use_unique(H, mlp_tc_prefers_unique(M, H, n_x), eloc_tc_workspace(H, n_x, false), H->has_index ? eloc_tc_workspace(H, n_x, true) : 0,
                     ws_bytes);
 }
 
@@ -1899,6 +1899,18 @@ int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const
   return ANQS_OK;
 }
 
+// Marking, listing and summing cost 20 to 60 us more than the sort of a few
+// connected determinants, unless every prefix of the sector is taken; what a
+// connected determinant costs beyond that grows with its slots and their layers.
+// Both forms take the same time (width 128, 3 layers, us) at 10 orbitals, 5 + 5
+// electrons, 32 samples (79), 14 orbitals, 7 + 7, 4 samples (101), 18 orbitals,
+// 2 + 2, 4 samples (87); width 64, 2 layers: 10 orbitals, 70 samples (80).
+bool mlp_tc_prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  if (!unique_applies(H, n_x)) return false;
+  const double work = double(n_x) * H->v.K * H->v.n * double(M->d.n_hidden) * M->d.width;
+  return unique_full(H, n_x) || work >= 6.7e7;
+}
+
 size_t eloc_tc_workspace(const anqs_ham* H, uint64_t n_x, bool unique) {
   Arena A(nullptr, 0);
   if (unique) {
@@ -1951,7 +1963,7 @@ static int plan_ws(const anqs_ham* H, Count n_x, void* ws, size_t ws_bytes, Eloc
 // kernel, on the stream of the histogram and the assembly that use them.
 int eloc_tc_pre(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, void* ws, size_t ws_bytes,
                 cudaStream_t s, bool fork) {
-  if (nodes_form(H, n_x.n, ws_bytes)) {
+  if (nodes_form(M, H, n_x.n, ws_bytes)) {
     NodeWs v;
     ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
     return launch_unique(H, x, n_x, v.u, s);
@@ -1992,9 +2004,9 @@ int eloc_tc_pre(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count
   return r;
 }
 
-int eloc_tc_post(const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim, const uint64_t* counts,
-                 double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
-  if (nodes_form(H, n_x.n, ws_bytes)) {
+int eloc_tc_post(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
+                 const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
+  if (nodes_form(M, H, n_x.n, ws_bytes)) {
     NodeWs v;
     ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
     ANQS_TRY(launch_path_sums(H, v.u, v.terms, v.mid, v.sums, s));
@@ -2013,7 +2025,7 @@ int eloc_tc_post(const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, d
 int run_eloc_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                 const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
   ANQS_TRY(eloc_tc_pre(M, H, x, n_x, ws, ws_bytes, s, true));
-  if (nodes_form(H, n_x.n, ws_bytes)) {
+  if (nodes_form(M, H, n_x.n, ws_bytes)) {
     NodeWs v;
     ANQS_TRY(plan_nodes_ws(H, n_x, ws, ws_bytes, v));
     ANQS_TRY(launch_mlp_tc_nodes(M, H->v, v.u.nodes, v.terms, s));
@@ -2024,7 +2036,7 @@ int run_eloc_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count
     ProfScope ps(PROF_TC_SUFFIX, s);
     ANQS_TRY(tv.W == 128 ? launch_ws_w<128>(tv, H->v, w, s) : launch_ws_w<64>(tv, H->v, w, s));
   }
-  return eloc_tc_post(H, x, n_x, ere, eim, counts, stats, ws, ws_bytes, s);
+  return eloc_tc_post(M, H, x, n_x, ere, eim, counts, stats, ws, ws_bytes, s);
 }
 
 // Tensor-memory columns of the adjoint at width 128: dW_1 takes what its widest
@@ -2111,7 +2123,7 @@ int launch_mlp_tc_multi(const MultiEloc* q, int n, int chunk, int dynamic, void*
     if (tv.W != W) return set_error(ANQS_ERR_ARG, "multi-problem launch needs one network width");
     a.prob[k].tv = tv;
     a.prob[k].hv = q[k].ham->v;
-    a.prob[k].nodes = nodes_form(q[k].ham, q[k].n_x, q[k].ws_bytes) ? 1 : 0;
+    a.prob[k].nodes = nodes_form(q[k].model, q[k].ham, q[k].n_x, q[k].ws_bytes) ? 1 : 0;
     if (a.prob[k].nodes) {
       NodeWs v;
       ANQS_TRY(plan_nodes_ws(q[k].ham, host_count(q[k].n_x), q[k].ws, q[k].ws_bytes, v));
