@@ -507,6 +507,7 @@ int anqs_hamiltonian_create(anqs_ham** out, int n, int na, int nb, const double*
   v.e_nuc = e_nuc;
   v.mu_lv = n;
   v.nz = 0;
+  trie_level_nodes(v, H->tree_nodes);
   if (build_sector(H) != ANQS_OK) {
     delete H;
     return ANQS_ERR_SECTOR;
@@ -899,30 +900,30 @@ int anqs_stats_combine(const double* stats_in, int world, double* stats_out, voi
 // prefix-reuse local energy: the BF16 forms and the NADE
 static bool uses_tc_eloc(const anqs_model* M) { return M->d.form == ANQS_FORM_BF16 || M->d.kind == ANQS_MODEL_NADE; }
 
-static size_t eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique) {
-  if (!uses_tc_eloc(M)) return plain_ws_bytes(M, H, n_x, unique);
-  if (M->d.kind == ANQS_MODEL_NADE) return nade_eloc_workspace(H, n_x, unique);
-  return M->d.kind == ANQS_MODEL_TF ? tf_tc_eloc_workspace(M, H, n_x, unique) : eloc_tc_workspace(H, n_x, unique);
-}
-
-static bool prefers_unique(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
-  if (!uses_tc_eloc(M)) return plain_prefers_unique(M, H, n_x);
-  return M->d.kind == ANQS_MODEL_MLP ? mlp_tc_prefers_unique(M, H, n_x) : unique_applies(H, n_x);
+// bytes of the form that a call of n_x samples prefers, and of the one with the least scratch
+static size_t eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool least) {
+  if (uses_tc_eloc(M) && M->d.kind == ANQS_MODEL_TF)
+    return least ? tf_tc_eloc_workspace_least(M, H, n_x) : tf_tc_eloc_workspace(M, H, n_x);
+  auto bytes = [&](bool unique) {
+    if (!uses_tc_eloc(M)) return plain_ws_bytes(M, H, n_x, unique);
+    return M->d.kind == ANQS_MODEL_NADE ? nade_eloc_workspace(H, n_x, unique) : eloc_tc_workspace(H, n_x, unique);
+  };
+  if (least) return H->has_index ? std::min(bytes(false), bytes(true)) : bytes(false);
+  if (!uses_tc_eloc(M)) return bytes(plain_prefers_unique(M, H, n_x));
+  return bytes(M->d.kind == ANQS_MODEL_NADE ? unique_applies(H, n_x) : mlp_tc_prefers_unique(M, H, n_x));
 }
 
 int anqs_local_energy_workspace_size(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t* bytes) {
   ANQS_TRY(check_pair(M, H));
   if (!bytes) return set_error(ANQS_ERR_ARG, "null output");
-  *bytes = eloc_workspace(M, H, n_x, prefers_unique(M, H, n_x));
+  *bytes = eloc_workspace(M, H, n_x, false);
   return ANQS_OK;
 }
 
 // a workspace large enough for one of the call's forms
 static int check_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, const void* ws, size_t ws_bytes) {
-  const bool pref = prefers_unique(M, H, n_x);
-  const size_t need = eloc_workspace(M, H, n_x, pref);
-  if (ws && ws_bytes >= need) return ANQS_OK;
-  if (ws && H->has_index && ws_bytes >= eloc_workspace(M, H, n_x, !pref)) return ANQS_OK;
+  const size_t need = eloc_workspace(M, H, n_x, false);
+  if (ws && (ws_bytes >= need || ws_bytes >= eloc_workspace(M, H, n_x, true))) return ANQS_OK;
   return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", need);
 }
 

@@ -401,6 +401,7 @@ struct anqs_ham {
   uint64_t* d_full_x = nullptr;     // all prefixes of levels 0..n,
   uint32_t* d_full_off = nullptr;   // their level offsets [n + 2]
   std::vector<uint32_t> full_off;
+  uint64_t tree_nodes[ANQS_MAX_ORB + 1] = {};  // trie_level_nodes
   unsigned* d_status;  // HamView::status
   double* d_h;
   double* d_g;
@@ -598,6 +599,7 @@ struct TrieWs {
   double* part;                       // [n_x][TRIE_PARTS][2]
   int parts;
 };
+void trie_level_nodes(const HamView& hv, uint64_t* nodes);
 // max_nodes: bound on the nodes below level n - 1 of a group (at least one sample)
 void plan_trie(const anqs_ham* H, uint64_t n_x, uint64_t max_nodes, Arena& A, TrieWs& w);
 // level p of group c, after level p - 1
@@ -667,12 +669,14 @@ int launch_js_sort(const uint8_t* js, Count mc, int n, uint32_t* ctl, uint32_t* 
                    uint32_t* perm, cudaStream_t s);
 int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const uint8_t* js, const float* cache,
                          const float2* T, const double* hval, const double* hdiag, const float* la_x,
-                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s);
+                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s,
+                         bool tsum = false);
 // BF16 transformer form
 int tf_tc_pack_alloc(anqs_model* m);
 int tf_tc_pack(anqs_model* m, cudaStream_t s);
 int tf_tc_status(const anqs_model* M, int* status);
-size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique);
+size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x);        // of the preferred form
+size_t tf_tc_eloc_workspace_least(const anqs_model* M, const anqs_ham* H, uint64_t n_x);  // of the one with the least
 int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                    const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s);
 int launch_tf_tc_logpsi(const anqs_model* M, const HamView& hv, const uint64_t* x, uint64_t n_x, float* la,

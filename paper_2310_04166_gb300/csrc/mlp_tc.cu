@@ -1389,7 +1389,9 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
 // parent slot-j term of v'_j + the terms T[x'][p] of the slots p > j; then
 // E_loc(x) = H_xx + sum H_xx' exp(log psi(x') - log psi(x)) with the ratio in
 // float32 and the sum in FP64, reduced in a fixed order (deterministic).  The
-// suffix terms come per (x', slot).  With so.counts set, the last CTA to
+// suffix terms come per (x', slot) (T[x'][p], MLP and NADE) or already summed
+// per x' (T[x'], `tsum`: the transformer, whose suffix kernel holds a
+// sequence's positions in one tile).  With so.counts set, the last CTA to
 // finish also reduces the statistics of the sample set over every row.
 constexpr int AT = 128;
 __global__ void __launch_bounds__(AT) eloc_assemble_kernel(int n, uint32_t K, Count n_x_, const uint64_t* __restrict__ xp,
@@ -1400,7 +1402,7 @@ __global__ void __launch_bounds__(AT) eloc_assemble_kernel(int n, uint32_t K, Co
                                                            const double* __restrict__ hdiag,
                                                            const float* __restrict__ la_x,
                                                            const float* __restrict__ ph_x, double* __restrict__ ere,
-                                                           double* __restrict__ eim, StatsOut so) {
+                                                           double* __restrict__ eim, int tsum, StatsOut so) {
   ANQS_PDL_ENTRY();
   __shared__ double red[2][AT / 32];
   __shared__ int s_last;
@@ -1416,16 +1418,24 @@ __global__ void __launch_bounds__(AT) eloc_assemble_kernel(int n, uint32_t K, Co
       const float* cc = cache + (l * n + j) * CACHE_F;
       const int vj = int((x >> (2 * j)) & 3ull);
       float la = cc[0] + cc[2 + vj], ph = cc[1] + cc[6 + vj];
-      // the terms of slots j+1 .. n-1, eight loads in flight at a time,
-      // added in slot order (the padding adds zeros)
-      for (int p0 = j + 1; p0 < n; p0 += 8) {
-        float2 tv[8];
+      if (tsum) {
+        if (j + 1 < n) {  // determinants with j = n - 1 have no suffix positions (and no T entry)
+          const float2 tv = T[row];
+          la += tv.x;
+          ph += tv.y;
+        }
+      } else {
+        // the terms of slots j+1 .. n-1, eight loads in flight at a time,
+        // added in slot order (the padding adds zeros)
+        for (int p0 = j + 1; p0 < n; p0 += 8) {
+          float2 tv[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tv[e] = p0 + e < n ? T[row * n + p0 + e] : make_float2(0.f, 0.f);
+          for (int e = 0; e < 8; ++e) tv[e] = p0 + e < n ? T[row * n + p0 + e] : make_float2(0.f, 0.f);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          la += tv[e].x;
-          ph += tv[e].y;
+          for (int e = 0; e < 8; ++e) {
+            la += tv[e].x;
+            ph += tv[e].y;
+          }
         }
       }
       const double h = hval[row];
@@ -1892,10 +1902,10 @@ int launch_js_sort(const uint8_t* js, Count mc, int n, uint32_t* ctl, uint32_t* 
 
 int launch_eloc_assemble(int n, uint32_t K, Count n_x, const uint64_t* xp, const uint8_t* js, const float* cache,
                          const float2* T, const double* hval, const double* hdiag, const float* la_x,
-                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s) {
+                         const float* ph_x, double* ere, double* eim, const StatsOut& so, cudaStream_t s, bool tsum) {
   uint64_t blocks = n_x.n;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  ANQS_CUDA_LAUNCH("eloc_assemble_kernel", launch_k(eloc_assemble_kernel, dim3(unsigned(blocks ? blocks : 1)), dim3(AT), 0, s, n, K, n_x, xp, js, cache, T, hval, hdiag, la_x, ph_x, ere, eim, so));
+  ANQS_CUDA_LAUNCH("eloc_assemble_kernel", launch_k(eloc_assemble_kernel, dim3(unsigned(blocks ? blocks : 1)), dim3(AT), 0, s, n, K, n_x, xp, js, cache, T, hval, hdiag, la_x, ph_x, ere, eim, tsum ? 1 : 0, so));
   return ANQS_OK;
 }
 

@@ -35,9 +35,17 @@
 //           own prefixes (levels < p, found through its table) and to itself;
 //           keeps its keys and values for the later levels and writes the
 //           masked half-log-probability and the phase of each outcome.
+//   SUFFIX  connected determinants x', grouped by first differing slot j:
+//           positions t = j+1..n-1 only (positions <= j see the same tokens as
+//           in the parent x, Eq. anqs_def); the keys and values of positions
+//           <= j are the parent's (kept by FULL); writes the sum over those
+//           positions of the masked slot terms, one (log|psi|, phase) pair
+//           T[x'] per connected determinant.  Three launches instead of four
+//           per level: the form of few samples (run_eloc_tf_tc).
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 
 #include "common.cuh"
@@ -51,9 +59,11 @@ size_t tf128_packed_bytes(const anqs_model* M);
 int tf128_pack(anqs_model* M, cudaStream_t s);
 int tf128_status_offset(const anqs_model* M);
 int launch_tf128_full(const anqs_model* M, const HamView& hv, const uint64_t* x, Count n_seq, int P, int last_only,
-                      float* raw, int prof, cudaStream_t s);
+                      float* raw, int prof, cudaStream_t s, __half* kv = nullptr);
 int launch_tf128_nodes(const anqs_model* M, const HamView& hv, const TrieLevel& lv, __half* kv, float2* terms,
                        cudaStream_t s);
+int launch_tf128_suffix(const anqs_model* M, const HamView& hv, const uint64_t* xp, const uint32_t* perm,
+                        const uint32_t* offsets, uint32_t K, __half* kv, float2* T, uint64_t m_max, cudaStream_t s);
 
 namespace {
 
@@ -79,7 +89,7 @@ constexpr uint32_t OFF_LP = OFF_HEAD + (8 * D + 8) * 4;    // every block's, the
 constexpr uint32_t SMEM_BYTES = OFF_LP + (kMaxL * LP_FLOATS + 2 * D) * 4;
 constexpr uint32_t TMEM_WG = 256;  // columns per warpgroup: [0,192) qkv / o / f1 buffers, [192,256) acc2
 constexpr uint64_t kWaitNs = 2000000000ull;
-constexpr int MODE_FULL = 0, MODE_NODES = 1;
+constexpr int MODE_FULL = 0, MODE_NODES = 1, MODE_SUFFIX = 2;
 static_assert(2 * A_BYTES <= KV_BYTES, "hidden chunks live in the k|v region");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
@@ -94,12 +104,17 @@ struct Args {
   Count n_seq;
   int P, last_only;  // NODES: P = the level
   float* raw;
+  __half* kv;           // NODES: [node][L][2 D]; FULL and SUFFIX: [sequence (parent)][L][n][2 D]
+  int keep_kv;          // the rows' keys and values are needed by a later launch
   // NODES (x, n_seq: the level's prefixes)
   const uint32_t* anc;  // [row][TRIE_ANC] node ids of the prefix's own prefixes, levels 0..P-1
-  __half* kv;           // [node][L][2 D]
   uint64_t node0;       // id of the level's first node
-  int keep_kv;          // the level's keys and values are needed by a later one
   float2* terms;        // [node][4]
+  // SUFFIX (x: the connected determinants)
+  const uint32_t* perm;     // them in ascending first differing slot
+  const uint32_t* offsets;  // offsets[j]: those with a smaller one
+  uint32_t K;
+  float2* T;
   int* status;
 };
 
@@ -223,7 +238,7 @@ __device__ __forceinline__ void f16x8_to_f32(const uint4 u, float (&f)[8]) {
   }
 }
 
-template <int DH>
+template <int DH, int MODE>
 __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
   constexpr int H = D / DH;
   constexpr uint32_t IDESC_QKV = tc::idesc_f16_f32(MT, 3 * D);
@@ -269,13 +284,23 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
     }
     for (int i = threadIdx.x; i < 2 * D; i += NT) s_lp[kMaxL * LP_FLOATS + i] = a.params[tail + i];
   }
-  const int P = a.mode == MODE_FULL ? a.P : 1;     // rows per sequence
-  const int t0 = a.mode == MODE_FULL ? 0 : a.P;    // their first position
-  const int S = MT / P;                            // sequences per tile
-  const uint64_t n_seq = a.n_seq.get(), total = (n_seq + S - 1) / S;
+  int P = MODE == MODE_FULL ? a.P : 1;          // rows per sequence
+  int t0 = MODE == MODE_NODES ? a.P : 0;        // their first position
+  int S = MT / P;                               // sequences per tile
+  uint64_t n_seq = MODE == MODE_SUFFIX ? 0 : a.n_seq.get(), total = (n_seq + S - 1) / S;
+  __shared__ uint64_t s_tiles[MODE == MODE_SUFFIX ? ANQS_MAX_ORB + 1 : 1];  // SUFFIX: first tile of each group
+  if (MODE == MODE_SUFFIX && threadIdx.x == 0) {
+    uint64_t k = 0;
+    s_tiles[0] = 0;
+    for (int j = 0; j < n - 1; ++j) {  // n - 1 - j positions each
+      const uint32_t cnt = __ldcg(a.offsets + j + 1) - __ldcg(a.offsets + j), per = uint32_t(MT / (n - 1 - j));
+      s_tiles[j + 1] = k += (cnt + per - 1) / per;
+    }
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  if constexpr (MODE == MODE_SUFFIX) total = s_tiles[n - 1];
   const uint32_t tmem = s_tmem + uint32_t(wg) * TMEM_WG;
   const uint32_t lane_base = uint32_t((t & ~31)) << 16;
   unsigned char* sA = smem + OFF_WG + wg * WG_BYTES;
@@ -297,8 +322,24 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
     const bool more = pair + gridDim.x < n_pairs;
     // ---- this warpgroup's tile and this thread's row ----
     const uint64_t tile = 2 * pair + wg;
-    const uint64_t seq = tile * S + t / P;
-    const bool valid = t / P < S && seq < n_seq;
+    uint64_t seq, parent = 0;
+    bool valid;
+    if constexpr (MODE == MODE_SUFFIX) {
+      int g = 0;
+      P = 1, S = MT, t0 = 1;
+      valid = tile < total;
+      if (valid) {
+        while (s_tiles[g + 1] <= tile) ++g;
+        P = n - 1 - g, S = MT / P, t0 = g + 1;
+      }
+      const uint64_t at = valid ? __ldcg(a.offsets + g) + (tile - s_tiles[g]) * S + t / P : 0;
+      valid = valid && t / P < S && at < __ldcg(a.offsets + g + 1);
+      seq = valid ? a.perm[at] : 0;
+      parent = seq / a.K;
+    } else {
+      seq = tile * S + t / P;
+      valid = t / P < S && seq < n_seq;
+    }
     const int pos = valid ? t0 + t % P : 0;
     const uint64_t x = valid ? a.x[seq] : 0;
     const int row0 = t - t % P;  // tile row of this sequence's first position
@@ -358,7 +399,8 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
         if (valid && a.keep_kv) {
-          uint4* g = reinterpret_cast<uint4*>(a.kv + ((a.node0 + seq) * L + l) * (2 * D) + (c0 - D));
+          const uint64_t at = MODE == MODE_FULL ? (seq * L + l) * P + pos : (a.node0 + seq) * L + l;
+          uint4* g = reinterpret_cast<uint4*>(a.kv + at * (2 * D) + (c0 - D));
 #pragma unroll
           for (int q = 0; q < 4; ++q) g[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
         }
@@ -366,6 +408,9 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
       __syncthreads();
       // causal attention of this row over the keys 0..pos
       const uint32_t* anc = a.anc + seq * TRIE_ANC;
+      auto key_node = [&](int u) -> uint32_t {
+        return MODE == MODE_SUFFIX ? uint32_t(u) : __ldcg(anc + u);
+      };
 #pragma unroll 1
       for (int hd = 0; hd < H; ++hd) {
         float q[DH];
@@ -407,15 +452,16 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
           }
           m = mn;
         };
-        // keys of positions < t0 (NODES) from the nodes' keys and values in
+        // keys of positions < t0 (NODES, SUFFIX) from the nodes' keys and values in
         // global memory (the next key's words are loaded before this key's
         // arithmetic), then the tile's own keys from shared memory
         const int n_anc = min(upto + 1, t0);
         if (n_anc > 0) {
-          const uint4* gp = reinterpret_cast<const uint4*>(a.kv) + size_t(l) * (2 * D / 8) + (hd * DH) / 8;
-          const size_t node = size_t(L) * (2 * D / 8);
-          uint32_t id = __ldcg(anc + (n_anc > 1 ? 1 : 0));
-          const uint4* p = gp + __ldcg(anc) * node;
+          const size_t first = MODE == MODE_SUFFIX ? (parent * L + l) * n : size_t(l);
+          const uint4* gp = reinterpret_cast<const uint4*>(a.kv) + first * (2 * D / 8) + (hd * DH) / 8;
+          const size_t node = MODE == MODE_SUFFIX ? 2 * D / 8 : size_t(L) * (2 * D / 8);
+          uint32_t id = key_node(n_anc > 1 ? 1 : 0);
+          const uint4* p = gp + key_node(0) * node;
           uint4 kw[DH / 8], vw[DH / 8];
 #pragma unroll
           for (int e = 0; e < DH / 8; ++e) kw[e] = __ldg(p + e), vw[e] = __ldg(p + D / 8 + e);
@@ -423,7 +469,7 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
           for (int u = 0; u < n_anc; ++u) {
             uint4 kn[DH / 8], vn[DH / 8];
             p = gp + id * node;
-            id = __ldcg(anc + min(u + 2, n_anc - 1));
+            id = key_node(min(u + 2, n_anc - 1));
 #pragma unroll
             for (int e = 0; e < DH / 8; ++e) kn[e] = __ldg(p + e), vn[e] = __ldg(p + D / 8 + e);
             step(kw, vw);
@@ -584,7 +630,7 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
         for (int o = 0; o < 8; ++o) out[o] = fmaf(y, s_head[o * D + c], out[o]);
       }
       if (valid) {
-        if (a.mode == MODE_FULL) {
+        if constexpr (MODE == MODE_FULL) {
           if (!a.last_only || pos == a.P - 1) {
             float4* dst = reinterpret_cast<float4*>(a.raw + (a.last_only ? seq : seq * a.P + pos) * 8);
             dst[0] = make_float4(out[0], out[1], out[2], out[3]);
@@ -608,10 +654,31 @@ __global__ void __launch_bounds__(NT, 1) tf_tc_kernel(Args a) {
           float tm[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) tm[u] = ((pmk >> u) & 1u) ? 0.5f * (out[u] - lse) : -INFINITY;
-          float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
-          dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
-          dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
+          if constexpr (MODE == MODE_NODES) {
+            float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
+            dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
+            dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
+          } else {
+            // the row's term to shared memory (the k|v region is free now); the
+            // sequence's first row adds its positions' terms below
+            const int v = int((x >> (2 * pos)) & 3ull);
+            reinterpret_cast<float2*>(sKV)[t] =
+                make_float2(v == 0 ? tm[0] : v == 1 ? tm[1] : v == 2 ? tm[2] : tm[3],
+                            v == 0 ? out[4] : v == 1 ? out[5] : v == 2 ? out[6] : out[7]);
+          }
         }
+      }
+    }
+    if constexpr (MODE == MODE_SUFFIX) {
+      __syncthreads();
+      if (valid && pos == t0) {
+        const float2* tr = reinterpret_cast<const float2*>(sKV) + t;
+        float sl = 0.f, sp = 0.f;
+        for (int i = 0; i < P; ++i) {
+          sl += tr[i].x;
+          sp += tr[i].y;
+        }
+        a.T[seq] = make_float2(sl, sp);
       }
     }
     __syncthreads();  // shared k|v and hidden buffers are rewritten by the next tile
@@ -647,13 +714,16 @@ int launch(const anqs_model* M, Args a, uint64_t max_tiles, int prof, cudaStream
   const unsigned grid = unsigned(std::max<uint64_t>(1, std::min<uint64_t>(pairs, uint64_t(sms()))));
   const int dh = D / M->d.n_heads;
   ProfScope ps(prof, s);
-  if (dh == 16) {
-    ANQS_CUDA(cudaFuncSetAttribute(tf_tc_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES)));
-    ANQS_CUDA_LAUNCH("tf_tc_kernel", launch_k(tf_tc_kernel<16>, dim3(grid), dim3(NT), SMEM_BYTES, s, a));
-  } else {
-    ANQS_CUDA(cudaFuncSetAttribute(tf_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES)));
-    ANQS_CUDA_LAUNCH("tf_tc_kernel", launch_k(tf_tc_kernel<32>, dim3(grid), dim3(NT), SMEM_BYTES, s, a));
-  }
+  auto go = [&](auto kern) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES));
+    return e != cudaSuccess ? e : launch_k(kern, dim3(grid), dim3(NT), SMEM_BYTES, s, a);
+  };
+  auto mode = [&](auto dh_c) -> cudaError_t {
+    constexpr int DH = decltype(dh_c)::value;
+    if (a.mode == MODE_FULL) return go(tf_tc_kernel<DH, MODE_FULL>);
+    return a.mode == MODE_NODES ? go(tf_tc_kernel<DH, MODE_NODES>) : go(tf_tc_kernel<DH, MODE_SUFFIX>);
+  };
+  ANQS_CUDA_LAUNCH("tf_tc_kernel", dh == 16 ? mode(std::integral_constant<int, 16>{}) : mode(std::integral_constant<int, 32>{}));
   return ANQS_OK;
 }
 
@@ -704,6 +774,108 @@ size_t plan_leaves(const anqs_ham* H, uint64_t n_x, Arena& A, TfLeafWs& w) {
   w.tab = A.take<float2>(w.u.max_leaves * (n + 1));
   w.counts = A.take<uint64_t>((w.u.max_leaves + kChunk - 1) / kChunk);
   return A.off;
+}
+
+// Scratch of the form over every connected determinant's own positions
+struct TfSuffixWs {
+  uint64_t* xp;
+  double* hv;
+  uint8_t* js;
+  double* hd;
+  float *la_x, *ph_x, *raw, *cache;
+  float2* T;  // per connected determinant
+  uint32_t *perm, *hist, *cursor, *offsets, *ticket;
+  __half* kv;  // [n_x][L][n][2 d]
+};
+
+size_t plan_suffix(const anqs_model* M, const anqs_ham* H, uint64_t n_x, Arena& A, TfSuffixWs& w) {
+  const uint64_t n = H->v.n, m = n_x * H->v.K;
+  w.xp = A.take<uint64_t>(m);
+  w.hv = A.take<double>(m);
+  w.js = A.take<uint8_t>(m);
+  w.hd = A.take<double>(n_x);
+  w.la_x = A.take<float>(n_x);
+  w.ph_x = A.take<float>(n_x);
+  w.raw = A.take<float>(n_x * n * 8);
+  w.cache = A.take<float>(n_x * n * TC_CACHE_F);
+  w.T = A.take<float2>(m);
+  w.perm = A.take<uint32_t>(m);
+  w.cursor = A.take<uint32_t>(ANQS_MAX_ORB);
+  w.offsets = A.take<uint32_t>(ANQS_MAX_ORB + 1);
+  w.hist = A.take<uint32_t>(TC_CTL_WORDS);
+  w.ticket = w.hist + TC_CTL_STATS_TICKET;
+  w.kv = A.take<__half>(n_x * uint64_t(M->d.n_layers) * n * 2 * uint64_t(M->d.d_model));
+  return A.off;
+}
+
+// The three forms of a local energy: every position of every distinct
+// determinant (sectors with a prefix index), each sample's prefix tree level by
+// level, the positions after the first difference of every connected
+// determinant.
+enum TfForm { TF_LEAVES, TF_TREE, TF_SUFFIX };
+
+size_t form_bytes(const anqs_model* M, const anqs_ham* H, uint64_t n_x, TfForm f) {
+  Arena A(nullptr, 0);
+  if (f == TF_LEAVES) {
+    TfLeafWs w;
+    return plan_leaves(H, n_x, A, w);
+  }
+  if (f == TF_TREE) {
+    TfTrieWs w;
+    return plan_trie_tf(M, H, n_x, A, w);
+  }
+  TfSuffixWs w;
+  return plan_suffix(M, H, n_x, A, w);
+}
+
+// Which form takes the least time.
+//
+// Distinct determinants, in sectors with an index: few samples share hardly any
+// determinant, and then a position costs about as much as one of the suffixes,
+// of which there are 0.85 (n - 1) per connected determinant against n.  Both
+// meet at about 24 samples of 64 dimensions and one block, fewer of larger
+// models (us, 13 orbitals, 4 + 4 electrons, distinct and suffixes: one block, 4
+// samples 220 and 142, 16 samples 334 and 309; two blocks, 4 samples 282 and
+// 229, 16 samples 457 and 522; 128 dimensions and two blocks, 8 samples 569 and
+// 657).  One wave of tiles is always the better one (131 and 150, 10 orbitals,
+// 7 + 7 electrons).
+//
+// Prefix trees take four launches per level, each waiting for the one before,
+// and 0.34 to 0.45 as many rows as the suffixes: the times below fit 508
+// measurements of 5 to 32 orbitals, 1 to 872 samples, 1 to 4 blocks, and choose
+// the slower form for ten of them, by 14% at most.  26 orbitals, 9 + 9
+// electrons, 64 dimensions, two blocks: one sample 1.7 ms by suffixes, 2.5 by
+// trees, eight 10.9 and 7.4.
+TfForm preferred_form(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  const int n = H->v.n, L = M->d.n_layers;
+  const bool wide = M->d.d_model == 128;
+  const double K = H->v.K, m = double(n_x);
+  if (unique_applies(H, n_x)) {
+    const double wave = double(MT / n) * sms() * (wide ? 1 : 2);
+    const double sector = double(H->sv.na_p[n]) * H->sv.nb_p[n];
+    if (unique_full(H, n_x) || std::min(sector, m * (K + 1)) <= wave || n_x * uint64_t(L) * (wide ? 2 : 1) >= 24)
+      return TF_LEAVES;
+  }
+  TfTrieWs w;
+  Arena A(nullptr, 0);
+  plan_trie_tf(M, H, n_x, A, w);
+  const double groups = double((n_x + w.t.group - 1) / w.t.group), rows_t = double(w.t.node0[n]) / double(w.t.group) * m;
+  const double rows_s = 0.85 * (n - 1) * K * m;
+  // us per level, ns per row and block
+  const double level = wide ? 20 + L * (12 + 0.88 * n) : 15 + L * (8 + 1.1 * n);
+  const double row_t = wide ? 0.5 + 0.07 * n : 0.25 + 0.05 * n, row_s = wide ? 1.1 + 0.045 * n : 0.33 + 0.0245 * n;
+  const double tree = groups * n * level + 1e-3 * rows_t * L * row_t, suffix = 100 + 1e-3 * rows_s * L * row_s;
+  return tree < suffix ? TF_TREE : TF_SUFFIX;
+}
+
+// the preferred form if its scratch fits into the workspace, else the first
+// that does (a workspace may have been sized for another number of samples, or
+// to be small)
+TfForm form_of(const anqs_model* M, const anqs_ham* H, uint64_t n_x, size_t ws_bytes) {
+  const TfForm pref = preferred_form(M, H, n_x);
+  for (TfForm f : {pref, TF_LEAVES, TF_TREE, TF_SUFFIX})
+    if ((f != TF_LEAVES || H->has_index) && form_bytes(M, H, n_x, f) <= ws_bytes) return f;
+  return pref;
 }
 
 }  // namespace
@@ -765,21 +937,71 @@ int launch_tf_tc_slot_logits(const anqs_model* M, int p, const uint64_t* pre, co
   return launch(M, a, (max_rows + S - 1) / S, PROF_TF_TC_SLOT, s);
 }
 
-size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x, bool unique) {
-  Arena A(nullptr, 0);
-  if (unique) {
-    TfLeafWs v;
-    return plan_leaves(H, n_x, A, v);
+size_t tf_tc_eloc_workspace(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  return form_bytes(M, H, n_x, preferred_form(M, H, n_x));
+}
+
+size_t tf_tc_eloc_workspace_least(const anqs_model* M, const anqs_ham* H, uint64_t n_x) {
+  const size_t least = std::min(form_bytes(M, H, n_x, TF_TREE), form_bytes(M, H, n_x, TF_SUFFIX));
+  return H->has_index ? std::min(least, form_bytes(M, H, n_x, TF_LEAVES)) : least;
+}
+
+static int run_suffix(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
+                      const uint64_t* counts, double* stats, const TfSuffixWs& w, cudaStream_t s) {
+  const int n = H->v.n;
+  const uint64_t K = H->v.K;
+  const Count mc = scaled(n_x, K);
+  ANQS_TRY(launch_connected(H->v, x, n_x, w.xp, w.hv, w.js, w.hd, s, w.hist));
+  if (M->d.d_model == 128) {
+    ANQS_TRY(launch_tf128_full(M, H->v, x, n_x, n, 0, w.raw, PROF_TF_TC_PARENT, s, w.kv));
+  } else {
+    Args a = full_args(x, n_x, n, 0, w.raw, H->v);
+    a.kv = w.kv;
+    a.keep_kv = 1;
+    ANQS_TRY(launch(M, a, (n_x.n + MT / n - 1) / (MT / n), PROF_TF_TC_PARENT, s));
   }
-  TfTrieWs w;
-  return plan_trie_tf(M, H, n_x, A, w);
+  {
+    ProfScope ps(PROF_TC_FINALIZE, s);
+    ANQS_TRY(launch_tc_finalize(H->v, x, n_x, w.raw, w.la_x, w.ph_x, w.cache, s));
+  }
+  {
+    ProfScope ps(PROF_TC_SORT, s);
+    ANQS_TRY(launch_js_sort(w.js, mc, n, w.hist, w.cursor, w.offsets, w.perm, s));
+  }
+  if (M->d.d_model == 128) {
+    ANQS_TRY(launch_tf128_suffix(M, H->v, w.xp, w.perm, w.offsets, uint32_t(K), w.kv, w.T, mc.n, s));
+  } else {
+    Args a{};
+    a.mode = MODE_SUFFIX;
+    a.hv = H->v;
+    a.x = w.xp;
+    a.perm = w.perm;
+    a.offsets = w.offsets;
+    a.K = uint32_t(K);
+    a.kv = w.kv;
+    a.T = w.T;
+    uint64_t tiles = 0;  // upper bound over the groups
+    for (int j = 0; j + 1 < n; ++j) tiles += mc.n / uint64_t(MT / (n - 1 - j)) + 1;
+    ANQS_TRY(launch(M, a, tiles, PROF_TF_TC_SUFFIX, s));
+  }
+  ProfScope ps(PROF_TC_ELOC, s);
+  return launch_eloc_assemble(n, uint32_t(K), n_x, w.xp, w.js, w.cache, w.T, w.hv, w.hd, w.la_x, w.ph_x, ere, eim,
+                              StatsOut{counts, stats, w.ticket}, s, true);
 }
 
 int run_eloc_tf_tc(const anqs_model* M, const anqs_ham* H, const uint64_t* x, Count n_x, double* ere, double* eim,
                    const uint64_t* counts, double* stats, void* ws, size_t ws_bytes, cudaStream_t s) {
   Arena A(ws, ws_bytes);
-  if (use_unique(H, unique_applies(H, n_x.n), tf_tc_eloc_workspace(M, H, n_x.n, false),
-                 H->has_index ? tf_tc_eloc_workspace(M, H, n_x.n, true) : 0, ws_bytes)) {
+  const TfForm form = form_of(M, H, n_x.n, ws_bytes);
+  if (form == TF_SUFFIX) {
+    TfSuffixWs v;
+    plan_suffix(M, H, n_x.n, A, v);
+    if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);
+    if (n_x.n * H->v.K > 0xffffffffull)
+      return set_error(ANQS_ERR_UNSUPPORTED, "more than 2^32 connected determinants per call");
+    return run_suffix(M, H, x, n_x, ere, eim, counts, stats, v, s);
+  }
+  if (form == TF_LEAVES) {
     TfLeafWs v;
     plan_leaves(H, n_x.n, A, v);
     if (!A.fits()) return set_error(ANQS_ERR_CAPACITY, "workspace needs %zu bytes", A.off);

@@ -44,9 +44,14 @@
 //           own prefixes (levels < p, found through its table) and to itself;
 //           keeps its keys and values for the later levels and writes the
 //           masked half-log-probability and the phase of each outcome.
+//   SUFFIX  connected determinants x' grouped by first differing slot j:
+//           positions j+1..n-1 only, keys and values of positions <= j from
+//           the parent's (kept by FULL); writes the sums T[x'] of the masked
+//           slot terms (the form of few samples).
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cmath>
 
 #include "common.cuh"
@@ -78,7 +83,7 @@ constexpr uint32_t OFF_LP = OFF_HX + MT * 8 * 4;              // the layer's Lay
 constexpr uint32_t LP_FLOATS = 14 * D;                         // ln1 g,b | bq bk bv bo | ln2 g,b | b1 (4D) | b2
 constexpr uint32_t SMEM_BYTES = OFF_LP + LP_FLOATS * 4;
 constexpr uint64_t kWaitNs = 2000000000ull;
-constexpr int MODE_FULL = 0, MODE_NODES = 1;
+constexpr int MODE_FULL = 0, MODE_NODES = 1, MODE_SUFFIX = 2;
 // chunk indices within a layer
 enum { C_Q = 0, C_K, C_V, C_O, C_W1_0, C_W1_1, C_W2_0, C_W1_2, C_W2_1, C_W1_3, C_W2_2, C_W2_3 };
 static_assert(2 * A_BYTES <= KV_BYTES, "hidden chunks live in the k|v region");
@@ -95,12 +100,17 @@ struct Args {
   Count n_seq;
   int P, last_only;  // NODES: P = the level
   float* raw;
+  __half* kv;           // NODES: [node][L][2 D]; FULL and SUFFIX: [sequence (parent)][L][n][2 D]
+  int keep_kv;          // the rows' keys and values are needed by a later launch
   // NODES (x, n_seq: the level's prefixes)
   const uint32_t* anc;  // [row][TRIE_ANC] node ids of the prefix's own prefixes, levels 0..P-1
-  __half* kv;           // [node][L][2 D]
   uint64_t node0;       // id of the level's first node
-  int keep_kv;          // the level's keys and values are needed by a later one
   float2* terms;        // [node][4]
+  // SUFFIX (x: the connected determinants)
+  const uint32_t* perm;     // them in ascending first differing slot
+  const uint32_t* offsets;  // offsets[j]: those with a smaller one
+  uint32_t K;
+  float2* T;
   int* status;
 };
 
@@ -363,13 +373,23 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
     const size_t tail = 5 * size_t(D) + size_t(n) * D + size_t(L) * layer_floats();
     for (int i = threadIdx.x; i < 8 * D + 8; i += NT) s_head[i] = a.params[tail + 2 * D + i];
   }
-  const int P = MODE == MODE_FULL ? a.P : 1;     // rows per sequence
-  const int t0 = MODE == MODE_FULL ? 0 : a.P;    // their first position
-  const int S = MT / P;                            // sequences per tile
-  const uint64_t n_seq = a.n_seq.get(), total = (n_seq + S - 1) / S;
+  int P = MODE == MODE_FULL ? a.P : 1;          // rows per sequence
+  int t0 = MODE == MODE_NODES ? a.P : 0;        // their first position
+  int S = MT / P;                               // sequences per tile
+  uint64_t n_seq = MODE == MODE_SUFFIX ? 0 : a.n_seq.get(), total = (n_seq + S - 1) / S;
+  __shared__ uint64_t s_tiles[MODE == MODE_SUFFIX ? ANQS_MAX_ORB + 1 : 1];  // SUFFIX: first tile of each group
+  if (MODE == MODE_SUFFIX && threadIdx.x == 0) {
+    uint64_t k = 0;
+    s_tiles[0] = 0;
+    for (int j = 0; j < n - 1; ++j) {  // n - 1 - j positions each
+      const uint32_t cnt = __ldcg(a.offsets + j + 1) - __ldcg(a.offsets + j), per = uint32_t(MT / (n - 1 - j));
+      s_tiles[j + 1] = k += (cnt + per - 1) / per;
+    }
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  if constexpr (MODE == MODE_SUFFIX) total = s_tiles[n - 1];
   const uint32_t w_addr = tc::smem_u32(smem + OFF_W);
   const uint32_t bar_full = tc::smem_u32(&bars[0]), bar_empty = tc::smem_u32(&bars[NS]);
   const uint32_t bar_m = tc::smem_u32(&bars[2 * NS]), bar_2 = tc::smem_u32(&bars[2 * NS + 1]);
@@ -395,8 +415,20 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
     const int cb = h * HD;  // this half's first model dimension
     for (uint64_t tile = blockIdx.x; ok && tile < total; tile += gridDim.x) {
       // ---- this thread's row
-      const uint64_t seq = tile * S + t / P;
-      const bool valid = t / P < S && seq < n_seq;
+      uint64_t seq, parent = 0;
+      bool valid;
+      if constexpr (MODE == MODE_SUFFIX) {
+        int g = 0;
+        while (s_tiles[g + 1] <= tile) ++g;
+        P = n - 1 - g, S = MT / P, t0 = g + 1;
+        const uint64_t at = __ldcg(a.offsets + g) + (tile - s_tiles[g]) * S + t / P;
+        valid = t / P < S && at < __ldcg(a.offsets + g + 1);
+        seq = valid ? a.perm[at] : 0;
+        parent = seq / a.K;
+      } else {
+        seq = tile * S + t / P;
+        valid = t / P < S && seq < n_seq;
+      }
       const int pos = valid ? t0 + t % P : 0;
       const uint64_t x = valid ? a.x[seq] : 0;
       const int row0 = t - t % P;  // tile row of this sequence's first position
@@ -587,6 +619,11 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
               uint4* dst = reinterpret_cast<uint4*>(sKV + t * KV_STRIDE + off * 2);
 #pragma unroll
               for (int q = 0; q < 4; ++q) dst[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+              if (MODE == MODE_FULL && valid && a.keep_kv) {
+                uint4* gd = reinterpret_cast<uint4*>(a.kv + ((seq * L + l) * P + pos) * (2 * D) + off);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) gd[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+              }
             }
           }
           csync();
@@ -633,7 +670,26 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
               }
               m = mn;
             };
-            // the sequence's keys from shared memory
+            // SUFFIX: keys of positions < t0 from the parent's in global memory
+            // (the next key's words are loaded before this key's arithmetic)
+            const int n_par = MODE == MODE_SUFFIX ? min(upto + 1, t0) : 0;
+            if (n_par > 0) {
+              const uint4* gp = reinterpret_cast<const uint4*>(a.kv) + (parent * L + l) * n * (2 * D / 8) + (hd * DH) / 8;
+              uint4 kw[DH / 8], vw[DH / 8];
+#pragma unroll
+              for (int e = 0; e < DH / 8; ++e) kw[e] = __ldg(gp + e), vw[e] = __ldg(gp + D / 8 + e);
+#pragma unroll 1
+              for (int u = 0; u < n_par; ++u) {
+                uint4 kn[DH / 8], vn[DH / 8];
+                const uint4* np = gp + min(u + 1, n_par - 1) * (2 * D / 8);
+#pragma unroll
+                for (int e = 0; e < DH / 8; ++e) kn[e] = __ldg(np + e), vn[e] = __ldg(np + D / 8 + e);
+                step(kw, vw);
+#pragma unroll
+                for (int e = 0; e < DH / 8; ++e) kw[e] = kn[e], vw[e] = vn[e];
+              }
+            }
+            // the sequence's own keys from shared memory
 #pragma unroll 1
             for (int u = t0; u <= upto; ++u) {
               const uint4* sp = reinterpret_cast<const uint4*>(sKV + (row0 + u - t0) * KV_STRIDE);
@@ -797,10 +853,31 @@ __global__ void __launch_bounds__(NT, 1) tf128_kernel(Args a) {
             float tm[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) tm[u] = ((pmk >> u) & 1u) ? 0.5f * (out[u] - lse) : -INFINITY;
-            float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
-            dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
-            dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
+            if constexpr (MODE == MODE_NODES) {
+              float4* dst = reinterpret_cast<float4*>(a.terms + (a.node0 + seq) * 4);
+              dst[0] = make_float4(tm[0], out[4], tm[1], out[5]);
+              dst[1] = make_float4(tm[2], out[6], tm[3], out[7]);
+            } else {
+              // the row's term to its own exchange slot (read above); the
+              // sequence's first row adds its positions' terms below
+              const int v = int((x >> (2 * pos)) & 3ull);
+              reinterpret_cast<float2*>(s_hx + t * 8)[0] =
+                  make_float2(v == 0 ? tm[0] : v == 1 ? tm[1] : v == 2 ? tm[2] : tm[3],
+                              v == 0 ? out[4] : v == 1 ? out[5] : v == 2 ? out[6] : out[7]);
+            }
           }
+        }
+      }
+      if constexpr (MODE == MODE_SUFFIX) {
+        csync();
+        if (h == 0 && valid && pos == t0) {
+          float sl = 0.f, sp = 0.f;
+          for (int i = 0; i < P; ++i) {
+            const float2 tv = reinterpret_cast<const float2*>(s_hx + (t + i) * 8)[0];
+            sl += tv.x;
+            sp += tv.y;
+          }
+          a.T[seq] = make_float2(sl, sp);
         }
       }
       csync();  // shared k|v, hidden buffers and exchange slots are rewritten by the next tile
@@ -839,9 +916,12 @@ int launch(const anqs_model* M, Args a, uint64_t max_tiles, int prof, cudaStream
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(SMEM_BYTES));
     return e != cudaSuccess ? e : launch_k(kern, dim3(grid), dim3(NT), SMEM_BYTES, s, a);
   };
-  ANQS_CUDA_LAUNCH("tf128_kernel", a.mode == MODE_NODES
-                                       ? (dh == 16 ? go(tf128_kernel<16, MODE_NODES>) : go(tf128_kernel<32, MODE_NODES>))
-                                       : (dh == 16 ? go(tf128_kernel<16, MODE_FULL>) : go(tf128_kernel<32, MODE_FULL>)));
+  auto mode = [&](auto dh_c) -> cudaError_t {
+    constexpr int DH = decltype(dh_c)::value;
+    if (a.mode == MODE_FULL) return go(tf128_kernel<DH, MODE_FULL>);
+    return a.mode == MODE_NODES ? go(tf128_kernel<DH, MODE_NODES>) : go(tf128_kernel<DH, MODE_SUFFIX>);
+  };
+  ANQS_CUDA_LAUNCH("tf128_kernel", dh == 16 ? mode(std::integral_constant<int, 16>{}) : mode(std::integral_constant<int, 32>{}));
   return ANQS_OK;
 }
 
@@ -875,8 +955,10 @@ int tf128_pack(anqs_model* M, cudaStream_t s) {
 int tf128_status_offset(const anqs_model* M) { return int(size_t(M->d.n_layers) * LAYER_BYTES); }
 
 int launch_tf128_full(const anqs_model* M, const HamView& hv, const uint64_t* x, Count n_seq, int P, int last_only,
-                      float* raw, int prof, cudaStream_t s) {
+                      float* raw, int prof, cudaStream_t s, __half* kv) {
   Args a = full_args(x, n_seq, P, last_only, raw, hv);
+  a.kv = kv;
+  a.keep_kv = kv != nullptr;
   const uint64_t S = MT / P;
   return launch(M, a, (n_seq.n + S - 1) / S, prof, s);
 }
@@ -895,6 +977,22 @@ int launch_tf128_nodes(const anqs_model* M, const HamView& hv, const TrieLevel& 
   a.keep_kv = lv.p + 1 < hv.n;
   a.terms = terms;
   return launch(M, a, (lv.rows.n + MT - 1) / MT, PROF_TF_TC_SUFFIX, s);
+}
+
+int launch_tf128_suffix(const anqs_model* M, const HamView& hv, const uint64_t* xp, const uint32_t* perm,
+                        const uint32_t* offsets, uint32_t K, __half* kv, float2* T, uint64_t m_max, cudaStream_t s) {
+  Args a{};
+  a.mode = MODE_SUFFIX;
+  a.hv = hv;
+  a.x = xp;
+  a.perm = perm;
+  a.offsets = offsets;
+  a.K = K;
+  a.kv = kv;
+  a.T = T;
+  uint64_t tiles = 0;  // upper bound over the groups
+  for (int j = 0; j + 1 < hv.n; ++j) tiles += m_max / uint64_t(MT / (hv.n - 1 - j)) + 1;
+  return launch(M, a, tiles, PROF_TF_TC_SUFFIX, s);
 }
 
 }  // namespace anqs

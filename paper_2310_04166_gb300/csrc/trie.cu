@@ -383,43 +383,45 @@ __global__ void __launch_bounds__(FT) trie_finish_kernel(Count n_x_, int parts, 
   cta_energy_stats<FT>(ere, eim, counts, n_x, stats);
 }
 
-uint64_t choose(int n, int k) {
-  if (k < 0 || k > n) return 0;
-  uint64_t r = 1;
-  for (int i = 1; i <= k; ++i) r = r * uint64_t(n - k + i) / uint64_t(i);
-  return r;
-}
-
-// Most distinct prefixes of t slots that one sample's connected determinants
-// (and the sample) can have, over how many electrons the sample has there
-uint64_t level_nodes(const HamView& hv, int t) {
-  // prefixes of one spin that take k moves, for a of ne electrons in the t slots
-  auto count = [&](int a, int ne, int k) {
-    const int occ = ne - a, vir = hv.n - t - occ;
-    uint64_t c = 0;
-    for (int r = 0; r <= k; ++r)
-      for (int s = 0; s <= k; ++s)
-        if (std::max(r, s) == k && k - r <= occ && k - s <= vir) c += choose(a, r) * choose(t - a, s);
-    return c;
-  };
-  uint64_t best = 0;
-  for (int a = std::max(0, hv.na - (hv.n - t)); a <= std::min(t, hv.na); ++a)
-    for (int b = std::max(0, hv.nb - (hv.n - t)); b <= std::min(t, hv.nb); ++b) {
-      uint64_t c = 0;
-      for (int k = 0; k <= 2; ++k)
-        for (int m = 0; k + m <= 2; ++m) c += count(a, hv.na, k) * count(b, hv.nb, m);
-      best = std::max(best, c);
-    }
-  return best;
-}
-
 }  // namespace
+
+// Most distinct prefixes of t = 0..n slots that one sample's connected
+// determinants (and the sample) can have, over how many electrons the sample
+// has there.  Once per Hamiltonian: a call asks for them several times.
+void trie_level_nodes(const HamView& hv, uint64_t* nodes) {
+  const int n = hv.n;
+  for (int t = 0; t <= n; ++t) {
+    // prefixes of one spin that take k moves, for a of ne electrons in the t slots: r removed and s added, k the
+    // larger, and the missing k - r and k - s still possible in the later slots
+    auto spin = [&](int a, int ne, uint64_t (&c)[3]) {
+      const int occ = ne - a, vir = n - t - occ, e = t - a;
+      const uint64_t A[3] = {1, uint64_t(a), uint64_t(a) * uint64_t(a > 0 ? a - 1 : 0) / 2};
+      const uint64_t B[3] = {1, uint64_t(e), uint64_t(e) * uint64_t(e > 0 ? e - 1 : 0) / 2};
+      for (int k = 0; k <= 2; ++k) {
+        c[k] = 0;
+        for (int r = 0; r <= k; ++r)
+          for (int s = 0; s <= k; ++s)
+            if (std::max(r, s) == k && k - r <= occ && k - s <= vir) c[k] += A[r] * B[s];
+      }
+    };
+    uint64_t cb[ANQS_MAX_ORB + 1][3], best = 0;
+    const int b0 = std::max(0, hv.nb - (n - t)), b1 = std::min(t, hv.nb);
+    for (int b = b0; b <= b1; ++b) spin(b, hv.nb, cb[b]);
+    for (int a = std::max(0, hv.na - (n - t)); a <= std::min(t, hv.na); ++a) {
+      uint64_t ca[3];
+      spin(a, hv.na, ca);
+      for (int b = b0; b <= b1; ++b)
+        best = std::max(best, ca[0] * (cb[b][0] + cb[b][1] + cb[b][2]) + ca[1] * (cb[b][0] + cb[b][1]) + ca[2] * cb[b][0]);
+    }
+    nodes[t] = best;
+  }
+}
 
 void plan_trie(const anqs_ham* H, uint64_t n_x, uint64_t max_nodes, Arena& A, TrieWs& w) {
   const int n = H->v.n;
   w = TrieWs{};
-  uint64_t per[ANQS_MAX_ORB + 1], inner = 0;
-  for (int p = 0; p <= n; ++p) per[p] = level_nodes(H->v, p);
+  const uint64_t* per = H->tree_nodes;
+  uint64_t inner = 0;
   for (int p = 0; p + 1 < n; ++p) inner += per[p];
   w.group = std::max<uint64_t>(1, inner ? max_nodes / inner : n_x);
   w.group = std::min(w.group, std::max<uint64_t>(1, (1ull << 31) / (uint64_t(H->v.K) + 1)));
