@@ -1,5 +1,6 @@
 // C ABI entry points of libanqs: argument checks, handles, sector table,
 // workspace planning and the order of kernel launches for each call.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -384,32 +385,25 @@ static int build_prefix_table(anqs_ham* H) {
 
 // Ranks of the sector's prefixes (SectorView) for up to IDX_MAX_ORB orbitals
 // and 2^30 determinants, and the list of all prefixes when levels 0..n-1 hold
-// at most kPrefixTable of them and level n at most four times that.
+// at most kPrefixTable of them and level n at most four times that.  One buffer,
+// filled in place, one allocation and one copy: a program that scans geometries
+// pays for it once per Hamiltonian (18 orbitals: 4 MB per spin, shared by two
+// spins of equally many electrons).
 static int build_index(anqs_ham* H) {
   const int n = H->v.n;
   if (n > IDX_MAX_ORB) return ANQS_OK;
   SectorView& sv = H->sv;
   sv.n = n;
-  std::vector<uint32_t> tab[2], str[2];  // rank tables, strings
+  const bool same = H->v.na == H->v.nb;
+  size_t strings[2] = {0, 0};
   for (int s = 0; s < 2; ++s) {
     const int ne = s ? H->v.nb : H->v.na;
-    tab[s].assign(size_t(2) << n, 0u);
-    // level p + 1's strings from level p's, in the order of the slots (slot 0
-    // first), so that neighbours share prefixes
-    std::vector<uint32_t> cur{0u}, nxt;
-    for (int p = 0;; ++p) {
-      (s ? sv.sob : sv.soa)[p] = uint32_t(str[s].size());
-      (s ? sv.nb_p : sv.na_p)[p] = uint32_t(cur.size());
-      for (size_t r = 0; r < cur.size(); ++r) tab[s][(size_t(1) << p) + cur[r]] = uint32_t(r);
-      str[s].insert(str[s].end(), cur.begin(), cur.end());
-      if (p == n) break;
-      nxt.clear();
-      for (uint32_t v : cur)
-        for (uint32_t bit = 0; bit < 2; ++bit) {
-          const int e = __builtin_popcount(v) + int(bit);
-          if (e <= ne && e + (n - p - 1) >= ne) nxt.push_back(v | bit << p);
-        }
-      cur.swap(nxt);
+    for (int p = 0; p <= n; ++p) {
+      uint64_t c = 0;  // strings of p slots that can still reach ne electrons
+      for (int e = std::max(0, ne - (n - p)); e <= std::min(p, ne); ++e) c += binom(p, e);
+      (s ? sv.sob : sv.soa)[p] = uint32_t(strings[s]);
+      (s ? sv.nb_p : sv.na_p)[p] = uint32_t(c);
+      strings[s] += size_t(c);
     }
   }
   uint64_t words = 0, below = 0;
@@ -423,7 +417,31 @@ static int build_index(anqs_ham* H) {
   sv.woff[n + 1] = uint32_t(words);
   const uint64_t leaves = uint64_t(sv.na_p[n]) * sv.nb_p[n];
   const bool full = below <= kPrefixTable && leaves <= 4 * kPrefixTable;
-  std::vector<uint64_t> xs;
+  // all prefixes (64 bits each) | rank tables | strings | level offsets
+  const size_t listed = full ? size_t(below + leaves) : 0, ranks = size_t(2) << n;
+  const size_t rk0 = 2 * listed, rk1 = same ? rk0 : rk0 + ranks, st0 = rk1 + ranks;
+  const size_t st1 = same ? st0 : st0 + strings[0], of0 = st1 + strings[same ? 0 : 1];
+  std::vector<uint32_t> all(of0 + (full ? size_t(n) + 2 : 0));
+  for (int s = 0; s < (same ? 1 : 2); ++s) {
+    const int ne = s ? H->v.nb : H->v.na;
+    const uint32_t *off = s ? sv.sob : sv.soa, *cnt = s ? sv.nb_p : sv.na_p;
+    uint32_t *rank = all.data() + (s ? rk1 : rk0), *str = all.data() + (s ? st1 : st0);
+    // level p + 1's strings from level p's, in the order of the slots (slot 0
+    // first), so that neighbours share prefixes
+    str[0] = 0u;
+    for (int p = 0; p < n; ++p) {
+      const uint32_t* cur = str + off[p];
+      uint32_t* nxt = str + off[p + 1];
+      for (uint32_t r = 0; r < cnt[p]; ++r) {
+        rank[(size_t(1) << p) + cur[r]] = r;
+        for (uint32_t bit = 0; bit < 2; ++bit) {
+          const int e = __builtin_popcount(cur[r]) + int(bit);
+          if (e <= ne && e + (n - p - 1) >= ne) *nxt++ = cur[r] | bit << p;
+        }
+      }
+    }
+    for (uint32_t r = 0; r < cnt[n]; ++r) rank[(size_t(1) << n) + str[off[n] + r]] = r;
+  }
   if (full) {
     auto spread = [](uint64_t x) {
       x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
@@ -432,33 +450,28 @@ static int build_index(anqs_ham* H) {
       x = (x | (x << 2)) & 0x3333333333333333ull;
       return (x | (x << 1)) & 0x5555555555555555ull;
     };
-    xs.reserve(below + leaves);
+    size_t k = 0;
     for (int p = 0; p <= n; ++p) {
-      H->full_off.push_back(uint32_t(xs.size()));
+      H->full_off.push_back(uint32_t(k));
       for (uint32_t a = 0; a < sv.na_p[p]; ++a) {
-        const uint64_t xa = spread(str[0][sv.soa[p] + a]);
-        for (uint32_t b = 0; b < sv.nb_p[p]; ++b) xs.push_back(xa | spread(str[1][sv.sob[p] + b]) << 1);
+        const uint64_t xa = spread(all[st0 + sv.soa[p] + a]);
+        for (uint32_t b = 0; b < sv.nb_p[p]; ++b, ++k) {
+          const uint64_t x = xa | spread(all[st1 + sv.sob[p] + b]) << 1;
+          memcpy(&all[2 * k], &x, sizeof(x));
+        }
       }
     }
-    H->full_off.push_back(uint32_t(xs.size()));
+    H->full_off.push_back(uint32_t(k));
+    std::copy(H->full_off.begin(), H->full_off.end(), all.begin() + ptrdiff_t(of0));
   }
-  // one allocation and copy: prefixes | rank tables | strings | level offsets
-  std::vector<uint32_t> all(2 * xs.size());
-  if (full) memcpy(all.data(), xs.data(), xs.size() * sizeof(uint64_t));
-  const size_t rk0 = all.size();
-  for (int s = 0; s < 2; ++s) all.insert(all.end(), tab[s].begin(), tab[s].end());
-  const size_t st0 = all.size();
-  for (int s = 0; s < 2; ++s) all.insert(all.end(), str[s].begin(), str[s].end());
-  const size_t of0 = all.size();
-  all.insert(all.end(), H->full_off.begin(), H->full_off.end());
   ANQS_CUDA(cudaMalloc(&H->d_idx, all.size() * sizeof(uint32_t)));
   ANQS_CUDA(cudaMemcpy(H->d_idx, all.data(), all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
   H->d_full_x = reinterpret_cast<uint64_t*>(H->d_idx);
   H->d_full_off = H->d_idx + of0;
   sv.rka = H->d_idx + rk0;
-  sv.rkb = sv.rka + tab[0].size();
+  sv.rkb = H->d_idx + rk1;
   sv.sta = H->d_idx + st0;
-  sv.stb = sv.sta + str[0].size();
+  sv.stb = H->d_idx + st1;
   H->has_index = true;
   H->has_full = full;
   return ANQS_OK;

@@ -393,3 +393,15 @@ def test_without_excitations(A, kind, form, n, na, nb, m):
     ere, eim, st = A.local_energy(model, ham, x, torch.ones_like(x))
     assert torch.allclose(ere, ref.expand(m), rtol=1e-13) and not eim.any()
     assert torch.allclose(st, torch.tensor([ref.item(), 0.0, 0.0, m], dtype=torch.float64, device="cuda"), rtol=1e-13)
+
+
+def test_transformer_leaves_in_chunks(A):
+    """More determinants than one chunk of 2^20 may hold (14 orbitals, 400 samples: a bound of 1.35e6), and the same
+    buffers with 30 rows, whose determinants leave the second chunk empty."""
+    model, ham = _tf16(A, 14, 7, 7, 64, 1, 3)
+    x = _dets(14, 7, 7, 400, 4)
+    assert x.numel() * (ham.n_connected + 1) > 1 << 20
+    e, bound = _reference(A, model, ham, x)
+    _agrees(A, model, ham, x, e, bound)
+    ere, eim, _ = A.local_energy(model, ham, x, n_dev=torch.tensor([30], dtype=torch.int64, device="cuda"))
+    assert torch.all((ere[:30] - e.real[:30]).abs() <= bound[:30]) and torch.all((eim[:30] - e.imag[:30]).abs() <= bound[:30])
