@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(NT, 1) mlp_tc_multi_kernel(const __grid_consta
 // kFlush tiles instead of once per tile; a reduction over the slabs follows.
 // Where a tile's scale is another than the sums', these are multiplied by the
 // quotient, a power of two, while the first layer's MMAs run (24 qubits, 20,000
-// samples: 200 us, 185 with one scale, 334 with a slab per tile).
+// samples: 198 us, 185 with one scale, 334 with a slab per tile).
 // One tile is a serial chain of MMA, wait and epilogue; what a tile cost
 // beyond it before was reading and writing its 150 KB of partial gradients,
 // fetching its 84 KB of weights and 128 instead of 256 threads in each
@@ -1033,6 +1033,20 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   const uint32_t tiles = uint32_t((n_x + MT - 1) / MT);
   const MlpPtrTc P = slot_ptrs_tc(a.m, p);
   float* gbase = a.part + uint64_t(blockIdx.x) * a.n_params;
+  // The next tile's row: the first while the weights come in, the others while
+  // the tile before them runs.  The first half alone takes the cotangents: from
+  // the statistics that is an FP64 division per row, 1 us of a tile's on this
+  // GPU when both halves do it.
+  uint64_t nx = 0;
+  float2 ncot = make_float2(0.f, 0.f);
+  auto load_row = [&](uint32_t tile) {
+    const uint64_t row = uint64_t(tile) * MT + t;
+    const bool in = tile < tiles && row < n_x;
+    nx = in ? a.xs[row] : 0ull;
+    ncot = make_float2(0.f, 0.f);
+    if (in && h == 0) cot_of(a.cot, row, ncot.x, ncot.y);
+  };
+  load_row(blockIdx.x);
   bool ok = __syncthreads_and(wait_bar(bar_w, 0));
   uint32_t ph = 0;
   auto mma_wait = [&]() -> bool {
@@ -1129,12 +1143,13 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
 
   uint32_t in_tmem = 0;  // tiles summed in tensor memory
   for (uint32_t tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
-    const uint64_t row = uint64_t(tile) * MT + t;
-    const bool valid = row < n_x;
-    const uint64_t x = valid ? a.xs[row] : 0ull;
-    float cla = 0.f, cph = 0.f;
-    if (valid) cot_of(a.cot, row, cla, cph);
-    const int e2 = scale_exponent(fmaxf(fabsf(cla), fabsf(cph)), e_sum);
+    const bool valid = uint64_t(tile) * MT + t < n_x;
+    const uint64_t x = nx;
+    float2* s_cot = reinterpret_cast<float2*>(DO);  // free until this tile's dout
+    if (h == 0) s_cot[t] = ncot;
+    const int e2 = scale_exponent(fmaxf(fabsf(ncot.x), fabsf(ncot.y)), e_sum);
+    const float cla = s_cot[t].x, cph = s_cot[t].y;  // written before the barrier in scale_exponent
+    load_row(tile + gridDim.x);
     if (in_tmem && abs(e2 - e_sum) > 64) {  // beyond what the sums can follow exactly
       flush();
       in_tmem = 0;
