@@ -315,7 +315,7 @@ TRAFFIC = {("h2o", "bf16"): {"mlp_tc_slot_kernel": 663808, "mlp_tc_grad_kernel":
 
 # kernel families that evaluate the connected determinants' amplitudes, in
 # order of preference for the headline roofline
-AMPLITUDE_FAMILIES = ("mlp_tc_suffix_kernel", "tf_tc_suffix_kernel", "nade_suffix_kernel", "tf_fp32_kernel")
+AMPLITUDE_FAMILIES = ("mlp_tc_amplitude_kernels", "tf_tc_amplitude_kernels", "nade_amplitude_kernels", "tf_fp32_kernel")
 
 
 def _make_model(A, w, params, form):
@@ -716,7 +716,7 @@ def _batch32(args, dev, quick=False):
             flop = 0.0
             for sp, pr in zip(specs, probs):
                 nu = int(pr.nu.item())
-                flop += _tc_work(A, pr.ham, pr.model, sp, pr.x[:nu].contiguous())["mlp_tc_suffix_kernel"]
+                flop += _tc_work(A, pr.ham, pr.model, sp, pr.x[:nu].contiguous())["mlp_tc_amplitude_kernels"]
             peaks, src = _peaks()
             best = min(t)
             ach = flop / (best / 1e3) / 1e12
@@ -979,8 +979,8 @@ def _tf_work(A, ham, w, x):
     out = {"tf_tc_parent_kernel": parent, "tf_tc_slot_kernel": slot, "tf_fp32_grad_kernels": 3.0 * parent}
     if n <= INDEX_MAX_ORB:
         full = _distinct_prefixes(A, ham, x)[n] * cf[n]
-        return dict(out, tf_tc_suffix_kernel=full, tf_fp32_kernel=full + slot,
-                    eloc_assemble_kernel=_eloc_bytes(len(x), ham.n_connected))
+        return dict(out, tf_tc_amplitude_kernels=full, tf_fp32_kernel=full + slot,
+                    eloc_kernels=_eloc_bytes(len(x), ham.n_connected))
     nodes = np.zeros(n)  # each sample's own distinct prefixes
     for xi, xp in zip(x, A.connected(ham, x)[0]):
         u = torch.cat([xi[None], xp])
@@ -988,8 +988,8 @@ def _tf_work(A, ham, w, x):
             u = torch.unique(u & ((1 << (2 * p)) - 1))
             nodes[p] += u.numel()
     m = len(x) * ham.n_connected
-    return dict(out, tf_tc_suffix_kernel=float((nodes * f).sum()), tf_fp32_kernel=m * cf[n] + parent + slot,
-                eloc_assemble_kernel=_eloc_bytes(len(x), ham.n_connected),
+    return dict(out, tf_tc_amplitude_kernels=float((nodes * f).sum()), tf_fp32_kernel=m * cf[n] + parent + slot,
+                eloc_kernels=_eloc_bytes(len(x), ham.n_connected),
                 connected_kernel=float(m * (8 + 8 + 1) + len(x) * 8))
 
 
@@ -1016,8 +1016,8 @@ def _tc_work(A, ham, model, w, x):
         slot += len(pre) * f[p]
     out = {"mlp_tc_slot_kernel": slot, "mlp_fp32_grad_kernel": 3.0 * parent, "mlp_tc_grad_kernel": 3.0 * parent}
     if n <= INDEX_MAX_ORB:
-        out["mlp_tc_suffix_kernel"] = float((_distinct_prefixes(A, ham, x)[:n] * f).sum())
-        out["eloc_assemble_kernel"] = _eloc_bytes(len(x), ham.n_connected)
+        out["mlp_tc_amplitude_kernels"] = float((_distinct_prefixes(A, ham, x)[:n] * f).sum())
+        out["eloc_kernels"] = _eloc_bytes(len(x), ham.n_connected)
     return out
 
 
@@ -1040,7 +1040,7 @@ def _nade_work(A, ham, w, x):
     for p in range(n):
         pre = np.unique(xs & np.uint64((1 << (2 * p)) - 1)) if p else np.zeros(1, np.uint64)
         samp += len(pre) * slot[p]
-    return {"nade_parent_kernel": len(xs) * slot.sum(), "nade_suffix_kernel": float((_distinct_prefixes(A, ham, x)[1:] * path).sum()),
+    return {"nade_parent_kernel": len(xs) * slot.sum(), "nade_amplitude_kernels": float((_distinct_prefixes(A, ham, x)[1:] * path).sum()),
             "nade_slot_kernel": samp, "nade_grad_kernel": 3.0 * len(xs) * f.sum()}
 
 

@@ -26,7 +26,6 @@ enum ProfId {
   PROF_MLP_FP32_SLOT,
   PROF_MLP_FP32_GRAD,
   PROF_TABLE,
-  PROF_ELOC_SUM,
   PROF_STATS,
   PROF_COTANGENT,
   PROF_SAMPLER,
@@ -38,7 +37,6 @@ enum ProfId {
   PROF_TF,
   PROF_TC_FINALIZE,
   PROF_GRAD_REDUCE,
-  PROF_SAMPLER_NET_FP32,
   PROF_TF_GRAD,
   PROF_TF_TC_PARENT,
   PROF_TF_TC_SUFFIX,

@@ -11,7 +11,7 @@
 namespace anqs {
 
 constexpr int MAXS = 256;  // singles of one spin: at most 16 x 16
-constexpr int MAXP = 512;  // pairs of a list: at most C(31, 2) = 465
+constexpr int MAXP = 512;  // pairs of a list: at most C(32, 2) = 496 (a spin without electrons)
 
 // Per-sample tables in shared memory.  A single (i, a) of spin s has index
 // r_i * n_virt + r_a in the order of the occupied and virtual lists.
@@ -28,8 +28,10 @@ struct Exc {
   uint32_t own[2];        // rank(alpha) * nb_p[n], rank(beta)
 };
 
-// q = v / d for v < 2^24, d <= 512 by multiplication with ceil(2^32 / d): the
-// product's excess over v / d is below v / 2^32 * 1 < 1 / d.
+// q = v / d for v d <= 2^32 by multiplication with ceil(2^32 / d): the product's
+// excess over v / d is v e / (2^32 d) with e < d, below 1 / d.  The largest here:
+// pairs of pairs, v < 120^2, d <= 496; singles of both spins, v < 2^16, d <= 256;
+// excitations and row variants, v < 2^17, d <= 32.
 struct FastDiv {
   uint32_t d, m;
 };

@@ -26,13 +26,13 @@ uint64_t g_count[PROF_COUNT];
 
 const char* kNames[PROF_COUNT] = {
     "connected_kernel",       "diagonal_kernel",      "mlp_fp32_logpsi_kernel", "mlp_fp32_slot_logits_kernel",
-    "mlp_fp32_grad_kernel",   "table_kernels",        "eloc_sum_kernel",        "stats_kernel",
-    "cotangent_kernel",       "sampler_draw_kernels", "mlp_tc_parent_kernel",   "mlp_tc_suffix_kernel",
-    "tc_sort_kernels",        "eloc_assemble_kernel", "mlp_tc_slot_kernel",     "tf_fp32_kernel",
-    "finalize_kernel",        "grad_partial_sum_kernel", "unused",              "tf_fp32_grad_kernels",
-    "tf_tc_parent_kernel",    "tf_tc_suffix_kernel",  "tf_tc_slot_kernel",
-    "nade_logpsi_kernel", "nade_grad_kernel", "nade_slot_kernel",
-    "nade_parent_kernel",    "nade_suffix_kernel",   "mlp_tc_grad_kernel"};
+    "mlp_fp32_grad_kernel",   "table_kernels",        "stats_kernel",           "cotangent_kernel",
+    "sampler_draw_kernels",   "mlp_tc_parent_kernel", "mlp_tc_amplitude_kernels",  // over prefixes or suffixes
+    "tc_sort_kernels",        "eloc_kernels",         "mlp_tc_slot_kernel",     "tf_fp32_kernel",
+    "finalize_kernel",        "grad_partial_sum_kernel", "tf_fp32_grad_kernels", "tf_tc_parent_kernel",
+    "tf_tc_amplitude_kernels",  // over determinants, prefixes or suffixes
+    "tf_tc_slot_kernel",      "nade_logpsi_kernel",   "nade_grad_kernel",       "nade_slot_kernel",
+    "nade_parent_kernel",     "nade_amplitude_kernels", "mlp_tc_grad_kernel"};
 
 cudaEvent_t get_event() {
   if (!g_pool.empty()) {

@@ -323,7 +323,7 @@ def test_transformer_forms_without_an_index(A, n, na, nb, m, d):
     small = m * (29 * ham.n_connected + 16 + n * (32 + 40 + 4 * blocks * d)) + 8192
     for ws, launches in ((need, n if d == 128 else None), (small, 1)):
         buf = torch.empty(ws, dtype=torch.uint8, device="cuda")
-        _, ran = _launches(A, "tf_tc_suffix_kernel", lambda: _agrees(A, model, ham, x, e, bound, workspace=buf))
+        _, ran = _launches(A, "tf_tc_amplitude_kernels", lambda: _agrees(A, model, ham, x, e, bound, workspace=buf))
         assert launches is None or ran == launches, (ws, ran)
     with pytest.raises(A.AnqsError):
         A.local_energy(model, ham, x, workspace=buf[:small // 2])
