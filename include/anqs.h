@@ -90,13 +90,14 @@ enum {
 enum { ANQS_MODEL_MLP = 0, ANQS_MODEL_TF = 1, ANQS_MODEL_TABLE = 2, ANQS_MODEL_NADE = 3 };
 
 /* Arithmetic form of a model's network evaluation.
- * FP32: plain SIMT float32 kernels, every configuration evaluated over all
- *       slots (no prefix reuse), except the NADE, whose local energy reuses
- *       the parent's slots for its connected determinants.
+ * FP32: plain SIMT float32 kernels.  A local energy evaluates each distinct
+ *       connected determinant once where that takes less than one by one (the
+ *       MLP and the NADE each distinct prefix); the results are the same bits.
  * BF16: the 16-bit form: tensor-core (tcgen05, TMEM accumulators) 16-bit
  *       GEMMs with float32 accumulation, float32 activations/softmax/phase
- *       heads, and reuse of the parent determinant's slots for its connected
- *       determinants.  GEMM operands are fp16, the same MMA instruction and
+ *       heads.  A local energy shares prefixes: among the samples' distinct
+ *       connected determinants, within each sample's, or with few samples
+ *       between a connected determinant and its parent.  GEMM operands are fp16, the same MMA instruction and
  *       rate as bfloat16 with three more significand bits (the bf16 rounding
  *       of activations put the gradient's error above 1e-3 relative L2):
  *       the MLP's weights (layer 1 as two fp16 parts) and tanh activations,
@@ -355,7 +356,12 @@ ANQS_API int anqs_test_sampler_barrier(unsigned extra_arrivals, uint64_t limit_n
  * If counts_dev is not NULL, stats_dev receives 4 doubles
  *   (Re E, Im E, Var, S) with S = sum_l n_l, E = sum_l n_l eloc_l / S,
  *   Var = sum_l n_l |eloc_l - E|^2 / S.
- * n_x >= 1.  Workspace from anqs_local_energy_workspace_size(n_x).
+ * n_x >= 1.  Workspace from anqs_local_energy_workspace_size(n_x): that of
+ * the form which takes the least time for n_x samples (a 16-bit transformer
+ * keeps up to about 8 GiB of keys and values).  A smaller one, or one sized for
+ * more samples, runs another form that it holds; the smallest is 24 to 29 bytes
+ * per connected determinant and the samples' own outputs (16-bit MLP and NADE
+ * also 8 n_orb bytes per connected determinant).  ANQS_ERR_CAPACITY below that.
  * Row count on the device: when n_x_dev is not NULL, only the first *n_x_dev
  * rows (read on the device, at most n_x) are processed and n_x is the
  * capacity that sizes launches and the workspace; e.g. pass the sampler's
@@ -363,8 +369,8 @@ ANQS_API int anqs_test_sampler_barrier(unsigned extra_arrivals, uint64_t limit_n
  * in one CUDA graph.  Outputs beyond *n_x_dev are left untouched.
  * The statistics are reduced in a fixed order (deterministic), in one pass
  * shifted by eloc_0 (equal to the two-pass form up to rounding).
- * The 16-bit MLP form runs part of the call on a second stream owned by the
- * model, forked from `stream` and joined back into it with events: the call
+ * With few samples or without a prefix index the 16-bit MLP form runs part of
+ * the call on a second stream owned by the model, forked from `stream` and joined back into it with events: the call
  * still orders with the work queued on `stream` and can be captured in a
  * CUDA graph, but one model must not be used by several host threads at once.
  * ------------------------------------------------------------------------- */
