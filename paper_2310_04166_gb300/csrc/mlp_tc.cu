@@ -984,7 +984,10 @@ __host__ __device__ constexpr uint32_t idesc_f16_mn(int M, int N, bool a_mn, boo
 
 constexpr int GNT = 2 * MT;
 
-template <int W>
+// MULTI: several tiles per CTA, summed in tensor memory.  A form of its own,
+// because a short call with a cold cache waits for its instructions too: with
+// the sums' code in its way the 14-qubit call's kernel took 35 us, without 29.
+template <int W, bool MULTI>
 __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_constant__ GradArgs a) {
   static_assert(W == 128, "the weight GEMMs put the layer width on the MMA's M = 128");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -1033,21 +1036,7 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   const uint32_t tiles = uint32_t((n_x + MT - 1) / MT);
   const MlpPtrTc P = slot_ptrs_tc(a.m, p);
   float* gbase = a.part + uint64_t(blockIdx.x) * a.n_params;
-  // The next tile's row: the first while the weights come in, the others while
-  // the tile before them runs.  The first half alone takes the cotangents: from
-  // the statistics that is an FP64 division per row, 1 us of a tile's on this
-  // GPU when both halves do it.
-  uint64_t nx = 0;
-  float2 ncot = make_float2(0.f, 0.f);
-  auto load_row = [&](uint32_t tile) {
-    const uint64_t row = uint64_t(tile) * MT + t;
-    const bool in = tile < tiles && row < n_x;
-    nx = in ? a.xs[row] : 0ull;
-    ncot = make_float2(0.f, 0.f);
-    if (in && h == 0) cot_of(a.cot, row, ncot.x, ncot.y);
-  };
-  load_row(blockIdx.x);
-  bool ok = __syncthreads_and(wait_bar(bar_w, 0));
+  bool ok = true;
   uint32_t ph = 0;
   auto mma_wait = [&]() -> bool {
     const bool r = __syncthreads_and(wait_bar(bar_m, ph));
@@ -1085,7 +1074,7 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   // each warp's access covers 32 consecutive columns of one row.  The halves
   // take alternate chunks.
   uint32_t flushes = 0;
-  auto put = [&](float* d, float v) { *d = flushes ? *d + v * inv_sc : v * inv_sc; };
+  auto put = [&](float* d, float v) { *d = MULTI && flushes ? *d + v * inv_sc : v * inv_sc; };
   auto flush = [&]() {
     float* stage = reinterpret_cast<float*>(h ? P2 : P1);  // [128][33]
     for (int k = 1; k <= L; ++k) {
@@ -1142,23 +1131,35 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
   };
 
   uint32_t in_tmem = 0;  // tiles summed in tensor memory
-  for (uint32_t tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
-    const bool valid = uint64_t(tile) * MT + t < n_x;
-    const uint64_t x = nx;
+  for (uint32_t tile = blockIdx.x;; tile += gridDim.x) {
+    const bool end = tile >= tiles;
+    const uint64_t row = uint64_t(tile) * MT + t;
+    const bool valid = !end && row < n_x;
+    const uint64_t x = valid ? a.xs[row] : 0ull;
+    // The first half takes the cotangents and hands them over: from the
+    // statistics that is an FP64 division per row.
+    float2 cot = make_float2(0.f, 0.f);
+    if (valid && h == 0) cot_of(a.cot, row, cot.x, cot.y);
+    if (tile == blockIdx.x) ok = __syncthreads_and(wait_bar(bar_w, 0));
+    if (!ok) break;
     float2* s_cot = reinterpret_cast<float2*>(DO);  // free until this tile's dout
-    if (h == 0) s_cot[t] = ncot;
-    const int e2 = scale_exponent(fmaxf(fabsf(ncot.x), fabsf(ncot.y)), e_sum);
-    const float cla = s_cot[t].x, cph = s_cot[t].y;  // written before the barrier in scale_exponent
-    load_row(tile + gridDim.x);
-    if (in_tmem && abs(e2 - e_sum) > 64) {  // beyond what the sums can follow exactly
+    int e2 = e_sum;
+    if (!end) {
+      if (h == 0) s_cot[t] = cot;
+      e2 = scale_exponent(fmaxf(fabsf(cot.x), fabsf(cot.y)), e_sum);
+    }
+    // beyond a quotient of 2^64 the sums cannot follow exactly
+    if (in_tmem && (end || (MULTI && (in_tmem == kFlush || abs(e2 - e_sum) > 64)))) {
       flush();
       in_tmem = 0;
     }
-    const float follow = in_tmem ? ldexpf(1.f, e2 - e_sum) : 1.f;
+    if (end) break;
+    const float cla = s_cot[t].x, cph = s_cot[t].y;  // written before the barrier in scale_exponent
+    const float follow = MULTI && in_tmem ? ldexpf(1.f, e2 - e_sum) : 1.f;
     e_sum = e2;
     sc = ldexpf(1.f, e2);
     inv_sc = ldexpf(1.f, -e2);
-    const uint32_t acc = in_tmem ? 1u : 0u;
+    const uint32_t acc = MULTI && in_tmem ? 1u : 0u;
     // the sums to this tile's scale; every MMA on them is done, and the next ones come after a barrier
     auto rescale = [&]() {
       __syncwarp();
@@ -1192,7 +1193,7 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
           tc::mma_commit(bar_m);
         }
       }
-      if (layer == 0 && follow != 1.f) rescale();
+      if (MULTI && layer == 0 && follow != 1.f) rescale();
       if (K > 0) ok = mma_wait();
       if (!ok || layer == L - 1) break;
       unsigned char* dst = Hb + uint32_t(layer) * TILE;
@@ -1387,10 +1388,7 @@ __global__ void __launch_bounds__(GNT, 1) mlp_tc_grad_kernel(const __grid_consta
       Zn = tmp;
     }
     if (!ok) break;
-    if (++in_tmem == kFlush || tile + gridDim.x >= tiles) {
-      flush();
-      in_tmem = 0;
-    }
+    ++in_tmem;
   }
   if (!ok && threadIdx.x == 0) atomicExch(a.tv.status, ST_TIMEOUT);
   tc::fence_before_sync();
@@ -2116,11 +2114,11 @@ int launch_mlp_tc_grad(const anqs_model* M, const HamView& hv, const uint64_t* x
     ANQS_TRY(launch_grad_cotangents(cot.ere, cot.eim, cot.counts, cot.stats, n_x, cl, cp, s));
     a.cot = CotSrc{cl, cp, nullptr, nullptr, nullptr, nullptr};
   }
-  ANQS_CUDA(cudaFuncSetAttribute(mlp_tc_grad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
+  const auto kern = tiles > slabs ? mlp_tc_grad_kernel<128, true> : mlp_tc_grad_kernel<128, false>;
+  ANQS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm)));
   {
     ProfScope ps(PROF_MLP_TC_GRAD, s);
-    ANQS_CUDA_LAUNCH("mlp_tc_grad_kernel", launch_k(mlp_tc_grad_kernel<128>, dim3(slabs, unsigned(M->d.n_orb)),
-                                                    dim3(GNT), sm, s, a));
+    ANQS_CUDA_LAUNCH("mlp_tc_grad_kernel", launch_k(kern, dim3(slabs, unsigned(M->d.n_orb)), dim3(GNT), sm, s, a));
   }
   return launch_grad_partial_sum(part, n_x, a.n_params, MT, slabs, grad, s);
 }
