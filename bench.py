@@ -479,9 +479,11 @@ def _run_form(A, lib, args, w, form, ham, params, dev, rank, dist, stream_clocks
 
 
 def _oracle_model(w):
-    from oracle.anqs import MLPAnsatz, TFAnsatz
+    from oracle.anqs import MLPAnsatz, NADEAnsatz, TFAnsatz
     from oracle.sector import molecular_isphys
     ip = molecular_isphys(w["n"], w["n_alpha"], w["n_beta"])
+    if w["kind"] == "nade":
+        return NADEAnsatz(w["params_struct"], w["n"], ip), ip
     om = MLPAnsatz(w["params_struct"], w["n"]) if w["kind"] == "mlp" else TFAnsatz(w["params_struct"], w["n"],
                                                                                     w["n_heads"])
     return om, ip
@@ -499,7 +501,10 @@ def _grad_vs_oracle(A, model, ham, w, x, cnt, e_ref):
     g = A.grad(model, ham, x, c, ere, eim, st).cpu().numpy().astype(np.float64)
     xs = x.cpu().numpy().astype(np.uint64)
     s_ref = energy_stats(e_ref, cnt)
-    g_ref = np.concatenate([t.reshape(-1).numpy() for t in gradient(om, ip, xs, cnt, e_ref, s_ref)])
+    parts = [t.numpy() for t in gradient(om, ip, xs, cnt, e_ref, s_ref)]
+    if w["kind"] == "nade":  # (re, im) interleaved in the flat layout
+        parts = [np.stack(p, axis=-1) for p in zip(parts[0::2], parts[1::2])]
+    g_ref = np.concatenate([p.reshape(-1) for p in parts])
     return float(np.linalg.norm(g - g_ref) / np.linalg.norm(g_ref))
 
 
