@@ -283,6 +283,7 @@ struct NodeView {
   const uint64_t* x;    // [nodes] prefix bits
   const uint32_t* off;  // [n + 2], device
   const uint2* packed;
+  uint32_t cover;       // connected determinants per determinant of the sector from which all are nodes (covers_sector)
 };
 #ifdef __CUDACC__
 // even bits of x, packed

@@ -67,19 +67,27 @@ __device__ __forceinline__ void mark_det(const HamView& hv, const SectorView& sv
 // connected one (6.6e6 of a 14,400-determinant sector: 126 us).  From the
 // device's count: a buffer may hold fewer samples than it has room for.
 // Not with Z2 symmetries, where the index also holds other sectors' prefixes.
-__device__ __forceinline__ bool covers_sector(const HamView& hv, const SectorView& sv, uint64_t n_x) {
-  return hv.nz == 0 && n_x * uint64_t(hv.K) >= 4ull * sv.na_p[sv.n] * sv.nb_p[sv.n];
+// How often (cover) depends on what a determinant costs the network: the sets
+// of samples that follow its distribution leave a third of the sector out at
+// four connected determinants per one, a tenth at twelve.  16-bit MLP, 12
+// orbitals, 5 + 5 electrons (us, all and marked): 274 and 202 at 1.5 per one,
+// 284 and 304 at 4, 337 and 439 at 12; FP32 MLP 5,990 and 3,870 at 4, 6,050
+// and 5,330 at 12, where marking takes 100.
+constexpr uint32_t kCover = 32;  // 16-bit MLP: kCoverMlpTc
+__device__ __forceinline__ bool covers_sector(const HamView& hv, const SectorView& sv, uint32_t cover, uint64_t n_x) {
+  return hv.nz == 0 && n_x * uint64_t(hv.K) >= uint64_t(cover) * sv.na_p[sv.n] * sv.nb_p[sv.n];
 }
 
 constexpr int MT_ = 128;
 
 __global__ void __launch_bounds__(MT_) mark_kernel(HamView hv, SectorView sv, const uint64_t* __restrict__ xs,
-                                                   Count n_x_, int splits, uint32_t* __restrict__ bits, int levels) {
+                                                   Count n_x_, int splits, uint32_t* __restrict__ bits, int levels,
+                                                   uint32_t cover) {
   ANQS_PDL_ENTRY();
   __shared__ Exc E;
   const uint64_t items = n_x_.get() * uint64_t(splits);
   const uint32_t K = hv.K;
-  if (covers_sector(hv, sv, n_x_.get())) {
+  if (covers_sector(hv, sv, cover, n_x_.get())) {
     for (int p = levels ? 0 : sv.n; p <= sv.n; ++p) {
       const uint32_t all = sv.na_p[p] * sv.nb_p[p], words = (all + 31u) / 32u;
       for (uint32_t w = blockIdx.x * MT_ + threadIdx.x; w < words; w += gridDim.x * MT_)
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(ET) eloc_direct_kernel(HamView hv, SectorView 
   const FastDiv dvar = fast_div(var);
   uint32_t leaf0 = 0;
   if constexpr (RANK) leaf0 = __ldcg(nv.off + n);
-  const bool all = !nv.packed || covers_sector(hv, sv, n_x);  // every determinant of the sector has a row
+  const bool all = !nv.packed || covers_sector(hv, sv, nv.cover, n_x);  // every determinant of the sector has a row
   // row of determinant index idx in the amplitude tables; false if it is not there
   auto leaf = [&](uint32_t idx, uint32_t& r) -> bool {
     if (all) {
@@ -777,7 +785,7 @@ void plan_unique(const anqs_ham* H, uint64_t n_x, bool levels, Arena& A, UniqueW
   w.node_x = A.take<uint64_t>(w.max_nodes);
   w.leaf_x = w.node_x;  // without levels, the determinants are the only nodes
   w.off = A.take<uint32_t>(n + 2);
-  w.nodes = w.full ? NodeView{H->d_full_x, H->d_full_off, nullptr} : NodeView{w.node_x, w.off, w.packed};
+  w.nodes = w.full ? NodeView{H->d_full_x, H->d_full_off, nullptr, kCover} : NodeView{w.node_x, w.off, w.packed, kCover};
 }
 
 int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueWs& w, cudaStream_t s) {
@@ -787,7 +795,7 @@ int launch_unique(const anqs_ham* H, const uint64_t* x, Count n_x, const UniqueW
   {
     ProfScope ps(PROF_CONNECT, s);
     const unsigned grid = unsigned(std::min<uint64_t>(n_x.n * splits, 152 * 12));
-    ANQS_CUDA_LAUNCH("mark_kernel", launch_k(mark_kernel, dim3(grid), dim3(MT_), 0, s, H->v, H->sv, x, n_x, splits, w.bits, w.levels ? 1 : 0));
+    ANQS_CUDA_LAUNCH("mark_kernel", launch_k(mark_kernel, dim3(grid), dim3(MT_), 0, s, H->v, H->sv, x, n_x, splits, w.bits, w.levels ? 1 : 0, w.nodes.cover));
   }
   ProfScope ps(PROF_TC_SORT, s);
   const uint32_t words = uint32_t(index_words(H)), cw = words_per_cta(words);
@@ -841,7 +849,7 @@ void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w) {
   w.bsum = A.take<uint32_t>((words + words_per_cta(uint32_t(words)) - 1) / words_per_cta(uint32_t(words)));
   w.node_x = A.take<uint64_t>(w.max_rows);
   w.off = A.take<uint32_t>(n + 1);
-  w.nodes = NodeView{w.node_x, w.off, w.packed};
+  w.nodes = NodeView{w.node_x, w.off, w.packed, kCover};
 }
 
 int launch_tree(const anqs_ham* H, const uint64_t* x, Count n_x, const TreeWs& w, cudaStream_t s) {

@@ -1774,6 +1774,7 @@ size_t plan_eloc(const anqs_ham* H, uint64_t n_x, Arena& A, ElocWs& w) {
 }
 
 // Scratch of the form over distinct prefixes (eloc_unique.cu)
+constexpr uint32_t kCoverMlpTc = 4;  // NodeView::cover
 struct NodeWs {
   UniqueWs u;
   float2 *terms, *mid, *sums;
@@ -1781,6 +1782,7 @@ struct NodeWs {
 
 size_t plan_nodes(const anqs_ham* H, uint64_t n_x, Arena& A, NodeWs& w) {
   plan_unique(H, n_x, true, A, w.u);
+  w.u.nodes.cover = kCoverMlpTc;
   w.terms = A.take<float2>((w.u.max_nodes - w.u.max_leaves) * 4);
   w.mid = A.take<float2>(path_sums_mid(H, n_x));
   w.sums = A.take<float2>(w.u.max_leaves);

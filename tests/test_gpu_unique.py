@@ -405,3 +405,16 @@ def test_transformer_leaves_in_chunks(A):
     _agrees(A, model, ham, x, e, bound)
     ere, eim, _ = A.local_energy(model, ham, x, n_dev=torch.tensor([30], dtype=torch.int64, device="cuda"))
     assert torch.all((ere[:30] - e.real[:30]).abs() <= bound[:30]) and torch.all((eim[:30] - e.imag[:30]).abs() <= bound[:30])
+
+
+@pytest.mark.parametrize("kind,form", [("mlp", "bf16"), ("nade", "fp32"), ("tf", "bf16")])
+@pytest.mark.parametrize("n,na,nb,m", [(11, 4, 5, 560), (11, 4, 5, 500), (9, 4, 5, 1100)])
+def test_reuse_forms_that_cover_the_sector(A, kind, form, n, na, nb, m):
+    """Just above and below four connected determinants per determinant of the sector, and above 32: every bit set
+    without looking, or marked; then room for as many samples with nine there."""
+    model, ham = _problem(A, kind, form, n, na, nb, 80 + n)
+    x = _dets(n, na, nb, m, n)
+    e, bound = _reference(A, model, ham, x)
+    _agrees(A, model, ham, x, e, bound)
+    ere, eim, _ = A.local_energy(model, ham, x, n_dev=torch.tensor([9], dtype=torch.int64, device="cuda"))
+    assert torch.all((ere[:9] - e.real[:9]).abs() <= bound[:9]) and torch.all((eim[:9] - e.imag[:9]).abs() <= bound[:9])
