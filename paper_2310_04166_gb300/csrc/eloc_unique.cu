@@ -728,12 +728,21 @@ int split_of(uint64_t n_x, uint32_t K) {
 uint64_t index_words(const anqs_ham* H) { return H->sv.woff[H->sv.n + 1]; }
 
 // every prefix of a small sector is evaluated when the call's connected
-// determinants outnumber the sector's at least fourfold
+// determinants outnumber the sector's at least fourfold.  Below that it is the
+// better form too where it was measured (7 orbitals, 5 + 5 electrons, half a
+// connected determinant per determinant: 16-bit MLP 39 us against 69 marked,
+// FP32 MLP 57 against 91, NADE 52 against 77, transformer 66 against 81); the
+// line keeps a call of few samples from a sector's whole network work.
 bool use_full(const anqs_ham* H, uint64_t n_x) {
   return H->has_full && n_x * uint64_t(H->v.K) >= 4ull * H->sv.na_p[H->v.n] * H->sv.nb_p[H->v.n];
 }
 
-constexpr int kMidSlots = 3;  // last slots of a determinant's path summed from its level n - 3 prefix
+// The last slots of a determinant's path are summed from its level n - 3 prefix
+// where the extra launch pays.  Two steps against one, 16-bit MLP: 4,900
+// determinants 41 us against 38 (hence the 16,384), 63,504 94 against 90, 213,444
+// 140 against 142, 853,776 379 against 402; FP32 MLP (32 places): 63,504 645
+// against 696.
+constexpr int kMidSlots = 3;
 
 int mid_level(const anqs_ham* H, uint64_t leaves) {
   return H->v.n > 2 * kMidSlots && leaves > 16384 ? H->v.n - kMidSlots : 0;
@@ -747,7 +756,11 @@ uint64_t level_bound(const anqs_ham* H, uint64_t n_x, int p) {
 }  // namespace
 
 // The bitmap's fixed cost (zeroing, scanning: 20 bytes per word) against the
-// connected set's own (at least 29 bytes per determinant without it)
+// connected set's own (at least 29 bytes per determinant without it).  A line on
+// scratch before time.  Index against list, 16-bit MLP 3 x 128: 14 orbitals 7 + 7
+// (1.05 M words), 4 samples 99 us against 101, 64 samples 217 against 431; 16
+// orbitals 6 + 6 (5.93 M words), 4 samples (words = 292 m) 185 against 148, 16
+// samples (73 m) 255 against 274, 256 samples (4.6 m) 761 against 2,633.
 bool unique_applies(const anqs_ham* H, uint64_t n_x) {
   if (!H->has_index) return false;
   if (use_full(H, n_x)) return true;
@@ -833,7 +846,12 @@ bool use_unique(const anqs_ham* H, bool preferred, size_t plain, size_t unique, 
   return preferred ? unique <= ws_bytes || plain > ws_bytes : plain > ws_bytes && unique <= ws_bytes;
 }
 
-// the samples' prefixes; 2^21 bitmap words cost about 20 us to clear and scan
+// The samples' prefixes: what marking and listing them costs is repaid where
+// many samples share them.  Prefixes against rows, transformer d 64, 2 blocks, 14
+// orbitals 7 + 7: 1 sample 367 us against 295, 256 samples 508 against 451, 4,000
+// samples 1,163 against 1,816; 18 orbitals 6 + 6, far beyond the line: 681
+// against 301, 777 against 487, 1,828 against 2,383.  2^21 bitmap words cost
+// about 20 us to clear and scan.
 bool tree_applies(const anqs_ham* H) { return H->has_index && H->sv.woff[H->v.n] <= (1u << 21); }
 
 void plan_tree(const anqs_ham* H, uint64_t n_x, Arena& A, TreeWs& w) {
